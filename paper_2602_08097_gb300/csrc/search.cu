@@ -1,10 +1,14 @@
 // Batched GreedySearch (Algorithm 2) and k-recall@k (§4).
 //
-// One warp runs one query at a time; warps take queries from an atomic
-// counter.  The search list is kept sorted by (distance, id) in shared
-// memory, so "the closest unexpanded member" of Algorithm 2 is the first
-// member without its visited bit, and "retain the closest L" is a cut after
-// a merge.
+// Queries are taken from an atomic counter.  Two kernels hold the search list
+// differently:
+//   search_reg_kernel   L <= 256: the list lives in one warp's registers, sorted,
+//                       entry i in slot i % S of lane i / S.  Every entry sees
+//                       for itself whether it stays, moves up by one or makes
+//                       room for the new point, so adding a point takes two
+//                       shuffles and a few selects per slot.
+//   search_list_kernel  longer lists: in shared memory, sorted by (distance, id);
+//                       new points are sorted and merged 32 at a time.
 //
 // Algorithm 2 keeps a set: adding a point that is already in the list has
 // no effect.  A point that was in the list and was cut may be added again by
@@ -13,25 +17,30 @@
 // the point still lies behind it.  (An expanded point that is cut is the same
 // case: it comes back behind the L-th and is never the closest unexpanded
 // member.)  So the only membership test the search needs is "is v in the
-// list now?", which a binary search of the sorted list answers exactly at the
-// position where v would be merged.  A small direct-mapped cache of recently
-// met ids in shared memory skips most repeated distance computations; a miss
-// only costs one more distance, never a different result.
+// list now?".  A small direct-mapped cache of recently met ids in shared memory
+// skips most repeated distance computations; a miss only costs one more
+// distance, never a different result.
 //
-// Neighbours are added 32 at a time, each batch merged and cut to L before the
-// next; the L closest of a union are the L closest of the L closest of its
+// Neighbours are added one at a time or in batches, the list cut to L after
+// each; the L closest of a union are the L closest of the L closest of its
 // parts, so this equals adding the whole list and cutting once.
 //
-// Ordering: uint8 distances are exact integers.  float32 distances (summed
-// per 32-dimension slice) carry a rigorous single-precision error bound; when
-// two intervals overlap, both distances are recomputed in float-float
-// arithmetic (bound about d 2^-46 relative), and only if those intervals still
-// overlap in binary64 (index order, no fused multiply-add), so every
-// comparison agrees with the binary64 reading.
+// Distances (row_keys): 4, 8 or 32 lanes share a row (by its length), lane s of
+// G taking its 16-byte chunks s, s + G, ..., so that whole 32-byte sectors are
+// read and every load of a step is in flight at once.  Every kernel sums a
+// distance the same way, so a query's results do not depend on the kernel.
+//
+// Ordering: uint8 distances are exact integers.  float32 distances carry a
+// rigorous single-precision error bound (lane_rel_bound); when two intervals
+// overlap, both distances are recomputed in float-float arithmetic (bound about
+// d 2^-46 relative), and only if those intervals still overlap in binary64
+// (index order, no fused multiply-add), so every comparison agrees with the
+// binary64 reading.
 #include <cfloat>
 #include <map>
 #include <mutex>
 #include <tuple>
+#include <type_traits>
 
 #include "internal.h"
 
@@ -40,6 +49,7 @@ namespace rpk {
 namespace {
 
 constexpr int kWarps = 4;  // warps (queries in flight) per CTA
+constexpr int kTeam = 5;        // warps per query of the team form: the list's warp and four that read rows
 constexpr unsigned kVisited = 0x80000000u;
 constexpr unsigned kIdMask = 0x7fffffffu;
 
@@ -126,46 +136,128 @@ __device__ inline WarpSmem carve(unsigned char* base, int L, int64_t row_bytes, 
   return w;
 }
 
-// d2(q, v) in the search's working precision, as order-preserving bits.
-// uint8: d2 = |q|^2 + |x|^2 - 2 <q, x> from dp4a alone, `qn` = |q|^2 (an
-// identity of integers, exact in 32-bit modular arithmetic since d2 < 2^32).
+// Lanes that share a row of nch 16-byte chunks: 4 for rows of up to 384 bytes (a
+// step of eight rows then has at most six loads per lane), 8 up to 1 KB, else
+// the whole warp.
+__host__ __device__ constexpr int row_lanes(int nch) { return nch <= 24 ? 4 : nch <= 64 ? 8 : 32; }
+
+// Relative bound of a float distance as row_keys sums it: each term carries two
+// roundings of its difference, ceil(nch / G) fused adds into one of its lane's
+// four sums, two to join those and log2 G to join the lanes; six ulps more
+// cover the comparisons built on it.
+__device__ __forceinline__ float lane_rel_bound(int nch) {
+  const int G = row_lanes(nch);
+  return float((nch + G - 1) / G + 2 + (G == 4 ? 2 : G == 8 ? 3 : 5) + 8) * 5.9604645e-08f;
+}
+
+// What one lane has summed of a row's distance.  uint8: |x|^2 - 2 <q, x>,
+// exact in 32-bit modular arithmetic (d2 = |q|^2 + |x|^2 - 2 <q, x> < 2^32).
+// float: four sums of squared differences, one per component of a chunk.
 template <int DT>
-__device__ __forceinline__ unsigned dist_bits(const uint8_t* __restrict__ q, const uint8_t* __restrict__ x,
-                                              int64_t row_bytes, unsigned qn) {
-  const uint4* pq = reinterpret_cast<const uint4*>(q);
-  const uint4* px = reinterpret_cast<const uint4*>(x);
-  if constexpr (DT == kU8) {
-    unsigned dot = 0, xn = 0;
-    for (int64_t c = 0; c < row_bytes / 16; ++c) {
-      const uint4 a = pq[c], b = __ldg(px + c);
-      dot = __dp4a(a.x, b.x, dot);
-      dot = __dp4a(a.y, b.y, dot);
-      dot = __dp4a(a.z, b.z, dot);
-      dot = __dp4a(a.w, b.w, dot);
-      xn = __dp4a(b.x, b.x, xn);
-      xn = __dp4a(b.y, b.y, xn);
-      xn = __dp4a(b.z, b.z, xn);
-      xn = __dp4a(b.w, b.w, xn);
-    }
-    return qn + xn - 2u * dot;
-  } else {
-    // summed per 32-dimension slice (slice_rel_bound)
-    float acc = 0.f;
-    for (int64_t c0 = 0; c0 < row_bytes / 16; c0 += 8) {
-      float part = 0.f;
-      const int64_t c1 = c0 + 8 < row_bytes / 16 ? c0 + 8 : row_bytes / 16;
-      for (int64_t c = c0; c < c1; ++c) {
-        const uint4 a = pq[c], b = __ldg(px + c);
-        float t;
-        t = __uint_as_float(a.x) - __uint_as_float(b.x); part = fmaf(t, t, part);
-        t = __uint_as_float(a.y) - __uint_as_float(b.y); part = fmaf(t, t, part);
-        t = __uint_as_float(a.z) - __uint_as_float(b.z); part = fmaf(t, t, part);
-        t = __uint_as_float(a.w) - __uint_as_float(b.w); part = fmaf(t, t, part);
-      }
-      acc += part;
-    }
-    return __float_as_uint(acc);
+struct LaneSum;
+template <>
+struct LaneSum<kU8> {
+  unsigned dot = 0, xx = 0;
+  __device__ __forceinline__ void add(uint4 q, uint4 x) {
+    dot = __dp4a(q.x, x.x, dot);
+    dot = __dp4a(q.y, x.y, dot);
+    dot = __dp4a(q.z, x.z, dot);
+    dot = __dp4a(q.w, x.w, dot);
+    xx = __dp4a(x.x, x.x, xx);
+    xx = __dp4a(x.y, x.y, xx);
+    xx = __dp4a(x.z, x.z, xx);
+    xx = __dp4a(x.w, x.w, xx);
   }
+  template <int G>
+  __device__ __forceinline__ unsigned finish(unsigned qn) {  // over the G lanes of a row
+    unsigned v = xx - 2u * dot;
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return qn + v;
+  }
+};
+template <>
+struct LaneSum<kF32> {
+  float x = 0.f, y = 0.f, z = 0.f, w = 0.f;
+  __device__ __forceinline__ void add(uint4 q, uint4 b) {
+    float t;
+    t = __uint_as_float(q.x) - __uint_as_float(b.x); x = fmaf(t, t, x);
+    t = __uint_as_float(q.y) - __uint_as_float(b.y); y = fmaf(t, t, y);
+    t = __uint_as_float(q.z) - __uint_as_float(b.z); z = fmaf(t, t, z);
+    t = __uint_as_float(q.w) - __uint_as_float(b.w); w = fmaf(t, t, w);
+  }
+  template <int G>
+  __device__ __forceinline__ unsigned finish(unsigned) {
+    float v = (x + y) + (z + w);
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return __float_as_uint(v);
+  }
+};
+
+// Rows r, r + step, ... (U of them, those below nf) for each group of G lanes,
+// in blocks of KC chunks per lane; a block's loads are all issued before the
+// first is used.  Rows past nf repeat row nf - 1 and are not stored.  WHOLE:
+// nch = G KC, so that no load needs a test.
+template <int DT, int G, int KC, int U, bool WHOLE>
+__device__ __forceinline__ void row_keys_step(const uint8_t* __restrict__ X, int64_t row_bytes, int nch,
+                                              const uint8_t* q, const unsigned* cid, unsigned* ckey, int nf, int r,
+                                              int step, unsigned qn) {
+  const int sub = threadIdx.x & (G - 1);
+  const uint4* px[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    px[u] = reinterpret_cast<const uint4*>(X + int64_t(cid[min(r + u * step, nf - 1)]) * row_bytes) + sub;
+  const uint4* pq = reinterpret_cast<const uint4*>(q) + sub;
+  LaneSum<DT> a[U];
+  for (int c0 = 0; c0 < nch; c0 += G * KC) {
+    uint4 x[U][KC];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int c = 0; c < KC; ++c)
+        x[u][c] = WHOLE || sub + c0 + G * c < nch ? __ldg(px[u] + c0 + G * c) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int c = 0; c < KC; ++c) {
+      if (WHOLE || sub + c0 + G * c < nch) {
+        const uint4 qv = pq[c0 + G * c];
+#pragma unroll
+        for (int u = 0; u < U; ++u) a[u].add(qv, x[u][c]);
+      }
+    }
+    if (WHOLE) break;
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const unsigned k = a[u].template finish<G>(qn);
+    if (r + u * step < nf) ckey[r + u * step] = k;  // the same value from each of the G lanes
+  }
+}
+
+// d2(q, cid[r]) as order-preserving bits into ckey[r] for the rows r < nf that
+// fall to this warp, number `wi` of `nw` that share them.  All lanes of the
+// warp take part; cid, q and ckey are in shared memory.  W: the kernel's warps
+// per query (one: registers are short, so fewer loads at a time; 960-float rows,
+// 1,000 queries on teams of three: 4 loads per lane in flight 5.48 ms, 8 4.58 ms).
+template <int DT, int W>
+__device__ __forceinline__ void row_keys(const uint8_t* __restrict__ X, int64_t row_bytes, const uint8_t* q,
+                                         const unsigned* cid, unsigned* ckey, int nf, int wi, int nw, unsigned qn) {
+  const int lane = threadIdx.x & 31;
+  const int nch = int(row_bytes / 16);
+#define RP_ROWS(G, KC, U, WHOLE)                                  \
+  for (int b = (32 / G) * wi; b < nf; b += (32 / G) * U * nw)     \
+    row_keys_step<DT, G, KC, U, WHOLE>(X, row_bytes, nch, q, cid, ckey, nf, b + lane / G, (32 / G) * nw, qn)
+  if (nch <= 24) {  // row_lanes(nch) = 4: eight rows a step
+    if (nch == 8) RP_ROWS(4, 2, 2, true);
+    else if (nch == 24) RP_ROWS(4, 6, 1, true);
+    else if (nch == 16) RP_ROWS(4, 4, 1, true);
+    else RP_ROWS(4, 3, 1, false);
+  } else if (nch <= 64) {
+    RP_ROWS(8, 4, 1, false);
+  } else {
+    RP_ROWS(32, (W == 1 ? 4 : 8), (W == kTeam ? 2 : 1), false);
+  }
+#undef RP_ROWS
 }
 
 // Total order on (distance, id) entries.  For float data `d64a`/`d64b` point to
@@ -204,8 +296,11 @@ __device__ __forceinline__ bool entry_less(unsigned ka, unsigned ia, double* d64
   }
 }
 
+// The list in shared memory, for L > kRegL.  A batch of 32 neighbours: those
+// the id cache does not hold get their distances, those that enter the list
+// are sorted by a bitonic network and merged in place.
 template <int DT>
-__global__ void __launch_bounds__(kWarps * 32, 9) search_kernel(SearchArgs a) {
+__global__ void __launch_bounds__(kWarps * 32, 8) search_list_kernel(SearchArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool f32 = DT == kF32;
@@ -213,7 +308,7 @@ __global__ void __launch_bounds__(kWarps * 32, 9) search_kernel(SearchArgs a) {
                      a.cache_bits);
   const int cshift = 32 - a.cache_bits;
   const int centries = 1 << a.cache_bits;
-  const float E = slice_rel_bound(a.d), Eabs = abs_bound(a.d);
+  const float E = lane_rel_bound(int(a.row_bytes / 16)), Eabs = abs_bound(a.d);
   const double qnan = __longlong_as_double(0x7ff8000000000000ll);
 
   for (;;) {
@@ -254,11 +349,13 @@ __global__ void __launch_bounds__(kWarps * 32, 9) search_kernel(SearchArgs a) {
     int f = 0;  // the members before index f are all expanded
     if (lane == 0) {
       const unsigned s = unsigned(start);
-      keyc[0] = dist_bits<DT>(S.q, a.X + int64_t(s) * a.row_bytes, a.row_bytes, qn);
+      S.cid[0] = s;
       idc[0] = s;
       if (f32) dc[0] = qnan;
       S.cache[(s * 0x9E3779B1u) >> cshift] = s;
     }
+    __syncwarp();
+    row_keys<DT, 1>(a.X, a.row_bytes, S.q, S.cid, keyc, 1, 0, 1, qn);
     __syncwarp();
 
     int64_t iters = 0;
@@ -306,9 +403,15 @@ __global__ void __launch_bounds__(kWarps * 32, 9) search_kernel(SearchArgs a) {
           fresh = S.cache[h] != v;
           if (fresh) S.cache[h] = v;
         }
-        if (!__any_sync(0xffffffffu, fresh)) continue;
-        unsigned kv = 0xffffffffu;
-        if (fresh) kv = dist_bits<DT>(S.q, a.X + int64_t(v) * a.row_bytes, a.row_bytes, qn);
+        const unsigned frm = __ballot_sync(0xffffffffu, fresh);
+        if (!frm) continue;
+        const int fr = __popc(frm & ((1u << lane) - 1u));
+        if (fresh) S.cid[fr] = v;
+        __syncwarp();
+        row_keys<DT, 1>(a.X, a.row_bytes, S.q, S.cid, S.ckey, __popc(frm), 0, 1, qn);
+        __syncwarp();
+        const unsigned kv = fresh ? S.ckey[fr] : 0xffffffffu;
+        __syncwarp();
         // A full list keeps only entries before its L-th: a point behind it
         // would be cut right after the merge, so it skips the merge.
         bool enters = fresh;
@@ -465,6 +568,452 @@ __global__ void __launch_bounds__(kWarps * 32, 9) search_kernel(SearchArgs a) {
   }
 }
 
+// ---------------------------------------------------------------------------
+// the list in registers
+// ---------------------------------------------------------------------------
+constexpr int kRegL = 256;      // longest list of search_reg_kernel
+constexpr int kNbr = 64;        // neighbours taken at a time
+constexpr int kTeamQueriesPerSm = 3;
+constexpr int kSmallTeam = 3;   // the same with two that read rows
+constexpr int kSmallTeamCtas = 7;
+constexpr int kSmallTeamQueriesPerSm = 8;
+constexpr unsigned kEmptyId = 0xffffffffu;  // an empty slot: expanded, no point has its id
+
+struct RegSmem {
+  unsigned* cache;
+  uint8_t* q;
+  unsigned* cid;   // [kNbr] new ids
+  unsigned* ckey;  // [kNbr] their distances
+  int* ctl;        // team form: rows to read (-1: the query is done); [1] the query
+};
+
+__host__ __device__ inline size_t reg_bytes(int64_t row_bytes, int cache_bits) {
+  return ((size_t(4) << cache_bits) + size_t(row_bytes) + size_t(2 * kNbr) * 4 + 16 + 127) & ~size_t(127);
+}
+__device__ inline RegSmem reg_carve(unsigned char* p, int64_t row_bytes, int cache_bits) {
+  RegSmem w;
+  w.cache = reinterpret_cast<unsigned*>(p);
+  p += size_t(4) << cache_bits;
+  w.q = p;
+  p += row_bytes;
+  w.cid = reinterpret_cast<unsigned*>(p);
+  p += kNbr * 4;
+  w.ckey = reinterpret_cast<unsigned*>(p);
+  p += kNbr * 4;
+  w.ctl = reinterpret_cast<int*>(p);
+  return w;
+}
+
+// ff_d2 by one warp: lane l takes chunks l, l + 32, ...; the lanes' pairs are
+// joined by a butterfly of two-sums, each level's low sum off by at most
+// 3 2^-48 of the total.  A lane's 4 ceil(nch / 32) steps and the levels that
+// join nonzero pairs stay within the (3 d + 13) 2^-48 of one chain (ff_bound).
+// The same value in every lane.
+__device__ __forceinline__ double ff_d2_warp(const float* q, const float* __restrict__ x, int nch) {
+  const float4* pq = reinterpret_cast<const float4*>(q);
+  const float4* px = reinterpret_cast<const float4*>(x);
+  float sh = 0.f, sl = 0.f;
+  for (int c = threadIdx.x & 31; c < nch; c += 32) {
+    const float4 a = pq[c], b = __ldg(px + c);
+    ff_step(a.x, b.x, sh, sl);
+    ff_step(a.y, b.y, sh, sl);
+    ff_step(a.z, b.z, sh, sl);
+    ff_step(a.w, b.w, sh, sl);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float oh = __shfl_xor_sync(0xffffffffu, sh, o), ol = __shfl_xor_sync(0xffffffffu, sl, o);
+    const float s1 = __fadd_rn(sh, oh);  // two-sum of the high parts
+    const float bv = __fsub_rn(s1, sh);
+    const float e = __fadd_rn(__fsub_rn(sh, __fsub_rn(s1, bv)), __fsub_rn(oh, bv));
+    const float l1 = __fadd_rn(__fadd_rn(sl, ol), e);
+    sh = __fadd_rn(s1, l1);
+    sl = __fsub_rn(l1, __fsub_rn(sh, s1));
+  }
+  return __dadd_rn(double(sh), double(sl));
+}
+
+// Whether point `m` precedes point `c` in (distance, id) order, where their
+// single-precision intervals overlap: float-float distances, then binary64.
+// Called by a whole warp; out of line, since it is rare.
+__device__ __noinline__ bool precedes_fine(const uint8_t* Xb, int64_t row_bytes, int d, DevStatus* status,
+                                           const float* q, unsigned m, unsigned c) {
+  const int64_t stride = row_bytes / 4;
+  const float* xm = reinterpret_cast<const float*>(Xb) + int64_t(m) * stride;
+  const float* xc = reinterpret_cast<const float*>(Xb) + int64_t(c) * stride;
+  const int nch = int(row_bytes / 16);
+  const int o = slot_order(-ff_d2_warp(q, xm, nch), -ff_d2_warp(q, xc, nch), ff_bound(d));
+  if (o >= 0) return o == 1;
+  const double dm = canon_d2_f32(q, xm, d), dc = canon_d2_f32(q, xc, d);
+  if ((threadIdx.x & 31) == 0) atomicAdd(&status->fp64_search, 2ull);
+  return dm < dc || (dm == dc && m < c);
+}
+
+// The list of one query, held by a warp: entry i in slot i % S of lane i / S,
+// sorted by (distance, id), empty entries last (they have no point's id and
+// count as expanded).  Entries from L on have been cut: they are never expanded
+// or returned, and since nothing is ever taken out they cannot come back.
+// Slots are only indexed by constants, so they stay in registers.
+template <int DT, int S>
+struct RegList {
+  static constexpr unsigned kFull = 0xffffffffu;
+  unsigned key[S], idv[S];
+  unsigned inside;  // bit j: entry j of this lane lies before L
+
+  __device__ __forceinline__ void clear(int L, int lane) {
+    inside = 0;
+#pragma unroll
+    for (int j = 0; j < S; ++j) {
+      key[j] = DT == kU8 ? 0xffffffffu : 0x7f800000u;  // behind every point
+      idv[j] = kEmptyId;
+      inside |= lane * S + j < L ? 1u << j : 0u;
+    }
+  }
+  // Slot j of lane l: the key there, in every lane.
+  __device__ __forceinline__ unsigned key_at(int l, int j) const {
+    unsigned v = 0;
+#pragma unroll
+    for (int i = 0; i < S; ++i) v |= i == j ? key[i] : 0u;
+    return __shfl_sync(kFull, v, l);
+  }
+  // This lane's unexpanded entries before L, as bits.
+  __device__ __forceinline__ unsigned open_bits() const {
+    unsigned v = 0;
+#pragma unroll
+    for (int j = 0; j < S; ++j) v |= (idv[j] >> 31) << j;
+    return inside & ~v;
+  }
+  // The point at the lowest of `u`'s bits in the first lane that has any.
+  __device__ __forceinline__ unsigned first_of(unsigned u, unsigned who) const {
+    unsigned v = idv[S - 1];
+#pragma unroll
+    for (int j = S - 2; j >= 0; --j) v = (u >> j) & 1u ? idv[j] : v;
+    return __shfl_sync(kFull, v, __ffs(who) - 1);
+  }
+  // The closest unexpanded member, marked expanded (kEmptyId: none is left), and
+  // if `next` is asked for the one after it.
+  template <bool NEXT>
+  __device__ __forceinline__ unsigned pop(unsigned& next, int lane) {
+    unsigned u = open_bits();
+    const unsigned who = __ballot_sync(kFull, u != 0);
+    if (!who) return kEmptyId;
+    const unsigned p = first_of(u, who);
+    const unsigned low = lane == __ffs(who) - 1 ? u & (0u - u) : 0u;
+#pragma unroll
+    for (int j = 0; j < S; ++j) idv[j] |= (low << (31 - j)) & kVisited;
+    if constexpr (NEXT) {
+      u &= ~low;
+      const unsigned who2 = __ballot_sync(kFull, u != 0);
+      next = who2 ? first_of(u, who2) : kEmptyId;
+    }
+    return p;
+  }
+  // Puts point c at distance kc in its place.  stay: bit j = this lane's entry j
+  // precedes it; before: so does the entry before this lane's first.
+  __device__ __forceinline__ void place(unsigned kc, unsigned c, unsigned stay, bool before, unsigned pk, unsigned pi) {
+#pragma unroll
+    for (int j = S - 1; j >= 0; --j) {
+      const bool here = (stay >> j) & 1u;
+      const bool prev = j > 0 ? (stay >> (j > 0 ? j - 1 : 0)) & 1u : before;
+      const unsigned mk = j > 0 ? key[j > 0 ? j - 1 : 0] : pk, mi = j > 0 ? idv[j > 0 ? j - 1 : 0] : pi;
+      key[j] = here ? key[j] : prev ? kc : mk;
+      idv[j] = here ? idv[j] : prev ? c : mi;
+    }
+  }
+  // Adds point c at distance kc unless it is a member.  An entry whose key lies
+  // below kc (1 - E2) - A2 surely precedes it and one above kc (1 + E2) + A2
+  // surely follows (E2 = 2 E and four ulps, A2 = 4 Eabs: the two intervals are
+  // then apart); the rest, equal keys for uint8, are settled on ids or on finer
+  // distances, and the point itself is among them if it is a member.
+  __device__ __forceinline__ void add(unsigned kc, unsigned c, const SearchArgs& a, const uint8_t* q, float E2,
+                                      float A2, int lane) {
+    const unsigned pk = __shfl_up_sync(kFull, key[S - 1], 1), pi = __shfl_up_sync(kFull, idv[S - 1], 1);
+    bool less[S];
+    bool near = false, before;
+    if constexpr (DT == kU8) {
+#pragma unroll
+      for (int j = 0; j < S; ++j) {
+        less[j] = key[j] < kc;
+        near |= key[j] == kc;
+      }
+      before = pk < kc || lane == 0;
+    } else {
+      const float f = __uint_as_float(kc);
+      const float lo = f * (1.0f - E2) - A2, hi = f * (1.0f + E2) + A2;
+#pragma unroll
+      for (int j = 0; j < S; ++j) {
+        less[j] = __uint_as_float(key[j]) < lo;
+        near |= !less[j] && !(__uint_as_float(key[j]) > hi);
+      }
+      before = __uint_as_float(pk) < lo || lane == 0;
+    }
+    if (__any_sync(kFull, near)) {
+      add_near(kc, c, a, q, E2, A2, lane, pk, pi);
+      return;
+    }
+#pragma unroll
+    for (int j = S - 1; j >= 0; --j) {
+      const bool prev = j > 0 ? less[j > 0 ? j - 1 : 0] : before;
+      const unsigned mk = j > 0 ? key[j > 0 ? j - 1 : 0] : pk, mi = j > 0 ? idv[j > 0 ? j - 1 : 0] : pi;
+      key[j] = less[j] ? key[j] : prev ? kc : mk;
+      idv[j] = less[j] ? idv[j] : prev ? c : mi;
+    }
+  }
+  __device__ __forceinline__ void add_near(unsigned kc, unsigned c, const SearchArgs& a, const uint8_t* q, float E2,
+                                           float A2, int lane, unsigned pk, unsigned pi) {
+    unsigned stay = 0;
+    bool have = false;
+#pragma unroll
+    for (int j = 0; j < S; ++j) have |= (idv[j] & kIdMask) == c;
+    if (__any_sync(kFull, have)) return;
+    if constexpr (DT == kU8) {
+#pragma unroll
+      for (int j = 0; j < S; ++j)
+        stay |= key[j] < kc || (key[j] == kc && (idv[j] & kIdMask) < c) ? 1u << j : 0u;
+    } else {
+      const float f = __uint_as_float(kc);
+      const float lo = f * (1.0f - E2) - A2, hi = f * (1.0f + E2) + A2;
+#pragma unroll
+      for (int j = 0; j < S; ++j) {
+        const float fj = __uint_as_float(key[j]);
+        stay |= fj < lo ? 1u << j : 0u;
+        unsigned b = __ballot_sync(kFull, !(fj < lo) && !(fj > hi) && idv[j] != kEmptyId);
+        while (b) {
+          const int l = __ffs(b) - 1;
+          b &= b - 1;
+          const unsigned m = __shfl_sync(kFull, idv[j], l) & kIdMask;
+          const bool first = precedes_fine(a.X, a.row_bytes, a.d, a.status, reinterpret_cast<const float*>(q), m, c);
+          if (first && lane == l) stay |= 1u << j;
+        }
+      }
+    }
+    const unsigned ps = __shfl_up_sync(kFull, stay, 1);
+    place(kc, c, stay, lane == 0 || ((ps >> (S - 1)) & 1u), pk, pi);
+  }
+};
+
+// One query per warp (W = 1, four warps per CTA), or per CTA of W warps: warp 0
+// keeps the list and the others read the rows.
+//
+// What bounds it: with one warp per query, the instructions of an expansion (row
+// distances, adding points); with a team, the chain row bounds -> ids -> rows of
+// each expansion and the list's warp.  A team therefore knows the next member to
+// be expanded before the current one is done (only a closer new point displaces
+// it: 9 of 10 stay), loads its row bounds before the current rows are read and
+// its ids before they are added.  Without a team other queries hide that chain,
+// and the registers count for more.
+//
+// Measured, a list sorted in shared memory (32 neighbours at a time, one lane per
+// row) -> this kernel: 400,000 x 96 floats, L = 100, one query 585 -> 142 us,
+// 10,000 queries 2.57 -> 0.89 ms; 400,000 x 128 uint8, L = 128, 10,000 queries
+// 2.11 -> 1.13 ms; 30,000 x 960 floats, L = 200, 1,000 queries 23.2 -> 4.6 ms (36
+// GB of rows).  Also measured: an unordered list with its minimum and maximum by
+// warp reductions (one query 216 us, 10,000 1.84 ms).  Eight CTAs per SM of
+// one-warp queries (64 registers) beat six and ten (0.89 against 0.98 and 1.09 ms
+// on the float rows).
+template <int DT, int S, int W>
+__global__ void __launch_bounds__(W == 1 ? kWarps * 32 : W * 32, W == 1 ? 8 : W == kTeam ? 3 : kSmallTeamCtas)
+    search_reg_kernel(SearchArgs a) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const RegSmem M = reg_carve(smem_raw + (W == 1 ? size_t(warp) * reg_bytes(a.row_bytes, a.cache_bits) : 0),
+                              a.row_bytes, a.cache_bits);
+  const int cshift = 32 - a.cache_bits;
+  const int nch = int(a.row_bytes / 16);
+  const unsigned full = 0xffffffffu;
+  const float E2 = 2.0f * lane_rel_bound(nch) + 2.3841858e-07f, A2 = 4.0f * abs_bound(a.d);
+  const int wthreads = W == 1 ? 32 : W * 32, wt = W == 1 ? lane : int(threadIdx.x);
+
+  for (;;) {
+    unsigned qi = 0;
+    if constexpr (W == 1) {
+      if (lane == 0) qi = atomicAdd(a.work, 1u);
+      qi = __shfl_sync(full, qi, 0);
+    } else {
+      if (threadIdx.x == 0) M.ctl[1] = int(atomicAdd(a.work, 1u));
+      __syncthreads();
+      qi = unsigned(M.ctl[1]);
+    }
+    if (qi >= a.nq) break;
+    const uint4* src = reinterpret_cast<const uint4*>(
+        a.q_point ? a.X + int64_t(a.q_point[qi]) * a.row_bytes : a.Q + int64_t(qi) * a.row_bytes);
+    for (int c = wt; c < nch; c += wthreads) reinterpret_cast<uint4*>(M.q)[c] = src[c];
+    for (int c = wt; c < (1 << a.cache_bits); c += wthreads) M.cache[c] = kEmptyId;
+    if constexpr (W == 1) __syncwarp();
+    else __syncthreads();
+    unsigned qn = 0;  // uint8: |q|^2
+    if constexpr (DT == kU8) {
+      for (int w4 = lane; w4 < 4 * nch; w4 += 32) {
+        const unsigned qw = reinterpret_cast<const unsigned*>(M.q)[w4];
+        qn = __dp4a(qw, qw, qn);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) qn += __shfl_xor_sync(full, qn, o);
+    }
+    if (W > 1 && warp > 0) {
+      // the team: distances of the new rows, as warp 0 asks for them
+      for (;;) {
+        __syncthreads();
+        const int nf = M.ctl[0];
+        if (nf < 0) break;
+        row_keys<DT, W>(a.X, a.row_bytes, M.q, M.cid, M.ckey, nf, warp - 1, W - 1, qn);
+        __syncthreads();
+      }
+      __syncthreads();
+      continue;
+    }
+    const int64_t* __restrict__ row_ptr = a.row_ptr;
+    const int32_t* __restrict__ col = a.col;
+    unsigned start = unsigned(a.start);
+    if (a.q_graph) {
+      const SearchGraph sg = a.graphs[a.q_graph[qi]];
+      row_ptr = sg.row_ptr;
+      col = sg.col;
+      start = unsigned(sg.start);
+    }
+    RegList<DT, S> list;
+    const int L = a.q_L ? a.q_L[qi] : a.L;
+    list.clear(L, lane);
+    if (lane == 0) {
+      M.cid[0] = start;
+      M.cache[(start * 0x9E3779B1u) >> cshift] = start;
+    }
+    __syncwarp();
+    row_keys<DT, 1>(a.X, a.row_bytes, M.q, M.cid, M.ckey, 1, 0, 1, qn);
+    __syncwarp();
+    if (lane == 0) {
+      list.key[0] = M.ckey[0];
+      list.idv[0] = start;
+    }
+    __syncwarp();
+
+    // the expected next expansion: its point, row and first ids
+    unsigned nx = kEmptyId;
+    const int32_t* nx_ids = col;
+    int nx_deg = 0;
+    unsigned nx_v0 = 0, nx_v1 = 0;
+    int64_t iters = 0;
+    for (;;) {
+      unsigned after = kEmptyId;
+      const unsigned ps = list.template pop<(W > 1)>(after, lane);
+      if (ps == kEmptyId) break;
+      if (++iters > a.n + 1) {  // cannot happen: each point is expanded at most once
+        if (lane == 0) raise_status(a.status, kDevOverflow, qi);
+        break;
+      }
+      if (a.visited && lane == 0 && iters <= a.visited_cap)
+        a.visited[int64_t(qi) * a.visited_cap + iters - 1] = int32_t(ps);
+      // row v: its first id and its degree
+      auto bounds = [&](unsigned v, const int32_t*& ids, int& deg) {
+        if (a.adj_deg) {
+          ids = col + int64_t(v) * a.adj_stride;
+          deg = a.adj_deg[v];
+        } else {
+          const int64_t b = row_ptr[v];
+          ids = col + b;
+          deg = int(row_ptr[v + 1] - b);
+        }
+      };
+      const int32_t* ids;
+      int deg;
+      unsigned v0, v1;
+      if (W > 1 && ps == nx) {
+        ids = nx_ids;
+        deg = nx_deg;
+        v0 = nx_v0;
+        v1 = nx_v1;
+      } else {
+        bounds(ps, ids, deg);
+        v0 = lane < deg ? unsigned(ids[lane]) : 0u;
+        v1 = 32 + lane < deg ? unsigned(ids[32 + lane]) : 0u;
+      }
+      nx = after;
+      if (W > 1 && nx != kEmptyId) bounds(nx, nx_ids, nx_deg);
+      bool first = true;
+      for (int eb = 0; eb < deg || first; eb += kNbr) {
+        if (!first) {
+          v0 = eb + lane < deg ? unsigned(ids[eb + lane]) : 0u;
+          v1 = eb + 32 + lane < deg ? unsigned(ids[eb + 32 + lane]) : 0u;
+        }
+        // ---- the neighbours that the cache does not hold.  A row holds
+        // distinct ids, so lanes that share a cache entry hold different ids:
+        // whichever write lands, no lane skips a new id.
+        const unsigned below = (1u << lane) - 1u;
+        int nf = 0;
+        auto take = [&](unsigned v, bool in) {
+          const unsigned h = (v * 0x9E3779B1u) >> cshift;
+          const bool f = in && M.cache[h] != v;
+          const unsigned m = __ballot_sync(full, f);
+          if (f) {
+            M.cache[h] = v;
+            M.cid[nf + __popc(m & below)] = v;
+          }
+          nf += __popc(m);
+        };
+        take(v0, eb + lane < deg);
+        if (eb + 32 < deg) take(v1, eb + 32 + lane < deg);
+        if (nf > 0) {
+          if constexpr (W == 1) {
+            __syncwarp();
+            row_keys<DT, 1>(a.X, a.row_bytes, M.q, M.cid, M.ckey, nf, 0, 1, qn);
+          } else {
+            if (lane == 0) M.ctl[0] = nf;
+            __syncthreads();
+          }
+        }
+        if (W > 1 && first && nx != kEmptyId) {  // its row bounds are here by now
+          nx_v0 = lane < nx_deg ? unsigned(nx_ids[lane]) : 0u;
+          nx_v1 = 32 + lane < nx_deg ? unsigned(nx_ids[32 + lane]) : 0u;
+        }
+        first = false;
+        if (nf == 0) continue;
+        if constexpr (W == 1) __syncwarp();
+        else __syncthreads();
+        // ---- those that may come before the L-th entry (an empty one: all of
+        // them).  A distance that is no number, of a query that holds one, never
+        // displaces a member.
+        const unsigned kth = list.key_at((L - 1) / S, (L - 1) % S);
+        const float last = __uint_as_float(kth) * (1.0f + E2) + A2;
+        auto enters = [&](int i) {
+          if (i >= nf) return false;
+          if constexpr (DT == kU8) return M.ckey[i] <= kth;
+          else return __uint_as_float(M.ckey[i]) <= last || kth == 0x7f800000u;
+        };
+#pragma unroll 1
+        for (int base = 0; base < nf; base += 32) {
+          unsigned todo = __ballot_sync(full, enters(base + lane));
+          while (todo) {
+            const int at = base + __ffs(todo) - 1;
+            todo &= todo - 1;
+            list.add(M.ckey[at], M.cid[at], a, M.q, E2, A2, lane);
+          }
+        }
+        __syncwarp();
+      }
+    }
+    if constexpr (W > 1) {
+      if (lane == 0) M.ctl[0] = -1;
+      __syncthreads();
+    }
+    if (a.visited_cnt && lane == 0) a.visited_cnt[qi] = int32_t(iters < INT32_MAX ? iters : INT32_MAX);
+    // ---- the k closest members
+#pragma unroll
+    for (int j = 0; j < S; ++j) {
+      const int i = lane * S + j;
+      if (i < a.k) {
+        const bool have = list.idv[j] != kEmptyId;
+        const int64_t at = int64_t(qi) * a.k + i;
+        a.out_ids[at] = have ? int32_t(list.idv[j] & kIdMask) : -1;
+        if (a.out_dists)
+          a.out_dists[at] = !have ? __int_as_float(0x7f800000)
+                                  : (DT == kU8 ? float(list.key[j]) : __uint_as_float(list.key[j]));
+      }
+    }
+    if constexpr (W == 1) __syncwarp();
+    else __syncthreads();
+  }
+}
+
 __global__ void recall_kernel(const int32_t* __restrict__ found, int ld_found, const int32_t* __restrict__ truth,
                               int ld_truth, int64_t nq, int k, unsigned long long* hits) {
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -495,30 +1044,67 @@ constexpr int kMinCacheBits = 8, kMaxCacheBits = 12;
 // The default plan stops at 512 entries: a larger cache takes shared memory
 // that L1 would otherwise give to the neighbour rows and vectors, and measured
 // slower on 1M x 128 uint8 at L = 128 (1,024 entries 6% slower, 4,096 50%).
-constexpr int kDefaultMaxCacheBits = 9;
+constexpr int kDefaultMaxCacheBits = 10;
 
-// CTAs of search_kernel<DT> one SM holds with `bytes` of dynamic shared memory
-// (registers and shared memory both count), from the occupancy calculator.
+using SearchKernel = void (*)(SearchArgs);
+
+// The kernels of one data type: the list in registers in 4 or 8 slots, one
+// warp or a team per query, and the list in shared memory.
 template <int DT>
-cudaError_t resident_ctas(size_t bytes, size_t max_bytes, int* out) {
-  cudaError_t err = cudaFuncSetAttribute(search_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(max_bytes));
+SearchKernel search_kernel_of(bool reg, int slots, int warps) {
+  if (!reg) return search_list_kernel<DT>;
+  if (warps == kTeam) return slots <= 4 ? search_reg_kernel<DT, 4, kTeam> : search_reg_kernel<DT, 8, kTeam>;
+  if (warps == kSmallTeam) return slots <= 4 ? search_reg_kernel<DT, 4, kSmallTeam> : search_reg_kernel<DT, 8, kSmallTeam>;
+  return slots <= 4 ? search_reg_kernel<DT, 4, 1> : search_reg_kernel<DT, 8, 1>;
+}
+
+// Every kernel may use all the shared memory a block can have, set once per
+// device (which also loads them all, so that a later call inside a stream
+// capture finds its kernel loaded).
+cudaError_t prepare_kernels() {
+  static std::mutex mu;
+  static std::map<int, bool> done;
+  int dev = 0, most = 0;
+  cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, search_kernel<DT>, kWarps * 32, bytes);
+  std::lock_guard<std::mutex> g(mu);
+  if (done.count(dev)) return cudaSuccess;
+  if ((err = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return err;
+  const int warps[4] = {1, kSmallTeam, kTeam, 0};
+  for (int v = 0; v < 16; ++v) {
+    const int slots = (v & 2) ? 8 : 4, w = warps[v >> 2];
+    SearchKernel k = (v & 1) ? search_kernel_of<kF32>(w > 0, slots, w) : search_kernel_of<kU8>(w > 0, slots, w);
+    if ((err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return err;
+  }
+  done[dev] = true;
+  return cudaSuccess;
 }
 
 // Default plan: the queries in flight hide the latency of each expansion, so
 // the search first maximises the CTAs per SM, then takes the largest id cache
-// (256 or 512 entries per warp) that keeps that many.  Plans are remembered
-// per (dtype, L, row bytes); the occupancy queries run once for each.
+// (256 or 512 entries per query) that keeps that many.  Plans are remembered
+// per (kernel, L, row bytes); the occupancy queries run once for each.
 struct SearchPlan {
   int bits = kMinCacheBits;
   int ctas = 1;
 };
 
-cudaError_t default_plan(bool f32, int L, int64_t row_bytes, SearchPlan* plan) {
+struct SearchForm {
+  SearchKernel kern = nullptr;
+  int threads = 0;
+  int queries = 0;  // in flight per CTA
+  bool reg = false, f32 = false;
+  int L = 0;
+  int64_t row_bytes = 0;
+  size_t bytes(int bits) const {
+    return size_t(queries) * (reg ? reg_bytes(row_bytes, bits) : warp_bytes(L, row_bytes, f32, bits));
+  }
+};
+
+cudaError_t default_plan(const SearchForm& F, SearchPlan* plan) {
   static std::mutex mu;
-  static std::map<std::tuple<bool, int, int64_t>, SearchPlan> memo;
-  const auto key = std::make_tuple(f32, L, row_bytes);
+  static std::map<std::tuple<SearchKernel, int, int64_t>, SearchPlan> memo;
+  const auto key = std::make_tuple(F.kern, F.reg ? 0 : F.L, F.row_bytes);
   {
     std::lock_guard<std::mutex> g(mu);
     auto it = memo.find(key);
@@ -527,13 +1113,11 @@ cudaError_t default_plan(bool f32, int L, int64_t row_bytes, SearchPlan* plan) {
       return cudaSuccess;
     }
   }
-  const size_t max_bytes = warp_bytes(L, row_bytes, f32, kMaxCacheBits) * kWarps;
   SearchPlan best;
   int best_ctas = 0;
-  for (int b = kMinCacheBits; b <= kDefaultMaxCacheBits; ++b) {
+  for (int b = kMinCacheBits; b <= (F.queries == 1 ? kMaxCacheBits : kDefaultMaxCacheBits); ++b) {
     int nb = 0;
-    const size_t bytes = warp_bytes(L, row_bytes, f32, b) * kWarps;
-    cudaError_t err = f32 ? resident_ctas<kF32>(bytes, max_bytes, &nb) : resident_ctas<kU8>(bytes, max_bytes, &nb);
+    cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, F.kern, F.threads, F.bytes(b));
     if (err != cudaSuccess) return err;
     if (nb >= best_ctas && nb > 0) {  // ties go to the larger cache
       best_ctas = nb;
@@ -575,36 +1159,43 @@ cudaError_t launch_search(const SearchLaunch& L, cudaStream_t s) {
   a.visited = L.visited;
   a.visited_cnt = L.visited_cnt;
   a.visited_cap = L.visited_cap;
-  const bool f32 = L.data.dtype == kF32;
+  cudaError_t err = prepare_kernels();
+  if (err != cudaSuccess) return err;
+  SearchForm F;
+  F.f32 = L.data.dtype == kF32;
+  F.reg = L.L <= kRegL;
+  F.L = L.L;
+  F.row_bytes = L.data.row_bytes;
+  // Few queries: a team per query.  400,000 x 96 floats, one warp / team of
+  // three / team of five, in us: 152 queries 198 / 178 / 181, 456: 292 / 256 /
+  // 241, 800: 370 / 321 / 450, 1,216: 382 / 342 / 624, 1,824: 399 / 495 / 858;
+  // 128-byte uint8 rows alike.  The lines lie where a team's CTAs (3 and 7 per
+  // SM) no longer hold all queries at once.
+  const int warps = !F.reg ? 0
+                    : L.nq <= int64_t(L.num_sms) * kTeamQueriesPerSm      ? kTeam
+                    : L.nq <= int64_t(L.num_sms) * kSmallTeamQueriesPerSm ? kSmallTeam
+                                                                          : 1;
+  const int slots = (L.L + 31) / 32;
+  F.kern = F.f32 ? search_kernel_of<kF32>(F.reg, slots, warps) : search_kernel_of<kU8>(F.reg, slots, warps);
+  F.threads = (warps > 1 ? warps : kWarps) * 32;
+  F.queries = warps > 1 ? 1 : kWarps;
   SearchPlan plan;
   if (L.cache_bits >= kMinCacheBits && L.cache_bits <= kMaxCacheBits) {  // a configured plan (rp_set_search_config)
     plan.bits = L.cache_bits;
-    const size_t bytes = warp_bytes(L.L, L.data.row_bytes, f32, plan.bits) * kWarps;
-    cudaError_t err = f32 ? resident_ctas<kF32>(bytes, bytes, &plan.ctas) : resident_ctas<kU8>(bytes, bytes, &plan.ctas);
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&plan.ctas, F.kern, F.threads, F.bytes(plan.bits));
     if (err != cudaSuccess) return err;
     plan.ctas = std::min(plan.ctas, kMaxCtasPerSmCap);
-  } else {
-    cudaError_t err = default_plan(f32, L.L, L.data.row_bytes, &plan);
-    if (err != cudaSuccess) return err;
+  } else if ((err = default_plan(F, &plan)) != cudaSuccess) {
+    return err;
   }
   int base_ctas = plan.ctas;
   if (L.ctas_per_sm > 0) base_ctas = std::min(base_ctas, L.ctas_per_sm);
   base_ctas = std::max(base_ctas, 1);
   a.cache_bits = plan.bits;
-  const size_t bytes = warp_bytes(L.L, L.data.row_bytes, f32, plan.bits) * kWarps;
   const int64_t want = int64_t(L.num_sms) * base_ctas;
-  const int64_t need = (L.nq + kWarps - 1) / kWarps;
+  const int64_t need = (L.nq + F.queries - 1) / F.queries;
   const int grid = int(std::max<int64_t>(1, std::min(want, need)));
-  cudaError_t err;
-  if (f32) {
-    err = cudaFuncSetAttribute(search_kernel<kF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
-    if (err != cudaSuccess) return err;
-    search_kernel<kF32><<<grid, kWarps * 32, bytes, s>>>(a);
-  } else {
-    err = cudaFuncSetAttribute(search_kernel<kU8>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
-    if (err != cudaSuccess) return err;
-    search_kernel<kU8><<<grid, kWarps * 32, bytes, s>>>(a);
-  }
+  F.kern<<<grid, F.threads, F.bytes(plan.bits), s>>>(a);
   return cudaGetLastError();
 }
 
