@@ -339,7 +339,11 @@ __device__ __forceinline__ unsigned exact_threshold(unsigned k, unsigned long lo
   return static_cast<unsigned>(q);
 }
 
-// Nodes claimed at a time by a prune_tc_kernel CTA (one per lane of warp 0).
+// Most nodes claimed at a time by a prune_tc_kernel CTA (one per lane of warp
+// 0).  A launch with fewer than 4 x 32 nodes per CTA claims less, so that every
+// CTA gets about four claims: at 32 always, the 600-row launches of a Vamana
+// build kept 19 of 304 CTAs busy (30,000 x 96 float points, both passes: 53 ms of
+// 65..128-candidate launches, now 7.2 ms).
 constexpr int kClaim = 32;
 
 // Named barriers of prune_tc_kernel (0 is __syncthreads, unused in the loop).
@@ -396,7 +400,7 @@ __global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_ker
   const int lane = r & 31;
   unsigned char* opnd = smem_raw + L::off_opnd;
   int* misc = reinterpret_cast<int*>(smem_raw + L::off_misc);
-  // misc ints: [0..3] slot node (s*2+g), [4..7] slot degree, [12] claim queue head
+  // misc ints: [0..3] slot node (s*2+g), [4..7] slot degree, [12] claim queue head, [13] its first entry
   int64_t* misc64 = reinterpret_cast<int64_t*>(smem_raw + L::off_misc + 64);  // [0..3] slot row start
   int* qnode = reinterpret_cast<int*>(smem_raw + L::off_misc + L::q_node);
   int* qdeg = reinterpret_cast<int*>(smem_raw + L::off_misc + L::q_deg);
@@ -408,11 +412,12 @@ __global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_ker
   auto slot_base = [&](int s, int g) { return smem_raw + L::off_slots + (size_t(s) * NG + g) * L::s_bytes; };
   const float E_rel = slice_rel_bound(a.d), E_abs = abs_bound(a.d);
   const int count = *a.count;
-
   if (warp == 0) tmem_alloc(tmem_slot, kTmemCols);  // of the SM's 512 TMEM columns, for the kernel's life
   if (r == 0) {
     mbar_init(mbar, 1);
+    // the queue counts up to kClaim; a claim of fewer nodes fills its end
     misc[12] = kClaim;  // empty claim queue
+    misc[13] = kClaim - max(NG, min(kClaim, count / (int(gridDim.x) * 4) / NG * NG));
     rq_count[0] = rq_count[1] = 0;
   }
   tc_fence_before();
@@ -455,15 +460,17 @@ __global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_ker
       // the consumer has resolved this slot's queue of two rounds ago: empty it
       if (DT == kF32 && r == 0) rq_count[s] = 0;
       if (warp == 0) {
-        // next NG nodes from the claim queue; warp 0 refills it kClaim nodes at
-        // a time (one atomic, the row bounds loaded by all lanes at once)
+        // next NG nodes from the claim queue; warp 0 refills it kClaim nodes (or
+        // the launch's smaller share) at a time: one atomic, the row bounds
+        // loaded by all lanes at once
         int head = misc[12];
         if (head >= kClaim) {
+          const int skip = misc[13];
           unsigned base = 0;
-          if (lane == 0) base = atomicAdd(a.work, unsigned(kClaim));
+          if (lane == 0) base = atomicAdd(a.work, unsigned(kClaim - skip));
           base = __shfl_sync(0xffffffffu, base, 0);
-          const unsigned idx = base + unsigned(lane);
-          const int pn = idx < unsigned(count) ? a.nodes[idx] : -1;
+          const unsigned idx = base + unsigned(lane - skip);
+          const int pn = lane >= skip && idx < unsigned(count) ? a.nodes[idx] : -1;
           int deg = 0;
           int64_t e0n = 0;
           if (pn >= 0) {
@@ -478,7 +485,7 @@ __global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_ker
           qdeg[lane] = deg;
           qe0[lane] = e0n;
           __syncwarp();
-          head = 0;
+          head = skip;
         }
         if (lane < NG) {
           misc[s * 2 + lane] = dead ? -1 : qnode[head + lane];
