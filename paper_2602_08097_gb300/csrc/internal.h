@@ -79,6 +79,8 @@ cudaError_t launch_scan_counts(const int32_t* cnt, int64_t n, int64_t* row_ptr,
                                int64_t* block_sums, int32_t* max_deg, cudaStream_t s);
 cudaError_t launch_add_random_candidates(const int32_t* knn, int kk, int64_t n, int nr, uint64_t seed, int32_t* out,
                                          cudaStream_t s);
+// the largest out-degree into *out (zeroed by the caller)
+cudaError_t launch_max_degree(const int64_t* row_ptr, int64_t n, unsigned long long* out, cudaStream_t s);
 cudaError_t launch_slice_row_ptr(const int64_t* row_ptr, int64_t n, int64_t lo, int64_t hi, int64_t* out,
                                  cudaStream_t s);
 cudaError_t launch_medoid(const DevData& D, double* mean /* d */, double* block_best /* 2*nb */,

@@ -120,6 +120,21 @@ __global__ void clean_write_kernel(const int64_t* __restrict__ row_ptr, const in
   }
 }
 
+// The largest out-degree, as an atomicMax into *out (zeroed by the caller).
+__global__ void max_degree_kernel(const int64_t* __restrict__ row_ptr, int64_t n, unsigned long long* __restrict__ out) {
+  unsigned long long m = 0;
+  for (int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; p < n; p += int64_t(gridDim.x) * blockDim.x) {
+    const unsigned long long deg = static_cast<unsigned long long>(row_ptr[p + 1] - row_ptr[p]);
+    m = deg > m ? deg : m;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long v = __shfl_down_sync(0xffffffffu, m, o);
+    m = v > m ? v : m;
+  }
+  if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(out, m);
+}
+
 // counts -> exclusive row_ptr (one level per 4096-node block), plus max count
 constexpr int kChunk = 4096;
 constexpr int kThreads = 256;
@@ -530,6 +545,12 @@ __global__ void slice_row_ptr_kernel(const int64_t* __restrict__ row_ptr, int64_
     const int64_t e = row_ptr[i];
     out[i] = (e < e_lo ? e_lo : (e > e_hi ? e_hi : e)) - e_lo;
   }
+}
+
+cudaError_t launch_max_degree(const int64_t* row_ptr, int64_t n, unsigned long long* out, cudaStream_t s) {
+  const int64_t blocks = (n + 255) / 256;
+  max_degree_kernel<<<unsigned(blocks < 1 ? 1 : blocks < 1024 ? blocks : 1024), 256, 0, s>>>(row_ptr, n, out);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_slice_row_ptr(const int64_t* row_ptr, int64_t n, int64_t lo, int64_t hi, int64_t* out,

@@ -103,6 +103,11 @@ struct rp_ctx {
   uint8_t* qbuf = nullptr;
   int64_t qbuf_bytes = 0;
   unsigned long long* hits = nullptr;  // device [1]
+  // pinned host memory for what calls read back (a copy into it needs no
+  // staging by the driver): the status word and two more, then kPinData bytes
+  // for the rows and results of small searches.  Only touched by calls that
+  // wait for their copies before they return, under the context's lock.
+  uint8_t* pin = nullptr;
   std::vector<BatchPlan> plans;
   // prune configuration: autotuned per source graph, or fixed by rp_set_tuning
   int tuning_mode = RP_TUNING_AUTO;
@@ -197,10 +202,18 @@ rp_status grow(rp_ctx* c, T** buf, int64_t* have, int64_t need) {
   return RP_OK;
 }
 
-rp_status check_device_status(rp_ctx* c) {
+constexpr size_t kPinHead = 256;
+constexpr size_t kPinData = 256 << 10;
+static_assert(sizeof(DevStatus) + 16 <= kPinHead, "the pinned head holds the status word and two more words");
+
+// Reads the status word back with whatever else the stream holds: queue_status,
+// then one wait, then status_result.
+cudaError_t queue_status(rp_ctx* c) {
+  return cudaMemcpyAsync(c->pin, c->status, sizeof(DevStatus), cudaMemcpyDeviceToHost, c->stream);
+}
+rp_status status_result(rp_ctx* c) {
   DevStatus h;
-  CUDA_TRY(c, cudaMemcpyAsync(&h, c->status, sizeof h, cudaMemcpyDeviceToHost, c->stream));
-  CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  memcpy(&h, c->pin, sizeof h);
   if (h.code != 0) {
     const int zero = 0;
     CUDA_TRY(c, cudaMemcpyAsync(&c->status->code, &zero, sizeof zero, cudaMemcpyHostToDevice, c->stream));
@@ -213,6 +226,12 @@ rp_status check_device_status(rp_ctx* c) {
     return fail(c, RP_EDEVICE, "device status %d (%s) at index %lld", h.code, what, (long long)h.info);
   }
   return RP_OK;
+}
+
+rp_status check_device_status(rp_ctx* c) {
+  CUDA_TRY(c, queue_status(c));
+  CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  return status_result(c);
 }
 
 // Records a timing event; inside a stream capture it becomes an event-record
@@ -724,7 +743,23 @@ rp_status search_impl(rp_ctx* c, const rp_graph* graphs, int32_t ngraphs, const 
   const int64_t table_off = (qbytes + out_bytes + 255) / 256 * 256;
   const int64_t table_bytes = q_graph ? int64_t(ngraphs) * int64_t(sizeof(SearchGraph)) + 8 * nq + 16 : 0;
   if ((s = grow(c, &c->qbuf, &c->qbuf_bytes, table_off + table_bytes)) != RP_OK) return s;
-  if ((s = upload_rows(c, c->qbuf, D.row_bytes, queries, nq, D.d, D.dtype, mem_flags)) != RP_OK) return s;
+  // Device rows that already have the padded layout are read in place; a few
+  // host rows are padded into pinned memory and go up in one copy.
+  const size_t packed = size_t(D.d) * elem_size(D.dtype);
+  const uint8_t* rows = c->qbuf;
+  const bool small = mem_flags == RP_MEM_HOST && size_t(qbytes + out_bytes) <= kPinData;
+  uint8_t* const pin_rows = c->pin + kPinHead;
+  if (mem_flags == RP_MEM_DEVICE && int64_t(packed) == D.row_bytes && reinterpret_cast<uintptr_t>(queries) % 16 == 0) {
+    rows = static_cast<const uint8_t*>(queries);
+  } else if (small) {
+    for (int64_t i = 0; i < nq; ++i) {
+      memcpy(pin_rows + i * D.row_bytes, static_cast<const uint8_t*>(queries) + size_t(i) * packed, packed);
+      memset(pin_rows + i * D.row_bytes + packed, 0, size_t(D.row_bytes) - packed);
+    }
+    CUDA_TRY(c, cudaMemcpyAsync(c->qbuf, pin_rows, size_t(qbytes), cudaMemcpyHostToDevice, c->stream));
+  } else if ((s = upload_rows(c, c->qbuf, D.row_bytes, queries, nq, D.d, D.dtype, mem_flags)) != RP_OK) {
+    return s;
+  }
   SearchLaunch S;
   S.data = D.dev();
   S.row_ptr = Gs[0]->row_ptr;
@@ -744,7 +779,7 @@ rp_status search_impl(rp_ctx* c, const rp_graph* graphs, int32_t ngraphs, const 
     S.q_graph = reinterpret_cast<const int32_t*>(t + gb);
     S.q_L = reinterpret_cast<const int32_t*>(t + gb + size_t(nq) * 4);
   }
-  S.Q = c->qbuf;
+  S.Q = rows;
   S.nq = nq;
   S.L = L;
   S.k = k;
@@ -768,10 +803,21 @@ rp_status search_impl(rp_ctx* c, const rp_graph* graphs, int32_t ngraphs, const 
   c->ev_search = true;
   c->kernel_launches += 1;
   if (mem_flags == RP_MEM_HOST) {
-    CUDA_TRY(c, cudaMemcpyAsync(ids, dev_ids, size_t(nq * k) * 4, cudaMemcpyDeviceToHost, c->stream));
-    if (dists) CUDA_TRY(c, cudaMemcpyAsync(dists, dev_d, size_t(nq * k) * 4, cudaMemcpyDeviceToHost, c->stream));
+    const size_t nb = size_t(nq * k) * 4;
+    uint8_t* const pin_out = pin_rows + qbytes;
+    if (small) {  // ids and distances are one block behind the rows
+      CUDA_TRY(c, cudaMemcpyAsync(pin_out, dev_ids, 2 * nb, cudaMemcpyDeviceToHost, c->stream));
+    } else {
+      CUDA_TRY(c, cudaMemcpyAsync(ids, dev_ids, nb, cudaMemcpyDeviceToHost, c->stream));
+      if (dists) CUDA_TRY(c, cudaMemcpyAsync(dists, dev_d, nb, cudaMemcpyDeviceToHost, c->stream));
+    }
+    CUDA_TRY(c, queue_status(c));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    return check_device_status(c);
+    if (small) {
+      memcpy(ids, pin_out, nb);
+      if (dists) memcpy(dists, pin_out + nb, nb);
+    }
+    return status_result(c);
   }
   if (q_graph) {
     // the host tables were read by stream-ordered copies; finish them before returning
@@ -1299,6 +1345,7 @@ rp_status rp_create(rp_ctx** out, int32_t device, uint64_t hbm_budget_bytes, voi
     return RP_ECUDA;
   if (dalloc(c.get(), reinterpret_cast<void**>(&c->work), 8 * sizeof(unsigned)) != RP_OK) return RP_ECUDA;
   if (dalloc(c.get(), reinterpret_cast<void**>(&c->hits), sizeof(unsigned long long)) != RP_OK) return RP_ECUDA;
+  if (cudaMallocHost(reinterpret_cast<void**>(&c->pin), kPinHead + kPinData) != cudaSuccess) return RP_ECUDA;
   if (cudaMemsetAsync(c->status, 0, sizeof(DevStatus), c->stream) != cudaSuccess) return RP_ECUDA;
   if (cudaMemsetAsync(c->dropped, 0, 2 * sizeof(unsigned long long), c->stream) != cudaSuccess) return RP_ECUDA;
   for (auto& e : c->ev)
@@ -1339,6 +1386,7 @@ rp_status rp_destroy(rp_ctx* c) {
     for (auto& e : c->ev)
       if (e) cudaEventDestroy(e);
     if (c->own_stream) cudaStreamDestroy(c->stream);
+    if (c->pin) cudaFreeHost(c->pin);
   }
   delete c;
   return RP_OK;
@@ -1350,8 +1398,7 @@ rp_status rp_sync(rp_ctx* c) {
   if (!c) return RP_EINVAL;
   std::lock_guard<std::mutex> lk(c->mu);
   cudaSetDevice(c->device);
-  CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  return check_device_status(c);
+  return check_device_status(c);  // waits for the stream
 }
 
 rp_status rp_load_graph(rp_ctx* c, const void* vectors, int32_t dtype, int64_t n, int32_t d, const int64_t* row_ptr,
@@ -1524,19 +1571,27 @@ rp_status rp_graph_info(rp_ctx* c, rp_graph g, int64_t* n, int64_t* nnz, int32_t
   Graph* G = find_graph(c, g);
   if (!G) return fail(c, RP_ENOTFOUND, "unknown graph %lld", (long long)g);
   if (G->nnz < 0 || max_deg) {
-    std::vector<int64_t> h(size_t(G->n + 1));
-    CUDA_TRY(c, cudaMemcpyAsync(h.data(), G->row_ptr, size_t(G->n + 1) * 8, cudaMemcpyDeviceToHost, c->stream));
+    // The degrees are reduced on the device, and both words and the status come
+    // back in one wait.
+    int64_t* const words = reinterpret_cast<int64_t*>(c->pin + kPinHead - 16);
+    CUDA_TRY(c, cudaMemsetAsync(c->hits, 0, 8, c->stream));
+    CUDA_TRY(c, launch_max_degree(G->row_ptr, G->n, c->hits, c->stream));
+    c->kernel_launches += 1;
+    CUDA_TRY(c, cudaMemcpyAsync(words, G->row_ptr + G->n, 8, cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(c, cudaMemcpyAsync(words + 1, c->hits, 8, cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(c, queue_status(c));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    G->nnz = h[size_t(G->n)];
-    int64_t mx = 0;
-    for (int64_t p = 0; p < G->n; ++p) mx = std::max(mx, h[size_t(p + 1)] - h[size_t(p)]);
-    G->max_deg_bound = int(mx);
-    if (max_deg) *max_deg = int32_t(mx);
+    G->nnz = words[0];
+    G->max_deg_bound = int(words[1]);
+    if (max_deg) *max_deg = int32_t(words[1]);
+  } else {
+    CUDA_TRY(c, queue_status(c));
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   }
   if (n) *n = G->n;
   if (nnz) *nnz = G->nnz;
   if (start) *start = G->start;
-  return check_device_status(c);
+  return status_result(c);
 }
 
 rp_status rp_graph_export(rp_ctx* c, rp_graph g, int64_t* row_ptr, int32_t* col, int64_t col_cap,
@@ -1555,10 +1610,7 @@ rp_status rp_graph_export(rp_ctx* c, rp_graph g, int64_t* row_ptr, int32_t* col,
   const cudaMemcpyKind kind = mem_flags == RP_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
   CUDA_TRY(c, cudaMemcpyAsync(row_ptr, G->row_ptr, size_t(G->n + 1) * 8, kind, c->stream));
   if (G->nnz > 0) CUDA_TRY(c, cudaMemcpyAsync(col, G->col, size_t(G->nnz) * 4, kind, c->stream));
-  if (mem_flags == RP_MEM_HOST) {
-    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    return check_device_status(c);
-  }
+  if (mem_flags == RP_MEM_HOST) return check_device_status(c);  // waits for the copies
   return RP_OK;
 }
 
