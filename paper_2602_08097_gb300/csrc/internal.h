@@ -165,7 +165,7 @@ bool knn_tc_eligible(int dtype, int d, int k);
 // max |x| over n float rows, as the bits of a non-negative float (atomicMax into *out)
 cudaError_t launch_maxabs_f32(const uint8_t* X, int64_t row_bytes, int64_t n, int d, unsigned* out, cudaStream_t s);
 size_t knn_tc_scratch_bytes(int dtype, int d, int64_t n, int64_t nq_ext, int num_sms);
-cudaError_t launch_knn_tc(const KnnTcLaunch& K, cudaStream_t s);
+cudaError_t launch_knn_tc(const KnnTcLaunch& K, cudaStream_t s, int64_t* kernels /* launched */);
 
 // vamana.cu: batched Vamana construction (graph held as nbr[p * R ..], deg[p])
 cudaError_t launch_vamana_candidates(const int32_t* pts, int64_t nb, const int32_t* visited, const int32_t* vis_cnt,

@@ -296,27 +296,53 @@ __global__ void __launch_bounds__(kThreads) knn_kernel(KnnArgs a) {
 // tile already in the core-matrix order of the tcgen05 operand layout: uint8
 // values as they are (exact), float rows scaled by a power of two so that
 // |x| <= 1 and split into two f16 operands, hi = f16(x) and lo =
-// f16(2^11 (x - hi)), the tile holding hi then lo.  A CTA of 4 warps owns 128
-// queries (thread t = query t = TMEM lane t) and streams every point tile past
-// them: D = Q P^T on tcgen05 into one of two TMEM accumulator sets (float rows:
-// hi hi^T in one accumulator, hi lo^T + lo hi^T in a second, G~ = the first +
-// 2^-11 the second), the next tile's copy in flight meanwhile.  The split keeps
-// the Gram error near 2^-22 |q||p| instead of f16's 2^-11, so the candidate
-// window stays narrow on data whose neighbours lie close together.
+// f16(2^11 (x - hi)), the tile holding hi then lo.  The split keeps the Gram
+// error near 2^-22 |q||p| instead of f16's 2^-11, so the candidate window stays
+// narrow on data whose neighbours lie close together.
 //
-// From G~ the thread forms d2~ = |q|^2 + |p|^2 - 2 G~ (scaled units) and a
-// rigorous error bound err (zero for uint8 rows of d <= 128, where every
-// quantity is an exact integer below 2^24).  Point p is kept as a candidate
-// when its lower bound d2~ - err is at most tau, the k-th smallest upper bound
-// d2~ + err met so far: at least k points have d2 <= tau, so every true k
-// nearest neighbour passes when it is met (tau only decreases).  A query's
-// candidates live in a global buffer; when it could overflow, the query's
-// warp sorts the upper bounds, lowers tau and drops the candidates above it.
-// At the end the candidates are ranked by their exact keys (uint8: exact
-// integers; float: sums per 32-dim slice with near-tie runs re-ordered in
-// binary64), as the CUDA-core kernel ranks its lists.
-constexpr int kTcQ = 128;  // queries per CTA (rows of the MMA)
-constexpr int kTcP = 128;  // points per tile (columns of the MMA)
+// Scan (knn_scan_kernel): a step is one query tile against one point tile, D =
+// Q P^T on tcgen05 (float rows: hi hi^T in one accumulator, hi lo^T + lo hi^T in
+// a second, G~ = the first + 2^-11 the second).  The steps of a chunk of query
+// tiles, in order, are cut evenly over the CTAs, so that 79 query tiles (10,000
+// queries) keep every SM busy; a query tile's points are then scanned in a few
+// parts by neighbouring CTAs.  One warp copies the tiles in (bulk copies, two or
+// three in flight) and issues the MMAs one step ahead of the eight warps that
+// read the accumulators: two threads per query (TMEM lane), half the columns each.
+//
+// From G~ a thread forms d2~ = |q|^2 + |p|^2 - 2 G~ (scaled units) and a rigorous
+// error bound err (zero for uint8 rows of d <= 128, where every quantity is an
+// exact integer below 2^24).  Point p is kept as a candidate, as {d2~, id}, when
+// its lower bound may be at most tau, an upper bound of the k-th smallest
+// distance met so far by any part of the query (the k-th smallest d2~ of a part
+// plus the largest err it has met): at least k points have d2 <= tau, so every
+// true k nearest neighbour passes when it is met (tau only decreases).  Eight
+// columns at a time are tested branch-free (the sign of d2~ - threshold, shifted
+// into a mask), and the few that pass are stored by predicated instructions, if
+// any lane has one.  A query's candidates live in a global buffer per part, one
+// thread's from its start up, the other's from its end down; when it gets long, a
+// warp selects the k-th, lowers tau and drops the candidates above it.
+//
+// Rank (knn_rank_kernel), one warp per query: the candidates of its parts are
+// cut to the final tau and ranked by their exact keys (uint8: exact integers;
+// float: sums per 32-dim slice with near-tie runs re-ordered in binary64), as
+// the CUDA-core kernel ranks its lists.
+//
+// What bounds the scan: per step, the three split products (1,150 cycles of
+// MMA at d = 96) and the threads' 128 columns at four to five instructions
+// each.  10,000 queries x 400,000 points x 96 dims, k 100: 5.0 ms for the scan and
+// 0.34 for the ranking, 5.5 in all; one CTA per query tile, a lane per query row
+// and the tile's loads, products and cuts in turn took 47.6 (79 CTAs of 152, the
+// tensor cores idle through every cut).
+constexpr int kTcQ = 128;     // queries per tile (rows of the MMA)
+constexpr int kTcP = 128;     // points per tile (columns of the MMA)
+constexpr int kTcCand = 512;  // candidates a part keeps per query
+// A part's candidates are cut when they pass kTcCut (or what a cut left plus 96):
+// more candidates pass an old tau than a cut costs.  A tile adds at most kTcP.
+constexpr int kTcCut = 224;
+constexpr int kTcThreads = 288;
+constexpr int kTcNorms = 8;   // point-norm rows in shared memory
+constexpr int kTcMinSteps = 8;  // a CTA takes at least this many point tiles (if there are as many)
+constexpr int kRankCand = 1024;
 
 struct KnnTcArgs {
   const uint8_t* X;          // raw rows (exact ranking)
@@ -330,16 +356,23 @@ struct KnnTcArgs {
   const uint8_t* ptiles;     // packed point tiles
   int64_t tile_bytes;        // kTcP * dpad * 2 per operand: uint8 one (f16), float two (hi, lo)
   int ksteps;                // dpad / 16
+  int nbuf;                  // point tiles in shared memory, 2 or 3
   const float* qnorm;        // |q'|^2 per query (scaled)
   const float* pnorm;        // |p'|^2 per point, padded to whole tiles with 0
-  const float2* tmax;        // per point tile: (max |p'|^2, max |p'|)
+  const float2* tmax;        // per point tile: (max |p'|^2, max |p'|), then the same over all tiles
   int exact;                 // 1: G~ and d2~ are exact
   float eps_ip, eps_n, sub_abs;  // sub_abs: the subnormal-rounding term per unit of |q| + |p|
-  uint4* cand;               // per CTA: kTcQ x capc entries {lb, ub, id, 0}
-  int capc;
+  // this chunk: query tiles qt0 .. qt0 + nqt - 1, `per` steps per CTA.  The part
+  // of CTA c on the chunk's query tile t is part c + t: each is met once, since
+  // from one part to the next c or t or both grow.
+  int64_t qt0, nqt, per;
+  int kscan;                 // k, one more for base points, whose own row is met too
+  uint2* cand;               // [part][query][kTcCand] {d2~, id}
+  int* pcnt;                 // [part][query] candidates (from the start, << 16 from the end), zeroed: none
+                             // of a part that could not finish
+  unsigned* tauq;            // [chunk query] tau as an ordered key (fkey), lowered by every part
   int32_t* out_ids;
   float* out_dists;
-  unsigned* work;            // zeroed: next query tile
   DevStatus* status;
 };
 
@@ -365,246 +398,470 @@ __device__ __forceinline__ float tc_err(const KnnTcArgs& a, float nq, float sq, 
 // Operands per tile: uint8 rows one f16 operand, float rows two (hi, lo).
 __host__ __device__ constexpr int tc_nop(int dtype) { return dtype == kF32 ? 2 : 1; }
 
-size_t knn_tc_smem(int dtype, int64_t tile_bytes, int capc) {
-  // A tile, two B tiles, two point-norm rows, per-warp sort buffers, misc.
-  // uint8: at least a third of an SM's shared memory, so that at most two CTAs
-  // (each holding 256 of the SM's 512 TMEM columns) share an SM; float: more
-  // than half, one CTA holding all 512 (two sets of two accumulators).
-  const size_t need = size_t(tile_bytes) * 3 + 2 * kTcP * 4 + size_t(4) * capc * 8 + 256;
+// Entry i of a buffer that holds `a` entries from its start and the rest from
+// `gap` places on: gap = 0 for a plain list.
+__device__ __forceinline__ int entry_at(int i, int a, int gap) { return i < a ? i : i + gap; }
+
+// The k-th smallest distance of the m >= k entries as a key, by bisection on its
+// bits; the entries are read once, PER of them per lane.  One warp.
+template <int PER>
+__device__ __forceinline__ unsigned kth_of(const uint2* e, int m, int k, int a = kTcCand, int gap = 0) {
+  const int lane = threadIdx.x & 31;
+  unsigned u[PER];
+#pragma unroll
+  for (int i = 0; i < PER; ++i) u[i] = 32 * i + lane < m ? fkey(__uint_as_float(e[entry_at(32 * i + lane, a, gap)].x)) : 0xffffffffu;
+  unsigned lo = 0xffffffffu, hi = 0;
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    lo = min(lo, u[i]);
+    if (32 * i + lane < m) hi = max(hi, u[i]);
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  while (lo < hi) {  // the k-th smallest lies in [lo, hi]
+    const unsigned mid = lo + (hi - lo) / 2;
+    int c = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) c += u[i] <= mid;
+    if (__reduce_add_sync(0xffffffffu, c) >= k) hi = mid;
+    else lo = mid + 1;
+  }
+  return lo;
+}
+
+// An error bound as what is added to or taken from a d2~: e with the roundings of
+// that sum.
+__device__ __forceinline__ float cut_width(float e, float norms) { return e * 1.0001f + 4.7683716e-07f * norms; }
+
+// Drops the entries whose lower bound (d2~ - w) lies above tau and moves the rest
+// to the start; returns how many are left.  One warp.
+__device__ __forceinline__ int cut_above(uint2* e, int m, float tau, float w, int a = kTcCand, int gap = 0) {
+  const int lane = threadIdx.x & 31;
+  int kept = 0;
+  for (int i0 = 0; i0 < m; i0 += 32) {
+    const int i = i0 + lane;
+    uint2 v = make_uint2(0, 0);
+    if (i < m) v = e[entry_at(i, a, gap)];  // never before the place it may be moved to
+    const bool keep = i < m && __uint_as_float(v.x) - w <= tau;
+    const unsigned km = __ballot_sync(0xffffffffu, keep);
+    __syncwarp();
+    if (keep) e[kept + __popc(km & ((1u << lane) - 1))] = v;
+    kept += __popc(km);
+    __syncwarp();
+  }
+  return kept;
+}
+
+// *at = {x, y} and at += step bytes if `yes`, by predicated instructions: a branch per column costs
+// more than the stores it skips.
+__device__ __forceinline__ void push_if(unsigned yes, uint2*& at, long long step, unsigned x, unsigned y) {
+  unsigned long long p = reinterpret_cast<unsigned long long>(at);
+  asm volatile(
+      "{\n.reg .pred p;\nsetp.ne.u32 p, %1, 0;\n@p st.global.v2.u32 [%0], {%2, %3};\n@p add.s64 %0, %0, %4;\n}\n"
+      : "+l"(p)
+      : "r"(yes), "r"(x), "r"(y), "l"(step)
+      : "memory");
+  at = reinterpret_cast<uint2*>(p);
+}
+
+// A query tile, the point tiles, their norms, the barriers.  uint8: at least a
+// third of an SM's shared memory, so that at most two CTAs (each holding 256 of
+// the SM's 512 TMEM columns) share an SM; float: more than half, one CTA holding
+// all 512 (two sets of two accumulators).
+size_t knn_tc_smem(int dtype, int64_t tile_bytes, int nbuf) {
+  const size_t need = size_t(tile_bytes) * size_t(1 + nbuf) + kTcNorms * kTcP * 4 + 256 + 3 * kTcQ * 4;
   return std::max(need, dtype == kF32 ? size_t(228 * 1024 / 2 + 1024) : size_t(228 * 1024 / 3 + 1024));
 }
 
 template <int DT>
-__global__ void __launch_bounds__(128) knn_tc_kernel(KnnTcArgs a) {
+__global__ void __launch_bounds__(kTcThreads) knn_scan_kernel(KnnTcArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   // float rows: hi and lo operands, two accumulators per set (acc0 at column
   // 0 of the set, acc1 at 128)
   constexpr bool kSplit = DT == kF32;
   constexpr uint32_t kSetCols = kSplit ? 256u : 128u;
+  constexpr int kWait = 1 << 20;
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   unsigned char* sA = smem_raw;
-  unsigned char* sB0 = smem_raw + a.tile_bytes;
-  unsigned char* sB1 = smem_raw + 2 * a.tile_bytes;
-  float* sPn = reinterpret_cast<float*>(smem_raw + 3 * a.tile_bytes);                 // [2][kTcP]
-  unsigned long long* sSort = reinterpret_cast<unsigned long long*>(sPn + 2 * kTcP);  // [4][capc]
-  unsigned char* misc = reinterpret_cast<unsigned char*>(sSort + size_t(4) * a.capc);
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(misc);  // [2]
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 16);
-  int* qt_slot = reinterpret_cast<int*>(misc + 32);
+  unsigned char* sB = smem_raw + a.tile_bytes;
+  float* sPn = reinterpret_cast<float*>(smem_raw + (1 + a.nbuf) * a.tile_bytes);  // [kTcNorms][kTcP]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sPn + kTcNorms * kTcP);
+  uint64_t* full = bars;           // [3] point tile landed
+  uint64_t* afull = bars + 3;      // query tile landed
+  uint64_t* mma_done = bars + 4;   // [2] accumulator set written
+  uint64_t* acc_free = bars + 6;   // [2] accumulator set read (8 warps)
+  uint64_t* nfull = bars + 8;      // [kTcNorms] point norms landed
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 8 + kTcNorms);
+  int* sCnt = reinterpret_cast<int*>(bars + 32);               // [2][kTcQ] candidates, by half
+  float* sTau = reinterpret_cast<float*>(sCnt + 2 * kTcQ);     // [kTcQ] tau after a cut
   const int64_t npt = (a.n + kTcP - 1) / kTcP;
-  const int64_t nqt = (a.nq + kTcQ - 1) / kTcQ;
-  constexpr uint32_t idesc = umma_idesc_f16(128, 128);
-  constexpr uint32_t lbo = 16u * 128u;  // 16 row-groups of 128 bytes per k-chunk
+  const int64_t s0 = int64_t(blockIdx.x) * a.per;
+  const int64_t total = a.nqt * npt;
+  const int64_t s1 = s0 + a.per < total ? s0 + a.per : total;
+  const int steps = int(s1 > s0 ? s1 - s0 : 0);
+  const int q_first = int(s0 / npt), j_first = int(s0 - q_first * npt), ntile = int(npt);
 
   if (warp == 0) tmem_alloc(tmem_slot, 2 * kSetCols);  // two accumulator sets
   if (t == 0) {
-    mbar_init(&mbar[0], 1);
-    mbar_init(&mbar[1], 1);
+    for (int i = 0; i < 4; ++i) mbar_init(&full[i], 1);  // full[0..2], afull
+    for (int i = 0; i < 2; ++i) mbar_init(&mma_done[i], 1);
+    for (int i = 0; i < 2; ++i) mbar_init(&acc_free[i], 8);
+    for (int i = 0; i < kTcNorms; ++i) mbar_init(&nfull[i], 1);
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  uint32_t phase0 = 0u, phase1 = 0u;
-  unsigned long long* wsort = sSort + size_t(warp) * a.capc;
-  const float inf = __int_as_float(0x7f800000);
-  bool dead = false;
 
-  for (;;) {
-    if (t == 0) *qt_slot = int(atomicAdd(a.work, 1u));
-    __syncthreads();
-    const int64_t qt = *qt_slot;
-    __syncthreads();
-    if (qt >= nqt) break;
-    // ---- the query tile (operand A), resident for the whole scan
-    {
-      const uint4* src = reinterpret_cast<const uint4*>(a.qtiles + qt * a.tile_bytes);
-      uint4* dst = reinterpret_cast<uint4*>(sA);
-      for (int64_t i = t; i < a.tile_bytes / 16; i += 128) dst[i] = src[i];
-    }
-    const int64_t qi = qt * kTcQ + t;
-    const bool qlive = qi < a.nq;
-    const float nqq = qlive ? a.qnorm[qi] : 0.f;
-    const float sq = sqrtf(nqq);
-    float tau = inf;
-    int cnt = 0;
-    uint4* cbuf = a.cand + (int64_t(blockIdx.x) * kTcQ + t) * a.capc;
-    auto load_tile = [&](int64_t j, unsigned char* dstB, float* dstN) {
-      const unsigned char* src = a.ptiles + j * a.tile_bytes;
-      for (int64_t i = t; i < a.tile_bytes / 16; i += 128) cp_async16(dstB + i * 16, src + i * 16, 16);
-      if (t < kTcP / 4) cp_async16(dstN + 4 * t, a.pnorm + j * kTcP + 4 * t, 16);
-      cp_async_commit();
-    };
-    load_tile(0, sB0, sPn);
-    for (int64_t j = 0; j < npt; ++j) {
-      const int b = int(j & 1);
-      unsigned char* sB = b ? sB1 : sB0;
-      const float* pnb = sPn + b * kTcP;
-      cp_async_wait<0>();
-      fence_async_smem();
-      tc_fence_before();
-      __syncthreads();  // tile j in smem; every read of accumulator b (tile j - 2) finished
-      tc_fence_after();
-      if (t == 0) {
+  if (warp == 8) {
+    // ---------------- copies and MMAs, one lane ----------------
+    if (lane == 0 && steps > 0) {
+      constexpr uint32_t idesc = umma_idesc_f16(128, 128);
+      constexpr uint32_t lbo = 16u * 128u;  // 16 row-groups of 128 bytes per k-chunk
+      const uint32_t lo_off = uint32_t(a.tile_bytes / 2);  // float tiles: lo after hi
+      // A point tile goes into buffer (step % nbuf) once the MMA of the step
+      // that used it is done, its norms into row (step % kTcNorms): step s is
+      // loaded after the MMA of step s - 2 was issued, which waited until the
+      // accumulators of step s - 4 were read; whoever has read those is done with
+      // the norms of every step before, s - kTcNorms among them.
+      int loaded = 0, lj = j_first, lb = 0;
+      auto load_point_tile = [&]() {  // step `loaded` of this CTA
+        const int nb = loaded % kTcNorms;
+        mbar_expect(&full[lb], uint32_t(a.tile_bytes));
+        bulk_load(sB + lb * a.tile_bytes, a.ptiles + lj * a.tile_bytes, uint32_t(a.tile_bytes), &full[lb]);
+        mbar_expect(&nfull[nb], kTcP * 4u);
+        bulk_load(sPn + nb * kTcP, a.pnorm + int64_t(lj) * kTcP, kTcP * 4u, &nfull[nb]);
+        ++loaded;
+        if (++lj == ntile) lj = 0;
+        if (++lb == a.nbuf) lb = 0;
+      };
+      for (int i = 0; i < a.nbuf - 1 && loaded < steps; ++i) load_point_tile();
+      bool ok = true;
+      uint32_t aphase = 0, pphase = 0;
+      int q = q_first, j = j_first, pb = 0;
+      for (int it = 0; it < steps && ok; ++it) {
+        const int b = it & 1;
+        if (it == 0 || j == 0) {  // the next query tile, once the last MMA has read the old one
+          if (it > 0) ok = mbar_wait(&mma_done[b ^ 1], uint32_t((it - 1) >> 1) & 1u, kWait);
+          if (!ok) break;
+          mbar_expect(afull, uint32_t(a.tile_bytes));
+          bulk_load(sA, a.qtiles + (a.qt0 + q) * a.tile_bytes, uint32_t(a.tile_bytes), afull);
+          ok = mbar_wait(afull, aphase, kWait);
+          aphase ^= 1u;
+          if (!ok) break;
+        }
+        ok = mbar_wait(&full[pb], pphase, kWait);
+        if (ok && it >= 2) ok = mbar_wait(&acc_free[b], uint32_t((it >> 1) - 1) & 1u, kWait);
+        if (!ok) break;
+        tc_fence_after();
         const uint32_t acc = tmem + uint32_t(b) * kSetCols;
-        const uint32_t lo_off = uint32_t(a.tile_bytes / 2);  // float tiles: lo after hi
+        const unsigned char* B = sB + pb * a.tile_bytes;
         for (int kk = 0; kk < a.ksteps; ++kk) {
           const uint64_t da = umma_desc(smem_addr(sA) + uint32_t(kk) * 2u * lbo, lbo, 128u);
-          const uint64_t db = umma_desc(smem_addr(sB) + uint32_t(kk) * 2u * lbo, lbo, 128u);
+          const uint64_t db = umma_desc(smem_addr(B) + uint32_t(kk) * 2u * lbo, lbo, 128u);
           umma_f16(acc, da, db, idesc, kk > 0);
           if constexpr (kSplit) {  // the cross terms with the low halves
             const uint64_t dal = umma_desc(smem_addr(sA) + lo_off + uint32_t(kk) * 2u * lbo, lbo, 128u);
-            const uint64_t dbl = umma_desc(smem_addr(sB) + lo_off + uint32_t(kk) * 2u * lbo, lbo, 128u);
+            const uint64_t dbl = umma_desc(smem_addr(B) + lo_off + uint32_t(kk) * 2u * lbo, lbo, 128u);
             umma_f16(acc + 128u, da, dbl, idesc, kk > 0);
             umma_f16(acc + 128u, dal, db, idesc, true);
           }
         }
-        umma_commit(&mbar[b]);
+        umma_commit(&mma_done[b]);
+        if (loaded < steps) {  // into the buffer that step it - 1 has read
+          if (it > 0) ok = mbar_wait(&mma_done[b ^ 1], uint32_t((it - 1) >> 1) & 1u, kWait);
+          if (ok) load_point_tile();
+        }
+        if (++j == ntile) {
+          j = 0;
+          ++q;
+        }
+        if (++pb == a.nbuf) {
+          pb = 0;
+          pphase ^= 1u;
+        }
       }
-      // B[b ^ 1] held tile j - 1, whose MMA finished before its candidates were read
-      if (j + 1 < npt) load_tile(j + 1, b ? sB0 : sB1, sPn + (b ^ 1) * kTcP);
-      const bool ok = mbar_wait(&mbar[b], b ? phase1 : phase0, 1 << 24);
-      if (b) phase1 ^= 1u;
-      else phase0 ^= 1u;
-      if (!__syncthreads_and(ok)) {  // the MMA never completed: report, stop (uniform)
-        if (t == 0) raise_status(a.status, kDevOverflow, -3);
-        dead = true;
-        break;
+      if (!ok) {  // a wait ran out: report, let the copies in flight land, stop
+        raise_status(a.status, kDevOverflow, -3);
+        for (int s = loaded > a.nbuf ? loaded - a.nbuf : 0; s < loaded; ++s) {
+          mbar_wait(&full[s % a.nbuf], uint32_t(s / a.nbuf) & 1u, kWait);
+          mbar_wait(&nfull[s % kTcNorms], uint32_t(s / kTcNorms) & 1u, kWait);
+        }
       }
-      tc_fence_after();
-      // ---- this tile's candidates
+    }
+  } else {
+    // ---------------- candidates: threads tl and 128 + tl, query tl of the tile ----------------
+    const int tl = t & (kTcQ - 1), half = t >> 7, quad = warp & 3;
+    const long long dir = half ? -8 : 8;
+    const float inf = __int_as_float(0x7f800000);
+    float tau = inf, nqq = 0.f, sq = 0.f, width = 0.f;  // width: cut_width of every point met
+    int cnt = 0, limit = kTcCut;
+    int q = q_first, j = j_first;
+    int64_t qi = 0;
+    bool qlive = false;
+    uint2 *cbuf = nullptr, *cnext = nullptr;
+    unsigned* tq = nullptr;
+    bool ok = true;
+    float shared_tau = inf;  // of the query's other parts, loaded a step ahead, as the tile's norms are
+    float2 tm = steps > 0 ? a.tmax[j] : make_float2(0.f, 0.f);
+    // A warp whose wait runs out takes no more candidates, but stays with its
+    // partner's barriers to the end.
+    for (int it = 0; it < steps; ++it) {
+      const int b = it & 1;
+      if (it == 0 || j == 0) {  // a new part
+        qi = (a.qt0 + q) * kTcQ + tl;
+        qlive = qi < a.nq;
+        nqq = qlive ? a.qnorm[qi] : 0.f;
+        sq = sqrtf(nqq);
+        cbuf = a.cand + (int64_t(blockIdx.x + q) * kTcQ + tl) * kTcCand;
+        tq = a.tauq + int64_t(q) * kTcQ + tl;
+        if (half) cbuf += kTcCand - 1;  // this thread's own start
+        cnext = cbuf;
+        cnt = 0;
+        limit = kTcCut;
+        tau = inf;
+        width = 0.f;
+        shared_tau = fkey_inv(__ldcg(tq));
+      }
+      // tau as lowered meanwhile by the query's other parts (any value that was
+      // ever there is a valid one; not a number: none yet)
+      tau = fminf(tau, shared_tau);
       float thr = tau;
       if (!a.exact) {
-        const float2 tm = a.tmax[j];
-        thr = (tau + tc_err(a, nqq, sq, tm.x, tm.y)) * 1.000001f;  // never below tau + err of a point
+        // never below the upper end of what lb <= tau admits, with the roundings of the test itself
+        const float e = tc_err(a, nqq, sq, tm.x, tm.y);
+        width = fmaxf(width, cut_width(e, nqq + tm.x));
+        thr = (tau + e) * 1.000002f + 4.7683716e-07f * (nqq + tm.x);
+      } else {
+        thr = tau + 1.f;  // integers: d2 <= tau as d2 - (tau + 1) < 0
       }
-      const int64_t p0 = j * kTcP;
+      const bool tail = int64_t(j + 1) * kTcP > a.n;
+      const float base = nqq - thr;
+      const float* pnb = sPn + (it % kTcNorms) * kTcP;
+      ok = ok && mbar_wait(&nfull[it % kTcNorms], uint32_t(it / kTcNorms) & 1u, kWait);
+      ok = ok && mbar_wait(&mma_done[b], uint32_t(it >> 1) & 1u, kWait);
+      ok = __all_sync(0xffffffffu, ok);
+      tc_fence_after();
+      shared_tau = fkey_inv(__ldcg(tq));
+      tm = a.tmax[j + 1 < ntile ? j + 1 : 0];
+      const int64_t p0 = int64_t(j) * kTcP;
 #pragma unroll 1
-      for (int c0 = 0; c0 < kTcP; c0 += 32) {
+      for (int c0 = half * (kTcP / 2); ok && c0 < (half + 1) * (kTcP / 2); c0 += 32) {
         uint32_t v[32], v2[kSplit ? 32 : 1];
-        const uint32_t acc = tmem + (uint32_t(32 * warp) << 16) + uint32_t(b) * kSetCols + uint32_t(c0);
+        const uint32_t acc = tmem + (uint32_t(32 * quad) << 16) + uint32_t(b) * kSetCols + uint32_t(c0);
         tmem_ld32(acc, v);
         if constexpr (kSplit) tmem_ld32(acc + 128u, *reinterpret_cast<uint32_t(*)[32]>(v2));
         tmem_ld_wait();
-        if (!qlive) continue;
+        if (c0 + 32 == (half + 1) * (kTcP / 2)) {  // the last read of this set
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&acc_free[b]);
+        }
+        // float rows: hi hi^T + 2^-11 (hi lo^T + lo hi^T), scaled units
+        if constexpr (kSplit) {
 #pragma unroll
-        for (int jj = 0; jj < 32; ++jj) {
-          const int c = c0 + jj;
-          const float pn = pnb[c];
-          // float rows: hi hi^T + 2^-11 (hi lo^T + lo hi^T), scaled units
-          const float G = kSplit ? fmaf(__uint_as_float(v2[jj]), 4.8828125e-04f, __uint_as_float(v[jj]))
-                                 : __uint_as_float(v[jj]);
-          const float d2 = fmaf(-2.f, G, nqq + pn);
-          if (d2 <= thr) {
-            const int64_t pid = p0 + c;
-            if (pid >= a.n || (!a.Qraw && pid == qi)) continue;
-            float lb = d2, ub = d2;
-            if (!a.exact) {
-              const float err = tc_err(a, nqq, sq, pn, sqrtf(pn));
-              lb = d2 - err;
-              ub = d2 + err;
-            }
-            if (lb <= tau) {
-              if (cnt < a.capc) cbuf[cnt++] = make_uint4(__float_as_uint(lb), __float_as_uint(ub), unsigned(pid), 0u);
-              else raise_status(a.status, kDevOverflow, qi);
-            }
+          for (int jj = 0; jj < 32; ++jj)
+            v[jj] = __float_as_uint(fmaf(__uint_as_float(v2[jj]), 4.8828125e-04f, __uint_as_float(v[jj])));
+        }
+#pragma unroll
+        for (int g = 0; g < 32; g += 8) {
+          const float4 pa = *reinterpret_cast<const float4*>(pnb + c0 + g);
+          const float4 pb = *reinterpret_cast<const float4*>(pnb + c0 + g + 4);
+          const float pn[8] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w};
+          unsigned m = 0;
+#pragma unroll
+          for (int e = 7; e >= 0; --e)
+            m = __funnelshift_l(__float_as_uint(fmaf(-2.f, __uint_as_float(v[g + e]), base + pn[e])), m, 1);
+          if (!qlive) m = 0;
+          if (tail) {  // the last tile: columns past n
+            const int64_t left = a.n - (p0 + c0 + g);
+            m &= left >= 8 ? 0xffu : left > 0 ? (1u << int(left)) - 1u : 0u;
           }
+          if (!__any_sync(0xffffffffu, m != 0)) continue;
+          const unsigned id0 = unsigned(p0) + unsigned(c0 + g);
+#pragma unroll
+          for (int e = 0; e < 8; ++e)  // at most kTcP more a tile: the buffer has room
+            push_if((m >> e) & 1u, cnext, dir, __float_as_uint(fmaf(-2.f, __uint_as_float(v[g + e]), nqq + pn[e])),
+                    id0 + unsigned(e));
         }
       }
-      // ---- buffers that could overflow on the next tile: lower tau, drop what lies above it
-      unsigned need = __ballot_sync(0xffffffffu, cnt > a.capc - kTcP);
-      __syncwarp();  // candidates written by one lane are read by the whole warp below
-      while (need) {
-        const int L = __ffs(need) - 1;
-        need &= need - 1;
-        const int cL = __shfl_sync(0xffffffffu, cnt, L);
-        uint4* bL = a.cand + (int64_t(blockIdx.x) * kTcQ + warp * 32 + L) * a.capc;
-        for (int i = lane; i < cL; i += 32)
-          wsort[i] = (static_cast<unsigned long long>(fkey(__uint_as_float(bL[i].y))) << 32) | unsigned(i);
-        __syncwarp();
-        warp_sort(wsort, cL);
-        const float tnew = cL >= a.k ? fkey_inv(unsigned(wsort[a.k - 1] >> 32)) : inf;
-        __syncwarp();
-        int w = 0;
-        for (int i0 = 0; i0 < cL; i0 += 32) {
-          const int i = i0 + lane;
-          uint4 e = make_uint4(0, 0, 0, 0);
-          bool keep = false;
-          if (i < cL) {
-            e = bL[i];
-            keep = __uint_as_float(e.x) <= tnew;
+      // ---- both threads of a query know its length
+      cnt = half ? int(cbuf - cnext) : int(cnext - cbuf);
+      sCnt[half * kTcQ + tl] = cnt;
+      named_sync(1 + quad, 64);  // and what either has stored
+      const int other = sCnt[(half ^ 1) * kTcQ + tl];
+      // ---- long buffers: lower tau, drop what lies above it; every other one of
+      // the quadrant's by either warp
+      const unsigned need = __ballot_sync(0xffffffffu, cnt + other > limit);
+      if (need) {  // the same in both warps
+        named_sync(1 + quad, 64);  // sCnt read
+        int nth = 0;
+        for (unsigned todo = need; todo; todo &= todo - 1, ++nth) {
+          if ((nth & 1) != half) continue;
+          const int L = __ffs(int(todo)) - 1;
+          const int own = __shfl_sync(0xffffffffu, cnt, L), oth = __shfl_sync(0xffffffffu, other, L);
+          const float wL = __shfl_sync(0xffffffffu, width, L);
+          const int nA = half ? oth : own, cL = own + oth, ql = quad * 32 + L;
+          uint2* bL = a.cand + (int64_t(blockIdx.x + q) * kTcQ + ql) * kTcCand;
+          // cL > kTcCut >= kscan
+          const float tnew = fkey_inv(kth_of<kTcCand / 32>(bL, cL, a.kscan, nA, kTcCand - cL)) + wL;
+          const int w = cut_above(bL, cL, tnew, wL, nA, kTcCand - cL);
+          if (lane == 0) {
+            sCnt[ql] = w;
+            sTau[ql] = tnew;
+            atomicMin(a.tauq + int64_t(q) * kTcQ + ql, fkey(tnew));
+            if (w > kTcCand - kTcP) raise_status(a.status, kDevOverflow, (a.qt0 + q) * kTcQ + ql);
           }
-          const unsigned km = __ballot_sync(0xffffffffu, keep);
-          __syncwarp();
-          if (keep) bL[w + __popc(km & ((1u << lane) - 1))] = e;
-          w += __popc(km);
           __syncwarp();
         }
-        if (lane == L) {
-          cnt = w;
-          tau = fminf(tau, tnew);
-          if (cnt > a.capc - kTcP) raise_status(a.status, kDevOverflow, qi);
+        named_sync(1 + quad, 64);
+        if ((need >> lane) & 1u) {
+          const int w = sCnt[tl];
+          cnt = half ? 0 : w;
+          cnext = half ? cbuf : cbuf + w;
+          tau = fminf(tau, sTau[tl]);
+          limit = min(max(kTcCut, w + 96), kTcCand - kTcP);
+          if (w > kTcCand - kTcP) qlive = false;  // no room for the next tile: reported, take no more
         }
-        __syncwarp();
+      }
+      if (it + 1 == steps || j + 1 == ntile) {
+        // the part's candidates; `other` as it stands after a cut
+        const int second = half ? cnt : (need >> lane) & 1u ? 0 : other;
+        if (!half) a.pcnt[int64_t(blockIdx.x + q) * kTcQ + tl] = cnt | (second << 16);
+      }
+      named_sync(1 + quad, 64);  // sCnt and sTau read before the next step writes them
+      if (++j == ntile) {
+        j = 0;
+        ++q;
       }
     }
-    if (dead) break;
-    // ---- exact ranking of each query's candidates, one warp per query in turn
-    for (int L = 0; L < 32; ++L) {
-      const int64_t qg = qt * kTcQ + warp * 32 + L;
-      if (qg >= a.nq) break;
-      const int cL = __shfl_sync(0xffffffffu, cnt, L);
-      const float tL = __shfl_sync(0xffffffffu, tau, L);
-      const uint4* bL = a.cand + (int64_t(blockIdx.x) * kTcQ + warp * 32 + L) * a.capc;
-      const uint8_t* qrow = a.Qraw ? a.Qraw + qg * a.row_bytes : a.X + qg * a.row_bytes;
-      int m = 0;
-      for (int i0 = 0; i0 < cL; i0 += 32) {
-        const int i = i0 + lane;
-        bool keep = false;
-        unsigned long long key = 0;
-        if (i < cL) {
-          const uint4 e = bL[i];
-          keep = __uint_as_float(e.x) <= tL;
-          if (keep) {
-            const uint2* x2 = reinterpret_cast<const uint2*>(qrow);
-            const uint2* y2 = reinterpret_cast<const uint2*>(a.X + int64_t(e.z) * a.row_bytes);
-            unsigned acc = 0;
-            for (int64_t s0 = 0; s0 < a.row_bytes / 8; s0 += 16) {  // per 128-byte slice, as the CUDA-core kernel
-              unsigned part = 0;
-              for (int w8 = 0; w8 < 16; ++w8) acc_pair<DT>(x2[s0 + w8], y2[s0 + w8], part);
-              if constexpr (DT == kU8) acc += part;
-              else acc = __float_as_uint(__uint_as_float(acc) + __uint_as_float(part));
-            }
-            key = (static_cast<unsigned long long>(acc) << 32) | e.z;
-          }
-        }
-        const unsigned km = __ballot_sync(0xffffffffu, keep);
-        if (keep) wsort[m + __popc(km & ((1u << lane) - 1))] = key;
-        m += __popc(km);
-      }
-      __syncwarp();
-      warp_sort(wsort, m);
-      const int nc = min(m, a.k);
-      if constexpr (DT == kF32) {
-        if (lane == 0) fix_near_ties(a.X, a.row_bytes, a.d, a.status, wsort, m, reinterpret_cast<const float*>(qrow), qg);
-        __syncwarp();
-      }
-      for (int j = lane; j < a.k; j += 32) {
-        const bool have = j < nc;
-        a.out_ids[qg * a.k + j] = have ? int32_t(unsigned(wsort[j])) : -1;
-        if (a.out_dists) {
-          const unsigned kb = unsigned(wsort[j] >> 32);
-          a.out_dists[qg * a.k + j] = !have ? inf : (DT == kU8 ? float(kb) : __uint_as_float(kb));
-        }
-      }
-      __syncwarp();
-    }
+    if (!ok && lane == 0) raise_status(a.status, kDevOverflow, -4);
   }
-  cp_async_wait<0>();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   if (warp == 0) tmem_dealloc(tmem, 2 * kSetCols);
+}
+
+template <int DT>
+__global__ void __launch_bounds__(128) knn_rank_kernel(KnnTcArgs a) {
+  __shared__ uint2 sbuf[4][kRankCand];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t ql = int64_t(blockIdx.x) * 4 + warp;  // query of the chunk
+  const int64_t qg = a.qt0 * kTcQ + ql;
+  if (ql >= a.nqt * kTcQ || qg >= a.nq) return;
+  const int64_t npt = (a.n + kTcP - 1) / kTcP, qt = ql / kTcQ;
+  const int t = int(ql % kTcQ);
+  const float inf = __int_as_float(0x7f800000);
+  uint2* e = sbuf[warp];
+  float tau = fminf(inf, fkey_inv(a.tauq[ql]));  // never lowered: all ones, not a number
+  float w = 0.f;
+  if (!a.exact) {
+    const float nqq = a.qnorm[qg];
+    const float2 tm = a.tmax[npt];  // over all points
+    w = cut_width(tc_err(a, nqq, sqrtf(nqq), tm.x, tm.y), nqq + tm.x);
+  }
+  // ---- the candidates of the query's parts, cut to the smallest tau
+  int m = 0;
+  bool over = false;
+  auto lower = [&]() {  // tau from what is held
+    if (m < a.k) return;
+    const float tnew = fkey_inv(kth_of<kRankCand / 32>(e, m, a.k, kRankCand)) + w;
+    tau = fminf(tau, tnew);
+    m = cut_above(e, m, tau, w, kRankCand);
+  };
+  const int64_t c1 = ((qt + 1) * npt - 1) / a.per;
+  for (int64_t c = qt * npt / a.per; c <= c1; ++c) {
+    const int64_t part = (c + qt) * kTcQ + t;
+    const int nA = a.pcnt[part] & 0xffff, cn = nA + (a.pcnt[part] >> 16), gap = kTcCand - cn;
+    const uint2* src = a.cand + part * kTcCand;
+    for (int i0 = 0; i0 < cn; i0 += 32) {
+      if (m > kRankCand - 32) {
+        __syncwarp();
+        lower();
+        if (m > kRankCand - 32) {
+          over = true;
+          break;
+        }
+      }
+      const int i = i0 + lane;
+      uint2 v = make_uint2(0, 0);
+      if (i < cn) v = src[entry_at(i, nA, gap)];
+      const bool self = !a.Qraw && int64_t(v.y) == qg;
+      const bool keep = i < cn && !self && __uint_as_float(v.x) - w <= tau;
+      const unsigned km = __ballot_sync(0xffffffffu, keep);
+      if (keep) e[m + __popc(km & ((1u << lane) - 1))] = v;
+      m += __popc(km);
+      __syncwarp();
+    }
+  }
+  if (over && lane == 0) raise_status(a.status, kDevOverflow, qg);
+  lower();
+  // ---- exact keys: four lanes per row
+  unsigned long long* keys = reinterpret_cast<unsigned long long*>(e);
+  const uint8_t* qrow = a.Qraw ? a.Qraw + qg * a.row_bytes : a.X + qg * a.row_bytes;
+  const int ns = int(a.row_bytes / 128);  // at most four slices of 128 bytes
+  const int sub = lane & 3;
+  for (int i0 = 0; i0 < m; i0 += 8) {
+    const int i = i0 + (lane >> 2);
+    const unsigned id = e[i < m ? i : m - 1].y;
+    const uint4* x = reinterpret_cast<const uint4*>(qrow);
+    const uint4* y = reinterpret_cast<const uint4*>(a.X + int64_t(id) * a.row_bytes);
+    unsigned key;
+    if constexpr (DT == kU8) {
+      unsigned part = 0;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const uint4 p = __ldg(x + sub + 4 * h), q = __ldg(y + sub + 4 * h);
+        acc_pair<DT>(make_uint2(p.x, p.y), make_uint2(q.x, q.y), part);
+        acc_pair<DT>(make_uint2(p.z, p.w), make_uint2(q.z, q.w), part);
+      }
+      part += __shfl_xor_sync(0xffffffffu, part, 1);
+      part += __shfl_xor_sync(0xffffffffu, part, 2);
+      key = part;
+    } else {
+      // a lane sums one slice in index order; the slice sums are added in order,
+      // as the CUDA-core kernel does
+      unsigned part = 0;
+      if (sub < ns) {
+        uint4 p[8], q[8];
+#pragma unroll
+        for (int h = 0; h < 8; ++h) {
+          p[h] = __ldg(x + 8 * sub + h);
+          q[h] = __ldg(y + 8 * sub + h);
+        }
+#pragma unroll
+        for (int h = 0; h < 8; ++h) {
+          acc_pair<DT>(make_uint2(p[h].x, p[h].y), make_uint2(q[h].x, q[h].y), part);
+          acc_pair<DT>(make_uint2(p[h].z, p[h].w), make_uint2(q[h].z, q[h].w), part);
+        }
+      }
+      float acc = 0.f;
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        const float ps = __uint_as_float(__shfl_sync(0xffffffffu, part, (lane & ~3) + s));
+        if (s < ns) acc += ps;
+      }
+      key = __float_as_uint(acc);
+    }
+    __syncwarp();
+    if (sub == 0 && i < m) keys[i] = (static_cast<unsigned long long>(key) << 32) | id;
+    __syncwarp();
+  }
+  warp_sort(keys, m);
+  const int nc = min(m, a.k);
+  if constexpr (DT == kF32) {
+    if (lane == 0) fix_near_ties(a.X, a.row_bytes, a.d, a.status, keys, m, reinterpret_cast<const float*>(qrow), qg);
+    __syncwarp();
+  }
+  for (int j = lane; j < a.k; j += 32) {
+    const bool have = j < nc;
+    a.out_ids[qg * a.k + j] = have ? int32_t(unsigned(keys[j])) : -1;
+    if (a.out_dists) {
+      const unsigned kb = unsigned(keys[j] >> 32);
+      a.out_dists[qg * a.k + j] = !have ? inf : (DT == kU8 ? float(kb) : __uint_as_float(kb));
+    }
+  }
 }
 
 // ---- packing: f16 operand tiles, scaled squared norms, per-tile maxima
@@ -638,19 +895,24 @@ __global__ void pack_f16_kernel(const uint8_t* __restrict__ X, int64_t row_bytes
   const int64_t op_bytes = int64_t(kTcP) * dpad * 2;
   uint8_t* tb = tiles + tile * op_bytes * tc_nop(DT);
   float acc = 0.f;
+  const uint8_t* row = X + i * row_bytes;  // padded with zeros past d, and row_bytes covers dpad
   for (int kc = 0; kc < dpad / 8; ++kc) {
-    float v[8];
+    float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (i < n) {
+      if constexpr (DT == kU8) {
+        const uint2 w = *reinterpret_cast<const uint2*>(row + kc * 8);
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int c = kc * 8 + e;
-      float x = 0.f;
-      if (i < n && c < d) {
-        if constexpr (DT == kU8) x = float(X[i * row_bytes + c]);
-        else x = reinterpret_cast<const float*>(X + i * row_bytes)[c] * s;
+        for (int e = 0; e < 8; ++e) v[e] = float(((e < 4 ? w.x : w.y) >> (8 * (e & 3))) & 0xffu);
+      } else {
+        const float4 p = *reinterpret_cast<const float4*>(row + kc * 32);
+        const float4 q = *reinterpret_cast<const float4*>(row + kc * 32 + 16);
+        const float x[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = x[e] * s;
       }
-      v[e] = x;
-      acc = fmaf(x, x, acc);
     }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc = fmaf(v[e], v[e], acc);
     const int64_t at = (int64_t(kc) * 16 + r / 8) * 128 + (r % 8) * 16;
     if constexpr (DT == kF32) {
       uint4 hi, lo;
@@ -668,7 +930,8 @@ __global__ void pack_f16_kernel(const uint8_t* __restrict__ X, int64_t row_bytes
   norms[i] = acc;
 }
 
-// per tile: (max |x'|^2, max |x'|), the latter rounded up
+// per tile: (max |x'|^2, max |x'|), the latter rounded up; out[ntile], zeroed
+// before, takes the largest of each
 __global__ void tile_max_kernel(const float* __restrict__ norms, int64_t ntile, float2* __restrict__ out) {
   const int64_t tile = int64_t(blockIdx.x) * (blockDim.x / 32) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -677,7 +940,13 @@ __global__ void tile_max_kernel(const float* __restrict__ norms, int64_t ntile, 
   for (int r = lane; r < kTcP; r += 32) m = fmaxf(m, norms[tile * kTcP + r]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) out[tile] = make_float2(m, sqrtf(m) * 1.000001f);
+  if (lane == 0) {
+    const float root = sqrtf(m) * 1.000001f;
+    out[tile] = make_float2(m, root);
+    unsigned* all = reinterpret_cast<unsigned*>(out + ntile);  // bits of non-negative floats
+    atomicMax(all, __float_as_uint(m));
+    atomicMax(all + 1, __float_as_uint(root));
+  }
 }
 
 }  // namespace
@@ -727,9 +996,9 @@ bool knn_tc_eligible(int dtype, int d, int k) {
 
 namespace {
 struct TcPlan {
-  int dpad, capc, ctas, grid;
-  int64_t ntile, nqtile, tile_bytes;
-  size_t off_ptiles, off_pnorm, off_tmax, off_qtiles, off_qnorm, off_cand, total;
+  int dpad, nbuf, ctas, grid;
+  int64_t ntile, nqtile, chunk, tile_bytes;
+  size_t off_ptiles, off_pnorm, off_tmax, off_qtiles, off_qnorm, off_cand, off_pcnt, off_tauq, total;
 };
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
@@ -737,28 +1006,56 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 TcPlan tc_plan(int dtype, int d, int64_t n, int64_t nq_ext, int num_sms) {
   TcPlan P{};
   P.dpad = (d + 15) / 16 * 16;
-  P.capc = 512;
   P.tile_bytes = int64_t(kTcP) * P.dpad * 2 * tc_nop(dtype);
-  const size_t smem = knn_tc_smem(dtype, P.tile_bytes, P.capc);
+  P.nbuf = knn_tc_smem(dtype, P.tile_bytes, 3) <= size_t(227) * 1024 ? 3 : 2;  // float rows past 112 dimensions: 2
+  if (dtype == kU8) P.nbuf = 2;                                              // two CTAs share an SM
+  const size_t smem = knn_tc_smem(dtype, P.tile_bytes, P.nbuf);
   P.ctas = int(std::max<size_t>(1, std::min<size_t>(2, size_t(228 * 1024) / (smem + 1024))));
   P.grid = num_sms * P.ctas;
+  // query tiles per launch: as many as there are CTAs, less four, which makes up
+  // to 2 grid - 4 parts of 512 KB
+  P.chunk = std::max(P.grid - 4, 1);
   P.ntile = (n + kTcP - 1) / kTcP;
   P.nqtile = (nq_ext + kTcQ - 1) / kTcQ;
-  size_t o = 256;  // header: max |x| bits at 0, query-tile counter at 64
+  const size_t parts = size_t(P.grid) + size_t(P.chunk);
+  size_t o = 256;  // header: max |x| bits at 0
   P.off_ptiles = o;
   o = align256(o + size_t(P.ntile) * P.tile_bytes);
   P.off_pnorm = o;
   o = align256(o + size_t(P.ntile) * kTcP * 4);
   P.off_tmax = o;
-  o = align256(o + size_t(P.ntile) * 8);
+  o = align256(o + size_t(P.ntile + 1) * 8);
   P.off_qtiles = o;
   o = align256(o + size_t(P.nqtile) * P.tile_bytes);
   P.off_qnorm = o;
   o = align256(o + size_t(P.nqtile) * kTcQ * 4);
   P.off_cand = o;
-  o = align256(o + size_t(P.grid) * kTcQ * P.capc * 16);
+  o = align256(o + parts * kTcQ * kTcCand * 8);
+  P.off_pcnt = o;
+  o = align256(o + parts * kTcQ * 4);
+  P.off_tauq = o;
+  o = align256(o + size_t(P.chunk) * kTcQ * 4);
   P.total = o;
   return P;
+}
+
+template <int DT>
+cudaError_t scan_and_rank(KnnTcArgs a, const TcPlan& P, cudaStream_t s) {
+  const size_t smem = knn_tc_smem(DT, P.tile_bytes, P.nbuf);
+  cudaError_t err = cudaFuncSetAttribute(knn_scan_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  if (err != cudaSuccess) return err;
+  const int64_t nqt = (a.nq + kTcQ - 1) / kTcQ;
+  for (a.qt0 = 0; a.qt0 < nqt; a.qt0 += P.chunk) {
+    a.nqt = std::min(P.chunk, nqt - a.qt0);
+    const int64_t total = a.nqt * P.ntile;
+    a.per = std::max<int64_t>((total + P.grid - 1) / P.grid, std::min<int64_t>(P.ntile, kTcMinSteps));
+    if ((err = cudaMemsetAsync(a.tauq, 0xff, size_t(a.nqt) * kTcQ * 4, s)) != cudaSuccess) return err;
+    if ((err = cudaMemsetAsync(a.pcnt, 0, size_t(P.grid + P.chunk) * kTcQ * 4, s)) != cudaSuccess) return err;
+    knn_scan_kernel<DT><<<unsigned((total + a.per - 1) / a.per), kTcThreads, smem, s>>>(a);
+    knn_rank_kernel<DT><<<unsigned(a.nqt * kTcQ / 4), 128, 0, s>>>(a);
+    if ((err = cudaGetLastError()) != cudaSuccess) return err;
+  }
+  return cudaSuccess;
 }
 }  // namespace
 
@@ -766,27 +1063,28 @@ size_t knn_tc_scratch_bytes(int dtype, int d, int64_t n, int64_t nq_ext, int num
   return tc_plan(dtype, d, n, nq_ext, num_sms).total;
 }
 
-cudaError_t launch_knn_tc(const KnnTcLaunch& K, cudaStream_t s) {
+cudaError_t launch_knn_tc(const KnnTcLaunch& K, cudaStream_t s, int64_t* kernels) {
   const bool f32 = K.data.dtype == kF32;
   const TcPlan P = tc_plan(K.data.dtype, K.data.d, K.data.n, K.Q ? K.nq : 0, K.num_sms);
   uint8_t* base = K.scratch;
   unsigned* maxbits = reinterpret_cast<unsigned*>(base);
-  unsigned* work = reinterpret_cast<unsigned*>(base + 64);
   cudaError_t err = cudaMemsetAsync(base, 0, 256, s);
   if (err != cudaSuccess) return err;
-  // the scale: a power of two that brings max |x| (points and queries) to at most 1
-  float scale = 1.f;
-  if (f32) {
-    maxabs_kernel<<<1024, 256, 0, s>>>(K.data.X, K.data.row_bytes, K.data.n, K.data.d, maxbits);
-    if (K.Q) maxabs_kernel<<<256, 256, 0, s>>>(K.Q, K.data.row_bytes, K.nq, K.data.d, maxbits);
+  // the scale: a power of two that brings max |x| (points, known since their
+  // load, and queries) to at most 1
+  float scale = f32 ? K.data.scale : 1.f;
+  if (f32 && K.Q) {
+    maxabs_kernel<<<256, 256, 0, s>>>(K.Q, K.data.row_bytes, K.nq, K.data.d, maxbits);
     unsigned mb = 0;
     if ((err = cudaMemcpyAsync(&mb, maxbits, 4, cudaMemcpyDeviceToHost, s)) != cudaSuccess) return err;
     if ((err = cudaStreamSynchronize(s)) != cudaSuccess) return err;
     float mx = 0.f;
     memcpy(&mx, &mb, 4);
     int e = 0;
-    if (mx > 0.f && std::isfinite(mx)) std::frexp(mx, &e);  // mx < 2^e
-    scale = std::ldexp(1.f, -e);
+    if (mx > 0.f && std::isfinite(mx)) {
+      std::frexp(mx, &e);  // mx < 2^e
+      scale = std::min(scale, std::ldexp(1.f, -e));
+    }
   }
   uint8_t* ptiles = base + P.off_ptiles;
   float* pnorm = reinterpret_cast<float*>(base + P.off_pnorm);
@@ -798,6 +1096,7 @@ cudaError_t launch_knn_tc(const KnnTcLaunch& K, cudaStream_t s) {
   else
     pack_f16_kernel<kU8><<<unsigned((rows + 255) / 256), 256, 0, s>>>(K.data.X, K.data.row_bytes, K.data.n, K.data.d,
                                                                      P.dpad, 1.f, ptiles, pnorm);
+  if ((err = cudaMemsetAsync(tmax + P.ntile, 0, 8, s)) != cudaSuccess) return err;
   tile_max_kernel<<<unsigned((P.ntile + 7) / 8), 256, 0, s>>>(pnorm, P.ntile, tmax);
   const uint8_t* qtiles = ptiles;
   const float* qnorm = pnorm;
@@ -827,10 +1126,12 @@ cudaError_t launch_knn_tc(const KnnTcLaunch& K, cudaStream_t s) {
   a.ptiles = ptiles;
   a.tile_bytes = P.tile_bytes;
   a.ksteps = P.dpad / 16;
+  a.nbuf = P.nbuf;
   a.qnorm = qnorm;
   a.pnorm = pnorm;
   a.tmax = tmax;
   a.exact = f32 ? 0 : 1;
+  a.kscan = K.Q ? K.k : K.k + 1;
   // Split Gram of scaled rows: |G~ - G| <= eps_ip |q'||p'| + 2^-36 sqrt(d) (|q'| + |p'|):
   // 2^-22 left by the split of each operand, 2^-22 for the dropped lo lo^T, 2^-23 for
   // the last sum, f32 accumulation d 2^-24 with a factor 4 allowance; the lo halves
@@ -838,25 +1139,15 @@ cudaError_t launch_knn_tc(const KnnTcLaunch& K, cudaStream_t s) {
   a.eps_ip = 4.f * 2.384185791015625e-07f + 1.1920929e-07f + float(K.data.d) * 2.384185791015625e-07f;
   a.eps_n = float(K.data.d + 2) * 5.9604645e-08f;
   a.sub_abs = std::sqrt(float(K.data.d)) * 1.001f * 2.910383e-11f;  // twice 2^-36 sqrt(d)
-  a.cand = reinterpret_cast<uint4*>(base + P.off_cand);
-  a.capc = P.capc;
+  a.cand = reinterpret_cast<uint2*>(base + P.off_cand);
+  a.pcnt = reinterpret_cast<int*>(base + P.off_pcnt);
+  a.tauq = reinterpret_cast<unsigned*>(base + P.off_tauq);
   a.out_ids = K.out_ids;
   a.out_dists = K.out_dists;
-  a.work = work;
   a.status = K.status;
-  const size_t smem = knn_tc_smem(K.data.dtype, P.tile_bytes, P.capc);
-  if (f32) {
-    if ((err = cudaFuncSetAttribute(knn_tc_kernel<kF32>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))) !=
-        cudaSuccess)
-      return err;
-    knn_tc_kernel<kF32><<<unsigned(P.grid), 128, smem, s>>>(a);
-  } else {
-    if ((err = cudaFuncSetAttribute(knn_tc_kernel<kU8>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))) !=
-        cudaSuccess)
-      return err;
-    knn_tc_kernel<kU8><<<unsigned(P.grid), 128, smem, s>>>(a);
-  }
-  return cudaGetLastError();
+  const int64_t chunks = ((K.nq + kTcQ - 1) / kTcQ + P.chunk - 1) / P.chunk;
+  *kernels = 2 + (K.Q ? (f32 ? 2 : 1) : 0) + 2 * chunks;
+  return f32 ? scan_and_rank<kF32>(a, P, s) : scan_and_rank<kU8>(a, P, s);
 }
 
 }  // namespace rpk

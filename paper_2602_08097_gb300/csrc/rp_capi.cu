@@ -696,10 +696,11 @@ rp_status run_knn(rp_ctx* c, const Dataset& D, const uint8_t* Q, int64_t nq, int
     K.status = c->status;
     K.num_sms = c->num_sms;
     K.scratch = static_cast<uint8_t*>(scratch);
-    const cudaError_t ce = launch_knn_tc(K, c->stream);
+    int64_t nk = 0;
+    const cudaError_t ce = launch_knn_tc(K, c->stream, &nk);
     dfree(c, scratch, bytes);
     if (ce != cudaSuccess) return fail(c, RP_ECUDA, "tensor-core kNN: %s", cudaGetErrorString(ce));
-    c->kernel_launches += D.dtype == RP_F32 ? 5 : 3;
+    c->kernel_launches += nk;
     c->last_knn_method = RP_KNN_TENSOR;
     return RP_OK;
   }
