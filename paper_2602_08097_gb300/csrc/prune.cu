@@ -140,6 +140,26 @@ __device__ __forceinline__ typename Acc<DT>::T row_d2(const uint8_t* a, const ui
   return acc;
 }
 
+// The same where either row may be in shared memory (plain loads).
+template <int DT>
+__device__ __forceinline__ typename Acc<DT>::T row_d2_any(const uint8_t* a, const uint8_t* b, int64_t row_bytes) {
+  typename Acc<DT>::T acc = 0;
+  const uint4* pa = reinterpret_cast<const uint4*>(a);
+  const uint4* pb = reinterpret_cast<const uint4*>(b);
+  const int nv = int(row_bytes / 16);
+  for (int c0 = 0; c0 < nv; c0 += 8) {
+    typename Acc<DT>::T part = 0;
+    if (c0 + 8 <= nv) {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) part = Acc<DT>::step4(pa[c0 + c], pb[c0 + c], part);
+    } else {
+      for (int c = c0; c < nv; ++c) part = Acc<DT>::step4(pa[c], pb[c], part);
+    }
+    acc += part;
+  }
+  return acc;
+}
+
 // The tiers past single precision for float rows.  First float-float
 // distances (error (3d + 13) 2^-48 relative, ff_bound), whose intervals settle
 // the canonical decision fl(A^2 d2a) <= fl(1e6 d2b) unless the two products'
@@ -1208,13 +1228,56 @@ __global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_ker
 // ---------------------------------------------------------------------------
 // generic path: one node per CTA, any degree up to RP_MAX_DEGREE
 // ---------------------------------------------------------------------------
+// The candidates are sorted once, then taken 32 at a time in processing order, one
+// per lane: first each of the batch is held against the points kept so far (a
+// warp takes every eighth of them), then the survivors against one another (a
+// warp takes every eighth survivor), and the batch's greedy scan runs on the
+// resulting bit masks.  So a node takes m / 32 rounds, not one per kept point,
+// and every candidate's row is read once.  The batch's rows, the next batch's and
+// the kept points' rows lie in shared memory as far as they fit, each padded by 16
+// bytes so that the lanes' 16-byte reads fall into different banks.
+//
+// What bounds it: a list of several hundred candidates (the point near the middle
+// of the data takes up to 512 back edges a batch in a Vamana build) occupies one
+// CTA and nothing else runs meanwhile.  30,000 x 96 float points, R 64: that list
+// (576 candidates) took 660 us with one round per kept point and rows from global
+// memory, now 105; all of the build's lists of more than 128 36.9 ms, now 6.3.
+constexpr int kGenThreads = 256;
+constexpr int kGenWarps = kGenThreads / 32;
+constexpr int kGenBatch = 32;
 struct GenericLayout {
-  // sort keys and, once sorted, the binary64 pivot-key cache share one array
-  __host__ __device__ static size_t bytes(int M2) { return size_t(M2) * 22 + 64; }
+  // sort keys and, once sorted, the binary64 pivot-key cache share one array; then
+  // ids, the order, the keys, the kept ranks, near-tie links; per batch: one mask
+  // per candidate, the dominated ones; misc
+  __host__ __device__ static size_t masks(int M2) { return size_t(M2) * 23 + (size_t(M2) & 3); }
+  __host__ __device__ static size_t rows(int M2) { return (masks(M2) + (kGenBatch + 2 + 16) * 4 + 127) & ~size_t(127); }
 };
 
+// d2 of row `b` from rows a0 and a1 (any of them in shared memory, plain loads),
+// summed as row_d2 sums them.
 template <int DT>
-__global__ void __launch_bounds__(256) prune_generic_kernel(PruneArgs a, int M2) {
+__device__ __forceinline__ void row_d2_two(const uint8_t* a0, const uint8_t* a1, const uint8_t* b, int64_t row_bytes,
+                                           typename Acc<DT>::T& s0, typename Acc<DT>::T& s1) {
+  const uint4* p0 = reinterpret_cast<const uint4*>(a0);
+  const uint4* p1 = reinterpret_cast<const uint4*>(a1);
+  const uint4* pb = reinterpret_cast<const uint4*>(b);
+  const int nv = int(row_bytes / 16);  // a multiple of 8
+  s0 = s1 = 0;
+  for (int c0 = 0; c0 < nv; c0 += 8) {
+    typename Acc<DT>::T t0 = 0, t1 = 0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const uint4 v = pb[c0 + c];
+      t0 = Acc<DT>::step4(p0[c0 + c], v, t0);
+      t1 = Acc<DT>::step4(p1[c0 + c], v, t1);
+    }
+    s0 += t0;
+    s1 += t1;
+  }
+}
+
+template <int DT>
+__global__ void __launch_bounds__(kGenThreads) prune_generic_kernel(PruneArgs a, int M2, int stage_rows) {
   using AT = typename Acc<DT>::T;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned long long* skey = reinterpret_cast<unsigned long long*>(smem_raw);
@@ -1222,10 +1285,19 @@ __global__ void __launch_bounds__(256) prune_generic_kernel(PruneArgs a, int M2)
   int32_t* ids = reinterpret_cast<int32_t*>(smem_raw + size_t(M2) * 8);
   int32_t* perm = reinterpret_cast<int32_t*>(smem_raw + size_t(M2) * 12);
   AT* key = reinterpret_cast<AT*>(smem_raw + size_t(M2) * 16);
-  unsigned char* alive = smem_raw + size_t(M2) * 20;
-  unsigned char* lnk = smem_raw + size_t(M2) * 21;
-  int* misc = reinterpret_cast<int*>(smem_raw + size_t(M2) * 22);
-  const int t = threadIdx.x, NT = blockDim.x;
+  uint16_t* kept_at = reinterpret_cast<uint16_t*>(smem_raw + size_t(M2) * 20);  // ranks of the kept points
+  unsigned char* lnk = smem_raw + size_t(M2) * 22;
+  unsigned* dmask = reinterpret_cast<unsigned*>(smem_raw + GenericLayout::masks(M2));  // [kGenBatch]
+  unsigned* dword = dmask + kGenBatch;                                                 // [2] dominated by kept points
+  int* misc = reinterpret_cast<int*>(dword + 2);
+  unsigned char* stage = smem_raw + GenericLayout::rows(M2);
+  const int64_t stride = a.row_bytes + 16;  // of a staged row
+  // staged rows: one or two batches, the rest for kept points
+  const int nbuf = stage_rows >= 3 * kGenBatch ? 2 : stage_rows >= kGenBatch ? 1 : 0;
+  const int kept_rows = stage_rows - nbuf * kGenBatch;
+  unsigned char* kept_stage = stage + nbuf * kGenBatch * stride;
+  const int nch = int(a.row_bytes / 16);
+  const int t = threadIdx.x, NT = kGenThreads, lane = t & 31, warp = t >> 5;
   const int count = *a.count;
   const float E = rel_bound(a.d), Eabs = abs_bound(a.d);
   long long done = 0;
@@ -1252,12 +1324,26 @@ __global__ void __launch_bounds__(256) prune_generic_kernel(PruneArgs a, int M2)
     // largest, sized for its longest list; the others sort no more than their own)
     int Mp = 1;
     while (Mp < m) Mp <<= 1;
+    for (int j = t; j < m; j += NT) ids[j] = a.col[e0 + j];
+    __syncthreads();
+    // pivot keys: four lanes per row, eight rows a warp at a time (rel_bound holds
+    // for any order of the sum)
+    for (int j0 = 8 * warp; j0 < m; j0 += 8 * kGenWarps) {
+      const int j = j0 + (lane >> 2);
+      const uint4* x = reinterpret_cast<const uint4*>(a.X + int64_t(ids[j < m ? j : m - 1]) * a.row_bytes);
+      const uint4* q = reinterpret_cast<const uint4*>(xp);
+      AT acc = 0;
+#pragma unroll 4
+      for (int c = lane & 3; c < nch; c += 4) acc = Acc<DT>::step4(__ldg(x + c), __ldg(q + c), acc);
+      acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+      acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+      if ((lane & 3) == 0 && j < m) key[j] = acc;
+    }
+    __syncthreads();
     for (int j = t; j < Mp; j += NT) {
       if (j < m) {
-        const int32_t v = a.col[e0 + j];
-        ids[j] = v;
-        const AT kv = row_d2<DT>(xp, a.X + int64_t(v) * a.row_bytes, a.row_bytes);
-        key[j] = kv;
+        const int32_t v = ids[j];
+        const AT kv = key[j];
         skey[j] = a.variant == 0 ? (Acc<DT>::bits(kv) << 32) | unsigned(v) : (unsigned long long)j;
       } else {
         skey[j] = ~0ull;
@@ -1328,49 +1414,106 @@ __global__ void __launch_bounds__(256) prune_generic_kernel(PruneArgs a, int M2)
     }
     __syncthreads();
 
+    // the rows of ranks i0 .. i0 + 31 into batch buffer b
+    auto load_batch = [&](int i0, int b) {
+      const int nb = min(kGenBatch, m - i0);
+      for (int i = t; i < nb * nch; i += NT) {
+        const int r = i / nch, c = i - r * nch;
+        cp_async16(stage + (b * kGenBatch + r) * stride + c * 16,
+                   a.X + int64_t(ids[perm[i0 + r]]) * a.row_bytes + c * 16, 16);
+      }
+      cp_async_commit();
+    };
     for (int tt = 0; tt < a.T; ++tt) {
       const int64_t A2 = int64_t(a.A[tt]) * a.A[tt];
       const int R = a.R[tt];
       int32_t* out = a.out_col[tt] + e0;
-      for (int j = t; j < m; j += NT) alive[j] = 1;
-      if (t == 0) misc[1] = 0;  // cursor
-      __syncthreads();
       int kept = 0;
-      for (;;) {
-        if (t == 0) {
-          int c = misc[1];
-          while (c < m && !alive[c]) ++c;
-          misc[1] = c;
-          misc[3] = c;
-          if (c < m) {
-            out[kept] = ids[perm[c]];
-            alive[c] = 0;
-          }
-        }
-        __syncthreads();
-        const int i = misc[3];
-        if (i >= m) break;
-        ++kept;
-        if (kept == R) break;
-        const int32_t ui = ids[perm[i]];
-        const uint8_t* xu = a.X + int64_t(ui) * a.row_bytes;
-        for (int j = i + 1 + t; j < m; j += NT) {
-          if (!alive[j]) continue;
-          const int pj = perm[j];
-          const AT d2a = row_d2<DT>(xu, a.X + int64_t(ids[pj]) * a.row_bytes, a.row_bytes);
-          bool dom;
+      if (nbuf > 0) load_batch(0, 0);
+      for (int i0 = 0, round = 0; i0 < m && kept < R; i0 += kGenBatch, ++round) {
+        const int nb = min(kGenBatch, m - i0), b = nbuf == 2 ? round & 1 : 0;
+        if (nbuf > 0) cp_async_wait<0>();
+        if (t == 0) *dword = 0u;
+        __syncthreads();  // this batch's rows; the kept rows; every reader of the other buffer is done
+        if (nbuf == 2 && i0 + kGenBatch < m) load_batch(i0 + kGenBatch, b ^ 1);
+        auto batch_row = [&](int c) -> const uint8_t* {
+          return nbuf > 0 ? stage + (b * kGenBatch + c) * stride : a.X + int64_t(ids[perm[i0 + c]]) * a.row_bytes;
+        };
+        auto kept_row = [&](int k) -> const uint8_t* {
+          return k < kept_rows ? kept_stage + k * stride : a.X + int64_t(ids[perm[kept_at[k]]]) * a.row_bytes;
+        };
+        // this lane's candidate
+        const int c = lane < nb ? lane : nb - 1;
+        const int pc = perm[i0 + c];
+        const AT kc = key[pc];
+        const uint8_t* xc = batch_row(c);
+        // whether point u (stored position pu) removes it
+        auto removes = [&](int pu, AT d2a) -> bool {
           if constexpr (DT == kU8) {
-            dom = static_cast<unsigned long long>(A2) * d2a <= 1000000ull * static_cast<unsigned long long>(key[pj]);
+            return static_cast<unsigned long long>(A2) * d2a <= 1000000ull * static_cast<unsigned long long>(kc);
           } else {
-            const int r = sure_dominates(float(A2), d2a, key[pj], E, Eabs);
-            dom = r >= 0 ? (r == 1) : fine_dominates(a, ui, ids[pj], ppt, &key64[pj], double(A2));
+            const int r = sure_dominates(float(A2), d2a, kc, E, Eabs);
+            return r >= 0 ? r == 1 : fine_dominates(a, ids[pu], ids[pc], ppt, &key64[pc], double(A2));
           }
-          if (dom) alive[j] = 0;
+        };
+        // ---- the batch against the points kept so far
+        bool dom = lane >= nb;
+        for (int k = warp; k < kept && !__all_sync(0xffffffffu, dom); k += 2 * kGenWarps) {
+          const int k1 = k + kGenWarps < kept ? k + kGenWarps : k;
+          if (!dom) {
+            AT d0, d1;
+            row_d2_two<DT>(kept_row(k), kept_row(k1), xc, a.row_bytes, d0, d1);
+            dom = removes(perm[kept_at[k]], d0) || removes(perm[kept_at[k1]], d1);
+          }
+        }
+        const unsigned db = __ballot_sync(0xffffffffu, dom);
+        if (lane == 0 && db) atomicOr(dword, db);
+        __syncthreads();
+        const unsigned alive = ~*dword;
+        // ---- the survivors against one another
+        int at = 0;
+        for (unsigned mm = alive; mm; mm &= mm - 1, ++at) {
+          if (at % kGenWarps != warp) continue;
+          const int u = __ffs(int(mm)) - 1;
+          bool rm = false;
+          if (lane > u && ((alive >> lane) & 1u))
+            rm = removes(perm[i0 + u], row_d2_any<DT>(batch_row(u), xc, a.row_bytes));
+          const unsigned rb = __ballot_sync(0xffffffffu, rm);
+          if (lane == 0) dmask[u] = rb;
         }
         __syncthreads();
+        // ---- the batch's greedy scan (every thread; the masks are the same for all)
+        unsigned keep = 0;
+        int now = kept;
+        for (unsigned live = alive; live && now < R; ++now) {
+          const int u = __ffs(int(live)) - 1;
+          keep |= 1u << u;
+          live &= ~(dmask[u] | (1u << u));
+        }
+        if (t < kGenBatch && ((keep >> t) & 1u)) {
+          const int k = kept + __popc(keep & ((1u << t) - 1u));
+          kept_at[k] = uint16_t(i0 + t);
+          out[k] = ids[perm[i0 + t]];
+        }
+        // their rows, if there is room and a batch to come
+        if (i0 + kGenBatch < m && now < R) {
+          int k = kept;
+          for (unsigned mm = keep; mm && k < kept_rows; mm &= mm - 1, ++k) {
+            if (k % kGenWarps != warp) continue;
+            const uint8_t* x = batch_row(__ffs(int(mm)) - 1);
+            for (int ch = lane; ch < nch; ch += 32)
+              *reinterpret_cast<uint4*>(kept_stage + k * stride + ch * 16) = *reinterpret_cast<const uint4*>(x + ch * 16);
+          }
+        }
+        kept = now;
+        if (nbuf == 1 && i0 + kGenBatch < m && kept < R) {
+          __syncthreads();  // every reader of the one buffer is done
+          load_batch(i0 + kGenBatch, 0);
+        }
       }
-      if (t == 0) a.out_cnt[tt][p] = kept;
+      cp_async_wait<0>();  // a next batch that was not needed
       __syncthreads();
+      if (t == 0) a.out_cnt[tt][p] = kept;
     }
     ++done;
   }
@@ -1640,17 +1783,26 @@ static cudaError_t run_generic(const PruneArgs& args, int num_sms, int64_t host_
   if (host_count <= 0) return cudaSuccess;
   int M2 = 256;
   while (M2 < max_degree) M2 <<= 1;
-  const size_t bytes = GenericLayout::bytes(M2);
+  // Staged rows: two batches and 64 kept points where two CTAs still share an SM
+  // (128 rows of 96 floats are 50 KB), else what leaves room for one; at least a
+  // batch, or none.
+  const size_t head = GenericLayout::rows(M2);
+  const size_t row = size_t(args.row_bytes) + 16;
+  const size_t half = size_t(113) * 1024, whole = size_t(227) * 1024;
+  size_t rows = std::min<size_t>(2 * kGenBatch + 64, head < half ? (half - head) / row : 0);
+  if (rows < 2 * kGenBatch + 32) rows = std::min<size_t>(2 * kGenBatch + 64, head < whole ? (whole - head) / row : 0);
+  if (rows < size_t(kGenBatch)) rows = 0;
+  const size_t bytes = head + rows * row;
   auto kern = prune_generic_kernel<DT>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
   if (err != cudaSuccess) return err;
   err = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   if (err != cudaSuccess) return err;
   int per_sm = 0;
-  err = resident_ctas(kern, 256, bytes, 8, &per_sm);
+  err = resident_ctas(kern, kGenThreads, bytes, 8, &per_sm);
   if (err != cudaSuccess) return err;
   const int64_t grid = std::min<int64_t>(int64_t(num_sms) * per_sm, host_count);
-  kern<<<unsigned(grid), 256, bytes, s>>>(args, M2);
+  kern<<<unsigned(grid), kGenThreads, bytes, s>>>(args, M2, int(rows));
   return cudaGetLastError();
 }
 
