@@ -17,13 +17,23 @@ namespace rpk {
 
 namespace {
 
+// Packed rows (src_rb bytes) -> padded ones (dst_rb, a multiple of 4), a 4-byte
+// word per step; WORDS: src_rb is a multiple of 4 too.
+template <bool WORDS>
 __global__ void pad_rows_kernel(const uint8_t* __restrict__ src, int64_t n, int64_t src_rb,
                                 uint8_t* __restrict__ dst, int64_t dst_rb) {
-  const int64_t total = n * dst_rb;
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < total;
-       i += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t r = i / dst_rb, c = i % dst_rb;
-    dst[i] = c < src_rb ? src[r * src_rb + c] : 0;
+  const unsigned words = unsigned(dst_rb / 4);
+  for (int64_t r = int64_t(blockIdx.x) * blockDim.y + threadIdx.y; r < n; r += int64_t(gridDim.x) * blockDim.y) {
+    const uint8_t* x = src + r * src_rb;
+    for (unsigned w = threadIdx.x; w < words; w += blockDim.x) {
+      unsigned v = 0;
+      if constexpr (WORDS) {
+        if (4 * w < src_rb) v = reinterpret_cast<const unsigned*>(x)[w];
+      } else {
+        for (unsigned b = 0; b < 4 && 4 * w + b < src_rb; ++b) v |= unsigned(x[4 * w + b]) << (8 * b);
+      }
+      reinterpret_cast<unsigned*>(dst + r * dst_rb)[w] = v;
+    }
   }
 }
 
@@ -318,9 +328,27 @@ __global__ void mean_u8_finish_kernel(const unsigned long long* __restrict__ sum
 // and takes the first nonzero value exactly; a subnormal s takes real additions.
 // Every step consumes at least one row, so the loop ends.
 //
-// One warp per column (grid = d). Rows arrive in blocks of kMeanBlock through
-// shared memory, the next block loaded into registers while this one is summed.
-constexpr int kMeanBlock = 1024;
+// Many more rows go at once where nothing happens.  A CTA per column (grid = d)
+// takes blocks of kMeanBlock rows, eight rows a thread, and adds a whole block by
+// one of two rules:
+//   one binade  no value of the block is a tie and every running T of the block
+//               stays in [2^52 + 1, 2^53 - 1] (each thread's running sum's least
+//               and largest value, on the CTA's prefix of the threads' totals);
+//   exact       with 2^e above |s| + the sum of |x|, s and every x are multiples
+//               of 2^(e - 53): then so is every partial sum, each has at most 53
+//               bits, and no addition rounds at all.  Sums that change binade or
+//               sign often (a column whose mean is near zero) are small against
+//               2^53 times their values' last bits, so this takes them.
+// A block that neither takes goes to warp 0: 256 rows at a time by the first rule
+// and 64 by the step above where that fails too.
+//
+// What bounds it: one block's chain, load to verdict, about 2 us for 2,048 rows;
+// the next block's loads are in flight meanwhile.  200,000 x 96 rows: one warp
+// per column with 64-row steps took 3.76 ms, its slowest column (3,650 changes of
+// binade in 118,000 rows) at every change; this one 0.56.
+constexpr int kMeanThreads = 256;
+constexpr int kMeanPer = 8;
+constexpr int kMeanBlock = kMeanThreads * kMeanPer;
 
 // q = rne(x / 2^e52) in the sign frame of s (neg), or false when x / 2^e52 is a
 // tie or too large to be kept anyway (the caller then adds x in binary64).
@@ -346,108 +374,272 @@ __device__ __forceinline__ bool mean_units(float x, int e52, unsigned neg, long 
   return ok;
 }
 
-__global__ void __launch_bounds__(32) mean_f32_kernel(const uint8_t* __restrict__ X, int64_t n,
-                                                      int64_t row_bytes, int d, double* __restrict__ mean) {
-  __shared__ float buf[kMeanBlock];
-  const int j = blockIdx.x;
-  const int lane = threadIdx.x;
+// One step of up to 64 rows x[0, avail), avail >= 1, onto s; returns how many
+// were added.  One warp; s and the result are the same in every lane.
+__device__ __forceinline__ int mean_step64(const float* x, int avail, double& s) {
+  const int lane = threadIdx.x & 31;
+  const long long kLo = (1ll << 52) + 1, kHi = 1ll << 53;
+  const bool ha = 2 * lane < avail, hb = 2 * lane + 1 < avail;
+  const float xa = ha ? x[2 * lane] : 0.f;
+  const float xb = hb ? x[2 * lane + 1] : 0.f;
+  const unsigned long long sb = (unsigned long long)__double_as_longlong(s);
+  const int eb = int((sb >> 52) & 0x7ff);
+  if (sb == 0) {  // s = +0
+    const unsigned nza = __ballot_sync(0xffffffffu, ha && (__float_as_uint(xa) & 0x7fffffffu) != 0);
+    const unsigned nzb = __ballot_sync(0xffffffffu, hb && (__float_as_uint(xb) & 0x7fffffffu) != 0);
+    if ((nza | nzb) == 0) return avail;
+    const int l = __ffs(int(nza | nzb)) - 1;
+    const bool at_a = (nza >> l) & 1u;
+    s = double(__shfl_sync(0xffffffffu, at_a ? xa : xb, l));  // 0 + x = x exactly
+    return 2 * l + (at_a ? 0 : 1) + 1;
+  }
+  if (eb == 0 || eb == 0x7ff) {  // subnormal s (or a non-finite one): a real addition
+    s = __dadd_rn(s, double(__shfl_sync(0xffffffffu, xa, 0)));
+    return 1;
+  }
+  const int e52 = eb - 1075;
+  const unsigned neg = unsigned(sb >> 63);
+  const long long S = (long long)((sb & ((1ull << 52) - 1)) | (1ull << 52));
+  long long qa, qb;
+  const bool oka = mean_units(xa, e52, neg, qa) && ha;
+  const bool okb = mean_units(xb, e52, neg, qb) && hb;
+  if (!ha) qa = 0;
+  if (!hb) qb = 0;
+  long long pre = qa + qb;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long v = __shfl_up_sync(0xffffffffu, pre, o);
+    if (lane >= o) pre += v;
+  }
+  const long long Tb = S + pre, Ta = Tb - qb;
+  const bool va = oka && Ta >= kLo && Ta <= kHi;
+  const bool vb = okb && Tb >= kLo && Tb <= kHi;
+  const unsigned inva = __ballot_sync(0xffffffffu, !va), invb = __ballot_sync(0xffffffffu, !vb);
+  const unsigned enda = __ballot_sync(0xffffffffu, va && Ta == kHi);
+  const unsigned endb = __ballot_sync(0xffffffffu, vb && Tb == kHi);
+  int fi = 64, fe = 64;  // first element kept by no T, first element at 2^53
+  if (inva | invb) {
+    const int l = __ffs(int(inva | invb)) - 1;
+    fi = 2 * l + (((inva >> l) & 1u) ? 0 : 1);
+  }
+  if (enda | endb) {
+    const int l = __ffs(int(enda | endb)) - 1;
+    fe = 2 * l + (((enda >> l) & 1u) ? 0 : 1);
+  }
+  const int c = fi < fe + 1 ? fi : fe + 1;  // elements kept, c <= fi <= avail
+  if (c > 0) {
+    const int e = c - 1;
+    const long long T = __shfl_sync(0xffffffffu, (e & 1) ? Tb : Ta, e >> 1);
+    const unsigned long long sign = (unsigned long long)neg << 63;
+    s = __longlong_as_double((long long)(T == kHi ? sign | ((unsigned long long)(eb + 1) << 52)
+                                                 : sign | ((unsigned long long)eb << 52) |
+                                                       (unsigned long long)(T - (1ll << 52))));
+  }
+  int used = c;
+  if (c < avail && c == fi) {
+    s = __dadd_rn(s, double(__shfl_sync(0xffffffffu, (c & 1) ? xb : xa, c >> 1)));
+    used = c + 1;
+  }
+  return used;
+}
+
+// A thread's kMeanPer rows x (the first `have` of them exist) in units of s: the
+// total, the least and largest running sum (of rows that exist) and whether no
+// value was a tie or too large.  At most 2^57 in magnitude.
+__device__ __forceinline__ bool mean_run(const float (&x)[kMeanPer], int have, int e52, unsigned neg, long long& tot,
+                                         long long& lo, long long& hi) {
+  tot = 0;
+  lo = 0x7fffffffffffffffll;
+  hi = -0x7fffffffffffffffll;
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < kMeanPer; ++k) {
+    if (k < have) {
+      long long q;
+      ok &= mean_units(x[k], e52, neg, q);
+      tot += q;
+      lo = tot < lo ? tot : lo;
+      hi = tot > hi ? tot : hi;
+    }
+  }
+  return ok;
+}
+
+// The inclusive prefix sum over the warp's totals.  32 totals stay below 2^62.
+__device__ __forceinline__ long long warp_prefix(long long v) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long u = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += u;
+  }
+  return v;
+}
+
+// Every T = base + (a running sum) inside [2^52 + 1, 2^53 - 1]?  |base| <= 2^62.
+__device__ __forceinline__ bool mean_inside(long long base, long long lo, long long hi, int have) {
+  return have == 0 || (base + lo >= (1ll << 52) + 1 && base + hi <= (1ll << 53) - 1);
+}
+
+__device__ __forceinline__ double mean_join(unsigned long long sb, long long T) {  // the sign and binade of sb
+  return __longlong_as_double((long long)((sb & ~((1ull << 52) - 1)) | (unsigned long long)(T - (1ll << 52))));
+}
+
+// x as a multiple of 2^g, or false if it is none; |x| < 2^(g + 53).
+__device__ __forceinline__ bool mean_multiple(float x, int g, long long& q) {
+  const unsigned xb = __float_as_uint(x);
+  const int ex = int((xb >> 23) & 0xff);
+  const unsigned m = (xb & 0x7fffffu) | (ex ? 0x800000u : 0u);
+  const int k = (ex ? ex : 1) - 150 - g;  // x = m 2^k 2^g
+  long long v = 0;
+  bool ok = true;
+  if (k >= 0) {
+    v = (long long)m << (k < 53 ? k : 53);  // k <= 52 where m != 0
+  } else if (-k < 24) {
+    v = (long long)(m >> -k);
+    ok = (m & ((1u << -k) - 1u)) == 0;
+  } else {
+    ok = m == 0;
+  }
+  q = (xb >> 31) ? -v : v;
+  return ok;
+}
+
+__global__ void __launch_bounds__(kMeanThreads) mean_f32_kernel(const uint8_t* __restrict__ X, int64_t n,
+                                                                int64_t row_bytes, int d, double* __restrict__ mean) {
+  __shared__ __align__(16) float buf[kMeanBlock];
+  __shared__ long long wtot[kMeanThreads / 32];
+  __shared__ float wabs[kMeanThreads / 32];
+  __shared__ double s_sh;
+  const int j = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const float* F = reinterpret_cast<const float*>(X) + j;
   const int64_t stride = row_bytes / 4;
-  const long long kLo = (1ll << 52) + 1, kHi = 1ll << 53;
-  float nxt[kMeanBlock / 32];
+  float x[kMeanPer], nxt[kMeanPer];
+  auto load = [&](int64_t base, float (&v)[kMeanPer]) {
 #pragma unroll
-  for (int t = 0; t < kMeanBlock / 32; ++t) {
-    const int64_t r = int64_t(32 * t + lane);
-    nxt[t] = r < n ? __ldg(F + r * stride) : 0.f;
-  }
+    for (int k = 0; k < kMeanPer; ++k) {
+      const int64_t r = base + int64_t(t) * kMeanPer + k;
+      v[k] = r < n ? __ldg(F + r * stride) : 0.f;
+    }
+  };
+  load(0, nxt);
   double s = 0.0;
   for (int64_t base = 0; base < n; base += kMeanBlock) {
-    __syncwarp();
 #pragma unroll
-    for (int t = 0; t < kMeanBlock / 32; ++t) buf[32 * t + lane] = nxt[t];
-    __syncwarp();
-    if (base + kMeanBlock < n) {
+    for (int k = 0; k < kMeanPer; ++k) x[k] = nxt[k];
+    if (base + kMeanBlock < n) load(base + kMeanBlock, nxt);
+    const int count = int(n - base < kMeanBlock ? n - base : kMeanBlock);
+    const int left = count - t * kMeanPer;
+    const int have = left < 0 ? 0 : left < kMeanPer ? left : kMeanPer;
+    const unsigned long long sb = (unsigned long long)__double_as_longlong(s);
+    const int eb = int((sb >> 52) & 0x7ff);
+    const long long S = (long long)((sb & ((1ull << 52) - 1)) | (1ull << 52));
+    bool ok = eb != 0 && eb != 0x7ff;  // the same in every thread
+    long long total = 0;
+    if (ok) {
+      long long tot, lo, hi;
+      ok = mean_run(x, have, eb - 1075, unsigned(sb >> 63), tot, lo, hi);
+      const long long incl = warp_prefix(tot);
+      if (lane == 31) wtot[warp] = incl;
+      __syncthreads();
+      long long before = S;
 #pragma unroll
-      for (int t = 0; t < kMeanBlock / 32; ++t) {
-        const int64_t r = base + kMeanBlock + 32 * t + lane;
-        nxt[t] = r < n ? __ldg(F + r * stride) : 0.f;
-      }
-    }
-    const int64_t bend = n < base + kMeanBlock ? n : base + kMeanBlock;
-    int64_t i = base;
-    while (i < bend) {  // s, i and every branch below are uniform over the warp
-      const int avail = bend - i < 64 ? int(bend - i) : 64;
-      const int off = int(i - base);
-      const bool ha = 2 * lane < avail, hb = 2 * lane + 1 < avail;
-      const float xa = ha ? buf[off + 2 * lane] : 0.f;
-      const float xb = hb ? buf[off + 2 * lane + 1] : 0.f;
-      const unsigned long long sb = (unsigned long long)__double_as_longlong(s);
-      const int eb = int((sb >> 52) & 0x7ff);
-      if (sb == 0) {  // s = +0
-        const unsigned nza = __ballot_sync(0xffffffffu, ha && (__float_as_uint(xa) & 0x7fffffffu) != 0);
-        const unsigned nzb = __ballot_sync(0xffffffffu, hb && (__float_as_uint(xb) & 0x7fffffffu) != 0);
-        if ((nza | nzb) == 0) {
-          i += avail;
-          continue;
+      for (int w = 0; w < kMeanThreads / 32; ++w) {
+        const long long v = wtot[w];
+        if (v > (1ll << 53) || v < -(1ll << 53)) {  // leaves the binade (and the sums here could overflow)
+          ok = false;
+        } else {
+          if (w < warp) before += v;
+          total += v;
         }
-        const int l = __ffs(int(nza | nzb)) - 1;
-        const bool at_a = (nza >> l) & 1u;
-        s = double(__shfl_sync(0xffffffffu, at_a ? xa : xb, l));  // 0 + x = x exactly
-        i += 2 * l + (at_a ? 0 : 1) + 1;
-        continue;
       }
-      if (eb == 0 || eb == 0x7ff) {  // subnormal s (or a non-finite one): a real addition
-        s = __dadd_rn(s, double(__shfl_sync(0xffffffffu, xa, 0)));
-        i += 1;
-        continue;
-      }
-      const int e52 = eb - 1075;
-      const unsigned neg = unsigned(sb >> 63);
-      const long long S = (long long)((sb & ((1ull << 52) - 1)) | (1ull << 52));
-      long long qa, qb;
-      const bool oka = mean_units(xa, e52, neg, qa) && ha;
-      const bool okb = mean_units(xb, e52, neg, qb) && hb;
-      if (!ha) qa = 0;
-      if (!hb) qb = 0;
-      long long pre = qa + qb;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const long long v = __shfl_up_sync(0xffffffffu, pre, o);
-        if (lane >= o) pre += v;
-      }
-      const long long Tb = S + pre, Ta = Tb - qb;
-      const bool va = oka && Ta >= kLo && Ta <= kHi;
-      const bool vb = okb && Tb >= kLo && Tb <= kHi;
-      const unsigned inva = __ballot_sync(0xffffffffu, !va), invb = __ballot_sync(0xffffffffu, !vb);
-      const unsigned enda = __ballot_sync(0xffffffffu, va && Ta == kHi);
-      const unsigned endb = __ballot_sync(0xffffffffu, vb && Tb == kHi);
-      int fi = 64, fe = 64;  // first element kept by no T, first element at 2^53
-      if (inva | invb) {
-        const int l = __ffs(int(inva | invb)) - 1;
-        fi = 2 * l + (((inva >> l) & 1u) ? 0 : 1);
-      }
-      if (enda | endb) {
-        const int l = __ffs(int(enda | endb)) - 1;
-        fe = 2 * l + (((enda >> l) & 1u) ? 0 : 1);
-      }
-      const int c = fi < fe + 1 ? fi : fe + 1;  // elements kept, c <= fi <= avail
-      if (c > 0) {
-        const int e = c - 1;
-        const long long T = __shfl_sync(0xffffffffu, (e & 1) ? Tb : Ta, e >> 1);
-        const unsigned long long sign = (unsigned long long)neg << 63;
-        s = __longlong_as_double((long long)(T == kHi ? sign | ((unsigned long long)(eb + 1) << 52)
-                                                     : sign | ((unsigned long long)eb << 52) |
-                                                           (unsigned long long)(T - (1ll << 52))));
-      }
-      int used = c;
-      if (c < avail && c == fi) {
-        s = __dadd_rn(s, double(__shfl_sync(0xffffffffu, (c & 1) ? xb : xa, c >> 1)));
-        used = c + 1;
-      }
-      i += used;
+      ok = ok && mean_inside(before + incl - tot, lo, hi, have);
     }
+    if (__syncthreads_and(ok)) {
+      s = mean_join(sb, S + total);
+      continue;
+    }
+    // ---- the exact rule
+    float mag = 0.f;
+#pragma unroll
+    for (int k = 0; k < kMeanPer; ++k) mag += fabsf(x[k]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mag += __shfl_xor_sync(0xffffffffu, mag, o);
+    if (lane == 0) wabs[warp] = mag;
+    __syncthreads();
+    float top = 0.f;
+#pragma unroll
+    for (int w = 0; w < kMeanThreads / 32; ++w) top += wabs[w];
+    top = (top + fabsf(__double2float_ru(fabs(s)))) * 1.001f;  // the roundings above are below 2^-12 of it
+    bool exact = top > 0.f && top < 1.0e30f;  // the same in every thread
+    if (exact) {
+      int e;
+      frexpf(top, &e);  // top < 2^e
+      const int g = e - 53;
+      long long mine = 0;
+#pragma unroll
+      for (int k = 0; k < kMeanPer; ++k) {  // rows past n are zeros
+        long long q;
+        exact &= mean_multiple(x[k], g, q);
+        mine += q;
+      }
+      // s = ms 2^(es - 1075) with es - 1075 <= g, since |s| < 2^e
+      const long long ms = eb ? S : (long long)(sb & ((1ull << 52) - 1));
+      const int sh = g - ((eb ? eb : 1) - 1075);
+      long long s_units = 0;
+      if (sh < 53) {
+        s_units = ms >> sh;
+        exact &= (ms & ((1ll << sh) - 1)) == 0;
+      } else {
+        exact &= ms == 0;
+      }
+      if (sb >> 63) s_units = -s_units;
+      const long long incl = warp_prefix(mine);  // partial sums stay below 2^53 in magnitude
+      if (lane == 31) wtot[warp] = incl;
+      if (__syncthreads_and(exact)) {
+#pragma unroll
+        for (int w = 0; w < kMeanThreads / 32; ++w) s_units += wtot[w];
+        s = scalbn(double(s_units), g);  // exact: at most 53 bits
+        __syncthreads();  // wtot read before the next block writes it
+        continue;
+      }
+    }
+    // ---- row by row where something happens: warp 0
+#pragma unroll
+    for (int k = 0; k < kMeanPer; k += 4)
+      *reinterpret_cast<float4*>(buf + t * kMeanPer + k) = make_float4(x[k], x[k + 1], x[k + 2], x[k + 3]);
+    __syncthreads();
+    if (warp == 0) {
+      int i = 0;
+      bool smooth = true;  // the last 64-row step took all its rows
+      while (i < count) {  // s, i and every branch below are uniform over the warp
+        const unsigned long long b = (unsigned long long)__double_as_longlong(s);
+        const int e = int((b >> 52) & 0x7ff);
+        if (smooth && count - i >= 32 * kMeanPer && e != 0 && e != 0x7ff) {
+          float v[kMeanPer];
+#pragma unroll
+          for (int k = 0; k < kMeanPer; ++k) v[k] = buf[i + lane * kMeanPer + k];
+          long long tot, lo, hi;
+          const long long S0 = (long long)((b & ((1ull << 52) - 1)) | (1ull << 52));
+          const bool fine = mean_run(v, kMeanPer, e - 1075, unsigned(b >> 63), tot, lo, hi);
+          const long long incl = warp_prefix(tot);
+          if (__all_sync(0xffffffffu, fine && mean_inside(S0 + incl - tot, lo, hi, kMeanPer))) {
+            s = mean_join(b, S0 + __shfl_sync(0xffffffffu, incl, 31));
+            i += 32 * kMeanPer;
+            continue;
+          }
+        }
+        const int avail = count - i < 64 ? count - i : 64;
+        const int used = mean_step64(buf + i, avail, s);
+        smooth = used == avail;
+        i += used;
+      }
+      if (lane == 0) s_sh = s;
+    }
+    __syncthreads();
+    s = s_sh;
   }
-  if (lane == 0) mean[j] = __ddiv_rn(s, double(n));
+  if (t == 0) mean[j] = __ddiv_rn(s, double(n));
 }
 
 __global__ void nearest_mean_kernel(const uint8_t* __restrict__ X, int64_t n, int64_t row_bytes, int d,
@@ -490,20 +682,35 @@ __global__ void nearest_mean_kernel(const uint8_t* __restrict__ X, int64_t n, in
   }
 }
 
-__global__ void pick_medoid_kernel(const double* __restrict__ best, int64_t nb, int64_t* medoid) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// The best of the blocks' candidates: (distance, id) least, one CTA.
+__global__ void __launch_bounds__(256) pick_medoid_kernel(const double* __restrict__ best, int64_t nb, int64_t* medoid) {
+  __shared__ double sd[256];
+  __shared__ long long si[256];
   double bd = DBL_MAX;
   long long bi = -1;
-  for (int64_t b = 0; b < nb; ++b) {
+  for (int64_t b = threadIdx.x; b < nb; b += 256) {
     const double d2 = best[2 * b];
     const long long i2 = __double_as_longlong(best[2 * b + 1]);
-    if (i2 < 0) continue;
-    if (bi < 0 || d2 < bd || (d2 == bd && i2 < bi)) {
+    if (i2 >= 0 && (bi < 0 || d2 < bd || (d2 == bd && i2 < bi))) {
       bd = d2;
       bi = i2;
     }
   }
-  *medoid = bi;
+  sd[threadIdx.x] = bd;
+  si[threadIdx.x] = bi;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (threadIdx.x < o) {
+      const double d2 = sd[threadIdx.x + o];
+      const long long i2 = si[threadIdx.x + o];
+      if (i2 >= 0 && (si[threadIdx.x] < 0 || d2 < sd[threadIdx.x] || (d2 == sd[threadIdx.x] && i2 < si[threadIdx.x]))) {
+        sd[threadIdx.x] = d2;
+        si[threadIdx.x] = i2;
+      }
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) *medoid = si[0];
 }
 
 unsigned grid_for(int64_t work, int threads) {
@@ -514,9 +721,14 @@ unsigned grid_for(int64_t work, int threads) {
 
 cudaError_t launch_pad_rows(const void* src, int64_t n, int64_t src_rb, uint8_t* dst, int64_t dst_rb,
                             cudaStream_t s) {
-  if (src_rb == dst_rb) return cudaMemcpyAsync(dst, src, size_t(n * dst_rb), cudaMemcpyDeviceToDevice, s);
-  pad_rows_kernel<<<grid_for(n * dst_rb, 256), 256, 0, s>>>(static_cast<const uint8_t*>(src), n, src_rb, dst,
-                                                            dst_rb);
+  if (n <= 0) return cudaSuccess;
+  const dim3 block(32, 8);
+  const unsigned grid = unsigned(std::min<int64_t>((n + 7) / 8, 152 * 16));
+  const uint8_t* x = static_cast<const uint8_t*>(src);
+  if (src_rb % 4 == 0 && reinterpret_cast<uintptr_t>(src) % 4 == 0)
+    pad_rows_kernel<true><<<grid, block, 0, s>>>(x, n, src_rb, dst, dst_rb);
+  else
+    pad_rows_kernel<false><<<grid, block, 0, s>>>(x, n, src_rb, dst, dst_rb);
   return cudaGetLastError();
 }
 
@@ -631,11 +843,11 @@ cudaError_t launch_medoid(const DevData& D, double* mean, double* block_best, in
     mean_u8_sum_kernel<<<grid, 128, 0, s>>>(D.X, D.n, D.row_bytes, D.d, sums);
     mean_u8_finish_kernel<<<unsigned((D.d + 127) / 128), 128, 0, s>>>(sums, D.n, D.d, mean);
   } else {
-    mean_f32_kernel<<<unsigned(D.d), 32, 0, s>>>(D.X, D.n, D.row_bytes, D.d, mean);
+    mean_f32_kernel<<<unsigned(D.d), kMeanThreads, 0, s>>>(D.X, D.n, D.row_bytes, D.d, mean);
   }
   const int64_t nb = medoid_blocks(D.n);
   nearest_mean_kernel<<<unsigned(nb), 256, 0, s>>>(D.X, D.n, D.row_bytes, D.d, D.dtype, mean, block_best);
-  pick_medoid_kernel<<<1, 32, 0, s>>>(block_best, nb, medoid);
+  pick_medoid_kernel<<<1, 256, 0, s>>>(block_best, nb, medoid);
   return cudaGetLastError();
 }
 
