@@ -2,8 +2,9 @@
 // for every node p, each reading only the input graph) and the CSR emit.
 //
 // Per node p with m = |N_out(p)| candidates (Algorithm 1):
-//   a2 gather    each thread loads its candidate's row (and p's row) with
-//                16-byte vector loads and writes it as an f16 MMA operand;
+//   a2 gather    the candidates' rows are loaded with 16-byte vector loads and
+//                written as f16 MMA operands (uint8: a thread a row; float:
+//                four lanes a row, so that loads are coalesced);
 //   a3 keys      d2(p, v) for every candidate v, exactly / single precision;
 //   a5 Gram      G = A A^T for the candidates on the tensor cores (tcgen05,
 //                accumulator in TMEM), d2(u, v) = |u|^2 + |v|^2 - 2 G(u, v);
@@ -13,18 +14,16 @@
 //   a6 decide    for every target t and every pair u before v in that order,
 //                bit "u removes v": alpha_t * D(u, v) <= D(p, v);
 //   a7 scan      per target: keep the first live candidate, stop at R_t, drop
-//                every candidate the kept one removes (warp ballots over
-//                64-bit live masks; a6 is evaluated lazily inside this loop,
-//                only for rows some target keeps);
+//                every candidate the kept one removes (64-bit live masks);
 //   a8 emit      kept ids in kept order into per-target scratch, then counts
 //                -> row_ptr (scan) -> compacted col.
 // Because removal is only ever done by kept points, "take the argmin of the
 // live set" (Algorithm 1) and "walk the sorted order, skipping removed
 // points" pick the same sequence; the bit scan is the latter.
 //
-// Tensor-core path: m <= 64 (two nodes per 128-thread CTA, one 128 x 128
-// MMA) and 64 < m <= 128 (one node per CTA).  Larger degrees take the generic
-// path (one node per 256-thread CTA, lazy CUDA-core distances).
+// Tensor-core path: m <= 64 (two nodes per CTA, one 128 x 128 MMA) and 64 < m <=
+// 128 (one node per CTA), a kernel for uint8 rows and one for float rows.  Larger
+// degrees take the generic path (one node per 256-thread CTA, CUDA-core distances).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -195,6 +194,36 @@ __device__ __forceinline__ bool fine_dominates(const PruneArgs& a, int32_t u, in
   return canon_dominates(A2, d2a, d2b);
 }
 
+// fine_dominates by a whole warp (the same arguments in every lane).
+__device__ __noinline__ bool fine_dominates_warp(const PruneArgs& a, int32_t u, int32_t v, int32_t p, double* key64_v,
+                                                 double A2) {
+  const float* X = reinterpret_cast<const float*>(a.X);
+  const int64_t stride = a.row_bytes / 4;
+  const int nch = int(a.row_bytes / 16);
+  const float* xv = X + int64_t(v) * stride;
+  double sb = *key64_v;
+  __syncwarp();
+  if (isnan(sb)) {
+    sb = -ff_d2_warp(X + int64_t(p) * stride, xv, nch);
+    *key64_v = sb;
+  }
+  const double fa = -ff_d2_warp(X + int64_t(u) * stride, xv, nch);
+  const FFBound B = ff_bound(a.d);
+  double la, ha, lb, hb;
+  slot_interval(fa, B, &la, &ha);
+  slot_interval(sb, B, &lb, &hb);
+  if (__dmul_rn(A2, ha) <= __dmul_rn(1.0e6, lb)) return true;
+  if (__dmul_rn(A2, la) > __dmul_rn(1.0e6, hb)) return false;
+  const double d2a = canon_d2_f32(X + int64_t(u) * stride, xv, a.d);
+  double d2b = sb;
+  if (signbit(d2b)) {
+    d2b = canon_d2_f32(X + int64_t(p) * stride, xv, a.d);
+    *key64_v = d2b;
+  }
+  if ((threadIdx.x & 31) == 0) atomicAdd(&a.status->fp64_decisions, 1ull);
+  return canon_dominates(A2, d2a, d2b);
+}
+
 // An open pair of the float decision pass: row `t` against column `c` for the
 // distinct alphas u0 .. TA - 1 (ascending; the Gram tier found u0 of them
 // surely removing).  One single-precision difference-form distance from the
@@ -300,7 +329,7 @@ __device__ __forceinline__ float split_gram_value(uint32_t acc0, uint32_t acc1, 
   return fmaf(__uint_as_float(acc1), 4.8828125e-04f, __uint_as_float(acc0)) * inv_s2;
 }
 
-// Shared-memory plan of prune_tc_kernel.  Per node group the producer warps
+// Shared-memory plan of the tensor-core prune kernels.  Per node group the producer warps
 // keep norms and thresholds; per pipeline slot (2) and group they hand the
 // consumer warp the candidate ids, keys, binary64 key cache and masks.
 template <int MAXM, int TB, int NOP>
@@ -318,18 +347,18 @@ struct TcLayout {
   // per group, producer side
   static constexpr size_t p_norm = 0;
   static constexpr size_t p_sn = p_norm + size_t(MAXM) * 4;
-  // thresholds: [TB][MAXM] for uint8; [MAXM][TB4] for float (distinct alphas of a
-  // column contiguous, padded to a multiple of 4 for 16-byte reads)
+  // uint8: thresholds [TB][MAXM].  Float: a record per column, its lower and upper
+  // thresholds of every distinct alpha (TA rounded up to 4 of each), its key and
+  // the key's root; (2 TA4 + 4) floats apart, which spreads the 16-byte reads of
+  // eight consecutive columns over all banks for every TA4.
   static constexpr int TB4 = (TB + 3) / 4 * 4;
   static constexpr size_t p_qlo = p_sn + size_t(MAXM) * 4;
-  static constexpr size_t p_qhi = p_qlo + size_t(TB4) * MAXM * 4;
-  static constexpr size_t p_sk = p_qhi + size_t(TB4) * MAXM * 4;  // [MAXM] (key, id) in stored order
+  static constexpr size_t p_sk = p_qlo + size_t(2 * TB4 + 4) * MAXM * 4;  // [MAXM] (key, id) in stored order
   static constexpr size_t p_k64 = p_sk + size_t(MAXM) * 8;       // [MAXM] binary64 keys in stored order
-  static constexpr size_t p_cq = p_k64 + size_t(MAXM) * 8;        // [MAXM] float4 per column (float rows)
-  static constexpr size_t p_srt = p_cq + size_t(MAXM) * 16;       // [MAXM] float keys by rank (float rows)
-  static constexpr size_t p_rk = p_srt + size_t(MAXM) * 4;        // [MAXM] rank of each stored position (float rows)
+  static constexpr size_t p_srt = p_k64 + size_t(MAXM) * 8;       // [MAXM] float keys by rank (float rows)
+  static constexpr size_t p_rk = p_srt + size_t(MAXM) * 4;        // [MAXM] 4 x rank of each stored position (float rows)
   static constexpr size_t p_bytes = p_rk + size_t(MAXM) * 4;
-  static_assert(p_qlo % 16 == 0 && p_qhi % 16 == 0 && p_cq % 16 == 0 && p_rk % 16 == 0 && p_bytes % 16 == 0,
+  static_assert(p_qlo % 16 == 0 && p_sk % 16 == 0 && p_rk % 16 == 0 && p_bytes % 16 == 0,
                 "16-byte reads");
   static constexpr size_t off_prod = off_slots + 2 * NG * s_bytes;
   // small words: node/degree/row start per (slot, group), the claim queue's
@@ -359,58 +388,114 @@ __device__ __forceinline__ unsigned exact_threshold(unsigned k, unsigned long lo
   return static_cast<unsigned>(q);
 }
 
-// Most nodes claimed at a time by a prune_tc_kernel CTA (one per lane of warp
+// Most nodes claimed at a time by a tensor-core prune CTA (one per lane of warp
 // 0).  A launch with fewer than 4 x 32 nodes per CTA claims less, so that every
 // CTA gets about four claims: at 32 always, the 600-row launches of a Vamana
 // build kept 19 of 304 CTAs busy (30,000 x 96 float points, both passes: 53 ms of
 // 65..128-candidate launches, now 7.2 ms).
 constexpr int kClaim = 32;
 
-// Named barriers of prune_tc_kernel (0 is __syncthreads, unused in the loop).
-constexpr int kBarProd = 1;       // the 128 producer threads
-constexpr int kBarFull = 2;       // + slot: producers arrive, the consumer waits (160)
-constexpr int kBarFree = 4;       // + slot: the consumer arrives, producers wait (160)
+// Named barriers of the tensor-core prune kernels (0 is __syncthreads, unused in the loop).
+constexpr int kBarProd = 1;       // the producer threads
+constexpr int kBarFull = 2;       // + slot: producers arrive, the consumer waits (all threads)
+constexpr int kBarFree = 4;       // + slot: the consumer arrives, producers wait (all threads)
 
 __device__ __forceinline__ void bar_arrive(int id, int count) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
-// Producer barrier that also ORs a flag over the 128 producer threads.
-__device__ __forceinline__ bool prod_sync_or(bool flag) {
+// Producer barrier that also ORs a flag over the N producer threads.
+template <int N>
+__device__ __forceinline__ bool prod_sync_or_n(bool flag) {
   uint32_t res;
   asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.u32 p, %1, 0;\nbar.red.or.pred p, 1, 128, p;\nselp.u32 %0, 1, 0, p;\n}\n"
+      "{\n.reg .pred p;\nsetp.ne.u32 p, %1, 0;\nbar.red.or.pred p, 1, %2, p;\nselp.u32 %0, 1, 0, p;\n}\n"
       : "=r"(res)
-      : "r"(static_cast<uint32_t>(flag))
+      : "r"(static_cast<uint32_t>(flag)), "n"(N)
       : "memory");
   return res != 0;
 }
+__device__ __forceinline__ bool prod_sync_or(bool flag) { return prod_sync_or_n<128>(flag); }
 
-// One CTA = 4 producer warps + 1 consumer warp.  The producers handle NG =
-// 128 / MAXM nodes at a time, one candidate per thread: gather, pivot keys and
-// norms, the rank of each candidate in the processing order (a4), its f16
-// operand row, the tcgen05 Gram, per-column thresholds and one domination mask
-// per target (uint8) or distinct alpha (float) for every rank.  uint8 operand
-// rows sit at CTA row (group, rank) = TMEM lane, and each lane turns its Gram row
-// into mask bits straight from TMEM.  Float operand rows stay at the stored
-// position, so the MMA starts before the ranks are known; the Gram is then
-// staged in shared memory in rank order and decided with the pairs spread
-// evenly over the producers.  They hand ids and masks over through one of two
-// slots; the consumer warp resolves the slot's open float pairs and runs the
-// greedy loop per node and target (a7) while the producers work on the next
-// nodes.  4 CTAs per SM (the TMEM limit) need at most 96 registers per thread;
-// the kernels with more targets per launch, float rows (256 TMEM columns), or
-// one 128-candidate node per MMA (more shared memory per CTA) trade that for
+// The live candidates of one node as bits by rank, 64 a word.
+template <int MW>
+struct LiveBits {
+  unsigned long long w[MW];
+  __device__ __forceinline__ bool any() const { return MW == 1 ? w[0] != 0 : (w[0] | w[MW - 1]) != 0; }
+  // The lowest set bit (0 if there is none), taken out.
+  __device__ __forceinline__ int take() {
+    if (MW == 1 || w[0]) {
+      const int p = w[0] ? __ffsll(static_cast<long long>(w[0])) - 1 : 0;
+      w[0] &= w[0] - 1;
+      return p;
+    }
+    const int p = w[MW - 1] ? 64 + __ffsll(static_cast<long long>(w[MW - 1])) - 1 : 0;
+    w[MW - 1] &= w[MW - 1] - 1;
+    return p;
+  }
+  __device__ __forceinline__ bool has(int p) const {
+    return ((MW == 1 || p < 64 ? w[0] : w[MW - 1]) >> (p & 63)) & 1ull;
+  }
+};
+
+// Algorithm 1's loop over one node's live candidates for one target: the next in
+// order is kept and takes out those its mask names, until R are kept or none is
+// live.  Four steps a round: the masks and ids of the first four live candidates
+// are read together (one round trip to shared memory), and the second to fourth
+// are kept in turn unless a mask before them has taken them out.  A candidate's
+// own bit is dropped as it is kept.  For float rows, whose sweeps keep more
+// (400,000 nodes, two steps / four: eight float targets 9.17 / 8.96 ms; three uint8
+// ones, whose loop below takes two, 2.41 / 2.54 ms).
+template <int MW>
+__device__ __forceinline__ int greedy_scan(const unsigned long long (&al)[MW], const unsigned long long* mrow,
+                                           const int32_t* ids, int32_t* out, int R) {
+  LiveBits<MW> live;
+#pragma unroll
+  for (int w = 0; w < MW; ++w) live.w[w] = al[w];
+  int kept = 0;
+  while (kept < R && live.any()) {
+    LiveBits<MW> rest = live;
+    int p[4];
+    unsigned long long m[4][MW];
+    int32_t id[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) p[q] = rest.take();  // past the last live one: rank 0, never live again
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      id[q] = ids[p[q]];
+#pragma unroll
+      for (int w = 0; w < MW; ++w) m[q][w] = mrow[p[q] * MW + w];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (kept < R && live.has(p[q])) {
+        out[kept++] = id[q];
+#pragma unroll
+        for (int w = 0; w < MW; ++w) live.w[w] &= ~(m[q][w] | ((p[q] >> 6) == w ? 1ull << (p[q] & 63) : 0ull));
+      }
+    }
+  }
+  return kept;
+}
+
+// uint8 rows.  One CTA = 4 producer warps + 1 consumer warp.  The producers handle
+// NG = 128 / MAXM nodes at a time, one candidate per thread: gather, pivot keys
+// and norms, the rank of each candidate in the processing order (a4), its f16
+// operand row at CTA row (group, rank) = TMEM lane, the tcgen05 Gram, per-column
+// thresholds, and per target a domination mask for every rank, turned straight
+// from the lane's Gram row.  They hand ids and masks over through one of two
+// slots; the consumer warp runs the greedy loop per node and target (a7) while
+// the producers work on the next nodes.  4 CTAs per SM (the TMEM limit) need at
+// most 96 registers per thread; the kernels with more targets per launch, or one
+// 128-candidate node per MMA (more shared memory per CTA), trade that for
 // registers.
-template <int DT, int MAXM, int TB>
-constexpr int tc_min_ctas() { return (DT == kU8 && MAXM == 64 && TB <= 4) ? 4 : 2; }
+template <int MAXM, int TB>
+constexpr int tc_min_ctas() { return (MAXM == 64 && TB <= 4) ? 4 : 2; }
 
-template <int DT, int MAXM, int TB>
-__global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_kernel(PruneArgs a) {
-  // float rows: two f16 operands (hi, lo) and two accumulators (256 TMEM columns)
-  constexpr int kNop = DT == kF32 ? 2 : 1;
-  constexpr uint32_t kTmemCols = DT == kF32 ? 256u : 128u;
-  using L = TcLayout<MAXM, TB, kNop>;
-  using AT = typename Acc<DT>::T;
+template <int MAXM, int TB>
+__global__ void __launch_bounds__(160, tc_min_ctas<MAXM, TB>()) prune_u8_kernel(PruneArgs a) {
+  constexpr uint32_t kTmemCols = 128u;
+  using L = TcLayout<MAXM, TB, 1>;
+  using AT = typename Acc<kU8>::T;
   constexpr int NG = L::NG;
   constexpr int MW = L::MW;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -427,10 +512,7 @@ __global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_ker
   int64_t* qe0 = reinterpret_cast<int64_t*>(smem_raw + L::off_misc + L::q_e0);
   uint64_t* mbar = reinterpret_cast<uint64_t*>(smem_raw + L::off_misc + 128);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_raw + L::off_misc + 144);
-  int* rq_count = misc + 14;  // [2]: per slot parity
-  uint32_t* rq = reinterpret_cast<uint32_t*>(smem_raw + L::off_rq);
   auto slot_base = [&](int s, int g) { return smem_raw + L::off_slots + (size_t(s) * NG + g) * L::s_bytes; };
-  const float E_rel = slice_rel_bound(a.d), E_abs = abs_bound(a.d);
   const int count = *a.count;
   if (warp == 0) tmem_alloc(tmem_slot, kTmemCols);  // of the SM's 512 TMEM columns, for the kernel's life
   if (r == 0) {
@@ -438,7 +520,6 @@ __global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_ker
     // the queue counts up to kClaim; a claim of fewer nodes fills its end
     misc[12] = kClaim;  // empty claim queue
     misc[13] = kClaim - max(NG, min(kClaim, count / (int(gridDim.x) * 4) / NG * NG));
-    rq_count[0] = rq_count[1] = 0;
   }
   tc_fence_before();
   __syncthreads();
@@ -450,35 +531,15 @@ __global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_ker
     const int t = r % MAXM;
     unsigned char* pb = smem_raw + L::off_prod + g * L::p_bytes;
     AT* norm = reinterpret_cast<AT*>(pb + L::p_norm);
-    float* sn = reinterpret_cast<float*>(pb + L::p_sn);
     float* qlo = reinterpret_cast<float*>(pb + L::p_qlo);
-    float* qhi = reinterpret_cast<float*>(pb + L::p_qhi);
-    float4* cq = reinterpret_cast<float4*>(pb + L::p_cq);
     const uint32_t tmem = *tmem_slot;
-    // operands go in as f16: uint8 values exactly, float rows centred on the
-    // pivot, scaled by a power of two into [-1, 1] and split (issue_gram_slice)
-    const int64_t elems = a.row_bytes / (DT == kU8 ? 1 : 4);  // padded dims per row
+    const int64_t elems = a.row_bytes;  // padded dims per row
     const int nslices = int((elems + 127) / 128);
-    // Split f16 Gram of the scaled centred rows y = x - p, G' = hi hi^T + 2^-11
-    // (hi lo^T + lo hi^T): |G~ - <y_u, y_v>| <= eps_ip |y_u||y_v| + 2^-36 sqrt(d)
-    // (|y_u| + |y_v|) / scale (the f32 subtractions 2^-23 relative to
-    // |y_u||y_v|, the split 2^-22 per operand, the dropped lo lo^T term 2^-22,
-    // the last sum 2^-23, f32 accumulation d 2^-24 with a factor 4 allowance;
-    // subnormal lo).  The squared norms |y|^2 are the pivot keys, whose
-    // single-precision bound is E_rel relative (+ E_abs); eps_n adds the
-    // roundings that form d2 and its two bounds.
-    const float eps_ip = 5.f * 2.384185791015625e-07f + 1.1920929e-07f + float(a.d) * 2.384185791015625e-07f;
-    const float sub_abs = a.sqrt_d * 1.001f * 2.910383e-11f * a.inv_s;  // twice 2^-36 sqrt(d) / scale
-    const float eps_n = E_rel + 6.f * 5.9604645e-08f;
-    const float err_abs = 2.f * E_abs + float(a.d) * 2.3509887e-38f;  // + underflowed products, 2^-125 each
     uint32_t phase = 0;
     bool dead = false;
-    unsigned long long n_rechecks = 0;  // single-precision rechecks, added to the status once at the end
     for (int k = 0;; ++k) {
       const int s = k & 1;
       named_sync(kBarFree + s, 160);  // the consumer is done with this slot
-      // the consumer has resolved this slot's queue of two rounds ago: empty it
-      if (DT == kF32 && r == 0) rq_count[s] = 0;
       if (warp == 0) {
         // next NG nodes from the claim queue; warp 0 refills it kClaim nodes (or
         // the launch's smaller share) at a time: one atomic, the row bounds
@@ -524,7 +585,6 @@ __global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_ker
         break;
       }
       unsigned char* sb = slot_base(s, g);
-      double* key64 = reinterpret_cast<double*>(sb + L::s_key64);
       unsigned long long* masks = reinterpret_cast<unsigned long long*>(sb + L::s_masks);
       int32_t* ids = reinterpret_cast<int32_t*>(sb + L::s_ids);
       AT* key = reinterpret_cast<AT*>(sb + L::s_key);
@@ -548,7 +608,7 @@ __global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_ker
       // ---- a2 gather, a3 pivot key d2(p, x) and norm |x|^2 of candidate t
       AT kacc = 0, nacc = 0;
       uint4 xs[8];  // uint8, one slice: the row stays here for the operand pass
-      if constexpr (DT == kU8) {
+      {
         // d2(p, x) = |p|^2 + |x|^2 - 2 <p, x>: an identity of integers, exact in
         // 32-bit modular arithmetic since d2 < 2^32; |p|^2 is summed across the warp
         unsigned dacc = 0, pacc = 0;
@@ -578,80 +638,23 @@ __global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_ker
           }
         }
         kacc = pacc + nacc - 2u * dacc;
-      } else {
-        // Rows of one 128-dimension slice also write their split f16 operand
-        // here, at the stored position, so the row is read once.
-        const bool one_slice = nslices == 1;
-        if (live_row || one_slice) {
-          // The key is summed per 32-dimension slice (slice_rel_bound), each
-          // slice as two interleaved running sums of 16 squares added at its
-          // end: a bound of 17 roundings per slice, within the 32 allowed, and
-          // half the dependent chain.
-          float part = 0.f, part1 = 0.f;
-#pragma unroll 4
-          for (int c = 0; c < int(elems / 8); ++c) {
-            uint4 x0 = make_uint4(0, 0, 0, 0), x1 = x0, y0 = x0, y1 = x0;
-            if (live_row) {
-              const uint4* xq = reinterpret_cast<const uint4*>(xrow) + 2 * c;
-              const uint4* pq = reinterpret_cast<const uint4*>(prow) + 2 * c;
-              x0 = __ldg(xq);
-              x1 = __ldg(xq + 1);
-              y0 = __ldg(pq);
-              y1 = __ldg(pq + 1);
-            }
-            part = Acc<kF32>::step4(x0, y0, part);
-            part1 = Acc<kF32>::step4(x1, y1, part1);
-            if ((c & 3) == 3 || c == int(elems / 8) - 1) {
-              kacc += part + part1;
-              part = part1 = 0.f;
-            }
-            if (one_slice) {  // rows past the degree: zeros
-              const float xv[8] = {__uint_as_float(x0.x), __uint_as_float(x0.y), __uint_as_float(x0.z),
-                                   __uint_as_float(x0.w), __uint_as_float(x1.x), __uint_as_float(x1.y),
-                                   __uint_as_float(x1.z), __uint_as_float(x1.w)};
-              const float pv[8] = {__uint_as_float(y0.x), __uint_as_float(y0.y), __uint_as_float(y0.z),
-                                   __uint_as_float(y0.w), __uint_as_float(y1.x), __uint_as_float(y1.y),
-                                   __uint_as_float(y1.z), __uint_as_float(y1.w)};
-              store_split8_centred(opnd, g * MAXM + t, c, xv, pv, a.scale);
-            }
-          }
-        }
       }
       // ---- a4 processing order: the rank of (d2(p, x), id) among the m
       // candidates is x's place in Algorithm 1's argmin sequence (stored order
-      // for the unsorted variant).  Ids, keys, thresholds and masks below are
-      // laid out by rank; uint8 operand rows too, float operand rows stay at
-      // the stored position.
+      // for the unsorted variant).  Ids, keys, thresholds, masks and operand rows
+      // are laid out by rank.
       unsigned long long* sk = reinterpret_cast<unsigned long long*>(pb + L::p_sk);  // stored order
-      const unsigned long long my_sk = live_row ? (Acc<DT>::bits(kacc) << 32) | unsigned(my_id) : ~0ull;
+      const unsigned long long my_sk = live_row ? (Acc<kU8>::bits(kacc) << 32) | unsigned(my_id) : ~0ull;
       sk[t] = my_sk;
-      // Float rows of one slice have their operands in place: the Gram (a5)
-      // starts now and runs while the ranks are found.
-      const bool early_mma = DT == kF32 && nslices == 1;
-      if (early_mma) {
-        fence_async_smem();
-        tc_fence_before();
-      }
       named_sync(kBarProd, 128);
-      if (early_mma) {
-        tc_fence_after();
-        if (r == 0) {
-          issue_gram_slice<true>(tmem, opnd, int(elems), false);
-          umma_commit(mbar);
-        }
-      }
       int rank = t;
       // A list that Algorithm 1 wrote is already in its processing order
       // ((d2, id) ascending): then every rank is the stored position.  Checked,
-      // not assumed: each candidate against the one before it (for float keys,
-      // "surely less", which chains, so no two keys of the list can be near).
+      // not assumed: each candidate against the one before it.
       bool in_order = true;
       if (a.variant == 0) {
         bool inv = false;
-        if (live_row && t > 0) {
-          if constexpr (DT == kU8) inv = !(sk[t - 1] < my_sk);
-          else inv = !sure_less(__uint_as_float(unsigned(sk[t - 1] >> 32)), kacc, E_rel, E_abs);
-        }
+        if (live_row && t > 0) inv = !(sk[t - 1] < my_sk);
         in_order = !prod_sync_or(inv);
       }
       if (!in_order && live_row) {
@@ -666,83 +669,12 @@ __global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_ker
         }
         rank = cnt0 + cnt1;
       }
-      double my64 = __longlong_as_double(0x7ff8000000000000ll);
-      if constexpr (DT == kF32) {
-        // single-precision keys that might be out of order (intervals overlap):
-        // both ends of every such pair take a float-float key, and those pairs
-        // are ordered by it; only if two float-float intervals still meet do
-        // all such keys take their binary64 value (ties by id), as Algorithm 1
-        // reads d2 in binary64
-        // A key has a near partner iff a neighbour in single-precision order has
-        // one: sure_less is monotone, so every key between two near keys is near
-        // both.  The keys are laid out by rank (that order) and each thread looks
-        // at its two neighbours.
-        bool near = false;
-        if (!in_order) {
-          float* srt = reinterpret_cast<float*>(pb + L::p_srt);
-          if (live_row) srt[rank] = kacc;
-          named_sync(kBarProd, 128);
-          if (live_row)
-            near = (rank > 0 && !sure_less(srt[rank - 1], kacc, E_rel, E_abs)) ||
-                   (rank + 1 < m && !sure_less(kacc, srt[rank + 1], E_rel, E_abs));
-        }
-        if (!in_order && prod_sync_or(near)) {
-          double* k64s = reinterpret_cast<double*>(pb + L::p_k64);  // stored order
-          const FFBound fb = ff_bound(a.d);
-          if (near) my64 = -ff_d2(reinterpret_cast<const float*>(prow), reinterpret_cast<const float*>(xrow), a.row_bytes);
-          k64s[t] = my64;
-          named_sync(kBarProd, 128);
-          int cnt = 0;
-          bool open = false;
-          if (near) {
-            for (int j = 0; j < m; ++j) {
-              const float kj = __uint_as_float(unsigned(sk[j] >> 32));
-              if (sure_less(kj, kacc, E_rel, E_abs)) {
-                ++cnt;
-              } else if (j != t && !sure_less(kacc, kj, E_rel, E_abs)) {
-                const int o = slot_order(k64s[j], my64, fb);  // 1: j first
-                if (o < 0) open = true;
-                else cnt += o;
-              }
-            }
-          }
-          if (prod_sync_or(open)) {  // every reader of k64s has passed the barrier
-            if (near) {
-              my64 = canon_d2_f32(reinterpret_cast<const float*>(prow), reinterpret_cast<const float*>(xrow), a.d);
-              atomicAdd(&a.status->fp64_sort_keys, 1ull);
-            }
-            k64s[t] = my64;
-            named_sync(kBarProd, 128);
-            if (near) {
-              cnt = 0;
-              for (int j = 0; j < m; ++j) {
-                const float kj = __uint_as_float(unsigned(sk[j] >> 32));
-                if (sure_less(kj, kacc, E_rel, E_abs)) {
-                  ++cnt;
-                } else if (j != t && !sure_less(kacc, kj, E_rel, E_abs)) {
-                  const double dj = k64s[j];
-                  const int32_t idj = int32_t(unsigned(sk[j]));
-                  cnt += (dj < my64 || (dj == my64 && idj < my_id)) ? 1 : 0;
-                }
-              }
-            }
-          }
-          if (near) rank = cnt;
-        }
-      }
       if (live_row) {
         ids[rank] = my_id;
         key[rank] = kacc;
-        if constexpr (DT == kF32) {
-          // the centred rows' squared norms are the pivot keys
-          norm[rank] = kacc;
-          sn[rank] = sqrtf(kacc);
-          key64[rank] = my64;
-        } else {
-          norm[rank] = nacc;
-        }
+        norm[rank] = nacc;
       }
-      if constexpr (DT == kU8) {
+      {
         // ---- f16 operand row at position rank (rows past the degree stay zero);
         // a5 Gram on tcgen05, one MMA chain per 128-dim slice
         const int orow = g * MAXM + rank;
@@ -871,254 +803,14 @@ __global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_ker
         tc_fence_before();
         named_sync(kBarProd, 128);  // every producer's masks and TMEM reads are done
         tc_fence_after();
-      } else {
-        // ---- float rows: the operands stay at the stored position, so the
-        // Gram is in stored order; it is staged in shared memory in rank order
-        // and every pair (row before column) is decided from there, the pairs
-        // spread evenly over the 128 producer threads.
-        int* rank_of = reinterpret_cast<int*>(pb + L::p_rk);  // rank of each stored position
-        if (live_row) rank_of[t] = rank;
-        // rows of several 128-dimension slices: one MMA chain per slice, a
-        // slice's operands written once the previous MMA has read its own
-        for (int sl = 0; !early_mma && sl < nslices; ++sl) {
-          const int64_t rem = elems - int64_t(sl) * 128;
-          const int kd = int(rem < 128 ? rem : 128);  // a multiple of 16 here
-          if (sl > 0) {
-            const bool ok = mbar_wait(mbar, phase, 1 << 24);
-            if (prod_sync_or(!ok)) {  // the MMA never completed: report, stop after this slot (uniform)
-              if (r == 0) raise_status(a.status, kDevOverflow, -2);
-              dead = true;
-            }
-            phase ^= 1u;
-            tc_fence_after();
-            if (dead) break;
-          }
-#pragma unroll 4
-          for (int c = 0; c < kd / 8; ++c) {
-            uint4 x0 = make_uint4(0, 0, 0, 0), x1 = x0, y0 = x0, y1 = x0;
-            if (live_row) {  // rows past the degree stay zero
-              const uint4* xq = reinterpret_cast<const uint4*>(xrow + int64_t(sl) * 512) + 2 * c;
-              const uint4* pq = reinterpret_cast<const uint4*>(prow + int64_t(sl) * 512) + 2 * c;
-              x0 = __ldg(xq);
-              x1 = __ldg(xq + 1);
-              y0 = __ldg(pq);
-              y1 = __ldg(pq + 1);
-            }
-            const float xv[8] = {__uint_as_float(x0.x), __uint_as_float(x0.y), __uint_as_float(x0.z),
-                                 __uint_as_float(x0.w), __uint_as_float(x1.x), __uint_as_float(x1.y),
-                                 __uint_as_float(x1.z), __uint_as_float(x1.w)};
-            const float pv[8] = {__uint_as_float(y0.x), __uint_as_float(y0.y), __uint_as_float(y0.z),
-                                 __uint_as_float(y0.w), __uint_as_float(y1.x), __uint_as_float(y1.y),
-                                 __uint_as_float(y1.z), __uint_as_float(y1.w)};
-            store_split8_centred(opnd, g * MAXM + t, c, xv, pv, a.scale);
-          }
-          fence_async_smem();
-          tc_fence_before();
-          named_sync(kBarProd, 128);
-          tc_fence_after();
-          if (r == 0) {
-            issue_gram_slice<true>(tmem, opnd, kd, sl > 0);
-            umma_commit(mbar);
-          }
-        }
-        // while the MMA runs: the thresholds of column `rank` for every distinct
-        // alpha (a6).  The last factor of each (1 -+ 1e-6) covers the roundings
-        // of the pair's d2 - err and d2 + err, compared against them directly.
-        // a column's thresholds are TA4 = TA rounded up to 4 floats apart, so
-        // that consecutive columns' 16-byte reads are consecutive
-        const int TA4 = (a.TA + 3) & ~3;
-        if (live_row) {
-#pragma unroll
-          for (int u = 0; u < TB; ++u) {
-            if (u >= a.TA) break;
-            // kappa = 1e6 / A^2 carries one rounding and the product two more; the
-            // last factor (1 -+ 2e-6) covers them with room to spare, and the
-            // roundings of the pair's d2 - err and d2 + err, compared against
-            // these thresholds directly
-            qlo[rank * TA4 + u] = (kacc * (1.0f - E_rel) - E_abs) * a.kappa[u] * 0.999998f;
-            qhi[rank * TA4 + u] = (kacc * (1.0f + E_rel) + E_abs) * a.kappa[u] * 1.000002f;
-          }
-          // padding past the last alpha never counts (hi < -inf, lo > -inf)
-          for (int u = a.TA; u < TA4; ++u) qlo[rank * TA4 + u] = qhi[rank * TA4 + u] = -INFINITY;
-          cq[rank] = make_float4(kacc, sqrtf(kacc), 0.f, 0.f);  // the column's centred norm^2 and its root
-        }
-        if (next_id >= 0) {
-          const char* nrow = reinterpret_cast<const char*>(a.X + int64_t(next_id) * a.row_bytes);
-          for (int64_t off = 0; off < a.row_bytes; off += 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(nrow + off));
-        }
-        // the Gram's MMA (dead is uniform; a slot that is already dead has none
-        // outstanding)
-        const bool waited = !dead;
-        const bool ok = waited ? mbar_wait(mbar, phase, 1 << 24) : true;
-        // one barrier: every rank-indexed array is complete, and the wait's outcome is known to all
-        if (prod_sync_or(!ok)) {  // the MMA never completed: report, stop after this slot (uniform)
-          if (r == 0) raise_status(a.status, kDevOverflow, -2);
-          dead = true;
-        }
-        if (waited) phase ^= 1u;
-        tc_fence_after();
-        // The group's Gram, MAXM x MAXM in rank order over the operands (read by
-        // now), row R rotated by R: G~(R, c) at [R * MAXM + (c + R) % MAXM], the
-        // entries with R < c, in the operands' scaled units (G~ / inv_s2).
-        // tcgen05.ld is warp-collective: every lane issues it, live rows store.
-        float* Gs = reinterpret_cast<float*>(opnd) + size_t(g) * MAXM * MAXM;
-        if (!dead) {
-          const int cend = (m + 15) & ~15;  // the same for every lane of the warp (one node)
-          const uint32_t lane_base = tmem + (uint32_t(32 * warp) << 16) + uint32_t(g * MAXM);
-          float* grow = Gs + size_t(rank) * MAXM;
-          const int4* rk4 = reinterpret_cast<const int4*>(rank_of);
-#pragma unroll 1
-          for (int c0 = 0; c0 < cend; c0 += 16) {
-            uint32_t v[16], v2[16];
-            tmem_ld8(lane_base + uint32_t(c0), *reinterpret_cast<uint32_t(*)[8]>(v));
-            tmem_ld8(lane_base + uint32_t(c0 + 8), *reinterpret_cast<uint32_t(*)[8]>(v + 8));
-            tmem_ld8(lane_base + uint32_t(128 + c0), *reinterpret_cast<uint32_t(*)[8]>(v2));
-            tmem_ld8(lane_base + uint32_t(128 + c0 + 8), *reinterpret_cast<uint32_t(*)[8]>(v2 + 8));
-            tmem_ld_wait();
-            if (live_row) {
-#pragma unroll
-              for (int j4 = 0; j4 < 16; j4 += 4) {
-                const int4 r4 = rk4[(c0 + j4) / 4];  // ranks of four stored columns (past m: not used)
-                const int rc[4] = {r4.x, r4.y, r4.z, r4.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                  if (c0 + j4 + j < m && rc[j] > rank)  // in the scaled units (inv_s2 goes into the decision)
-                    grow[(rc[j] + rank) & (MAXM - 1)] = fmaf(__uint_as_float(v2[j4 + j]), 4.8828125e-04f,
-                                                             __uint_as_float(v[j4 + j]));
-              }
-            }
-          }
-          // rank row t's masks start empty (the rows of the group, one per thread)
-#pragma unroll
-          for (int u = 0; u < TB; ++u) {
-            if (u >= a.TA) break;
-#pragma unroll
-            for (int w = 0; w < MW; ++w) masks[(u * MAXM + t) * MW + w] = 0ull;
-          }
-        }
-        tc_fence_before();
-        named_sync(kBarProd, 128);  // the staged Gram, the cleared masks; TMEM read
-        tc_fence_after();
-        if (!dead) {
-          // Rows pair up as (q, MAXM - 1 - q): row q has MAXM - 1 - q later
-          // columns and row MAXM - 1 - q has q, MAXM - 1 in all, and the two
-          // threads of a pair take half each.  Thread h = 0 takes row q's first
-          // Q columns; thread h = 1 the rest of row q, then row MAXM - 1 - q.
-          // Item k of a thread is one (row, column) pair.
-          constexpr int Q = MAXM / 2;
-          const int q = t % Q, h = t / Q;
-          const int rA = q, rB = MAXM - 1 - q;
-          const int nItems = h == 0 ? Q : Q - 1;
-          const int nA = h == 0 ? Q : Q - 1 - q;        // items on row rA, the rest on row rB
-          const int cA = h == 0 ? rA + 1 : rA + Q + 1;  // row rA's first column
-          const int cB = rB + 1;                         // row rB's first column
-          // the d2 error bound as two multiply-adds: err = |c| At + |c|^2 eps_n + Bt
-          const float ntA = rA < m ? float(norm[rA]) : 0.f, stA = rA < m ? sn[rA] : 0.f;
-          const float ntB = rB < m ? float(norm[rB]) : 0.f, stB = rB < m ? sn[rB] : 0.f;
-          const float AtA = 2.f * eps_ip * stA * 1.0009765625f + sub_abs, BtA = sub_abs * stA + eps_n * ntA + err_abs;
-          const float AtB = 2.f * eps_ip * stB * 1.0009765625f + sub_abs, BtB = sub_abs * stB + eps_n * ntB + err_abs;
-          const int TA = a.TA;
-          const float m2inv_s2 = -2.f * a.inv_s2;
-          const float4* ql4 = reinterpret_cast<const float4*>(qlo);
-          const float4* qh4 = reinterpret_cast<const float4*>(qhi);
-          // Per distinct alpha u, bit k of mk[u] says that item k's column is
-          // surely removed at alpha u: hi < qlo(column, u).  Those tests are a
-          // prefix over u (the alphas ascend, the thresholds fall), so they are
-          // the row masks' bits as they stand.  "May be removed", !(lo >
-          // qhi(column, u)), is a prefix too; an item is open when some alpha may
-          // remove its column without surely doing so.
-          using IW = typename std::conditional<(Q <= 32), unsigned, unsigned long long>::type;
-          IW mk[TB], open = 0;
-#pragma unroll
-          for (int u = 0; u < TB; ++u) mk[u] = 0;
-          // straight-line items (the open ones are only marked), so that the
-          // reads of several items overlap
-#pragma unroll 2
-          for (int k = 0; k < Q; ++k) {
-            const bool onA = k < nA;
-            const int R = onA ? rA : rB;
-            const int c = onA ? cA + k : cB + (k - nA);
-            const bool valid = k < nItems && c < m;  // c > R, so the row is live too
-            const int ci = valid ? c : 0;            // the reads stay in range for every k
-            const float G = Gs[R * MAXM + ((ci + R) & (MAXM - 1))];
-            const float4 qc = cq[ci];
-            const float dv = fmaf(G, m2inv_s2, (onA ? ntA : ntB) + qc.x);  // G~ = G * inv_s2: exact scaling
-            const float err = fmaf(qc.y, onA ? AtA : AtB, fmaf(qc.x, eps_n, onA ? BtA : BtB));
-            const float lo = dv - err, hi = dv + err;
-            bool op = false;
-#pragma unroll
-            for (int u4 = 0; u4 < L::TB4; u4 += 4) {
-              if (u4 < TA) {  // uniform
-                const float4 l4 = ql4[(ci * TA4 + u4) / 4];
-                const float4 h4 = qh4[(ci * TA4 + u4) / 4];
-                const float lv[4] = {l4.x, l4.y, l4.z, l4.w}, hv[4] = {h4.x, h4.y, h4.z, h4.w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                  if (u4 + e >= TB) break;
-                  const bool sure = valid && hi < lv[e];  // padding past TA: -inf, never
-                  if (sure) mk[u4 + e] |= IW(1) << k;
-                  op |= valid && !sure && !(lo > hv[e]);
-                }
-              }
-            }
-            if (op) open |= IW(1) << k;
-          }
-          // open pairs (rare): the alphas from ts (the surely-removing count) on
-          // are decided exactly by the consumer warp before its scan; here if the
-          // slot's queue is full
-          while (open) {
-            const int k = int(__ffsll(static_cast<long long>(open))) - 1;
-            open &= open - 1;
-            const bool onA = k < nA;
-            const int R = onA ? rA : rB;
-            const int c = onA ? cA + k : cB + (k - nA);
-            int ts = 0;
-#pragma unroll
-            for (int u = 0; u < TB; ++u) ts += int((mk[u] >> k) & 1u);
-            const int qi = atomicAdd(rq_count + s, 1);
-            if (qi < L::rq_cap) {
-              rq[s * L::rq_cap + qi] = (unsigned(g * MAXM + R) << 16) | (unsigned(c) << 5) | unsigned(ts);
-            } else {
-              // removal is monotone in alpha: the alphas before the first that keeps the pair remove it
-              const int u1 = recheck_prefix_cold(a, ids, key, key64, R, c, ts, TA, ppt, E_rel, E_abs);
-              n_rechecks += recheck_tests(ts, u1, TA);
-#pragma unroll
-              for (int u = 0; u < TB; ++u)
-                if (u >= ts && u < u1) mk[u] |= IW(1) << k;
-            }
-          }
-          // item masks -> row masks: row rA's items are [0, nA) from column cA,
-          // row rB's [nA, nItems) from column cB
-          auto or_run = [&](unsigned long long* row, unsigned long long bits, int col) {
-            const int w0 = col >> 6, sh = col & 63;
-            if (bits << sh) atomicOr(row + w0, bits << sh);
-            if (MW > 1 && sh && w0 + 1 < MW && (bits >> (64 - sh))) atomicOr(row + w0 + 1, bits >> (64 - sh));
-          };
-#pragma unroll
-          for (int u = 0; u < TB; ++u) {
-            if (u >= TA) break;
-            const unsigned long long gt = mk[u];
-            const unsigned long long mA = nA >= 64 ? gt : (gt & ((1ull << nA) - 1));
-            const unsigned long long mB = nA >= 64 ? 0ull : (gt >> nA);
-            if (mA) or_run(masks + (u * MAXM + rA) * MW, mA, cA);
-            if (mB) or_run(masks + (u * MAXM + rB) * MW, mB, cB);
-          }
-        }
-        if (dead && t == 0) misc[s * 2 + g] = -1;  // nothing valid in this slot
       }
       bar_arrive(kBarFull + s, 160);
-    }
-    if constexpr (DT == kF32) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) n_rechecks += __shfl_xor_sync(0xffffffffu, n_rechecks, o);
-      if (lane == 0 && n_rechecks) atomicAdd(&a.status->spare[2], n_rechecks);
     }
   } else {
     // =========================== consumer warp ===========================
     bar_arrive(kBarFree + 0, 160);  // both slots start free
     bar_arrive(kBarFree + 1, 160);
     long long done = 0;
-    unsigned long long n_rechecks = 0;  // single-precision rechecks of the queued pairs
     for (int k = 0;; ++k) {
       const int s = k & 1;
       named_sync(kBarFull + s, 160);
@@ -1129,25 +821,6 @@ __global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_ker
         done += misc[s * 2 + q] >= 0;
       }
       if (!any) break;
-      if constexpr (DT == kF32) {
-        // the slot's open pairs, one per lane: each alpha that removes the
-        // column sets its bit in the row's mask for that alpha
-        const int nq = min(rq_count[s], L::rq_cap);
-        for (int i = lane; i < nq; i += 32) {
-          const uint32_t e = rq[s * L::rq_cap + i];
-          const int tr = int(e >> 16), c = int((e >> 5) & 0x7ffu), u0 = int(e & 31u);
-          const int gq = tr / MAXM, tq = tr % MAXM;
-          unsigned char* sbq = slot_base(s, gq);
-          const int u1 = recheck_prefix(a, reinterpret_cast<const int32_t*>(sbq + L::s_ids),
-                                        reinterpret_cast<const float*>(sbq + L::s_key),
-                                        reinterpret_cast<double*>(sbq + L::s_key64), tq, c, u0, a.TA,
-                                        point_of_row(a, misc[s * 2 + gq]), E_rel, E_abs);
-          n_rechecks += recheck_tests(u0, u1, a.TA);
-          unsigned long long* mrow = reinterpret_cast<unsigned long long*>(sbq + L::s_masks) + tq * MW + (c >> 6);
-          for (int u = u0; u < u1; ++u) atomicOr(mrow + u * MAXM * MW, 1ull << (c & 63));
-        }
-        __syncwarp();
-      }
       // ---- a7 greedy scan: lane (g * 16 + u) runs Algorithm 1's loop for node
       // g and target u.  Candidates are laid out by rank, so the next argmin of
       // the live set is its lowest set bit.
@@ -1168,7 +841,7 @@ __global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_ker
             al[w] = m > lo ? ((m - lo >= 64) ? ~0ull : ((1ull << (m - lo)) - 1)) : 0ull;
           }
           const int R = a.R[u];
-          const int mu = DT == kF32 ? a.amap[u] : u;  // the target's domination mask
+          const int mu = u;  // the target's domination mask
           int32_t* out = a.out_col[u] + e0;
           int kept = 0;
           if constexpr (MW == 1) {
@@ -1210,16 +883,687 @@ __global__ void __launch_bounds__(160, tc_min_ctas<DT, MAXM, TB>()) prune_tc_ker
       bar_arrive(kBarFree + s, 160);
     }
     if (lane == 0 && done) atomicAdd(&a.status->nodes_pruned, static_cast<unsigned long long>(done) * T);
-    if constexpr (DT == kF32) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) n_rechecks += __shfl_xor_sync(0xffffffffu, n_rechecks, o);
-      if (lane == 0 && n_rechecks) atomicAdd(&a.status->spare[2], n_rechecks);
-    }
   }
   // the TMEM columns go back once the producers are finished with them
   if (warp < 4) {
     tc_fence_before();
     named_sync(kBarProd, 128);
+    tc_fence_after();
+    if (warp == 0) tmem_dealloc(*tmem_slot, kTmemCols);
+  }
+}
+
+// Float rows.  One CTA = 4 H producer warps + 1 consumer warp over NG = 128 / MAXM
+// nodes at a time, candidates as the 128 rows of the MMA in stored order:
+//   gather   four lanes share a row (lane = 8 sub + row: eight rows a step, so
+//            that loads read whole 128-byte lines and the 16-byte operand stores
+//            of a phase fall into different banks); each row is read once: its
+//            pivot key and its split f16 operand come from the same registers,
+//            slice by slice, and the Gram of the last slice runs during the rest;
+//   rank     H threads per candidate;
+//   stage    the Gram goes from TMEM to shared memory in rank order, H warps per
+//            TMEM quadrant, a part of the columns each;
+//   decide   every pair (row before column) from there, the pairs spread evenly
+//            over the producers.
+// The consumer warp resolves the slot's open pairs and runs the greedy loop per
+// node and target (a7) while the producers work on the next nodes.
+//
+// What bounds it: issue and latency at two CTAs per SM (256 of the SM's 512 TMEM
+// columns and about 100 KB of shared memory each).  One kernel for both types, with
+// a thread to a row in the gather and a row of pairs, took 8.73 ms for 400,000 x 96
+// floats in lists of up to 64 at eight targets and 8.77 ms for 30,000 x 960 at nine;
+// this one 8.3 and 6.9.
+template <int MAXM, int TB, int H>
+__global__ void __launch_bounds__(128 * H + 32, 2) prune_f32_kernel(PruneArgs a) {
+  constexpr int kF32Prod = 128 * H, kF32Threads = kF32Prod + 32;
+  constexpr int kRows = 32 / H;       // rows a warp gathers
+  constexpr int kSteps = kRows / 8;   // eight at a time
+  constexpr uint32_t kTmemCols = 256u;  // two accumulators
+  using L = TcLayout<MAXM, TB, 2>;
+  constexpr int NG = L::NG;
+  constexpr int MW = L::MW;
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  const int T = a.T;
+  const int r = threadIdx.x;
+  const int warp = r >> 5;
+  const int lane = r & 31;
+  unsigned char* opnd = smem_raw + L::off_opnd;
+  int* misc = reinterpret_cast<int*>(smem_raw + L::off_misc);
+  // misc ints: [0..3] slot node (s*2+g), [4..7] slot degree, [12] claim queue head, [13] its first entry
+  int64_t* misc64 = reinterpret_cast<int64_t*>(smem_raw + L::off_misc + 64);  // [0..3] slot row start
+  int* qnode = reinterpret_cast<int*>(smem_raw + L::off_misc + L::q_node);
+  int* qdeg = reinterpret_cast<int*>(smem_raw + L::off_misc + L::q_deg);
+  int64_t* qe0 = reinterpret_cast<int64_t*>(smem_raw + L::off_misc + L::q_e0);
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(smem_raw + L::off_misc + 128);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_raw + L::off_misc + 144);
+  int* rq_count = misc + 14;  // [2]: per slot parity
+  uint32_t* rq = reinterpret_cast<uint32_t*>(smem_raw + L::off_rq);
+  auto slot_base = [&](int s, int g) { return smem_raw + L::off_slots + (size_t(s) * NG + g) * L::s_bytes; };
+  auto prod_base = [&](int g) { return smem_raw + L::off_prod + g * L::p_bytes; };
+  const float E_rel = slice_rel_bound(a.d), E_abs = abs_bound(a.d);
+  const int count = *a.count;
+
+  if (warp == 0) tmem_alloc(tmem_slot, kTmemCols);  // of the SM's 512 TMEM columns, for the kernel's life
+  if (r == 0) {
+    mbar_init(mbar, 1);
+    // the queue counts up to kClaim; a claim of fewer nodes fills its end
+    misc[12] = kClaim;  // empty claim queue
+    misc[13] = kClaim - max(NG, min(kClaim, count / (int(gridDim.x) * 4) / NG * NG));
+    rq_count[0] = rq_count[1] = 0;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+
+  if (warp < kF32Prod / 32) {
+    // =========================== producers ===========================
+    const uint32_t tmem = *tmem_slot;
+    const int64_t elems = a.row_bytes / 4;  // padded dims per row, a multiple of 32
+    const int nslices = int((elems + 127) / 128);
+    // Split f16 Gram of the scaled centred rows y = x - p, G' = hi hi^T + 2^-11
+    // (hi lo^T + lo hi^T): |G~ - <y_u, y_v>| <= eps_ip |y_u||y_v| + 2^-36 sqrt(d)
+    // (|y_u| + |y_v|) / scale (the f32 subtractions 2^-23 relative to
+    // |y_u||y_v|, the split 2^-22 per operand, the dropped lo lo^T term 2^-22,
+    // the last sum 2^-23, f32 accumulation d 2^-24 with a factor 4 allowance;
+    // subnormal lo).  The squared norms |y|^2 are the pivot keys, whose
+    // single-precision bound is E_rel relative (+ E_abs); eps_n adds the
+    // roundings that form d2 and its two bounds.
+    const float eps_ip = 5.f * 2.384185791015625e-07f + 1.1920929e-07f + float(a.d) * 2.384185791015625e-07f;
+    const float sub_abs = a.sqrt_d * 1.001f * 2.910383e-11f * a.inv_s;  // twice 2^-36 sqrt(d) / scale
+    const float eps_n = E_rel + 6.f * 5.9604645e-08f;
+    const float err_abs = 2.f * E_abs + float(a.d) * 2.3509887e-38f;  // + underflowed products, 2^-125 each
+    uint32_t phase = 0;
+    bool dead = false;
+    unsigned long long n_rechecks = 0;  // single-precision rechecks, added to the status once at the end
+    // candidate roles: threads H c .. H c + H - 1 for the CTA's row c, in warp c / kRows
+    const int g = (r / H) / MAXM, t = (r / H) % MAXM, half = r % H;
+    unsigned char* pb = prod_base(g);
+    float* norm = reinterpret_cast<float*>(pb + L::p_norm);
+    float* sn = reinterpret_cast<float*>(pb + L::p_sn);
+    float* rec = reinterpret_cast<float*>(pb + L::p_qlo);  // per column: thresholds, key, root
+    unsigned long long* sk = reinterpret_cast<unsigned long long*>(pb + L::p_sk);  // (key, id) in stored order
+    for (int k = 0;; ++k) {
+      const int s = k & 1;
+      named_sync(kBarFree + s, kF32Threads);  // the consumer is done with this slot
+      // the consumer has resolved this slot's queue of two rounds ago: empty it
+      if (r == 0) rq_count[s] = 0;
+      if (warp == 0) {
+        // next NG nodes from the claim queue; warp 0 refills it kClaim nodes (or
+        // the launch's smaller share) at a time: one atomic, the row bounds
+        // loaded by all lanes at once
+        int head = misc[12];
+        if (head >= kClaim) {
+          const int skip = misc[13];
+          unsigned base = 0;
+          if (lane == 0) base = atomicAdd(a.work, unsigned(kClaim - skip));
+          base = __shfl_sync(0xffffffffu, base, 0);
+          const unsigned idx = base + unsigned(lane - skip);
+          const int pn = lane >= skip && idx < unsigned(count) ? a.nodes[idx] : -1;
+          int deg = 0;
+          int64_t e0n = 0;
+          if (pn >= 0) {
+            e0n = a.row_ptr[pn];
+            deg = int(a.row_ptr[pn + 1] - e0n);
+          }
+          if (deg > MAXM) {  // bucketing never sends such a node here; skip it, report it
+            raise_status(a.status, kDevBadDegree, pn);
+            deg = 0;
+          }
+          qnode[lane] = pn;
+          qdeg[lane] = deg;
+          qe0[lane] = e0n;
+          __syncwarp();
+          head = skip;
+        }
+        if (lane < NG) {
+          misc[s * 2 + lane] = dead ? -1 : qnode[head + lane];
+          misc[4 + s * 2 + lane] = dead ? 0 : qdeg[head + lane];
+          misc64[s * 2 + lane] = qe0[head + lane];
+        }
+        __syncwarp();
+        if (lane == 0) misc[12] = head + NG;
+      }
+      named_sync(kBarProd, kF32Prod);
+      bool any = false;
+#pragma unroll
+      for (int q = 0; q < NG; ++q) any |= misc[s * 2 + q] >= 0;
+      if (!any) {  // tell the consumer there is nothing more, and stop
+        bar_arrive(kBarFull + s, kF32Threads);
+        break;
+      }
+      unsigned char* sb = slot_base(s, g);
+      double* key64 = reinterpret_cast<double*>(sb + L::s_key64);
+      unsigned long long* masks = reinterpret_cast<unsigned long long*>(sb + L::s_masks);
+      int32_t* ids = reinterpret_cast<int32_t*>(sb + L::s_ids);
+      float* key = reinterpret_cast<float*>(sb + L::s_key);
+      const int p = misc[s * 2 + g];
+      const int m = misc[4 + s * 2 + g];
+      const int64_t e0 = misc64[s * 2 + g];
+      const bool live_row = t < m;  // this thread's row is stored candidate t
+      const int32_t ppt = p >= 0 ? point_of_row(a, p) : 0;  // the point being pruned
+      const uint8_t* prow = a.X + int64_t(ppt) * a.row_bytes;
+      // The next slot's node of this group, if the claim queue already holds it:
+      // its candidate ids are loaded now and their rows prefetched into L2 while
+      // this slot waits on its Gram, so the next gather finds them there.
+      int32_t next_id = -1;
+      {
+        const int nh = misc[12] + g;
+        if (nh < kClaim && t < qdeg[nh]) next_id = a.col[qe0[nh] + t];
+      }
+      // ---- a2 gather, a3 pivot keys, split operands, a5 Gram: warp w has the
+      // rows from kRows w on, all of one node (its threads' own), eight at a time
+      {
+        const int sub = lane >> 3;
+        bool lv[kSteps];
+        int32_t gid[kSteps];
+        float kacc[kSteps];
+#pragma unroll
+        for (int q = 0; q < kSteps; ++q) {
+          const int row = kRows * warp + 8 * q + (lane & 7);
+          lv[q] = row % MAXM < m;
+          gid[q] = lv[q] ? a.col[e0 + row % MAXM] : 0;
+          kacc[q] = 0.f;
+        }
+        const uint4* pp = reinterpret_cast<const uint4*>(prow);
+        for (int sl = 0; sl < nslices; ++sl) {
+          if (sl > 0) {  // the operands are free once the previous slice's MMA has read them
+            const bool ok = mbar_wait(mbar, phase, 1 << 24);
+            if (prod_sync_or_n<kF32Prod>(!ok)) {  // the MMA never completed: report, stop after this slot (uniform)
+              if (r == 0) raise_status(a.status, kDevOverflow, -2);
+              dead = true;
+            }
+            phase ^= 1u;
+            tc_fence_after();
+            if (dead) break;
+          }
+          const int64_t rem = elems - int64_t(sl) * 128;
+          const int np = int(rem < 128 ? rem : 128) / 8;  // groups of eight dimensions, a multiple of four
+          // The key of a slice: two running sums per lane (the two halves of each
+          // group), joined, then over the four lanes: at most 16 + 1 + 2 roundings,
+          // within the 32 of slice_rel_bound (fewer dimensions take fewer).
+          float part[kSteps][2];
+#pragma unroll
+          for (int q = 0; q < kSteps; ++q) part[q][0] = part[q][1] = 0.f;
+#pragma unroll 1
+          for (int c = sub; c < np; c += 4) {
+            const int64_t at = int64_t(sl) * 32 + 2 * c;
+            const uint4 y0 = __ldg(pp + at), y1 = __ldg(pp + at + 1);
+            uint4 x0[kSteps], x1[kSteps];
+#pragma unroll
+            for (int q = 0; q < kSteps; ++q) {
+              const uint4* px = reinterpret_cast<const uint4*>(a.X + int64_t(gid[q]) * a.row_bytes) + at;
+              x0[q] = lv[q] ? __ldg(px) : y0;  // rows past the degree: the pivot, centred zeros
+              x1[q] = lv[q] ? __ldg(px + 1) : y1;
+            }
+            const float pv[8] = {__uint_as_float(y0.x), __uint_as_float(y0.y), __uint_as_float(y0.z),
+                                 __uint_as_float(y0.w), __uint_as_float(y1.x), __uint_as_float(y1.y),
+                                 __uint_as_float(y1.z), __uint_as_float(y1.w)};
+#pragma unroll
+            for (int q = 0; q < kSteps; ++q) {
+              const float xv[8] = {__uint_as_float(x0[q].x), __uint_as_float(x0[q].y), __uint_as_float(x0[q].z),
+                                   __uint_as_float(x0[q].w), __uint_as_float(x1[q].x), __uint_as_float(x1[q].y),
+                                   __uint_as_float(x1[q].z), __uint_as_float(x1[q].w)};
+              float y[8];
+#pragma unroll
+              for (int e = 0; e < 8; ++e) y[e] = xv[e] - pv[e];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                part[q][0] = fmaf(y[e], y[e], part[q][0]);
+                part[q][1] = fmaf(y[4 + e], y[4 + e], part[q][1]);
+              }
+              store_split8(opnd, kRows * warp + 8 * q + (lane & 7), c, y, a.scale);
+            }
+          }
+#pragma unroll
+          for (int q = 0; q < kSteps; ++q) {
+            float v = part[q][0] + part[q][1];
+            v += __shfl_xor_sync(0xffffffffu, v, 8);
+            v += __shfl_xor_sync(0xffffffffu, v, 16);
+            kacc[q] += v;
+          }
+          if (sl == nslices - 1 && sub == 0) {
+#pragma unroll
+            for (int q = 0; q < kSteps; ++q) {
+              const int row = kRows * warp + 8 * q + lane;
+              sk[row % MAXM] =
+                  lv[q] ? (static_cast<unsigned long long>(__float_as_uint(kacc[q])) << 32) | unsigned(gid[q]) : ~0ull;
+            }
+          }
+          fence_async_smem();
+          tc_fence_before();
+          named_sync(kBarProd, kF32Prod);  // the slice's operands; after the last one, the keys
+          tc_fence_after();
+          if (r == 0) {
+            issue_gram_slice<true>(tmem, opnd, 8 * np, sl > 0);
+            umma_commit(mbar);
+          }
+        }
+      }
+      if (dead) {  // nothing valid in this slot
+        if (r < NG) misc[s * 2 + r] = -1;
+        named_sync(kBarProd, kF32Prod);
+        bar_arrive(kBarFull + s, kF32Threads);
+        continue;  // the claim queue gives no node any more
+      }
+      // ---- a4 processing order: the rank of (d2(p, x), id) among the m candidates
+      // is x's place in Algorithm 1's argmin sequence (stored order for the unsorted
+      // variant).  Ids, keys, thresholds, masks and the staged Gram are laid out by
+      // rank.  The threads of a candidate end with the same rank.
+      const unsigned long long my_sk = sk[t];  // ~0 past the degree
+      const int32_t my_id = int32_t(unsigned(my_sk));
+      const float kacc = __uint_as_float(unsigned(my_sk >> 32));
+      const uint8_t* xrow = a.X + int64_t(live_row ? my_id : 0) * a.row_bytes;
+      int rank = t;
+      // A list that Algorithm 1 wrote is already in its processing order
+      // ((d2, id) ascending): then every rank is the stored position.  Checked,
+      // not assumed: each candidate against the one before it ("surely less",
+      // which chains, so no two keys of the list can be near).
+      bool in_order = true;
+      if (a.variant == 0) {
+        bool inv = false;
+        if (live_row && t > 0 && half == 0)
+          inv = !sure_less(__uint_as_float(unsigned(sk[t - 1] >> 32)), kacc, E_rel, E_abs);
+        in_order = !prod_sync_or_n<kF32Prod>(inv);
+      }
+      if (!in_order) {
+        // entries past the degree hold ~0 and never count; the candidate's threads
+        // take every H-th pair of entries
+        const ulonglong2* sk2 = reinterpret_cast<const ulonglong2*>(sk);
+        int cnt0 = 0, cnt1 = 0;  // two sums, so the adds of successive entries overlap
+#pragma unroll 4
+        for (int j2 = half; j2 < (m + 1) / 2; j2 += H) {
+          const ulonglong2 v = sk2[j2];
+          cnt0 += int(v.x < my_sk);
+          cnt1 += int(v.y < my_sk);
+        }
+        cnt0 += cnt1;
+        if (H == 2) cnt0 += __shfl_xor_sync(0xffffffffu, cnt0, 1);
+        if (live_row) rank = cnt0;
+      }
+      double my64 = __longlong_as_double(0x7ff8000000000000ll);
+      // single-precision keys that might be out of order (intervals overlap):
+      // both ends of every such pair take a float-float key, and those pairs
+      // are ordered by it; only if two float-float intervals still meet do
+      // all such keys take their binary64 value (ties by id), as Algorithm 1
+      // reads d2 in binary64
+      // A key has a near partner iff a neighbour in single-precision order has
+      // one: sure_less is monotone, so every key between two near keys is near
+      // both.  The keys are laid out by rank (that order) and each thread looks
+      // at its two neighbours.
+      bool near = false;
+      if (!in_order) {
+        float* srt = reinterpret_cast<float*>(pb + L::p_srt);
+        if (live_row && half == 0) srt[rank] = kacc;
+        named_sync(kBarProd, kF32Prod);
+        if (live_row)
+          near = (rank > 0 && !sure_less(srt[rank - 1], kacc, E_rel, E_abs)) ||
+                 (rank + 1 < m && !sure_less(kacc, srt[rank + 1], E_rel, E_abs));
+      }
+      if (!in_order && prod_sync_or_n<kF32Prod>(near)) {
+        double* k64s = reinterpret_cast<double*>(pb + L::p_k64);  // stored order
+        const FFBound fb = ff_bound(a.d);
+        if (near) my64 = -ff_d2(reinterpret_cast<const float*>(prow), reinterpret_cast<const float*>(xrow), a.row_bytes);
+        if (half == 0) k64s[t] = my64;
+        named_sync(kBarProd, kF32Prod);
+        int cnt = 0;
+        bool open = false;
+        if (near) {
+          for (int j = 0; j < m; ++j) {
+            const float kj = __uint_as_float(unsigned(sk[j] >> 32));
+            if (sure_less(kj, kacc, E_rel, E_abs)) {
+              ++cnt;
+            } else if (j != t && !sure_less(kacc, kj, E_rel, E_abs)) {
+              const int o = slot_order(k64s[j], my64, fb);  // 1: j first
+              if (o < 0) open = true;
+              else cnt += o;
+            }
+          }
+        }
+        if (prod_sync_or_n<kF32Prod>(open)) {  // every reader of k64s has passed the barrier
+          if (near) {
+            my64 = canon_d2_f32(reinterpret_cast<const float*>(prow), reinterpret_cast<const float*>(xrow), a.d);
+            if (half == 0) atomicAdd(&a.status->fp64_sort_keys, 1ull);
+          }
+          if (half == 0) k64s[t] = my64;
+          named_sync(kBarProd, kF32Prod);
+          if (near) {
+            cnt = 0;
+            for (int j = 0; j < m; ++j) {
+              const float kj = __uint_as_float(unsigned(sk[j] >> 32));
+              if (sure_less(kj, kacc, E_rel, E_abs)) {
+                ++cnt;
+              } else if (j != t && !sure_less(kacc, kj, E_rel, E_abs)) {
+                const double dj = k64s[j];
+                const int32_t idj = int32_t(unsigned(sk[j]));
+                cnt += (dj < my64 || (dj == my64 && idj < my_id)) ? 1 : 0;
+              }
+            }
+          }
+        }
+        if (near) rank = cnt;
+      }
+      int* rank_of = reinterpret_cast<int*>(pb + L::p_rk);  // rank of each stored position
+      // a column's record: TA4 = TA rounded up to 4 lower thresholds, as many upper
+      // ones, its centred norm^2 (the pivot key) and the root of it
+      const int TA4 = (a.TA + 3) & ~3, rstride = 2 * TA4 + 4;
+      if (half == 0) rank_of[t] = live_row ? 4 * rank : -4;
+      if (live_row && half == 0) {
+        ids[rank] = my_id;
+        key[rank] = kacc;
+        norm[rank] = kacc;
+        const float root = sqrtf(kacc);
+        sn[rank] = root;
+        key64[rank] = my64;
+        *reinterpret_cast<float2*>(rec + rank * rstride + 2 * TA4) = make_float2(kacc, root);
+      }
+      // while the MMA runs: the thresholds of column `rank` for every distinct
+      // alpha (a6).  kappa = 1e6 / A^2 carries one rounding and the product two
+      // more; the last factor (1 -+ 2e-6, and an ulp or two, since lo = upper counts
+      // as above it) covers them with room to spare, and the roundings of the
+      // pair's d2 - err and d2 + err, compared against these thresholds directly.
+      if (live_row && half == H - 1) {
+        float* th = rec + rank * rstride;
+#pragma unroll
+        for (int u = 0; u < TB; ++u) {
+          if (u >= a.TA) break;
+          th[u] = (kacc * (1.0f - E_rel) - E_abs) * a.kappa[u] * 0.999998f;
+          th[TA4 + u] = (kacc * (1.0f + E_rel) + E_abs) * a.kappa[u] * 1.0000022f;
+        }
+        // padding past the last alpha never counts (hi - -inf, lo - -inf: no sign)
+        for (int u = a.TA; u < TA4; ++u) th[u] = th[TA4 + u] = -INFINITY;
+      }
+      // rank row masks start empty, one (row, target) word per step of a thread
+      for (int i = H * t + half; i < a.TA * MAXM * MW; i += H * MAXM) masks[i] = 0ull;
+      if (next_id >= 0) {
+        const char* nrow = reinterpret_cast<const char*>(a.X + int64_t(next_id) * a.row_bytes);
+        for (int64_t off = 128 * half; off < a.row_bytes; off += 128 * H)
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(nrow + off));
+      }
+      const bool ok = mbar_wait(mbar, phase, 1 << 24);
+      // one barrier: every rank-indexed array is complete, and the wait's outcome is known to all
+      if (prod_sync_or_n<kF32Prod>(!ok)) {  // the MMA never completed: report, stop after this slot (uniform)
+        if (r == 0) raise_status(a.status, kDevOverflow, -2);
+        dead = true;
+      }
+      phase ^= 1u;
+      tc_fence_after();
+      // The group's Gram, MAXM x MAXM in rank order over the operands (read by
+      // now), row R rotated by R: G~(R, c) at [R * MAXM + (c + R) % MAXM], the
+      // entries with R < c, in the operands' scaled units (G~ / inv_s2).
+      // tcgen05.ld is warp-collective: every lane issues it, live rows store.
+      // Warps w, w + 4, .. read TMEM lanes 32 (w % 4) .. + 31, a part of the columns each.
+      if (!dead) {
+        const int lrow = 32 * (warp & 3) + lane, gq = lrow / MAXM, tq = lrow % MAXM;
+        const int mq = misc[4 + s * 2 + gq];
+        const int* rank_q = reinterpret_cast<const int*>(prod_base(gq) + L::p_rk);
+        const bool live_q = tq < mq;
+        const int my_rank4 = live_q ? rank_q[tq] : 0;
+        const int cbeg = (warp >> 2) * (MAXM / H);
+        const int cend = min(cbeg + MAXM / H, (mq + 15) & ~15);  // the same for every lane of the warp (one node)
+        const uint32_t lane_base = tmem + (uint32_t(32 * (warp & 3)) << 16) + uint32_t(gq * MAXM);
+        float* grow = reinterpret_cast<float*>(opnd) + size_t(gq) * MAXM * MAXM + size_t(my_rank4 / 4) * MAXM;
+        const int4* rk4 = reinterpret_cast<const int4*>(rank_q);
+#pragma unroll 1
+        for (int c0 = cbeg; c0 < cend; c0 += 16) {
+          uint32_t v[16], v2[16];
+          tmem_ld8(lane_base + uint32_t(c0), *reinterpret_cast<uint32_t(*)[8]>(v));
+          tmem_ld8(lane_base + uint32_t(c0 + 8), *reinterpret_cast<uint32_t(*)[8]>(v + 8));
+          tmem_ld8(lane_base + uint32_t(128 + c0), *reinterpret_cast<uint32_t(*)[8]>(v2));
+          tmem_ld8(lane_base + uint32_t(128 + c0 + 8), *reinterpret_cast<uint32_t(*)[8]>(v2 + 8));
+          tmem_ld_wait();
+          if (live_q) {
+#pragma unroll
+            for (int j4 = 0; j4 < 16; j4 += 4) {
+              const int4 r4 = rk4[(c0 + j4) / 4];  // 4 x the ranks of four stored columns (past m: -4)
+              const int rc[4] = {r4.x, r4.y, r4.z, r4.w};
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                if (rc[j] > my_rank4)  // in the scaled units (inv_s2 goes into the decision)
+                  *reinterpret_cast<float*>(reinterpret_cast<char*>(grow) + ((rc[j] + my_rank4) & (4 * MAXM - 1))) =
+                      fmaf(__uint_as_float(v2[j4 + j]), 4.8828125e-04f, __uint_as_float(v[j4 + j]));
+            }
+          }
+        }
+      }
+      tc_fence_before();
+      named_sync(kBarProd, kF32Prod);  // the staged Gram; TMEM read
+      tc_fence_after();
+      if (!dead) {
+        // Rows pair up as (q, MAXM - 1 - q): row q has MAXM - 1 - q later columns
+        // and row MAXM - 1 - q has q, MAXM - 1 in all.  Item i of a pair is row q's
+        // column q + 1 + i while there are such, then row MAXM - 1 - q's; the 2 H
+        // threads of a pair take MAXM / (2 H) items each.  (Here g is the node of
+        // the thread's warps too: H MAXM threads each.)
+        constexpr int Q = MAXM / 2, CH = MAXM / (2 * H);
+        const float* Gs = reinterpret_cast<const float*>(opnd) + size_t(g) * MAXM * MAXM;
+        const int tt = r & (H * MAXM - 1);
+        const int q = tt % Q, h = tt / Q;
+        const int rA = q, rB = MAXM - 1 - q;
+        const int lenA = MAXM - 1 - q;                      // items on row rA
+        const int nItems = min(CH, MAXM - 1 - CH * h);      // this thread's
+        const int nA = max(0, min(CH, lenA - CH * h));      // of them on row rA, the rest on row rB
+        const int cA = rA + 1 + CH * h;                     // row rA's first column here
+        const int cB = rB + 1 + max(0, CH * h - lenA);      // row rB's first column here
+        // the d2 error bound as two multiply-adds: err = |c| At + |c|^2 eps_n + Bt
+        const float ntA = rA < m ? norm[rA] : 0.f, stA = rA < m ? sn[rA] : 0.f;
+        const float ntB = rB < m ? norm[rB] : 0.f, stB = rB < m ? sn[rB] : 0.f;
+        const float AtA = 2.f * eps_ip * stA * 1.0009765625f + sub_abs, BtA = sub_abs * stA + eps_n * ntA + err_abs;
+        const float AtB = 2.f * eps_ip * stB * 1.0009765625f + sub_abs, BtB = sub_abs * stB + eps_n * ntB + err_abs;
+        const int TA = a.TA;
+        const float m2inv_s2 = -2.f * a.inv_s2;
+        // Per distinct alpha u, bit k of mk[u] says that item k's column is surely
+        // removed at alpha u: hi < lower(column, u), the sign of their difference,
+        // shifted in.  Those tests are a prefix over u (the alphas ascend, the
+        // thresholds fall), so they are the row masks' bits as they stand.  "May be
+        // removed", lo < upper(column, u), is a prefix too; an item is open when some
+        // alpha may remove its column without surely doing so.  Items go in last to
+        // first, so item k ends at bit k.  Items past nItems or past the degree read
+        // other columns' records or rows within the group's arrays; their bits are
+        // masked out below.
+        constexpr int NW = CH > 32 ? CH / 32 : 1, CB = CH > 32 ? 32 : CH;  // words of items, items a word
+        unsigned mk[NW][TB], open[NW];
+        auto items = [&](auto only_a) {
+          constexpr bool kOnlyA = decltype(only_a)::value;  // every item lies on row rA
+#pragma unroll
+          for (int w = 0; w < NW; ++w) {
+#pragma unroll
+            for (int u = 0; u < TB; ++u) mk[w][u] = 0;
+            unsigned ow = 0;
+#pragma unroll 2
+            for (int k2 = CB * w + CB - 1; k2 >= CB * w; --k2) {
+              const bool onA = kOnlyA || k2 < nA;
+              const int R = onA ? rA : rB;
+              const int c = min((onA ? cA : cB - nA) + k2, MAXM - 1);
+              const float G = Gs[R * MAXM + ((c + R) & (MAXM - 1))];
+              const float* th = rec + c * rstride;
+              const float2 qc = *reinterpret_cast<const float2*>(th + 2 * TA4);
+              const float dv = fmaf(G, m2inv_s2, (onA ? ntA : ntB) + qc.x);  // G~ = G * inv_s2: exact scaling
+              const float err = fmaf(qc.y, onA ? AtA : AtB, fmaf(qc.x, eps_n, onA ? BtA : BtB));
+              const float lo = dv - err, hi = dv + err;
+              unsigned op = 0;
+#pragma unroll
+              for (int u4 = 0; u4 < L::TB4; u4 += 4) {
+                if (u4 < TA) {  // uniform
+                  const float4 l4 = *reinterpret_cast<const float4*>(th + u4);
+                  const float4 h4 = *reinterpret_cast<const float4*>(th + TA4 + u4);
+                  const float lw[4] = {l4.x, l4.y, l4.z, l4.w}, hw[4] = {h4.x, h4.y, h4.z, h4.w};
+#pragma unroll
+                  for (int e = 0; e < 4; ++e) {
+                    if (u4 + e >= TB) break;
+                    const unsigned sure = __float_as_uint(hi - lw[e]), may = __float_as_uint(lo - hw[e]);
+                    mk[w][u4 + e] = __funnelshift_l(sure, mk[w][u4 + e], 1);
+                    op |= may & ~sure;
+                  }
+                }
+              }
+              ow = __funnelshift_l(op, ow, 1);
+            }
+            open[w] = ow;
+          }
+        };
+        if (CH * h + CH <= MAXM / 2) items(std::true_type{});  // the same for every lane: lenA >= MAXM / 2
+        else items(std::false_type{});
+        // items that exist: [0, nA) with cA + k < m, then [nA, nItems) with cB + k - nA < m
+        auto low_bits = [](int n) -> unsigned long long { return n <= 0 ? 0ull : n >= 64 ? ~0ull : (1ull << n) - 1; };
+        const unsigned long long there = low_bits(min(nA, m - cA)) | (low_bits(min(nItems - nA, m - cB)) << (nA & 63));
+        // open pairs (rare): the alphas from ts (the surely-removing count) on are
+        // decided exactly by the consumer warp before its scan; here if the slot's
+        // queue is full
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+          unsigned ob = open[w] & unsigned(there >> (32 * w));
+          while (ob) {
+            const int kb = __ffs(int(ob)) - 1, k2 = CB * w + kb;
+            ob &= ob - 1;
+            const bool onA = k2 < nA;
+            const int R = onA ? rA : rB;
+            const int c = onA ? cA + k2 : cB + (k2 - nA);
+            int ts = 0;
+#pragma unroll
+            for (int u = 0; u < TB; ++u) ts += u < TA ? int((mk[w][u] >> kb) & 1u) : 0;
+            const int qi = atomicAdd(rq_count + s, 1);
+            if (qi < L::rq_cap) {
+              rq[s * L::rq_cap + qi] = (unsigned(g * MAXM + R) << 16) | (unsigned(c) << 5) | unsigned(ts);
+            } else {
+              // removal is monotone in alpha: the alphas before the first that keeps the pair remove it
+              const int u1 = recheck_prefix_cold(a, ids, key, key64, R, c, ts, TA, ppt, E_rel, E_abs);
+              n_rechecks += recheck_tests(ts, u1, TA);
+#pragma unroll
+              for (int u = 0; u < TB; ++u)
+                if (u >= ts && u < u1) mk[w][u] |= 1u << kb;
+            }
+          }
+        }
+        // item masks -> row masks: row rA's items are [0, nA) from column cA,
+        // row rB's [nA, nItems) from column cB
+        auto or_run = [&](unsigned long long* row, unsigned long long bits, int col) {
+          const int w0 = col >> 6, sh = col & 63;
+          if (bits << sh) atomicOr(row + w0, bits << sh);
+          if (MW > 1 && sh && w0 + 1 < MW && (bits >> (64 - sh))) atomicOr(row + w0 + 1, bits >> (64 - sh));
+        };
+#pragma unroll
+        for (int u = 0; u < TB; ++u) {
+          if (u >= TA) break;
+          unsigned long long gt = mk[0][u];
+          if (NW > 1) gt |= static_cast<unsigned long long>(mk[NW - 1][u]) << 32;
+          gt &= there;
+          const unsigned long long mA = gt & low_bits(nA), mB = nA >= 64 ? 0ull : gt >> nA;
+          if (mA) or_run(masks + (u * MAXM + rA) * MW, mA, cA);
+          if (mB) or_run(masks + (u * MAXM + rB) * MW, mB, cB);
+        }
+      }
+      if (dead && r < NG) misc[s * 2 + r] = -1;  // nothing valid in this slot
+      bar_arrive(kBarFull + s, kF32Threads);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) n_rechecks += __shfl_xor_sync(0xffffffffu, n_rechecks, o);
+    if (lane == 0 && n_rechecks) atomicAdd(&a.status->spare[2], n_rechecks);
+  } else {
+    // =========================== consumer warp ===========================
+    bar_arrive(kBarFree + 0, kF32Threads);  // both slots start free
+    bar_arrive(kBarFree + 1, kF32Threads);
+    long long done = 0;
+    unsigned long long n_rechecks = 0;  // single-precision rechecks of the queued pairs
+    for (int k = 0;; ++k) {
+      const int s = k & 1;
+      named_sync(kBarFull + s, kF32Threads);
+      bool any = false;
+#pragma unroll
+      for (int q = 0; q < NG; ++q) {
+        any |= misc[s * 2 + q] >= 0;
+        done += misc[s * 2 + q] >= 0;
+      }
+      if (!any) break;
+      {
+        // The slot's open pairs, four at a time: the warp reads the rows together
+        // (a lane per 16-byte chunk; few enough roundings for slice_rel_bound), and
+        // each alpha that removes the column sets its bit in the row's mask.  One
+        // pair per lane, its two rows read chunk by chunk, took longer than all the
+        // rest of a slot on long rows.
+        const int nq = min(rq_count[s], L::rq_cap), nch = int(a.row_bytes / 16);
+        for (int i0 = 0; i0 < nq; i0 += 4) {
+          const uint4 *pu[4], *pv[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint32_t e = rq[s * L::rq_cap + min(i0 + j, nq - 1)];
+            const int tr = int(e >> 16), c = int((e >> 5) & 0x7ffu);
+            const int32_t* idq = reinterpret_cast<const int32_t*>(slot_base(s, tr / MAXM) + L::s_ids);
+            pu[j] = reinterpret_cast<const uint4*>(a.X + int64_t(idq[tr % MAXM]) * a.row_bytes);
+            pv[j] = reinterpret_cast<const uint4*>(a.X + int64_t(idq[c]) * a.row_bytes);
+          }
+          float d2a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+          for (int c = lane; c < nch; c += 32) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) d2a[j] = Acc<kF32>::step4(__ldg(pu[j] + c), __ldg(pv[j] + c), d2a[j]);
+          }
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) d2a[j] += __shfl_xor_sync(0xffffffffu, d2a[j], o);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (i0 + j >= nq) break;
+            const uint32_t e = rq[s * L::rq_cap + i0 + j];
+            const int tr = int(e >> 16), c = int((e >> 5) & 0x7ffu), u0 = int(e & 31u);
+            const int gq = tr / MAXM, tq = tr % MAXM;
+            unsigned char* sbq = slot_base(s, gq);
+            const int32_t* idq = reinterpret_cast<const int32_t*>(sbq + L::s_ids);
+            const float kc = reinterpret_cast<const float*>(sbq + L::s_key)[c];
+            double* k64 = reinterpret_cast<double*>(sbq + L::s_key64) + c;
+            int u1 = u0;  // removal is monotone in alpha (recheck_prefix)
+            for (; u1 < a.TA; ++u1) {
+              const int64_t A2 = int64_t(a.Ad[u1]) * a.Ad[u1];
+              const int rr = sure_dominates(float(A2), d2a[j], kc, E_rel, E_abs);
+              if (!(rr >= 0 ? (rr == 1)
+                            : fine_dominates_warp(a, idq[tq], idq[c], point_of_row(a, misc[s * 2 + gq]), k64, double(A2))))
+                break;
+            }
+            if (lane == 0) n_rechecks += recheck_tests(u0, u1, a.TA);
+            unsigned long long* mrow = reinterpret_cast<unsigned long long*>(sbq + L::s_masks) + tq * MW + (c >> 6);
+            if (lane >= u0 && lane < u1) atomicOr(mrow + lane * MAXM * MW, 1ull << (c & 63));
+          }
+        }
+        __syncwarp();
+      }
+      // ---- a7 greedy scan: lane (g * 16 + u) runs Algorithm 1's loop for node
+      // g and target u.  Candidates are laid out by rank, so the next argmin of
+      // the live set is its lowest set bit.
+      {
+        const int g = NG == 2 ? lane >> 4 : 0;
+        const int u = NG == 2 ? (lane & 15) : lane;
+        const int p = misc[s * 2 + g];
+        if (p >= 0 && u < T) {
+          const int m = misc[4 + s * 2 + g];
+          const int64_t e0 = misc64[s * 2 + g];
+          unsigned char* sb = slot_base(s, g);
+          const unsigned long long* masks = reinterpret_cast<const unsigned long long*>(sb + L::s_masks);
+          const int32_t* ids = reinterpret_cast<const int32_t*>(sb + L::s_ids);
+          unsigned long long al[MW];
+#pragma unroll
+          for (int w = 0; w < MW; ++w) {
+            const int lo = 64 * w;
+            al[w] = m > lo ? ((m - lo >= 64) ? ~0ull : ((1ull << (m - lo)) - 1)) : 0ull;
+          }
+          const int R = a.R[u];
+          const int mu = a.amap[u];  // the target's domination mask
+          int32_t* out = a.out_col[u] + e0;
+          const int kept = greedy_scan<MW>(al, masks + mu * MAXM * MW, ids, out, R);
+          a.out_cnt[u][p] = kept;
+        }
+      }
+      __syncwarp();
+      bar_arrive(kBarFree + s, kF32Threads);
+    }
+    if (lane == 0 && done) atomicAdd(&a.status->nodes_pruned, static_cast<unsigned long long>(done) * T);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) n_rechecks += __shfl_xor_sync(0xffffffffu, n_rechecks, o);
+    if (lane == 0 && n_rechecks) atomicAdd(&a.status->spare[2], n_rechecks);
+  }
+  // the TMEM columns go back once the producers are finished with them
+  if (warp < kF32Prod / 32) {
+    tc_fence_before();
+    named_sync(kBarProd, kF32Prod);
     tc_fence_after();
     if (warp == 0) tmem_dealloc(*tmem_slot, kTmemCols);
   }
@@ -1719,6 +2063,8 @@ cudaError_t launch_bucket_nodes(const int64_t* row_ptr, int64_t n, int32_t* list
   return cudaGetLastError();
 }
 
+constexpr int64_t kF32WideBytes = 512;
+
 // CTAs of `kern` that fit on one SM, from its registers and dynamic shared
 // memory (computed directly: the occupancy query under-reports it for these
 // kernels when called while a stream is being captured).
@@ -1741,11 +2087,13 @@ static cudaError_t resident_ctas(K kern, int threads, size_t dyn_smem, int cap, 
   return cudaSuccess;
 }
 
-template <int DT, int MAXM, int TB>
+template <int DT, int MAXM, int TB, int H>
 static cudaError_t run_fast_t(const PruneArgs& args, int num_sms, int64_t host_count, int ctas_cap, cudaStream_t s) {
   const size_t bytes = TcLayout<MAXM, TB, DT == kF32 ? 2 : 1>::bytes;
-  auto kern = prune_tc_kernel<DT, MAXM, TB>;
-  constexpr int kThreadsTc = 160;  // 4 producer warps + 1 consumer warp
+  void (*kern)(PruneArgs);
+  if constexpr (DT == kU8) kern = prune_u8_kernel<MAXM, TB>;
+  else kern = prune_f32_kernel<MAXM, TB, H>;
+  constexpr int kThreadsTc = 128 * H + 32;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
   if (err != cudaSuccess) return err;
   // ask for the largest shared-memory carveout so the launch sees the whole 228 KB per SM
@@ -1762,6 +2110,14 @@ static cudaError_t run_fast_t(const PruneArgs& args, int num_sms, int64_t host_c
   return cudaGetLastError();
 }
 
+// Float rows of more than one 128-dimension slice: eight producer warps.
+template <int DT, int MAXM, int TB>
+static cudaError_t run_fast_h(const PruneArgs& args, int num_sms, int64_t host_count, int ctas_cap, cudaStream_t s) {
+  if (DT == kF32 && args.row_bytes > kF32WideBytes)
+    return run_fast_t<DT, MAXM, TB, DT == kF32 ? 2 : 1>(args, num_sms, host_count, ctas_cap, s);
+  return run_fast_t<DT, MAXM, TB, 1>(args, num_sms, host_count, ctas_cap, s);
+}
+
 // Picks the kernel instance whose per-node target slots cover T.
 template <int DT, int MAXM>
 static cudaError_t run_fast(const PruneArgs& args, int num_sms, int64_t host_count, int ctas_cap, cudaStream_t s) {
@@ -1770,11 +2126,11 @@ static cudaError_t run_fast(const PruneArgs& args, int num_sms, int64_t host_cou
   // target for uint8 rows, per distinct alpha for float rows (targets sharing
   // alpha share them; the consumer's lanes cover every target either way)
   const int nb = DT == kF32 ? args.TA : args.T;
-  if (nb <= 1) return run_fast_t<DT, MAXM, 1>(args, num_sms, host_count, ctas_cap, s);
-  if (nb <= 2) return run_fast_t<DT, MAXM, 2>(args, num_sms, host_count, ctas_cap, s);
-  if (nb <= 4) return run_fast_t<DT, MAXM, 4>(args, num_sms, host_count, ctas_cap, s);
-  if (nb <= 8) return run_fast_t<DT, MAXM, 8>(args, num_sms, host_count, ctas_cap, s);
-  return run_fast_t<DT, MAXM, kMaxTargets>(args, num_sms, host_count, ctas_cap, s);
+  if (nb <= 1) return run_fast_h<DT, MAXM, 1>(args, num_sms, host_count, ctas_cap, s);
+  if (nb <= 2) return run_fast_h<DT, MAXM, 2>(args, num_sms, host_count, ctas_cap, s);
+  if (nb <= 4) return run_fast_h<DT, MAXM, 4>(args, num_sms, host_count, ctas_cap, s);
+  if (nb <= 8) return run_fast_h<DT, MAXM, 8>(args, num_sms, host_count, ctas_cap, s);
+  return run_fast_h<DT, MAXM, kMaxTargets>(args, num_sms, host_count, ctas_cap, s);
 }
 
 template <int DT>

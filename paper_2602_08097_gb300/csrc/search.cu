@@ -604,35 +604,6 @@ __device__ inline RegSmem reg_carve(unsigned char* p, int64_t row_bytes, int cac
   return w;
 }
 
-// ff_d2 by one warp: lane l takes chunks l, l + 32, ...; the lanes' pairs are
-// joined by a butterfly of two-sums, each level's low sum off by at most
-// 3 2^-48 of the total.  A lane's 4 ceil(nch / 32) steps and the levels that
-// join nonzero pairs stay within the (3 d + 13) 2^-48 of one chain (ff_bound).
-// The same value in every lane.
-__device__ __forceinline__ double ff_d2_warp(const float* q, const float* __restrict__ x, int nch) {
-  const float4* pq = reinterpret_cast<const float4*>(q);
-  const float4* px = reinterpret_cast<const float4*>(x);
-  float sh = 0.f, sl = 0.f;
-  for (int c = threadIdx.x & 31; c < nch; c += 32) {
-    const float4 a = pq[c], b = __ldg(px + c);
-    ff_step(a.x, b.x, sh, sl);
-    ff_step(a.y, b.y, sh, sl);
-    ff_step(a.z, b.z, sh, sl);
-    ff_step(a.w, b.w, sh, sl);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float oh = __shfl_xor_sync(0xffffffffu, sh, o), ol = __shfl_xor_sync(0xffffffffu, sl, o);
-    const float s1 = __fadd_rn(sh, oh);  // two-sum of the high parts
-    const float bv = __fsub_rn(s1, sh);
-    const float e = __fadd_rn(__fsub_rn(sh, __fsub_rn(s1, bv)), __fsub_rn(oh, bv));
-    const float l1 = __fadd_rn(__fadd_rn(sl, ol), e);
-    sh = __fadd_rn(s1, l1);
-    sl = __fsub_rn(l1, __fsub_rn(sh, s1));
-  }
-  return __dadd_rn(double(sh), double(sl));
-}
-
 // Whether point `m` precedes point `c` in (distance, id) order, where their
 // single-precision intervals overlap: float-float distances, then binary64.
 // Called by a whole warp; out of line, since it is rare.
