@@ -51,6 +51,8 @@ struct PruneLaunch {
 cudaError_t launch_bucket_nodes(const int64_t* row_ptr, int64_t n, int32_t* lists /* 3*n */,
                                 int32_t* counts /* 3 */, cudaStream_t s);
 cudaError_t launch_prune(const PruneLaunch& L, cudaStream_t s);
+// the CTAs per SM that L's tile0 and ctas_per_sm come to for the degree <= 64 bucket
+cudaError_t prune_ctas_per_sm(const PruneLaunch& L, int* ctas);
 // counts -> row_ptr (per target) and compaction of kept ids into col.
 cudaError_t launch_emit_csr(int64_t n, int T, const int64_t* src_row_ptr,
                             int32_t* const* scratch_col, int32_t* const* cnt,

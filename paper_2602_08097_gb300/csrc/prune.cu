@@ -2088,7 +2088,8 @@ static cudaError_t resident_ctas(K kern, int threads, size_t dyn_smem, int cap, 
 }
 
 template <int DT, int MAXM, int TB, int H>
-static cudaError_t run_fast_t(const PruneArgs& args, int num_sms, int64_t host_count, int ctas_cap, cudaStream_t s) {
+static cudaError_t run_fast_t(const PruneArgs& args, int num_sms, int64_t host_count, int ctas_cap, cudaStream_t s,
+                              int* fit) {
   const size_t bytes = TcLayout<MAXM, TB, DT == kF32 ? 2 : 1>::bytes;
   void (*kern)(PruneArgs);
   if constexpr (DT == kU8) kern = prune_u8_kernel<MAXM, TB>;
@@ -2104,6 +2105,10 @@ static cudaError_t run_fast_t(const PruneArgs& args, int num_sms, int64_t host_c
   err = resident_ctas(kern, kThreadsTc, bytes, DT == kF32 ? 2 : 4, &per_sm);
   if (err != cudaSuccess) return err;
   if (ctas_cap > 0) per_sm = std::min(per_sm, ctas_cap);
+  if (fit) {  // asked for the CTAs per SM, not for a launch
+    *fit = per_sm;
+    return cudaSuccess;
+  }
   const int64_t groups_needed = (host_count + (128 / MAXM) - 1) / (128 / MAXM);
   const int64_t grid = std::min<int64_t>(int64_t(num_sms) * per_sm, groups_needed);
   kern<<<unsigned(grid), kThreadsTc, bytes, s>>>(args);
@@ -2112,25 +2117,27 @@ static cudaError_t run_fast_t(const PruneArgs& args, int num_sms, int64_t host_c
 
 // Float rows of more than one 128-dimension slice: eight producer warps.
 template <int DT, int MAXM, int TB>
-static cudaError_t run_fast_h(const PruneArgs& args, int num_sms, int64_t host_count, int ctas_cap, cudaStream_t s) {
+static cudaError_t run_fast_h(const PruneArgs& args, int num_sms, int64_t host_count, int ctas_cap, cudaStream_t s,
+                              int* fit) {
   if (DT == kF32 && args.row_bytes > kF32WideBytes)
-    return run_fast_t<DT, MAXM, TB, DT == kF32 ? 2 : 1>(args, num_sms, host_count, ctas_cap, s);
-  return run_fast_t<DT, MAXM, TB, 1>(args, num_sms, host_count, ctas_cap, s);
+    return run_fast_t<DT, MAXM, TB, DT == kF32 ? 2 : 1>(args, num_sms, host_count, ctas_cap, s, fit);
+  return run_fast_t<DT, MAXM, TB, 1>(args, num_sms, host_count, ctas_cap, s, fit);
 }
 
 // Picks the kernel instance whose per-node target slots cover T.
 template <int DT, int MAXM>
-static cudaError_t run_fast(const PruneArgs& args, int num_sms, int64_t host_count, int ctas_cap, cudaStream_t s) {
+static cudaError_t run_fast(const PruneArgs& args, int num_sms, int64_t host_count, int ctas_cap, cudaStream_t s,
+                            int* fit = nullptr) {
   if (host_count <= 0) return cudaSuccess;
   // TB bounds what the kernel keeps per target: one mask and threshold set per
   // target for uint8 rows, per distinct alpha for float rows (targets sharing
   // alpha share them; the consumer's lanes cover every target either way)
   const int nb = DT == kF32 ? args.TA : args.T;
-  if (nb <= 1) return run_fast_h<DT, MAXM, 1>(args, num_sms, host_count, ctas_cap, s);
-  if (nb <= 2) return run_fast_h<DT, MAXM, 2>(args, num_sms, host_count, ctas_cap, s);
-  if (nb <= 4) return run_fast_h<DT, MAXM, 4>(args, num_sms, host_count, ctas_cap, s);
-  if (nb <= 8) return run_fast_h<DT, MAXM, 8>(args, num_sms, host_count, ctas_cap, s);
-  return run_fast_h<DT, MAXM, kMaxTargets>(args, num_sms, host_count, ctas_cap, s);
+  if (nb <= 1) return run_fast_h<DT, MAXM, 1>(args, num_sms, host_count, ctas_cap, s, fit);
+  if (nb <= 2) return run_fast_h<DT, MAXM, 2>(args, num_sms, host_count, ctas_cap, s, fit);
+  if (nb <= 4) return run_fast_h<DT, MAXM, 4>(args, num_sms, host_count, ctas_cap, s, fit);
+  if (nb <= 8) return run_fast_h<DT, MAXM, 8>(args, num_sms, host_count, ctas_cap, s, fit);
+  return run_fast_h<DT, MAXM, kMaxTargets>(args, num_sms, host_count, ctas_cap, s, fit);
 }
 
 template <int DT>
@@ -2255,7 +2262,8 @@ cudaError_t launch_gram_probe(const DevData& D, const int32_t* rows, const int32
   return cudaGetLastError();
 }
 
-cudaError_t launch_prune(const PruneLaunch& L, cudaStream_t s) {
+// The arguments that every bucket of a launch shares.
+static PruneArgs prune_args(const PruneLaunch& L) {
   PruneArgs a{};
   a.X = L.data.X;
   a.row_bytes = L.data.row_bytes;
@@ -2295,6 +2303,20 @@ cudaError_t launch_prune(const PruneLaunch& L, cudaStream_t s) {
     }
     a.amap[t] = a.TA - 1;
   }
+  return a;
+}
+
+cudaError_t prune_ctas_per_sm(const PruneLaunch& L, int* ctas) {
+  const PruneArgs a = prune_args(L);
+  if (L.data.dtype == kU8)
+    return L.tile0 == 0 ? run_fast<kU8, 64>(a, L.num_sms, 1, L.ctas_per_sm, nullptr, ctas)
+                        : run_fast<kU8, 128>(a, L.num_sms, 1, L.ctas_per_sm, nullptr, ctas);
+  return L.tile0 == 0 ? run_fast<kF32, 64>(a, L.num_sms, 1, L.ctas_per_sm, nullptr, ctas)
+                      : run_fast<kF32, 128>(a, L.num_sms, 1, L.ctas_per_sm, nullptr, ctas);
+}
+
+cudaError_t launch_prune(const PruneLaunch& L, cudaStream_t s) {
+  PruneArgs a = prune_args(L);
   cudaError_t err = cudaSuccess;
   for (int b = 0; b < 3 && err == cudaSuccess; ++b) {
     a.nodes = L.bucket_nodes[b];

@@ -429,11 +429,20 @@ rp_status choose_config(rp_ctx* c, Graph* S, int T, const int32_t* A, const int3
     }
     const int cand[6][2] = {{0, 0}, {0, 3}, {0, 2}, {1, 0}, {1, 3}, {1, 2}};
     float best_ms = 0.f;
+    std::vector<std::pair<int, int>> tried;  // (tile, CTAs per SM)
     for (int i = 0; i < 6; ++i) {
       L.tile0 = cand[i][0];
       L.ctas_per_sm = cand[i][1];
+      // pairs that come to the same launch are timed once (float rows: two CTAs
+      // per SM whatever is asked for)
+      int fit = 0;
+      CUDA_TRY(c, prune_ctas_per_sm(L, &fit));
+      if (std::find(tried.begin(), tried.end(), std::make_pair(L.tile0, fit)) != tried.end()) continue;
+      bool loaded = false;
+      for (const auto& tr : tried) loaded |= tr.first == L.tile0;
+      tried.emplace_back(L.tile0, fit);
       float ms = 0.f;
-      for (int rep = 0; rep < 2; ++rep) {  // the first run loads the kernel
+      for (int rep = loaded ? 1 : 0; rep < 2; ++rep) {  // a tile's first run loads its kernel
         CUDA_TRY(c, cudaMemsetAsync(c->work, 0, 8 * sizeof(unsigned), c->stream));
         CUDA_TRY(c, cudaEventRecord(c->ev[0], c->stream));
         CUDA_TRY(c, launch_prune(L, c->stream));
