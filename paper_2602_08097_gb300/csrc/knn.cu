@@ -327,12 +327,14 @@ __global__ void __launch_bounds__(kThreads) knn_kernel(KnnArgs a) {
 // float: sums per 32-dim slice with near-tie runs re-ordered in binary64), as
 // the CUDA-core kernel ranks its lists.
 //
-// What bounds the scan: per step, the three split products (1,150 cycles of
-// MMA at d = 96) and the threads' 128 columns at four to five instructions
-// each.  10,000 queries x 400,000 points x 96 dims, k 100: 5.0 ms for the scan and
-// 0.34 for the ranking, 5.5 in all; one CTA per query tile, a lane per query row
-// and the tile's loads, products and cuts in turn took 47.6 (79 CTAs of 152, the
-// tensor cores idle through every cut).
+// What bounds the scan: the threads' 64 columns a step, read, tested and now and
+// then stored, about 2,400 of a step's 4,000 cycles (its products: 1,150 at d = 96),
+// and the cuts, which hold the other warps up through the accumulators.  10,000
+// queries x 400,000 points x 96 dims, k 100: 3.7 ms, of which the ranking 0.34; one
+// CTA per query tile, a lane per query row and the tile's loads, products and cuts
+// in turn took 47.6 (79 CTAs of 152, the tensor cores idle through every cut).  With
+// the exact k-th in a cut, its entries read twice, and a vote per eight columns it
+// took 5.4.  All 64 columns read at once, for one wait less, changed nothing.
 constexpr int kTcQ = 128;     // queries per tile (rows of the MMA)
 constexpr int kTcP = 128;     // points per tile (columns of the MMA)
 constexpr int kTcCand = 512;  // candidates a part keeps per query
@@ -405,11 +407,11 @@ __device__ __forceinline__ int entry_at(int i, int a, int gap) { return i < a ? 
 // The k-th smallest distance of the m >= k entries as a key, by bisection on its
 // bits; the entries are read once, PER of them per lane.  One warp.
 template <int PER>
-__device__ __forceinline__ unsigned kth_of(const uint2* e, int m, int k, int a = kTcCand, int gap = 0) {
+__device__ __forceinline__ unsigned kth_of(const uint2* e, int m, int k) {
   const int lane = threadIdx.x & 31;
   unsigned u[PER];
 #pragma unroll
-  for (int i = 0; i < PER; ++i) u[i] = 32 * i + lane < m ? fkey(__uint_as_float(e[entry_at(32 * i + lane, a, gap)].x)) : 0xffffffffu;
+  for (int i = 0; i < PER; ++i) u[i] = 32 * i + lane < m ? fkey(__uint_as_float(e[32 * i + lane].x)) : 0xffffffffu;
   unsigned lo = 0xffffffffu, hi = 0;
 #pragma unroll
   for (int i = 0; i < PER; ++i) {
@@ -435,19 +437,67 @@ __device__ __forceinline__ float cut_width(float e, float norms) { return e * 1.
 
 // Drops the entries whose lower bound (d2~ - w) lies above tau and moves the rest
 // to the start; returns how many are left.  One warp.
-__device__ __forceinline__ int cut_above(uint2* e, int m, float tau, float w, int a = kTcCand, int gap = 0) {
+__device__ __forceinline__ int cut_above(uint2* e, int m, float tau, float w) {
   const int lane = threadIdx.x & 31;
   int kept = 0;
   for (int i0 = 0; i0 < m; i0 += 32) {
     const int i = i0 + lane;
     uint2 v = make_uint2(0, 0);
-    if (i < m) v = e[entry_at(i, a, gap)];  // never before the place it may be moved to
+    if (i < m) v = e[i];  // never before the place it may be moved to
     const bool keep = i < m && __uint_as_float(v.x) - w <= tau;
     const unsigned km = __ballot_sync(0xffffffffu, keep);
     __syncwarp();
     if (keep) e[kept + __popc(km & ((1u << lane) - 1))] = v;
     kept += __popc(km);
     __syncwarp();
+  }
+  return kept;
+}
+
+// A part's m >= k candidates (`a` of them at the buffer's start, the rest up to its
+// end), PER per lane, read once: tau = an upper bound of the k-th smallest d2~, plus
+// w; the entries whose lower bound lies above it are dropped and the rest moved to
+// the start.  Returns how many are left.  The bisection stops at a value that k to
+// k + kCutSlack entries do not exceed, after 5 or 6 of its 25 steps; the few more
+// that stay cost less.  One warp.
+constexpr int kCutSlack = 8;
+template <int PER>
+__device__ __forceinline__ int cut_part(uint2* e, int m, int k, float w, int a, float& tau) {
+  const int lane = threadIdx.x & 31;
+  const int gap = kTcCand - m;
+  uint2 v[PER];
+#pragma unroll
+  for (int i = 0; i < PER; ++i)
+    v[i] = 32 * i + lane < m ? e[entry_at(32 * i + lane, a, gap)] : make_uint2(0x7fffffffu, 0);
+  unsigned lo = 0xffffffffu, hi = 0;
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    v[i].x = fkey(__uint_as_float(v[i].x));  // past m: above every distance
+    lo = min(lo, v[i].x);
+    if (32 * i + lane < m) hi = max(hi, v[i].x);
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  while (lo < hi) {  // the k-th smallest lies in [lo, hi]
+    const unsigned mid = lo + (hi - lo) / 2;
+    int c = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) c += v[i].x <= mid;
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (c >= k) hi = mid;
+    else lo = mid + 1;
+    if (c >= k && c <= k + kCutSlack) break;
+  }
+  tau = fkey_inv(hi) + w;
+  int kept = 0;
+  __syncwarp();  // every entry has been read
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    const float x = fkey_inv(v[i].x);
+    const bool keep = 32 * i + lane < m && x - w <= tau;
+    const unsigned km = __ballot_sync(0xffffffffu, keep);
+    if (keep) e[kept + __popc(km & ((1u << lane) - 1))] = make_uint2(__float_as_uint(x), v[i].y);
+    kept += __popc(km);
   }
   return kept;
 }
@@ -663,25 +713,34 @@ __global__ void __launch_bounds__(kTcThreads) knn_scan_kernel(KnnTcArgs a) {
           for (int jj = 0; jj < 32; ++jj)
             v[jj] = __float_as_uint(fmaf(__uint_as_float(v2[jj]), 4.8828125e-04f, __uint_as_float(v[jj])));
         }
+        unsigned m = 0;  // bit e: column c0 + e
 #pragma unroll
         for (int g = 0; g < 32; g += 8) {
           const float4 pa = *reinterpret_cast<const float4*>(pnb + c0 + g);
           const float4 pb = *reinterpret_cast<const float4*>(pnb + c0 + g + 4);
           const float pn[8] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w};
-          unsigned m = 0;
+          unsigned mg = 0;
 #pragma unroll
           for (int e = 7; e >= 0; --e)
-            m = __funnelshift_l(__float_as_uint(fmaf(-2.f, __uint_as_float(v[g + e]), base + pn[e])), m, 1);
-          if (!qlive) m = 0;
-          if (tail) {  // the last tile: columns past n
-            const int64_t left = a.n - (p0 + c0 + g);
-            m &= left >= 8 ? 0xffu : left > 0 ? (1u << int(left)) - 1u : 0u;
-          }
-          if (!__any_sync(0xffffffffu, m != 0)) continue;
+            mg = __funnelshift_l(__float_as_uint(fmaf(-2.f, __uint_as_float(v[g + e]), base + pn[e])), mg, 1);
+          m |= mg << g;
+        }
+        if (!qlive) m = 0;
+        if (tail) {  // the last tile: columns past n
+          const int64_t left = a.n - (p0 + c0);
+          m &= left >= 32 ? 0xffffffffu : left > 0 ? (1u << int(left)) - 1u : 0u;
+        }
+        const unsigned any = __reduce_or_sync(0xffffffffu, m);
+        if (any == 0) continue;
+#pragma unroll
+        for (int g = 0; g < 32; g += 4) {
+          if (((any >> g) & 0xfu) == 0) continue;
+          const float4 pa = *reinterpret_cast<const float4*>(pnb + c0 + g);
+          const float pn[4] = {pa.x, pa.y, pa.z, pa.w};
           const unsigned id0 = unsigned(p0) + unsigned(c0 + g);
 #pragma unroll
-          for (int e = 0; e < 8; ++e)  // at most kTcP more a tile: the buffer has room
-            push_if((m >> e) & 1u, cnext, dir, __float_as_uint(fmaf(-2.f, __uint_as_float(v[g + e]), nqq + pn[e])),
+          for (int e = 0; e < 4; ++e)  // at most kTcP more a tile: the buffer has room
+            push_if((m >> (g + e)) & 1u, cnext, dir, __float_as_uint(fmaf(-2.f, __uint_as_float(v[g + e]), nqq + pn[e])),
                     id0 + unsigned(e));
         }
       }
@@ -704,8 +763,9 @@ __global__ void __launch_bounds__(kTcThreads) knn_scan_kernel(KnnTcArgs a) {
           const int nA = half ? oth : own, cL = own + oth, ql = quad * 32 + L;
           uint2* bL = a.cand + (int64_t(blockIdx.x + q) * kTcQ + ql) * kTcCand;
           // cL > kTcCut >= kscan
-          const float tnew = fkey_inv(kth_of<kTcCand / 32>(bL, cL, a.kscan, nA, kTcCand - cL)) + wL;
-          const int w = cut_above(bL, cL, tnew, wL, nA, kTcCand - cL);
+          float tnew;
+          const int w = cL <= 256 ? cut_part<8>(bL, cL, a.kscan, wL, nA, tnew)
+                                  : cut_part<kTcCand / 32>(bL, cL, a.kscan, wL, nA, tnew);
           if (lane == 0) {
             sCnt[ql] = w;
             sTau[ql] = tnew;
@@ -766,9 +826,9 @@ __global__ void __launch_bounds__(128) knn_rank_kernel(KnnTcArgs a) {
   bool over = false;
   auto lower = [&]() {  // tau from what is held
     if (m < a.k) return;
-    const float tnew = fkey_inv(kth_of<kRankCand / 32>(e, m, a.k, kRankCand)) + w;
+    const float tnew = fkey_inv(kth_of<kRankCand / 32>(e, m, a.k)) + w;
     tau = fminf(tau, tnew);
-    m = cut_above(e, m, tau, w, kRankCand);
+    m = cut_above(e, m, tau, w);
   };
   const int64_t c1 = ((qt + 1) * npt - 1) / a.per;
   for (int64_t c = qt * npt / a.per; c <= c1; ++c) {
