@@ -149,16 +149,19 @@ __device__ __forceinline__ double ff_d2(const float* q, const float* __restrict_
   return __dadd_rn(double(sh), double(sl));
 }
 
-// ff_d2 by one warp: lane l takes chunks l, l + 32, ...; the lanes' pairs are
-// joined by a butterfly of two-sums, each level's low sum off by at most
-// 3 2^-48 of the total.  A lane's 4 ceil(nch / 32) steps and the levels that
-// join nonzero pairs stay within the (3 d + 13) 2^-48 of one chain (ff_bound).
-// The same value in every lane.
+// ff_d2 by W neighbouring lanes of a converged warp (32: the whole warp; 8: four
+// rows at a time): lane l takes chunks l, l + W, ...; the lanes' pairs are joined
+// by a butterfly of two-sums, each level's low sum off by at most 3 2^-48 of the
+// total.  A lane's 4 ceil(nch / W) steps and the levels that join nonzero pairs
+// stay within the (3 d + 13) 2^-48 of one chain (ff_bound).  The same value in
+// each of the W lanes.
+template <int W = 32>
 __device__ __forceinline__ double ff_d2_warp(const float* q, const float* __restrict__ x, int nch) {
   const float4* pq = reinterpret_cast<const float4*>(q);
   const float4* px = reinterpret_cast<const float4*>(x);
   float sh = 0.f, sl = 0.f;
-  for (int c = threadIdx.x & 31; c < nch; c += 32) {
+#pragma unroll 4
+  for (int c = threadIdx.x & (W - 1); c < nch; c += W) {
     const float4 a = pq[c], b = __ldg(px + c);
     ff_step(a.x, b.x, sh, sl);
     ff_step(a.y, b.y, sh, sl);
@@ -166,7 +169,7 @@ __device__ __forceinline__ double ff_d2_warp(const float* q, const float* __rest
     ff_step(a.w, b.w, sh, sl);
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
+  for (int o = W / 2; o > 0; o >>= 1) {
     const float oh = __shfl_xor_sync(0xffffffffu, sh, o), ol = __shfl_xor_sync(0xffffffffu, sl, o);
     const float s1 = __fadd_rn(sh, oh);  // two-sum of the high parts
     const float bv = __fsub_rn(s1, sh);

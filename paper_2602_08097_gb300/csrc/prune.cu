@@ -1202,9 +1202,25 @@ __global__ void __launch_bounds__(128 * H + 32, 2) prune_f32_kernel(PruneArgs a)
       if (!in_order && prod_sync_or_n<kF32Prod>(near)) {
         double* k64s = reinterpret_cast<double*>(pb + L::p_k64);  // stored order
         const FFBound fb = ff_bound(a.d);
-        if (near) my64 = -ff_d2(reinterpret_cast<const float*>(prow), reinterpret_cast<const float*>(xrow), a.row_bytes);
         if (half == 0) k64s[t] = my64;
+        __syncwarp();
+        // the warp's near rows (all of one node), eight lanes to a row
+        const int nch = int(a.row_bytes / 16);
+        for (unsigned todo = __ballot_sync(0xffffffffu, near && half == 0); todo;) {
+          unsigned own = todo;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if (q < (lane >> 3)) own &= own - 1;
+            todo &= todo - 1;
+          }
+          const int src = own ? __ffs(own) - 1 : 0;
+          const uint8_t* orow = a.X + int64_t(__shfl_sync(0xffffffffu, my_id, src)) * a.row_bytes;
+          const double v = ff_d2_warp<8>(reinterpret_cast<const float*>(prow), reinterpret_cast<const float*>(orow),
+                                         own ? nch : 0);
+          if (own && (lane & 7) == 0) k64s[(kRows * warp + src / H) % MAXM] = -v;
+        }
         named_sync(kBarProd, kF32Prod);
+        if (near) my64 = k64s[t];
         int cnt = 0;
         bool open = false;
         if (near) {
