@@ -912,7 +912,9 @@ __global__ void __launch_bounds__(160, tc_min_ctas<MAXM, TB>()) prune_u8_kernel(
 // columns and about 100 KB of shared memory each).  One kernel for both types, with
 // a thread to a row in the gather and a row of pairs, took 8.73 ms for 400,000 x 96
 // floats in lists of up to 64 at eight targets and 8.77 ms for 30,000 x 960 at nine;
-// this one 8.3 and 6.9.
+// this one 8.0 and 4.3.  Of that, the near keys' float-float distances by eight
+// lanes a row (a thread a row before, 32 lines per load and half of a slot of 960
+// dimensions) 6.9 -> 4.7, the gather's next step in flight 8.2 -> 8.0 and 4.7 -> 4.3.
 template <int MAXM, int TB, int H>
 __global__ void __launch_bounds__(128 * H + 32, 2) prune_f32_kernel(PruneArgs a) {
   constexpr int kF32Prod = 128 * H, kF32Threads = kF32Prod + 32;
@@ -1061,10 +1063,26 @@ __global__ void __launch_bounds__(128 * H + 32, 2) prune_f32_kernel(PruneArgs a)
         for (int q = 0; q < kSteps; ++q) {
           const int row = kRows * warp + 8 * q + (lane & 7);
           lv[q] = row % MAXM < m;
-          gid[q] = lv[q] ? a.col[e0 + row % MAXM] : 0;
+          gid[q] = lv[q] ? a.col[e0 + row % MAXM] : ppt;
           kacc[q] = 0.f;
         }
-        const uint4* pp = reinterpret_cast<const uint4*>(prow);
+        // step j of a lane: dimensions 8 (4 j + sub) .. + 7 of its rows and the pivot.
+        // The next step's loads are in flight while this one's values are split,
+        // also across slices.
+        const uint4* pp = reinterpret_cast<const uint4*>(prow) + 2 * sub;
+        const int64_t steps = elems / 32;
+        uint4 ny[2], nx[kSteps][2];
+        auto load_step = [&](int64_t j) {
+          ny[0] = __ldg(pp + 8 * j), ny[1] = __ldg(pp + 8 * j + 1);
+#pragma unroll
+          for (int q = 0; q < kSteps; ++q) {
+            // rows past the degree: the pivot, centred zeros
+            const uint4* px = reinterpret_cast<const uint4*>(a.X + int64_t(gid[q]) * a.row_bytes) + 2 * sub + 8 * j;
+            nx[q][0] = __ldg(px), nx[q][1] = __ldg(px + 1);
+          }
+        };
+        load_step(0);
+        int64_t j = 0;
         for (int sl = 0; sl < nslices; ++sl) {
           if (sl > 0) {  // the operands are free once the previous slice's MMA has read them
             const bool ok = mbar_wait(mbar, phase, 1 << 24);
@@ -1086,15 +1104,11 @@ __global__ void __launch_bounds__(128 * H + 32, 2) prune_f32_kernel(PruneArgs a)
           for (int q = 0; q < kSteps; ++q) part[q][0] = part[q][1] = 0.f;
 #pragma unroll 1
           for (int c = sub; c < np; c += 4) {
-            const int64_t at = int64_t(sl) * 32 + 2 * c;
-            const uint4 y0 = __ldg(pp + at), y1 = __ldg(pp + at + 1);
+            const uint4 y0 = ny[0], y1 = ny[1];
             uint4 x0[kSteps], x1[kSteps];
 #pragma unroll
-            for (int q = 0; q < kSteps; ++q) {
-              const uint4* px = reinterpret_cast<const uint4*>(a.X + int64_t(gid[q]) * a.row_bytes) + at;
-              x0[q] = lv[q] ? __ldg(px) : y0;  // rows past the degree: the pivot, centred zeros
-              x1[q] = lv[q] ? __ldg(px + 1) : y1;
-            }
+            for (int q = 0; q < kSteps; ++q) x0[q] = nx[q][0], x1[q] = nx[q][1];
+            if (++j < steps) load_step(j);
             const float pv[8] = {__uint_as_float(y0.x), __uint_as_float(y0.y), __uint_as_float(y0.z),
                                  __uint_as_float(y0.w), __uint_as_float(y1.x), __uint_as_float(y1.y),
                                  __uint_as_float(y1.z), __uint_as_float(y1.w)};
@@ -2079,8 +2093,6 @@ cudaError_t launch_bucket_nodes(const int64_t* row_ptr, int64_t n, int32_t* list
   return cudaGetLastError();
 }
 
-constexpr int64_t kF32WideBytes = 512;
-
 // CTAs of `kern` that fit on one SM, from its registers and dynamic shared
 // memory (computed directly: the occupancy query under-reports it for these
 // kernels when called while a stream is being captured).
@@ -2131,7 +2143,12 @@ static cudaError_t run_fast_t(const PruneArgs& args, int num_sms, int64_t host_c
   return cudaGetLastError();
 }
 
-// Float rows of more than one 128-dimension slice: eight producer warps.
+// Float rows of more than one 128-dimension slice: eight producer warps, which hide
+// more of the slices' loads; shorter rows four, whose 168 registers (eight: 96) hold
+// all of a step (four / eight: 30,000 x 960 floats 4.40 / 4.26 ms, 400,000 x 96 7.98 /
+// 8.31).
+constexpr int64_t kF32WideBytes = 512;
+
 template <int DT, int MAXM, int TB>
 static cudaError_t run_fast_h(const PruneArgs& args, int num_sms, int64_t host_count, int ctas_cap, cudaStream_t s,
                               int* fit) {
