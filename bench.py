@@ -616,7 +616,7 @@ def run_ours(args):
             "config": {"workload": workload_name(n, nq, args.workload), "n": n, "d": W["d"], "targets": TARGETS_W,
                        "queries": nq, "L": L_W, "k": k, "l2": "flushed (512 MB write) before every timed step",
                        "parallelism": f"node ranges x{ws} (all-gather of tuned slices)" if ws > 1 else "1 GPU"},
-            "roofline": {"bound": "hbm", "kernel": f"prune_tc_kernel<{W['dtype']}, 64, {kernel_tb(W['dtype'], TARGETS_W)}> "
+            "roofline": {"bound": "hbm", "kernel": f"prune_{W['dtype']}_kernel<64, {kernel_tb(W['dtype'], TARGETS_W)}> "
                                                    "(tcgen05 Gram)",
                          "achieved": achieved,
                          "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak, "traffic": traffic,
