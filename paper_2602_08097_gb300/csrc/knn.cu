@@ -523,8 +523,11 @@ size_t knn_tc_smem(int dtype, int64_t tile_bytes, int nbuf) {
   return std::max(need, dtype == kF32 ? size_t(228 * 1024 / 2 + 1024) : size_t(228 * 1024 / 3 + 1024));
 }
 
+// uint8 rows: registers for two CTAs on an SM, as its memory and TMEM allow (10,000
+// queries x 400,000 points x 128, k 100: one CTA's 130 registers 3.7 ms, 96 3.4; 500
+// queries x 200,000 x 96, k 10: 0.47 and 0.40).
 template <int DT>
-__global__ void __launch_bounds__(kTcThreads) knn_scan_kernel(KnnTcArgs a) {
+__global__ void __launch_bounds__(kTcThreads, DT == kU8 ? 2 : 1) knn_scan_kernel(KnnTcArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   // float rows: hi and lo operands, two accumulators per set (acc0 at column
   // 0 of the set, acc1 at 128)
