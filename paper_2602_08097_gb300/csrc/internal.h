@@ -151,7 +151,7 @@ struct KnnLaunch {
 cudaError_t launch_knn(const KnnLaunch& K, cudaStream_t s);
 
 // Exact kNN with the candidate filter on tcgen05 (uint8 rows of d <= 128,
-// float rows of at most 256 dimensions, k <= 128).
+// float rows of at most 128 dimensions, k <= 128).
 struct KnnTcLaunch {
   DevData data;
   const uint8_t* Q = nullptr;  // padded query rows, or nullptr for base points 0..nq-1

@@ -314,13 +314,21 @@ __global__ void __launch_bounds__(kThreads) knn_kernel(KnnArgs a) {
 // exact integer below 2^24).  Point p is kept as a candidate, as {d2~, id}, when
 // its lower bound may be at most tau, an upper bound of the k-th smallest
 // distance met so far by any part of the query (the k-th smallest d2~ of a part
-// plus the largest err it has met): at least k points have d2 <= tau, so every
+// plus the largest err of any point): at least k points have d2 <= tau, so every
 // true k nearest neighbour passes when it is met (tau only decreases).  Eight
 // columns at a time are tested branch-free (the sign of d2~ - threshold, shifted
 // into a mask), and the few that pass are stored by predicated instructions, if
 // any lane has one.  A query's candidates live in a global buffer per part, one
 // thread's from its start up, the other's from its end down; when it gets long, a
 // warp selects the k-th, lowers tau and drops the candidates above it.
+//
+// err grows with the square of p's norm, so that the largest err of all points says
+// nothing about most of them once one has a large norm.  The test therefore takes
+// each point's own, as a linear function of its squared norm (tc_err_linear: one
+// multiply-add in place of an add).  A cut, and the ranking, take the largest while
+// it is narrow against tau or leaves few; else every entry's own (from its norm):
+// tau is then the k-th smallest d2~ + err, and an entry stays if its d2~ - err is
+// not above it.
 //
 // Rank (knn_rank_kernel), one warp per query: the candidates of its parts are
 // cut to the final tau and ranked by their exact keys (uint8: exact integers;
@@ -361,7 +369,7 @@ struct KnnTcArgs {
   int nbuf;                  // point tiles in shared memory, 2 or 3
   const float* qnorm;        // |q'|^2 per query (scaled)
   const float* pnorm;        // |p'|^2 per point, padded to whole tiles with 0
-  const float2* tmax;        // per point tile: (max |p'|^2, max |p'|), then the same over all tiles
+  const float2* tmax;        // (max |p'|^2, max |p'|) over all points
   int exact;                 // 1: G~ and d2~ are exact
   float eps_ip, eps_n, sub_abs;  // sub_abs: the subnormal-rounding term per unit of |q| + |p|
   // this chunk: query tiles qt0 .. qt0 + nqt - 1, `per` steps per CTA.  The part
@@ -397,6 +405,22 @@ __device__ __forceinline__ float tc_err(const KnnTcArgs& a, float nq, float sq, 
          1e-30f;
 }
 
+// tc_err as linear in np, for the scan's test: err <= (1 - f) np + c, since
+// 2 sq sp <= nq + np and 2 sp <= np / sq + sq (2 sp <= np + 1 where sq is 0).  Both
+// also carry 2^-21 of nq and np for the roundings of the test.
+__device__ __forceinline__ void tc_err_linear(const KnnTcArgs& a, float nq, float& f, float& c) {
+  const float sq = sqrtf(nq), s = sq > 0.f ? sq : 1.f;
+  const float g = a.eps_ip * 1.001f + a.eps_n + 9.5367432e-07f;
+  f = 1.f - (g + 0.5f * a.sub_abs / s) * 1.0002f;
+  c = (g * nq + a.sub_abs * (sq + 0.5f * s)) * 1.0002f + 2e-30f;
+}
+
+// tc_err of point id (its norm read from global memory).
+__device__ __forceinline__ float own_err(const KnnTcArgs& a, float nq, float sq, unsigned id) {
+  const float np = __ldg(a.pnorm + id);
+  return tc_err(a, nq, sq, np, sqrtf(np));
+}
+
 // Operands per tile: uint8 rows one f16 operand, float rows two (hi, lo).
 __host__ __device__ constexpr int tc_nop(int dtype) { return dtype == kF32 ? 2 : 1; }
 
@@ -404,14 +428,14 @@ __host__ __device__ constexpr int tc_nop(int dtype) { return dtype == kF32 ? 2 :
 // `gap` places on: gap = 0 for a plain list.
 __device__ __forceinline__ int entry_at(int i, int a, int gap) { return i < a ? i : i + gap; }
 
-// The k-th smallest distance of the m >= k entries as a key, by bisection on its
-// bits; the entries are read once, PER of them per lane.  One warp.
-template <int PER>
-__device__ __forceinline__ unsigned kth_of(const uint2* e, int m, int k) {
+// The k-th smallest value(entry) of the m >= k entries as a key, by bisection on
+// its bits; the entries are read once, PER of them per lane.  One warp.
+template <int PER, typename F>
+__device__ __forceinline__ unsigned kth_of(const uint2* e, int m, int k, F value) {
   const int lane = threadIdx.x & 31;
   unsigned u[PER];
 #pragma unroll
-  for (int i = 0; i < PER; ++i) u[i] = 32 * i + lane < m ? fkey(__uint_as_float(e[32 * i + lane].x)) : 0xffffffffu;
+  for (int i = 0; i < PER; ++i) u[i] = 32 * i + lane < m ? fkey(value(e[32 * i + lane])) : 0xffffffffu;
   unsigned lo = 0xffffffffu, hi = 0;
 #pragma unroll
   for (int i = 0; i < PER; ++i) {
@@ -435,16 +459,17 @@ __device__ __forceinline__ unsigned kth_of(const uint2* e, int m, int k) {
 // that sum.
 __device__ __forceinline__ float cut_width(float e, float norms) { return e * 1.0001f + 4.7683716e-07f * norms; }
 
-// Drops the entries whose lower bound (d2~ - w) lies above tau and moves the rest
-// to the start; returns how many are left.  One warp.
-__device__ __forceinline__ int cut_above(uint2* e, int m, float tau, float w) {
+// Drops the entries whose lower bound, lower(entry), lies above tau and moves the
+// rest to the start; returns how many are left.  One warp.
+template <typename F>
+__device__ __forceinline__ int cut_above(uint2* e, int m, float tau, F lower) {
   const int lane = threadIdx.x & 31;
   int kept = 0;
   for (int i0 = 0; i0 < m; i0 += 32) {
     const int i = i0 + lane;
     uint2 v = make_uint2(0, 0);
     if (i < m) v = e[i];  // never before the place it may be moved to
-    const bool keep = i < m && __uint_as_float(v.x) - w <= tau;
+    const bool keep = i < m && lower(v) <= tau;
     const unsigned km = __ballot_sync(0xffffffffu, keep);
     __syncwarp();
     if (keep) e[kept + __popc(km & ((1u << lane) - 1))] = v;
@@ -454,27 +479,17 @@ __device__ __forceinline__ int cut_above(uint2* e, int m, float tau, float w) {
   return kept;
 }
 
-// A part's m >= k candidates (`a` of them at the buffer's start, the rest up to its
-// end), PER per lane, read once: tau = an upper bound of the k-th smallest d2~, plus
-// w; the entries whose lower bound lies above it are dropped and the rest moved to
-// the start.  Returns how many are left.  The bisection stops at a value that k to
-// k + kCutSlack entries do not exceed, after 5 or 6 of its 25 steps; the few more
-// that stay cost less.  One warp.
-constexpr int kCutSlack = 8;
+// A key that at least k of a warp's m entries do not exceed: the k-th smallest,
+// or one that k to k + slack entries do not exceed.  u: the entries' keys, PER per
+// lane, all ones past m.
 template <int PER>
-__device__ __forceinline__ int cut_part(uint2* e, int m, int k, float w, int a, float& tau) {
+__device__ __forceinline__ unsigned kth_key(const unsigned (&u)[PER], int m, int k, int slack) {
   const int lane = threadIdx.x & 31;
-  const int gap = kTcCand - m;
-  uint2 v[PER];
-#pragma unroll
-  for (int i = 0; i < PER; ++i)
-    v[i] = 32 * i + lane < m ? e[entry_at(32 * i + lane, a, gap)] : make_uint2(0x7fffffffu, 0);
   unsigned lo = 0xffffffffu, hi = 0;
 #pragma unroll
   for (int i = 0; i < PER; ++i) {
-    v[i].x = fkey(__uint_as_float(v[i].x));  // past m: above every distance
-    lo = min(lo, v[i].x);
-    if (32 * i + lane < m) hi = max(hi, v[i].x);
+    lo = min(lo, u[i]);
+    if (32 * i + lane < m) hi = max(hi, u[i]);
   }
   lo = __reduce_min_sync(0xffffffffu, lo);
   hi = __reduce_max_sync(0xffffffffu, hi);
@@ -482,21 +497,63 @@ __device__ __forceinline__ int cut_part(uint2* e, int m, int k, float w, int a, 
     const unsigned mid = lo + (hi - lo) / 2;
     int c = 0;
 #pragma unroll
-    for (int i = 0; i < PER; ++i) c += v[i].x <= mid;
+    for (int i = 0; i < PER; ++i) c += u[i] <= mid;
     c = __reduce_add_sync(0xffffffffu, c);
     if (c >= k) hi = mid;
     else lo = mid + 1;
-    if (c >= k && c <= k + kCutSlack) break;
+    if (c >= k && c <= k + slack) break;
   }
-  tau = fkey_inv(hi) + w;
+  return hi;
+}
+
+// A part's m >= k candidates (`n0` of them at the buffer's start, the rest up to its
+// end), PER per lane, read once: tau = an upper bound of the k-th smallest d2~, plus
+// w; the entries whose lower bound lies above it are dropped and the rest moved to
+// the start.  Returns how many are left.  The bisection stops at a value that k to
+// k + kCutSlack entries do not exceed, after 5 or 6 of its 25 steps; the few more
+// that stay cost less.  If w is wide and leaves more than k + kOwnSlack, every entry's
+// own bound takes its place (nq: the query's squared norm).  One warp.
+constexpr int kCutSlack = 8;
+constexpr int kOwnSlack = 64;
+constexpr float kNarrow = 0.0009765625f;  // a bound below this part of tau is not looked into
+template <int DT, int PER>
+__device__ __forceinline__ int cut_part(const KnnTcArgs& a, uint2* e, int m, float w, float nq, int n0, float& tau) {
+  const int lane = threadIdx.x & 31;
+  const int gap = kTcCand - m, k = a.kscan;
+  unsigned u[PER], id[PER];
+#pragma unroll
+  for (int i = 0; i < PER; ++i) {
+    const uint2 v = 32 * i + lane < m ? e[entry_at(32 * i + lane, n0, gap)] : make_uint2(0x7fffffffu, 0);
+    u[i] = fkey(__uint_as_float(v.x));  // past m: above every distance
+    id[i] = v.y;
+  }
+  tau = fkey_inv(kth_key<PER>(u, m, k, kCutSlack)) + w;
+  unsigned drop = 0;  // bit i: entry 32 i + lane goes
+  if (DT == kF32 && w > kNarrow * tau) {
+    int c = 0;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) c += 32 * i + lane < m && fkey_inv(u[i]) - w <= tau;
+    if (__reduce_add_sync(0xffffffffu, c) > k + kOwnSlack) {
+      const float sq = sqrtf(nq);
+      unsigned ub[PER];
+#pragma unroll
+      for (int i = 0; i < PER; ++i)
+        ub[i] = 32 * i + lane < m ? fkey(fkey_inv(u[i]) + own_err(a, nq, sq, id[i])) : 0xffffffffu;
+      tau = fkey_inv(kth_key<PER>(ub, m, k, 0));
+#pragma unroll
+      for (int i = 0; i < PER; ++i)
+        if (32 * i + lane < m && !(fkey_inv(u[i]) - own_err(a, nq, sq, id[i]) <= tau)) drop |= 1u << i;
+      w = __int_as_float(0x7f800000);  // the test below keeps the rest
+    }
+  }
   int kept = 0;
   __syncwarp();  // every entry has been read
 #pragma unroll
   for (int i = 0; i < PER; ++i) {
-    const float x = fkey_inv(v[i].x);
-    const bool keep = 32 * i + lane < m && x - w <= tau;
+    const float x = fkey_inv(u[i]);
+    const bool keep = 32 * i + lane < m && x - w <= tau && !((drop >> i) & 1u);
     const unsigned km = __ballot_sync(0xffffffffu, keep);
-    if (keep) e[kept + __popc(km & ((1u << lane) - 1))] = make_uint2(__float_as_uint(x), v[i].y);
+    if (keep) e[kept + __popc(km & ((1u << lane) - 1))] = make_uint2(__float_as_uint(x), id[i]);
     kept += __popc(km);
   }
   return kept;
@@ -647,7 +704,7 @@ __global__ void __launch_bounds__(kTcThreads, DT == kU8 ? 2 : 1) knn_scan_kernel
     const int tl = t & (kTcQ - 1), half = t >> 7, quad = warp & 3;
     const long long dir = half ? -8 : 8;
     const float inf = __int_as_float(0x7f800000);
-    float tau = inf, nqq = 0.f, sq = 0.f, width = 0.f;  // width: cut_width of every point met
+    float tau = inf, nqq = 0.f, width = 0.f, lin_f = 1.f, lin_c = 0.f;  // width: cut_width of any point
     int cnt = 0, limit = kTcCut;
     int q = q_first, j = j_first;
     int64_t qi = 0;
@@ -655,8 +712,8 @@ __global__ void __launch_bounds__(kTcThreads, DT == kU8 ? 2 : 1) knn_scan_kernel
     uint2 *cbuf = nullptr, *cnext = nullptr;
     unsigned* tq = nullptr;
     bool ok = true;
-    float shared_tau = inf;  // of the query's other parts, loaded a step ahead, as the tile's norms are
-    float2 tm = steps > 0 ? a.tmax[j] : make_float2(0.f, 0.f);
+    float shared_tau = inf;  // of the query's other parts, loaded a step ahead
+    const float2 tm = *a.tmax;
     // A warp whose wait runs out takes no more candidates, but stays with its
     // partner's barriers to the end.
     for (int it = 0; it < steps; ++it) {
@@ -665,7 +722,10 @@ __global__ void __launch_bounds__(kTcThreads, DT == kU8 ? 2 : 1) knn_scan_kernel
         qi = (a.qt0 + q) * kTcQ + tl;
         qlive = qi < a.nq;
         nqq = qlive ? a.qnorm[qi] : 0.f;
-        sq = sqrtf(nqq);
+        if constexpr (kSplit) {
+          tc_err_linear(a, nqq, lin_f, lin_c);
+          width = cut_width(tc_err(a, nqq, sqrtf(nqq), tm.x, tm.y), nqq + tm.x);
+        }
         cbuf = a.cand + (int64_t(blockIdx.x + q) * kTcQ + tl) * kTcCand;
         tq = a.tauq + int64_t(q) * kTcQ + tl;
         if (half) cbuf += kTcCand - 1;  // this thread's own start
@@ -673,21 +733,13 @@ __global__ void __launch_bounds__(kTcThreads, DT == kU8 ? 2 : 1) knn_scan_kernel
         cnt = 0;
         limit = kTcCut;
         tau = inf;
-        width = 0.f;
         shared_tau = fkey_inv(__ldcg(tq));
       }
       // tau as lowered meanwhile by the query's other parts (any value that was
       // ever there is a valid one; not a number: none yet)
       tau = fminf(tau, shared_tau);
-      float thr = tau;
-      if (!a.exact) {
-        // never below the upper end of what lb <= tau admits, with the roundings of the test itself
-        const float e = tc_err(a, nqq, sq, tm.x, tm.y);
-        width = fmaxf(width, cut_width(e, nqq + tm.x));
-        thr = (tau + e) * 1.000002f + 4.7683716e-07f * (nqq + tm.x);
-      } else {
-        thr = tau + 1.f;  // integers: d2 <= tau as d2 - (tau + 1) < 0
-      }
+      // passes: |q'|^2 + f |p'|^2 - 2 G~ below thr
+      const float thr = kSplit ? tau * 1.000001f + lin_c : tau + 1.f;  // integers: d2 <= tau as d2 - (tau + 1) < 0
       const bool tail = int64_t(j + 1) * kTcP > a.n;
       const float base = nqq - thr;
       const float* pnb = sPn + (it % kTcNorms) * kTcP;
@@ -696,7 +748,6 @@ __global__ void __launch_bounds__(kTcThreads, DT == kU8 ? 2 : 1) knn_scan_kernel
       ok = __all_sync(0xffffffffu, ok);
       tc_fence_after();
       shared_tau = fkey_inv(__ldcg(tq));
-      tm = a.tmax[j + 1 < ntile ? j + 1 : 0];
       const int64_t p0 = int64_t(j) * kTcP;
 #pragma unroll 1
       for (int c0 = half * (kTcP / 2); ok && c0 < (half + 1) * (kTcP / 2); c0 += 32) {
@@ -725,7 +776,8 @@ __global__ void __launch_bounds__(kTcThreads, DT == kU8 ? 2 : 1) knn_scan_kernel
           unsigned mg = 0;
 #pragma unroll
           for (int e = 7; e >= 0; --e)
-            mg = __funnelshift_l(__float_as_uint(fmaf(-2.f, __uint_as_float(v[g + e]), base + pn[e])), mg, 1);
+            mg = __funnelshift_l(__float_as_uint(fmaf(-2.f, __uint_as_float(v[g + e]),
+                                                      kSplit ? fmaf(pn[e], lin_f, base) : base + pn[e])), mg, 1);
           m |= mg << g;
         }
         if (!qlive) m = 0;
@@ -762,13 +814,13 @@ __global__ void __launch_bounds__(kTcThreads, DT == kU8 ? 2 : 1) knn_scan_kernel
           if ((nth & 1) != half) continue;
           const int L = __ffs(int(todo)) - 1;
           const int own = __shfl_sync(0xffffffffu, cnt, L), oth = __shfl_sync(0xffffffffu, other, L);
-          const float wL = __shfl_sync(0xffffffffu, width, L);
+          const float wL = __shfl_sync(0xffffffffu, width, L), nL = __shfl_sync(0xffffffffu, nqq, L);
           const int nA = half ? oth : own, cL = own + oth, ql = quad * 32 + L;
           uint2* bL = a.cand + (int64_t(blockIdx.x + q) * kTcQ + ql) * kTcCand;
           // cL > kTcCut >= kscan
           float tnew;
-          const int w = cL <= 256 ? cut_part<8>(bL, cL, a.kscan, wL, nA, tnew)
-                                  : cut_part<kTcCand / 32>(bL, cL, a.kscan, wL, nA, tnew);
+          const int w = cL <= 256 ? cut_part<DT, 8>(a, bL, cL, wL, nL, nA, tnew)
+                                  : cut_part<DT, kTcCand / 32>(a, bL, cL, wL, nL, nA, tnew);
           if (lane == 0) {
             sCnt[ql] = w;
             sTau[ql] = tnew;
@@ -818,20 +870,29 @@ __global__ void __launch_bounds__(128) knn_rank_kernel(KnnTcArgs a) {
   const float inf = __int_as_float(0x7f800000);
   uint2* e = sbuf[warp];
   float tau = fminf(inf, fkey_inv(a.tauq[ql]));  // never lowered: all ones, not a number
-  float w = 0.f;
+  float w = 0.f, nqq = 0.f, sq = 0.f;
   if (!a.exact) {
-    const float nqq = a.qnorm[qg];
-    const float2 tm = a.tmax[npt];  // over all points
-    w = cut_width(tc_err(a, nqq, sqrtf(nqq), tm.x, tm.y), nqq + tm.x);
+    nqq = a.qnorm[qg];
+    sq = sqrtf(nqq);
+    const float2 tm = *a.tmax;
+    w = cut_width(tc_err(a, nqq, sq, tm.x, tm.y), nqq + tm.x);
   }
   // ---- the candidates of the query's parts, cut to the smallest tau
   int m = 0;
   bool over = false;
   auto lower = [&]() {  // tau from what is held
     if (m < a.k) return;
-    const float tnew = fkey_inv(kth_of<kRankCand / 32>(e, m, a.k)) + w;
+    const float tnew =
+        fkey_inv(kth_of<kRankCand / 32>(e, m, a.k, [](uint2 v) { return __uint_as_float(v.x); })) + w;
     tau = fminf(tau, tnew);
-    m = cut_above(e, m, tau, w);
+    m = cut_above(e, m, tau, [&](uint2 v) { return __uint_as_float(v.x) - w; });
+    if constexpr (DT == kF32) {
+      if (m <= a.k + kOwnSlack) return;
+      const float own = fkey_inv(kth_of<kRankCand / 32>(
+          e, m, a.k, [&](uint2 v) { return __uint_as_float(v.x) + own_err(a, nqq, sq, v.y); }));
+      tau = fminf(tau, own);
+      m = cut_above(e, m, tau, [&](uint2 v) { return __uint_as_float(v.x) - own_err(a, nqq, sq, v.y); });
+    }
   };
   const int64_t c1 = ((qt + 1) * npt - 1) / a.per;
   for (int64_t c = qt * npt / a.per; c <= c1; ++c) {
@@ -993,9 +1054,8 @@ __global__ void pack_f16_kernel(const uint8_t* __restrict__ X, int64_t row_bytes
   norms[i] = acc;
 }
 
-// per tile: (max |x'|^2, max |x'|), the latter rounded up; out[ntile], zeroed
-// before, takes the largest of each
-__global__ void tile_max_kernel(const float* __restrict__ norms, int64_t ntile, float2* __restrict__ out) {
+// *out, zeroed before: (max |x'|^2, max |x'|), the latter rounded up
+__global__ void norm_max_kernel(const float* __restrict__ norms, int64_t ntile, float2* __restrict__ out) {
   const int64_t tile = int64_t(blockIdx.x) * (blockDim.x / 32) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (tile >= ntile) return;
@@ -1004,11 +1064,9 @@ __global__ void tile_max_kernel(const float* __restrict__ norms, int64_t ntile, 
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   if (lane == 0) {
-    const float root = sqrtf(m) * 1.000001f;
-    out[tile] = make_float2(m, root);
-    unsigned* all = reinterpret_cast<unsigned*>(out + ntile);  // bits of non-negative floats
-    atomicMax(all, __float_as_uint(m));
-    atomicMax(all + 1, __float_as_uint(root));
+    unsigned* bits = reinterpret_cast<unsigned*>(out);  // of non-negative floats
+    atomicMax(bits, __float_as_uint(m));
+    atomicMax(bits + 1, __float_as_uint(sqrtf(m) * 1.000001f));
   }
 }
 
@@ -1087,7 +1145,7 @@ TcPlan tc_plan(int dtype, int d, int64_t n, int64_t nq_ext, int num_sms) {
   P.off_pnorm = o;
   o = align256(o + size_t(P.ntile) * kTcP * 4);
   P.off_tmax = o;
-  o = align256(o + size_t(P.ntile + 1) * 8);
+  o = align256(o + sizeof(float2));
   P.off_qtiles = o;
   o = align256(o + size_t(P.nqtile) * P.tile_bytes);
   P.off_qnorm = o;
@@ -1159,8 +1217,8 @@ cudaError_t launch_knn_tc(const KnnTcLaunch& K, cudaStream_t s, int64_t* kernels
   else
     pack_f16_kernel<kU8><<<unsigned((rows + 255) / 256), 256, 0, s>>>(K.data.X, K.data.row_bytes, K.data.n, K.data.d,
                                                                      P.dpad, 1.f, ptiles, pnorm);
-  if ((err = cudaMemsetAsync(tmax + P.ntile, 0, 8, s)) != cudaSuccess) return err;
-  tile_max_kernel<<<unsigned((P.ntile + 7) / 8), 256, 0, s>>>(pnorm, P.ntile, tmax);
+  if ((err = cudaMemsetAsync(tmax, 0, sizeof(float2), s)) != cudaSuccess) return err;
+  norm_max_kernel<<<unsigned((P.ntile + 7) / 8), 256, 0, s>>>(pnorm, P.ntile, tmax);
   const uint8_t* qtiles = ptiles;
   const float* qnorm = pnorm;
   if (K.Q) {
