@@ -335,6 +335,15 @@ __global__ void __launch_bounds__(kThreads) knn_kernel(KnnArgs a) {
 // float: sums per 32-dim slice with near-tie runs re-ordered in binary64), as
 // the CUDA-core kernel ranks its lists.
 //
+// Redo (knn_redo_kernel): a part that met more than kTcCand - kTcP equal or nearly
+// equal distances before any other part had a better tau has no room left, though
+// the query as a whole has better points and needs few of them (a block of repeated
+// rows does that).  Such a query is marked, not ranked, and scanned again: one CTA
+// per query tile takes all points in order as one part, from the tau that the first
+// scan came to, with exact cuts, and ranks the marked queries.  A query is refused
+// only if that runs out of room.  With nothing marked, as good as always, it costs its
+// launch.
+//
 // What bounds the scan: the threads' 64 columns a step, read, tested and now and
 // then stored, about 2,400 of a step's 4,000 cycles (its products: 1,150 at d = 96),
 // and the cuts, which hold the other warps up through the accumulators.  10,000
@@ -381,6 +390,7 @@ struct KnnTcArgs {
   int* pcnt;                 // [part][query] candidates (from the start, << 16 from the end), zeroed: none
                              // of a part that could not finish
   unsigned* tauq;            // [chunk query] tau as an ordered key (fkey), lowered by every part
+  int* marked;               // [chunk query] not 0: to be scanned again (zeroed before the scan)
   int32_t* out_ids;
   float* out_dists;
   DevStatus* status;
@@ -516,7 +526,7 @@ __device__ __forceinline__ unsigned kth_key(const unsigned (&u)[PER], int m, int
 constexpr int kCutSlack = 8;
 constexpr int kOwnSlack = 64;
 constexpr float kNarrow = 0.0009765625f;  // a bound below this part of tau is not looked into
-template <int DT, int PER>
+template <int DT, int PER, bool REDO>
 __device__ __forceinline__ int cut_part(const KnnTcArgs& a, uint2* e, int m, float w, float nq, int n0, float& tau) {
   const int lane = threadIdx.x & 31;
   const int gap = kTcCand - m, k = a.kscan;
@@ -527,9 +537,9 @@ __device__ __forceinline__ int cut_part(const KnnTcArgs& a, uint2* e, int m, flo
     u[i] = fkey(__uint_as_float(v.x));  // past m: above every distance
     id[i] = v.y;
   }
-  tau = fkey_inv(kth_key<PER>(u, m, k, kCutSlack)) + w;
+  tau = fkey_inv(kth_key<PER>(u, m, k, REDO ? 0 : kCutSlack)) + w;
   unsigned drop = 0;  // bit i: entry 32 i + lane goes
-  if (DT == kF32 && w > kNarrow * tau) {
+  if (DT == kF32 && (REDO || w > kNarrow * tau)) {
     int c = 0;
 #pragma unroll
     for (int i = 0; i < PER; ++i) c += 32 * i + lane < m && fkey_inv(u[i]) - w <= tau;
@@ -580,12 +590,9 @@ size_t knn_tc_smem(int dtype, int64_t tile_bytes, int nbuf) {
   return std::max(need, dtype == kF32 ? size_t(228 * 1024 / 2 + 1024) : size_t(228 * 1024 / 3 + 1024));
 }
 
-// uint8 rows: registers for two CTAs on an SM, as its memory and TMEM allow (10,000
-// queries x 400,000 points x 128, k 100: one CTA's 130 registers 3.7 ms, 96 3.4; 500
-// queries x 200,000 x 96, k 10: 0.47 and 0.40).
-template <int DT>
-__global__ void __launch_bounds__(kTcThreads, DT == kU8 ? 2 : 1) knn_scan_kernel(KnnTcArgs a) {
-  extern __shared__ __align__(128) unsigned char smem_raw[];
+// The steps of one CTA.  REDO: of the marked queries only, its query tile's points as one part.
+template <int DT, bool REDO>
+__device__ __forceinline__ void scan_steps(const KnnTcArgs& a, unsigned char* smem_raw) {
   // float rows: hi and lo operands, two accumulators per set (acc0 at column
   // 0 of the set, acc1 at 128)
   constexpr bool kSplit = DT == kF32;
@@ -720,7 +727,7 @@ __global__ void __launch_bounds__(kTcThreads, DT == kU8 ? 2 : 1) knn_scan_kernel
       const int b = it & 1;
       if (it == 0 || j == 0) {  // a new part
         qi = (a.qt0 + q) * kTcQ + tl;
-        qlive = qi < a.nq;
+        qlive = qi < a.nq && (!REDO || a.marked[q * kTcQ + tl] != 0);
         nqq = qlive ? a.qnorm[qi] : 0.f;
         if constexpr (kSplit) {
           tc_err_linear(a, nqq, lin_f, lin_c);
@@ -819,13 +826,16 @@ __global__ void __launch_bounds__(kTcThreads, DT == kU8 ? 2 : 1) knn_scan_kernel
           uint2* bL = a.cand + (int64_t(blockIdx.x + q) * kTcQ + ql) * kTcCand;
           // cL > kTcCut >= kscan
           float tnew;
-          const int w = cL <= 256 ? cut_part<DT, 8>(a, bL, cL, wL, nL, nA, tnew)
-                                  : cut_part<DT, kTcCand / 32>(a, bL, cL, wL, nL, nA, tnew);
+          const int w = cL <= 256 ? cut_part<DT, 8, REDO>(a, bL, cL, wL, nL, nA, tnew)
+                                  : cut_part<DT, kTcCand / 32, REDO>(a, bL, cL, wL, nL, nA, tnew);
           if (lane == 0) {
             sCnt[ql] = w;
             sTau[ql] = tnew;
             atomicMin(a.tauq + int64_t(q) * kTcQ + ql, fkey(tnew));
-            if (w > kTcCand - kTcP) raise_status(a.status, kDevOverflow, (a.qt0 + q) * kTcQ + ql);
+            if (w > kTcCand - kTcP) {
+              if (REDO) raise_status(a.status, kDevOverflow, (a.qt0 + q) * kTcQ + ql);
+              else a.marked[q * kTcQ + ql] = 1;
+            }
           }
           __syncwarp();
         }
@@ -836,7 +846,7 @@ __global__ void __launch_bounds__(kTcThreads, DT == kU8 ? 2 : 1) knn_scan_kernel
           cnext = half ? cbuf : cbuf + w;
           tau = fminf(tau, sTau[tl]);
           limit = min(max(kTcCut, w + 96), kTcCand - kTcP);
-          if (w > kTcCand - kTcP) qlive = false;  // no room for the next tile: reported, take no more
+          if (w > kTcCand - kTcP) qlive = false;  // no room for the next tile: marked or reported, take no more
         }
       }
       if (it + 1 == steps || j + 1 == ntile) {
@@ -858,18 +868,15 @@ __global__ void __launch_bounds__(kTcThreads, DT == kU8 ? 2 : 1) knn_scan_kernel
   if (warp == 0) tmem_dealloc(tmem, 2 * kSetCols);
 }
 
-template <int DT>
-__global__ void __launch_bounds__(128) knn_rank_kernel(KnnTcArgs a) {
-  __shared__ uint2 sbuf[4][kRankCand];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t ql = int64_t(blockIdx.x) * 4 + warp;  // query of the chunk
+// Query ql of the chunk, by one warp with kRankCand entries of shared memory at e.
+template <int DT, bool REDO>
+__device__ __forceinline__ void rank_query(const KnnTcArgs& a, int64_t ql, uint2* e) {
+  const int lane = threadIdx.x & 31;
   const int64_t qg = a.qt0 * kTcQ + ql;
-  if (ql >= a.nqt * kTcQ || qg >= a.nq) return;
   const int64_t npt = (a.n + kTcP - 1) / kTcP, qt = ql / kTcQ;
   const int t = int(ql % kTcQ);
   const float inf = __int_as_float(0x7f800000);
-  uint2* e = sbuf[warp];
-  float tau = fminf(inf, fkey_inv(a.tauq[ql]));  // never lowered: all ones, not a number
+  float tau = fminf(inf, fkey_inv(__ldcg(a.tauq + ql)));  // never lowered: all ones, not a number
   float w = 0.f, nqq = 0.f, sq = 0.f;
   if (!a.exact) {
     nqq = a.qnorm[qg];
@@ -887,7 +894,7 @@ __global__ void __launch_bounds__(128) knn_rank_kernel(KnnTcArgs a) {
     tau = fminf(tau, tnew);
     m = cut_above(e, m, tau, [&](uint2 v) { return __uint_as_float(v.x) - w; });
     if constexpr (DT == kF32) {
-      if (m <= a.k + kOwnSlack) return;
+      if (!REDO && m <= a.k + kOwnSlack) return;
       const float own = fkey_inv(kth_of<kRankCand / 32>(
           e, m, a.k, [&](uint2 v) { return __uint_as_float(v.x) + own_err(a, nqq, sq, v.y); }));
       tau = fminf(tau, own);
@@ -919,7 +926,10 @@ __global__ void __launch_bounds__(128) knn_rank_kernel(KnnTcArgs a) {
       __syncwarp();
     }
   }
-  if (over && lane == 0) raise_status(a.status, kDevOverflow, qg);
+  if (!REDO && over) {
+    if (lane == 0) a.marked[ql] = 1;
+    return;
+  }
   lower();
   // ---- exact keys: four lanes per row
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(e);
@@ -988,7 +998,39 @@ __global__ void __launch_bounds__(128) knn_rank_kernel(KnnTcArgs a) {
   }
 }
 
-// ---- packing: f16 operand tiles, scaled squared norms, per-tile maxima
+// uint8 rows: registers for two CTAs on an SM, as its memory and TMEM allow (10,000
+// queries x 400,000 points x 128, k 100: one CTA's 130 registers 3.7 ms, 96 3.4; 500
+// queries x 200,000 x 96, k 10: 0.47 and 0.40).
+template <int DT>
+__global__ void __launch_bounds__(kTcThreads, DT == kU8 ? 2 : 1) knn_scan_kernel(KnnTcArgs a) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  scan_steps<DT, false>(a, smem_raw);
+}
+
+template <int DT>
+__global__ void __launch_bounds__(128) knn_rank_kernel(KnnTcArgs a) {
+  __shared__ uint2 sbuf[4][kRankCand];
+  const int warp = threadIdx.x >> 5;
+  const int64_t ql = int64_t(blockIdx.x) * 4 + warp;
+  if (ql >= a.nqt * kTcQ || a.qt0 * kTcQ + ql >= a.nq || a.marked[ql] != 0) return;
+  rank_query<DT, false>(a, ql, sbuf[warp]);
+}
+
+// The marked queries of query tile blockIdx.x of the chunk: a.per = all its points.
+template <int DT>
+__global__ void __launch_bounds__(kTcThreads, 1) knn_redo_kernel(KnnTcArgs a) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int64_t q0 = int64_t(blockIdx.x) * kTcQ;
+  if (!__syncthreads_or(threadIdx.x < kTcQ && a.marked[q0 + threadIdx.x] != 0)) return;
+  scan_steps<DT, true>(a, smem_raw);
+  __syncthreads();  // the candidates; shared memory is free
+  const int warp = threadIdx.x >> 5;
+  for (int q = warp; warp < 8 && q < kTcQ; q += 8)  // a query past nq is never marked
+    if (a.marked[q0 + q] != 0) rank_query<DT, true>(a, q0 + q, reinterpret_cast<uint2*>(smem_raw) + warp * kRankCand);
+}
+static_assert(8 * kRankCand * sizeof(uint2) <= 228 * 1024 / 3, "the redo's ranking fits in what every scan has");
+
+// ---- packing: f16 operand tiles, scaled squared norms, their maximum
 
 // max |x| over n rows of float data (bits of a non-negative float, atomicMax)
 __global__ void maxabs_kernel(const uint8_t* __restrict__ X, int64_t row_bytes, int64_t n, int d,
@@ -1119,7 +1161,7 @@ namespace {
 struct TcPlan {
   int dpad, nbuf, ctas, grid;
   int64_t ntile, nqtile, chunk, tile_bytes;
-  size_t off_ptiles, off_pnorm, off_tmax, off_qtiles, off_qnorm, off_cand, off_pcnt, off_tauq, total;
+  size_t off_ptiles, off_pnorm, off_tmax, off_qtiles, off_qnorm, off_cand, off_pcnt, off_marked, off_tauq, total;
 };
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
@@ -1153,7 +1195,9 @@ TcPlan tc_plan(int dtype, int d, int64_t n, int64_t nq_ext, int num_sms) {
   P.off_cand = o;
   o = align256(o + parts * kTcQ * kTcCand * 8);
   P.off_pcnt = o;
-  o = align256(o + parts * kTcQ * 4);
+  o = o + parts * kTcQ * 4;
+  P.off_marked = o;  // right behind: one fill for both
+  o = align256(o + size_t(P.chunk) * kTcQ * 4);
   P.off_tauq = o;
   o = align256(o + size_t(P.chunk) * kTcQ * 4);
   P.total = o;
@@ -1164,6 +1208,8 @@ template <int DT>
 cudaError_t scan_and_rank(KnnTcArgs a, const TcPlan& P, cudaStream_t s) {
   const size_t smem = knn_tc_smem(DT, P.tile_bytes, P.nbuf);
   cudaError_t err = cudaFuncSetAttribute(knn_scan_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  if (err == cudaSuccess)
+    err = cudaFuncSetAttribute(knn_redo_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (err != cudaSuccess) return err;
   const int64_t nqt = (a.nq + kTcQ - 1) / kTcQ;
   for (a.qt0 = 0; a.qt0 < nqt; a.qt0 += P.chunk) {
@@ -1171,9 +1217,11 @@ cudaError_t scan_and_rank(KnnTcArgs a, const TcPlan& P, cudaStream_t s) {
     const int64_t total = a.nqt * P.ntile;
     a.per = std::max<int64_t>((total + P.grid - 1) / P.grid, std::min<int64_t>(P.ntile, kTcMinSteps));
     if ((err = cudaMemsetAsync(a.tauq, 0xff, size_t(a.nqt) * kTcQ * 4, s)) != cudaSuccess) return err;
-    if ((err = cudaMemsetAsync(a.pcnt, 0, size_t(P.grid + P.chunk) * kTcQ * 4, s)) != cudaSuccess) return err;
+    if ((err = cudaMemsetAsync(a.pcnt, 0, size_t(P.grid + 2 * P.chunk) * kTcQ * 4, s)) != cudaSuccess) return err;
     knn_scan_kernel<DT><<<unsigned((total + a.per - 1) / a.per), kTcThreads, smem, s>>>(a);
     knn_rank_kernel<DT><<<unsigned(a.nqt * kTcQ / 4), 128, 0, s>>>(a);
+    a.per = P.ntile;
+    knn_redo_kernel<DT><<<unsigned(a.nqt), kTcThreads, smem, s>>>(a);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
   }
   return cudaSuccess;
@@ -1262,12 +1310,13 @@ cudaError_t launch_knn_tc(const KnnTcLaunch& K, cudaStream_t s, int64_t* kernels
   a.sub_abs = std::sqrt(float(K.data.d)) * 1.001f * 2.910383e-11f;  // twice 2^-36 sqrt(d)
   a.cand = reinterpret_cast<uint2*>(base + P.off_cand);
   a.pcnt = reinterpret_cast<int*>(base + P.off_pcnt);
+  a.marked = reinterpret_cast<int*>(base + P.off_marked);
   a.tauq = reinterpret_cast<unsigned*>(base + P.off_tauq);
   a.out_ids = K.out_ids;
   a.out_dists = K.out_dists;
   a.status = K.status;
   const int64_t chunks = ((K.nq + kTcQ - 1) / kTcQ + P.chunk - 1) / P.chunk;
-  *kernels = 2 + (K.Q ? (f32 ? 2 : 1) : 0) + 2 * chunks;
+  *kernels = 2 + (K.Q ? (f32 ? 2 : 1) : 0) + 3 * chunks;
   return f32 ? scan_and_rank<kF32>(a, P, s) : scan_and_rank<kU8>(a, P, s);
 }
 

@@ -65,3 +65,38 @@ def test_more_query_tiles_than_a_launch_takes(ctx, dtype, d, few):
     (ti, td), (ci, cd) = _both(ctx, g, Q, 20)
     assert np.array_equal(ti, ci) and np.array_equal(td, cd)
     rp.rp_graph_free(ctx, g)
+
+
+@pytest.mark.parametrize("dtype,nq", [("u8", 25600), ("f32", 12800)])
+def test_a_part_that_starts_among_repeated_rows(ctx, dtype, nq):
+    # The near points lie in the first tile, the rest is one row over and over.  With
+    # two thirds as many query tiles as CTAs, most queries' second part is scanned
+    # before their first: it meets nothing but equal distances.
+    rng = np.random.default_rng(11)
+    n, d, k = 2048, 32, 10
+    if dtype == "u8":
+        X, Q = rng.integers(0, 20, (n, d)).astype(np.uint8), rng.integers(0, 20, (nq, d)).astype(np.uint8)
+        X[128:] = 200
+    else:
+        X, Q = rng.normal(size=(n, d)).astype(np.float32), rng.normal(size=(nq, d)).astype(np.float32)
+        X[128:] = 10.0
+    g = rp.rp_load_graph(ctx, X)
+    (ti, td), (ci, cd) = _both(ctx, g, Q, k)
+    assert np.array_equal(ti, ci) and np.array_equal(td, cd)
+    sel = np.arange(0, nq, 97)
+    assert np.array_equal(ti[sel], oracle.knn(X, k, Q=np.ascontiguousarray(Q[sel]))[0])
+    rp.rp_graph_free(ctx, g)
+
+
+def test_more_equal_distances_than_the_scan_holds_are_refused(ctx):
+    X = np.full((3000, 16), 7, np.uint8)
+    X[:5] = 1
+    g = rp.rp_load_graph(ctx, X)
+    Q = np.full((3, 16), 8, np.uint8)
+    rp.rp_set_knn_method(ctx, rp.RP_KNN_TENSOR)
+    with pytest.raises(rp.RPError):
+        rp.rp_knn(ctx, g, Q, 10)
+    rp.rp_set_knn_method(ctx, rp.RP_KNN_AUTO)
+    Q[:] = 0  # the context goes on: the five others are nearest
+    assert np.array_equal(np.sort(rp.rp_knn(ctx, g, Q, 5)[0], axis=1), np.tile(np.arange(5), (3, 1)))
+    rp.rp_graph_free(ctx, g)
