@@ -155,12 +155,12 @@ __device__ __forceinline__ double ff_d2(const float* q, const float* __restrict_
 // total.  A lane's 4 ceil(nch / W) steps and the levels that join nonzero pairs
 // stay within the (3 d + 13) 2^-48 of one chain (ff_bound).  The same value in
 // each of the W lanes.
-template <int W = 32>
+template <int W = 32, int UNROLL = 4>
 __device__ __forceinline__ double ff_d2_warp(const float* q, const float* __restrict__ x, int nch) {
   const float4* pq = reinterpret_cast<const float4*>(q);
   const float4* px = reinterpret_cast<const float4*>(x);
   float sh = 0.f, sl = 0.f;
-#pragma unroll 4
+#pragma unroll UNROLL
   for (int c = threadIdx.x & (W - 1); c < nch; c += W) {
     const float4 a = pq[c], b = __ldg(px + c);
     ff_step(a.x, b.x, sh, sl);

@@ -98,7 +98,15 @@ struct SearchGraph {
   int64_t pad;
 };
 
+// Queries of L <= 256 over float rows that met too many near-equal distances are
+// left with the id kSearchRedo first in their row and searched again by a second
+// launch: with the first (kSearchBoth), or by a call of its own (kSearchAgain) where
+// the caller sees the ids of the first alone (kSearchOnce) and mostly needs none.
+enum SearchPass { kSearchBoth, kSearchOnce, kSearchAgain };
+constexpr int32_t kSearchRedo = -2;
+
 struct SearchLaunch {
+  SearchPass pass = kSearchBoth;
   DevData data;
   const int64_t* row_ptr = nullptr;
   const int32_t* col = nullptr;
@@ -128,7 +136,7 @@ struct SearchLaunch {
   int32_t* visited_cnt = nullptr;
   int visited_cap = 0;
 };
-cudaError_t launch_search(const SearchLaunch& S, cudaStream_t s);
+cudaError_t launch_search(const SearchLaunch& S, cudaStream_t s, int* kernels = nullptr /* launched */);
 cudaError_t launch_recall(const int32_t* found, int ld_found, const int32_t* truth, int ld_truth,
                           int64_t nq, int k, unsigned long long* hits, cudaStream_t s);
 

@@ -834,11 +834,14 @@ rp_status search_impl(rp_ctx* c, const rp_graph* graphs, int32_t ngraphs, const 
   S.status = c->status;
   CUDA_TRY(c, cudaMemsetAsync(c->work, 0, 8 * sizeof(unsigned), c->stream));
   CUDA_TRY(c, record(c->ev[3], c->stream));
-  CUDA_TRY(c, launch_search(S, c->stream));
+  int nk = 0;
+  // the host sees the ids: it asks for the second launch if one is marked
+  S.pass = mem_flags == RP_MEM_HOST ? kSearchOnce : kSearchBoth;
+  CUDA_TRY(c, launch_search(S, c->stream, &nk));
   CUDA_TRY(c, record(c->ev[4], c->stream));
   c->ev_search = true;
-  c->kernel_launches += 1;
-  if (mem_flags == RP_MEM_HOST) {
+  c->kernel_launches += nk;
+  while (mem_flags == RP_MEM_HOST) {
     const size_t nb = size_t(nq * k) * 4;
     uint8_t* const pin_out = pin_rows + qbytes;
     if (small) {  // ids and distances are one block behind the rows
@@ -853,7 +856,13 @@ rp_status search_impl(rp_ctx* c, const rp_graph* graphs, int32_t ngraphs, const 
       memcpy(ids, pin_out, nb);
       if (dists) memcpy(dists, pin_out + nb, nb);
     }
-    return status_result(c);
+    bool again = false;
+    for (int64_t q = 0; S.pass == kSearchOnce && q < nq && !again; ++q) again = ids[q * k] == kSearchRedo;
+    if (!again) return status_result(c);
+    S.pass = kSearchAgain;
+    CUDA_TRY(c, launch_search(S, c->stream, &nk));
+    CUDA_TRY(c, record(c->ev[4], c->stream));
+    c->kernel_launches += nk;
   }
   if (q_graph) {
     // the host tables were read by stream-ordered copies; finish them before returning
@@ -1149,7 +1158,8 @@ rp_status build_vamana(rp_ctx* c, rp_graph data, const int32_t* perm, int32_t np
       S.work = c->work;
       S.status = c->status;
       CUDA_TRY(c, cudaMemsetAsync(c->work, 0, 8 * sizeof(unsigned), c->stream));
-      CUDA_TRY(c, launch_search(S, c->stream));
+      int nk = 0;
+      CUDA_TRY(c, launch_search(S, c->stream, &nk));
       // candidates V_p u N_out(p) \ {p}, Algorithm 1 over them, write back
       CUDA_TRY(c, launch_vamana_candidates(pts, nb, vis, vis_cnt, vcap, nbr, deg, R, cand, ccnt, cut, c->stream));
       CUDA_TRY(c, launch_scan_counts(ccnt, nb, crp, bsum, maxd, c->stream));
@@ -1161,7 +1171,7 @@ rp_status build_vamana(rp_ctx* c, rp_graph data, const int32_t* perm, int32_t np
       // back edges
       CUDA_TRY(c, cudaMemsetAsync(nj, 0, 4, c->stream));
       CUDA_TRY(c, launch_back_count(pts, nb, nbr, deg, R, pend, slot, jlist, nj, c->stream));
-      c->kernel_launches += 8;
+      c->kernel_launches += 7 + nk;
       const int64_t nJ = read_i32(c, nj, &s);
       if (s != RP_OK) return s;
       if (nJ > 0) {

@@ -8,7 +8,9 @@
 //                       room for the new point, so adding a point takes two
 //                       shuffles and a few selects per slot.
 //   search_list_kernel  longer lists: in shared memory, sorted by (distance, id);
-//                       new points are sorted and merged 32 at a time.
+//                       new points are sorted and merged 32 at a time.  It also takes
+//                       the float queries that met so many near-equal distances that
+//                       the first kernel gave them up (kFineBudget).
 //
 // Algorithm 2 keeps a set: adding a point that is already in the list has
 // no effect.  A point that was in the list and was cut may be added again by
@@ -37,6 +39,7 @@
 // (index order, no fused multiply-add), so every comparison agrees with the
 // binary64 reading.
 #include <cfloat>
+#include <climits>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -52,6 +55,16 @@ constexpr int kWarps = 4;  // warps (queries in flight) per CTA
 constexpr int kTeam = 5;        // warps per query of the team form: the list's warp and four that read rows
 constexpr unsigned kVisited = 0x80000000u;
 constexpr unsigned kIdMask = 0x7fffffffu;
+// A float query's close decisions in search_reg_kernel are made one at a time by the
+// whole warp, which is dear where distances tie all the time (rows of zeros and ones,
+// rows many times over).  A query that has made more than kFineBudget of them, or met
+// one that binary64 has to settle, leaves kSearchRedo as its first id and is searched
+// again by search_list_kernel, which keeps such distances and settles 32 at a time.
+// The benchmark's shapes make 0.2 (400,000 x 96, L = 100) to 20 a query (30,000 x 960,
+// L = 200), and none of their queries is given up.  20,000 x 96 zeros and ones, L =
+// 100, 5,000 queries: every decision made here 2,963 ms, with the budget 55, by the
+// list kernel alone 55.
+constexpr int kFineBudget = 128;
 
 struct SearchArgs {
   const uint8_t* X;
@@ -83,6 +96,7 @@ struct SearchArgs {
   int32_t* visited;
   int32_t* visited_cnt;
   int visited_cap;
+  int fine_budget;            // search_reg_kernel: most that a query may spend on close decisions
 };
 
 struct WarpSmem {
@@ -299,7 +313,8 @@ __device__ __forceinline__ bool entry_less(unsigned ka, unsigned ia, double* d64
 // The list in shared memory, for L > kRegL.  A batch of 32 neighbours: those
 // the id cache does not hold get their distances, those that enter the list
 // are sorted by a bitonic network and merged in place.
-template <int DT>
+// REDO: any L, only the queries that hold kSearchRedo (spread over the grid's warps).
+template <int DT, bool REDO>
 __global__ void __launch_bounds__(kWarps * 32, 8) search_list_kernel(SearchArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -310,12 +325,27 @@ __global__ void __launch_bounds__(kWarps * 32, 8) search_list_kernel(SearchArgs 
   const int centries = 1 << a.cache_bits;
   const float E = lane_rel_bound(int(a.row_bytes / 16)), Eabs = abs_bound(a.d);
   const double qnan = __longlong_as_double(0x7ff8000000000000ll);
+  // REDO: lane l looks at query rb + l * rstep
+  const int64_t rstep = int64_t(gridDim.x) * kWarps;
+  int64_t rb = int64_t(w) * gridDim.x + blockIdx.x - 32 * rstep;
+  unsigned redo = 0;
 
   for (;;) {
     unsigned qi = 0;
-    if (lane == 0) qi = atomicAdd(a.work, 1u);
-    qi = __shfl_sync(0xffffffffu, qi, 0);
-    if (qi >= a.nq) break;
+    if constexpr (REDO) {
+      while (!redo) {
+        rb += 32 * rstep;
+        if (rb >= a.nq) return;
+        const int64_t q = rb + lane * rstep;
+        redo = __ballot_sync(0xffffffffu, q < a.nq && a.out_ids[q * a.k] == kSearchRedo);
+      }
+      qi = unsigned(rb + (__ffs(int(redo)) - 1) * rstep);
+      redo &= redo - 1;
+    } else {
+      if (lane == 0) qi = atomicAdd(a.work, 1u);
+      qi = __shfl_sync(0xffffffffu, qi, 0);
+      if (qi >= a.nq) break;
+    }
     const int64_t* __restrict__ row_ptr = a.row_ptr;
     const int32_t* __restrict__ col = a.col;
     int64_t start = a.start;
@@ -584,7 +614,7 @@ struct RegSmem {
   uint8_t* q;
   unsigned* cid;   // [kNbr] new ids
   unsigned* ckey;  // [kNbr] their distances
-  int* ctl;        // team form: rows to read (-1: the query is done); [1] the query
+  int* ctl;        // team form: rows to read (-1: the query is done); [1] the query; [2] what is left of kFineBudget
 };
 
 __host__ __device__ inline size_t reg_bytes(int64_t row_bytes, int cache_bits) {
@@ -604,20 +634,79 @@ __device__ inline RegSmem reg_carve(unsigned char* p, int64_t row_bytes, int cac
   return w;
 }
 
+// The float-float distance of a query and a row by a whole warp, as ff_d2_warp sums
+// it, and whether it is exact and equals the binary64 one: no difference, square or
+// sum has rounded in single precision, and the total is at most 2^28 times the least
+// square.  Every square is then a multiple of some power of two g > least 2^-24,
+// so that every partial sum in index order is below 2^52 g and binary64 never rounds
+// either.  (Whole numbers of moderate size, so that their many ties cost no more.)
+__device__ __forceinline__ double ff_d2_exact(const float* q, const float* __restrict__ x, int nch, bool& exact) {
+  const float4* pq = reinterpret_cast<const float4*>(q);
+  const float4* px = reinterpret_cast<const float4*>(x);
+  float sh = 0.f, sl = 0.f, lost = 0.f, least = __int_as_float(0x7f800000);
+  auto step = [&](float a, float b) {
+    const float th = __fsub_rn(a, b);
+    const float bv = __fsub_rn(th, a);
+    const float tl = __fadd_rn(__fsub_rn(a, __fsub_rn(th, bv)), __fsub_rn(__fsub_rn(0.f, b), bv));
+    const float ph = __fmul_rn(th, th), s1 = __fadd_rn(sh, ph), b1 = __fsub_rn(s1, sh);
+    const float e = __fadd_rn(__fsub_rn(sh, __fsub_rn(s1, b1)), __fsub_rn(ph, b1));
+    lost += fabsf(tl) + fabsf(__fmaf_rn(th, th, -ph)) + fabsf(e);
+    least = th != 0.f ? fminf(least, ph) : least;
+    ff_step(a, b, sh, sl);
+  };
+#pragma unroll 1
+  for (int c = threadIdx.x & 31; c < nch; c += 32) {
+    const float4 a = pq[c], b = __ldg(px + c);
+    step(a.x, b.x);
+    step(a.y, b.y);
+    step(a.z, b.z);
+    step(a.w, b.w);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float oh = __shfl_xor_sync(0xffffffffu, sh, o), ol = __shfl_xor_sync(0xffffffffu, sl, o);
+    const float s1 = __fadd_rn(sh, oh);
+    const float bv = __fsub_rn(s1, sh);
+    const float e = __fadd_rn(__fsub_rn(sh, __fsub_rn(s1, bv)), __fsub_rn(oh, bv));
+    const float l1 = __fadd_rn(__fadd_rn(sl, ol), e);
+    lost += fabsf(e);
+    sh = __fadd_rn(s1, l1);
+    sl = __fsub_rn(l1, __fsub_rn(sh, s1));
+  }
+  least = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(least)));
+  // squares that may have underflowed are not looked into
+  exact = __all_sync(0xffffffffu, lost == 0.f) && least >= 1.0e-30f && sh <= 268435456.f * least;
+  return __dadd_rn(double(sh), double(sl));
+}
+
 // Whether point `m` precedes point `c` in (distance, id) order, where their
-// single-precision intervals overlap: float-float distances, then binary64.
-// Called by a whole warp; out of line, since it is rare.
-__device__ __noinline__ bool precedes_fine(const uint8_t* Xb, int64_t row_bytes, int d, DevStatus* status,
-                                           const float* q, unsigned m, unsigned c) {
-  const int64_t stride = row_bytes / 4;
-  const float* xm = reinterpret_cast<const float*>(Xb) + int64_t(m) * stride;
-  const float* xc = reinterpret_cast<const float*>(Xb) + int64_t(c) * stride;
-  const int nch = int(row_bytes / 16);
-  const int o = slot_order(-ff_d2_warp(q, xm, nch), -ff_d2_warp(q, xc, nch), ff_bound(d));
-  if (o >= 0) return o == 1;
-  const double dm = canon_d2_f32(q, xm, d), dc = canon_d2_f32(q, xc, d);
-  if ((threadIdx.x & 31) == 0) atomicAdd(&status->fp64_search, 2ull);
-  return dm < dc || (dm == dc && m < c);
+// single-precision intervals overlap: by float-float distances, by id where those are
+// exact or the rows the same.  Where binary64 would have to decide, the query is given
+// up.  Called by a whole warp; out of line, since it is rare.  q lies in a RegSmem,
+// whose ctl[2] is what the query may still spend: once that is negative, any answer
+// does and rows of no dimensions are compared.
+__device__ __noinline__ bool precedes_fine(const uint8_t* Xb, int64_t row_bytes, int d, const float* q, unsigned m,
+                                           unsigned c) {
+  int* left = reinterpret_cast<int*>(const_cast<uint8_t*>(reinterpret_cast<const uint8_t*>(q)) + row_bytes) +
+              2 * kNbr + 2;
+  const int nch = *left < 0 ? 0 : int(row_bytes / 16);
+  const float* xm = reinterpret_cast<const float*>(Xb + int64_t(m) * row_bytes);
+  const float* xc = reinterpret_cast<const float*>(Xb + int64_t(c) * row_bytes);
+  // (every vote on the way of every call: one under a condition, or a return before
+  // the end, and ptxas spills in the search's loop, 1.43 to 1.58 ms where it takes 0.95)
+  bool differ = false;
+#pragma unroll 1
+  for (int i = threadIdx.x & 31; i < 4 * nch; i += 32) differ |= __ldg(xm + i) != __ldg(xc + i);
+  const bool same = !__any_sync(0xffffffffu, differ);
+  bool em, ec;
+  const double dm = ff_d2_exact(q, xm, nch, em), dc = ff_d2_exact(q, xc, nch, ec);
+  int o = slot_order(-dm, -dc, ff_bound(d));
+  if (em && ec) o = dm < dc || (dm == dc && m < c);
+  if (same) o = m < c;
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) *left = o < 0 ? -1 : *left - 1;
+  __syncwarp();
+  return o == 1;
 }
 
 // The list of one query, held by a warp: entry i in slot i % S of lane i / S,
@@ -733,7 +822,8 @@ struct RegList {
   __device__ __forceinline__ void add_near(unsigned kc, unsigned c, const SearchArgs& a, const uint8_t* q, float E2,
                                            float A2, int lane, unsigned pk, unsigned pi) {
     unsigned stay = 0;
-    bool have = false;
+    // a float query without budget: nothing more is added
+    bool have = DT == kF32 && reinterpret_cast<const int*>(q + a.row_bytes)[2 * kNbr + 2] < 0;
 #pragma unroll
     for (int j = 0; j < S; ++j) have |= (idv[j] & kIdMask) == c;
     if (__any_sync(kFull, have)) return;
@@ -744,17 +834,20 @@ struct RegList {
     } else {
       const float f = __uint_as_float(kc);
       const float lo = f * (1.0f - E2) - A2, hi = f * (1.0f + E2) + A2;
+      unsigned close = 0;  // this lane's entries to be settled
 #pragma unroll
       for (int j = 0; j < S; ++j) {
         const float fj = __uint_as_float(key[j]);
         stay |= fj < lo ? 1u << j : 0u;
-        unsigned b = __ballot_sync(kFull, !(fj < lo) && !(fj > hi) && idv[j] != kEmptyId);
-        while (b) {
-          const int l = __ffs(b) - 1;
-          b &= b - 1;
-          const unsigned m = __shfl_sync(kFull, idv[j], l) & kIdMask;
-          const bool first = precedes_fine(a.X, a.row_bytes, a.d, a.status, reinterpret_cast<const float*>(q), m, c);
-          if (first && lane == l) stay |= 1u << j;
+        close |= !(fj < lo) && !(fj > hi) && idv[j] != kEmptyId ? 1u << j : 0u;
+      }
+      while (const unsigned who = __ballot_sync(kFull, close != 0)) {
+        const unsigned low = close & (0u - close);
+        const unsigned m = first_of(close, who) & kIdMask;
+        const bool first = precedes_fine(a.X, a.row_bytes, a.d, reinterpret_cast<const float*>(q), m, c);
+        if (lane == __ffs(who) - 1) {
+          close ^= low;
+          stay |= first ? low : 0u;
         }
       }
     }
@@ -848,6 +941,7 @@ __global__ void __launch_bounds__(W == 1 ? kWarps * 32 : W * 32, W == 1 ? 8 : W 
     if (lane == 0) {
       M.cid[0] = start;
       M.cache[(start * 0x9E3779B1u) >> cshift] = start;
+      if (DT == kF32) M.ctl[2] = a.fine_budget;
     }
     __syncwarp();
     row_keys<DT, 1>(a.X, a.row_bytes, M.q, M.cid, M.ckey, 1, 0, 1, qn);
@@ -942,11 +1036,12 @@ __global__ void __launch_bounds__(W == 1 ? kWarps * 32 : W * 32, W == 1 ? 8 : W 
         else __syncthreads();
         // ---- those that may come before the L-th entry (an empty one: all of
         // them).  A distance that is no number, of a query that holds one, never
-        // displaces a member.
+        // displaces a member.  None once the query's budget is spent: it then soon
+        // runs out of members to expand.
         const unsigned kth = list.key_at((L - 1) / S, (L - 1) % S);
         const float last = __uint_as_float(kth) * (1.0f + E2) + A2;
         auto enters = [&](int i) {
-          if (i >= nf) return false;
+          if (i >= nf || (DT == kF32 && M.ctl[2] < 0)) return false;
           if constexpr (DT == kU8) return M.ckey[i] <= kth;
           else return __uint_as_float(M.ckey[i]) <= last || kth == 0x7f800000u;
         };
@@ -968,10 +1063,13 @@ __global__ void __launch_bounds__(W == 1 ? kWarps * 32 : W * 32, W == 1 ? 8 : W 
     }
     if (a.visited_cnt && lane == 0) a.visited_cnt[qi] = int32_t(iters < INT32_MAX ? iters : INT32_MAX);
     // ---- the k closest members
+    const bool redo = DT == kF32 && M.ctl[2] < 0;  // given up for search_list_kernel
 #pragma unroll
     for (int j = 0; j < S; ++j) {
       const int i = lane * S + j;
-      if (i < a.k) {
+      if (redo) {
+        if (i == 0) a.out_ids[int64_t(qi) * a.k] = kSearchRedo;
+      } else if (i < a.k) {
         const bool have = list.idv[j] != kEmptyId;
         const int64_t at = int64_t(qi) * a.k + i;
         a.out_ids[at] = have ? int32_t(list.idv[j] & kIdMask) : -1;
@@ -1023,7 +1121,7 @@ using SearchKernel = void (*)(SearchArgs);
 // warp or a team per query, and the list in shared memory.
 template <int DT>
 SearchKernel search_kernel_of(bool reg, int slots, int warps) {
-  if (!reg) return search_list_kernel<DT>;
+  if (!reg) return search_list_kernel<DT, false>;
   if (warps == kTeam) return slots <= 4 ? search_reg_kernel<DT, 4, kTeam> : search_reg_kernel<DT, 8, kTeam>;
   if (warps == kSmallTeam) return slots <= 4 ? search_reg_kernel<DT, 4, kSmallTeam> : search_reg_kernel<DT, 8, kSmallTeam>;
   return slots <= 4 ? search_reg_kernel<DT, 4, 1> : search_reg_kernel<DT, 8, 1>;
@@ -1047,6 +1145,8 @@ cudaError_t prepare_kernels() {
     SearchKernel k = (v & 1) ? search_kernel_of<kF32>(w > 0, slots, w) : search_kernel_of<kU8>(w > 0, slots, w);
     if ((err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return err;
   }
+  err = cudaFuncSetAttribute(search_list_kernel<kF32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (err != cudaSuccess) return err;
   done[dev] = true;
   return cudaSuccess;
 }
@@ -1104,7 +1204,7 @@ cudaError_t default_plan(const SearchForm& F, SearchPlan* plan) {
   return cudaSuccess;
 }
 
-cudaError_t launch_search(const SearchLaunch& L, cudaStream_t s) {
+cudaError_t launch_search(const SearchLaunch& L, cudaStream_t s, int* kernels) {
   SearchArgs a{};
   a.X = L.data.X;
   a.row_bytes = L.data.row_bytes;
@@ -1159,15 +1259,37 @@ cudaError_t launch_search(const SearchLaunch& L, cudaStream_t s) {
   } else if ((err = default_plan(F, &plan)) != cudaSuccess) {
     return err;
   }
-  int base_ctas = plan.ctas;
-  if (L.ctas_per_sm > 0) base_ctas = std::min(base_ctas, L.ctas_per_sm);
-  base_ctas = std::max(base_ctas, 1);
-  a.cache_bits = plan.bits;
-  const int64_t want = int64_t(L.num_sms) * base_ctas;
-  const int64_t need = (L.nq + F.queries - 1) / F.queries;
-  const int grid = int(std::max<int64_t>(1, std::min(want, need)));
-  F.kern<<<grid, F.threads, F.bytes(plan.bits), s>>>(a);
-  return cudaGetLastError();
+  // Float queries that search_reg_kernel gives up (none, where the other kernel's
+  // shared memory does not fit: long rows of few queries).
+  SearchForm R = F;
+  SearchPlan redo_plan;
+  bool redo = F.f32 && F.reg;
+  if (redo) {
+    R.kern = search_list_kernel<kF32, true>;
+    R.reg = false;
+    R.threads = kWarps * 32;
+    R.queries = kWarps;
+    err = default_plan(R, &redo_plan);
+    if (err != cudaSuccess && err != cudaErrorInvalidConfiguration) return err;
+    redo = err == cudaSuccess;
+  }
+  a.fine_budget = redo ? kFineBudget : INT_MAX;
+  if (L.pass == kSearchAgain && !redo) return cudaSuccess;
+  auto run = [&](const SearchForm& G, const SearchPlan& p) {
+    int base_ctas = p.ctas;
+    if (L.ctas_per_sm > 0) base_ctas = std::min(base_ctas, L.ctas_per_sm);
+    base_ctas = std::max(base_ctas, 1);
+    a.cache_bits = p.bits;
+    const int64_t want = int64_t(L.num_sms) * base_ctas;
+    const int64_t need = (L.nq + G.queries - 1) / G.queries;
+    const int grid = int(std::max<int64_t>(1, std::min(want, need)));
+    G.kern<<<grid, G.threads, G.bytes(p.bits), s>>>(a);
+    return cudaGetLastError();
+  };
+  const bool first = L.pass != kSearchAgain, again = redo && L.pass != kSearchOnce;
+  if (kernels) *kernels = int(first) + int(again);
+  err = first ? run(F, plan) : cudaSuccess;
+  return err == cudaSuccess && again ? run(R, redo_plan) : err;
 }
 
 cudaError_t launch_recall(const int32_t* found, int ld_found, const int32_t* truth, int ld_truth, int64_t nq, int k,
