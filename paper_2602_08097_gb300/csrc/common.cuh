@@ -181,6 +181,50 @@ __device__ __forceinline__ double ff_d2_warp(const float* q, const float* __rest
   return __dadd_rn(double(sh), double(sl));
 }
 
+// ff_d2_warp by a whole warp, and whether it is exact and equals the binary64 one: no difference, square or
+// sum has rounded in single precision, and the total is at most 2^28 times the least
+// square.  Every square is then a multiple of some power of two g > least 2^-24,
+// so that every partial sum in index order is below 2^52 g and binary64 never rounds
+// either.  (Whole numbers of moderate size, so that their many ties cost no more.)
+__device__ __forceinline__ double ff_d2_exact(const float* q, const float* __restrict__ x, int nch, bool& exact) {
+  const float4* pq = reinterpret_cast<const float4*>(q);
+  const float4* px = reinterpret_cast<const float4*>(x);
+  float sh = 0.f, sl = 0.f, lost = 0.f, least = __int_as_float(0x7f800000);
+  auto step = [&](float a, float b) {
+    const float th = __fsub_rn(a, b);
+    const float bv = __fsub_rn(th, a);
+    const float tl = __fadd_rn(__fsub_rn(a, __fsub_rn(th, bv)), __fsub_rn(__fsub_rn(0.f, b), bv));
+    const float ph = __fmul_rn(th, th), s1 = __fadd_rn(sh, ph), b1 = __fsub_rn(s1, sh);
+    const float e = __fadd_rn(__fsub_rn(sh, __fsub_rn(s1, b1)), __fsub_rn(ph, b1));
+    lost += fabsf(tl) + fabsf(__fmaf_rn(th, th, -ph)) + fabsf(e);
+    least = th != 0.f ? fminf(least, ph) : least;
+    ff_step(a, b, sh, sl);
+  };
+#pragma unroll 1
+  for (int c = threadIdx.x & 31; c < nch; c += 32) {
+    const float4 a = pq[c], b = __ldg(px + c);
+    step(a.x, b.x);
+    step(a.y, b.y);
+    step(a.z, b.z);
+    step(a.w, b.w);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float oh = __shfl_xor_sync(0xffffffffu, sh, o), ol = __shfl_xor_sync(0xffffffffu, sl, o);
+    const float s1 = __fadd_rn(sh, oh);
+    const float bv = __fsub_rn(s1, sh);
+    const float e = __fadd_rn(__fsub_rn(sh, __fsub_rn(s1, bv)), __fsub_rn(oh, bv));
+    const float l1 = __fadd_rn(__fadd_rn(sl, ol), e);
+    lost += fabsf(e);
+    sh = __fadd_rn(s1, l1);
+    sl = __fsub_rn(l1, __fsub_rn(sh, s1));
+  }
+  least = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(least)));
+  // squares that may have underflowed are not looked into
+  exact = __all_sync(0xffffffffu, lost == 0.f) && least >= 1.0e-30f && sh <= 268435456.f * least;
+  return __dadd_rn(double(sh), double(sl));
+}
+
 // Cached distance slots of float entries: NaN = not computed yet, sign bit
 // set = a float-float value (its magnitude), else the canonical binary64 one.
 // Order of two slots when their intervals allow it: 1 = a first, 0 = b first,

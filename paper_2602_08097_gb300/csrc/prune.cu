@@ -166,6 +166,27 @@ __device__ __forceinline__ typename Acc<DT>::T row_d2_any(const uint8_t* a, cons
 // canonical reading computes them.  `key64_v` caches d2(p, v) for column v as
 // the search's slots do: NaN, a float-float value (sign bit set) or the
 // binary64 value.  Every writer of a slot stores a valid value of its kind.
+// recheck_tests: the tests that found alphas u0 .. u1 - 1 to remove and u1, if any, not.
+__device__ __forceinline__ int recheck_tests(int u0, int u1, int TA) { return u1 - u0 + (u1 < TA ? 1 : 0); }
+// slot_dominates: the decision on two such slots, 1, 0 or -1 (open).
+__device__ __forceinline__ int slot_dominates(double A2, double fa, double sb, const FFBound& B) {
+  double la, ha, lb, hb;
+  slot_interval(fa, B, &la, &ha);
+  slot_interval(sb, B, &lb, &hb);
+  // rounding is monotone: fl(A2 d2a) <= fl(A2 ha) and fl(1e6 lb) <= fl(1e6 d2b)
+  if (__dmul_rn(A2, ha) <= __dmul_rn(1.0e6, lb)) return 1;
+  return __dmul_rn(A2, la) > __dmul_rn(1.0e6, hb) ? 0 : -1;
+}
+// The binary64 value of slot *key64_v.
+__device__ __forceinline__ double slot_canon(const float* xp, const float* xv, int d, double* key64_v) {
+  double d2b = *key64_v;
+  if (signbit(d2b) || isnan(d2b)) {
+    d2b = canon_d2_f32(xp, xv, d);
+    *key64_v = d2b;
+  }
+  return d2b;
+}
+
 __device__ __forceinline__ bool fine_dominates(const PruneArgs& a, int32_t u, int32_t v, int32_t p,
                                                double* key64_v, double A2) {
   const float* X = reinterpret_cast<const float*>(a.X);
@@ -176,52 +197,67 @@ __device__ __forceinline__ bool fine_dominates(const PruneArgs& a, int32_t u, in
     sb = -ff_d2(X + int64_t(p) * stride, xv, a.row_bytes);
     *key64_v = sb;
   }
-  const double fa = -ff_d2(X + int64_t(u) * stride, xv, a.row_bytes);
-  const FFBound B = ff_bound(a.d);
-  double la, ha, lb, hb;
-  slot_interval(fa, B, &la, &ha);
-  slot_interval(sb, B, &lb, &hb);
-  // rounding is monotone: fl(A2 d2a) <= fl(A2 ha) and fl(1e6 lb) <= fl(1e6 d2b)
-  if (__dmul_rn(A2, ha) <= __dmul_rn(1.0e6, lb)) return true;
-  if (__dmul_rn(A2, la) > __dmul_rn(1.0e6, hb)) return false;
+  const int o = slot_dominates(A2, -ff_d2(X + int64_t(u) * stride, xv, a.row_bytes), sb, ff_bound(a.d));
+  if (o >= 0) return o == 1;
   const double d2a = canon_d2_f32(X + int64_t(u) * stride, xv, a.d);
-  double d2b = sb;
-  if (signbit(d2b)) {
-    d2b = canon_d2_f32(X + int64_t(p) * stride, xv, a.d);
-    *key64_v = d2b;
-  }
   atomicAdd(&a.status->fp64_decisions, 1ull);
-  return canon_dominates(A2, d2a, d2b);
+  return canon_dominates(A2, d2a, slot_canon(X + int64_t(p) * stride, xv, a.d, key64_v));
 }
 
-// fine_dominates by a whole warp (the same arguments in every lane).
-__device__ __noinline__ bool fine_dominates_warp(const PruneArgs& a, int32_t u, int32_t v, int32_t p, double* key64_v,
-                                                 double A2) {
+// Up to 32 open pairs of the float decision pass, one per lane (`mine`): point u
+// against column v of pivot p, whose single-precision distance d2a left the alphas
+// from u1 on open.  Returns the first alpha that keeps the column (removal is
+// monotone in alpha).  float-float distances by the whole warp, a pair at a time, and
+// where they are exact they are the binary64 ones; what is open after that in binary64
+// by the lanes side by side: a binary64 sum's time is its chain of additions,
+// whatever the number of lanes that add.  One pair after the other in binary64, lists
+// of up to 64 over 20,000 x 96 zeros and ones took 114 ms and over rows 50 times over
+// 21.9; this way 6.4 and 3.4.
+__device__ __noinline__ int fine_prefix(const PruneArgs& a, bool mine, int32_t u, int32_t v, int32_t p, double* key64_v,
+                                        float d2a, float key, int u1, float E_rel, float E_abs) {
   const float* X = reinterpret_cast<const float*>(a.X);
   const int64_t stride = a.row_bytes / 4;
-  const int nch = int(a.row_bytes / 16);
-  const float* xv = X + int64_t(v) * stride;
-  double sb = *key64_v;
-  __syncwarp();
-  if (isnan(sb)) {
-    sb = -ff_d2_warp(X + int64_t(p) * stride, xv, nch);
-    *key64_v = sb;
-  }
-  const double fa = -ff_d2_warp(X + int64_t(u) * stride, xv, nch);
+  const int nch = int(a.row_bytes / 16), lane = threadIdx.x & 31;
   const FFBound B = ff_bound(a.d);
-  double la, ha, lb, hb;
-  slot_interval(fa, B, &la, &ha);
-  slot_interval(sb, B, &lb, &hb);
-  if (__dmul_rn(A2, ha) <= __dmul_rn(1.0e6, lb)) return true;
-  if (__dmul_rn(A2, la) > __dmul_rn(1.0e6, hb)) return false;
-  const double d2a = canon_d2_f32(X + int64_t(u) * stride, xv, a.d);
-  double d2b = sb;
-  if (signbit(d2b)) {
-    d2b = canon_d2_f32(X + int64_t(p) * stride, xv, a.d);
-    *key64_v = d2b;
+  double fa = 0.0;
+  for (unsigned todo = __ballot_sync(0xffffffffu, mine); todo; todo &= todo - 1) {
+    const int l = __ffs(int(todo)) - 1;
+    const float* xu = X + int64_t(__shfl_sync(0xffffffffu, u, l)) * stride;
+    const float* xv = X + int64_t(__shfl_sync(0xffffffffu, v, l)) * stride;
+    const float* xp = X + int64_t(__shfl_sync(0xffffffffu, p, l)) * stride;
+    bool exact;
+    const double f = ff_d2_exact(xu, xv, nch, exact);
+    if (lane == l) fa = exact ? f : -f;
+    if (__any_sync(0xffffffffu, lane == l && isnan(*key64_v))) {
+      const double g = ff_d2_exact(xp, xv, nch, exact);
+      if (lane == l) *key64_v = exact ? g : -g;
+      __syncwarp();
+    }
   }
-  if ((threadIdx.x & 31) == 0) atomicAdd(&a.status->fp64_decisions, 1ull);
-  return canon_dominates(A2, d2a, d2b);
+  bool open = false;
+  auto A2 = [&](int t) { return int64_t(a.Ad[t]) * a.Ad[t]; };
+  if (mine) {
+    const double sb = *key64_v;
+    for (; u1 < a.TA; ++u1) {
+      int o = sure_dominates(float(A2(u1)), d2a, key, E_rel, E_abs);
+      if (o < 0) o = slot_dominates(double(A2(u1)), fa, sb, B);
+      open = o < 0;
+      if (o != 1) break;
+    }
+  }
+  if (__any_sync(0xffffffffu, open)) {
+    __syncwarp();
+    if (open) {
+      const float* xv = X + int64_t(v) * stride;
+      const double c2a = signbit(fa) ? canon_d2_f32(X + int64_t(u) * stride, xv, a.d) : fa;
+      const double c2b = slot_canon(X + int64_t(p) * stride, xv, a.d, key64_v);
+      const int first = u1;
+      while (u1 < a.TA && canon_dominates(double(A2(u1)), c2a, c2b)) ++u1;
+      atomicAdd(&a.status->fp64_decisions, static_cast<unsigned long long>(recheck_tests(first, u1, a.TA)));
+    }
+    __syncwarp();
+  }
+  return u1;
 }
 
 // An open pair of the float decision pass: row `t` against column `c` for the
@@ -231,12 +267,12 @@ __device__ __noinline__ bool fine_dominates_warp(const PruneArgs& a, int32_t u, 
 // binary64.  Removal is monotone in alpha (removed at a larger alpha means
 // removed at every smaller one), so the alphas that remove the column are a
 // prefix: returns u1, the first that keeps it (TA if none), after
-// recheck_tests(u0, u1, TA) tests.  Inlined into the queue's resolution
-// loop; the in-place use below is out of line, since inlining it there let
-// the mask loop unroll fully and the larger code ran slower.
-__device__ __forceinline__ int recheck_prefix(const PruneArgs& a, const int32_t* ids, const float* key,
-                                              double* key64, int t, int c, int u0, int TA, int p, float E_rel,
-                                              float E_abs) {
+// recheck_tests(u0, u1, TA) tests.  For the pairs decided in place when the queue
+// is full; out of line, since inlining it there let the mask loop unroll fully and
+// the larger code ran slower.
+__device__ __noinline__ int recheck_prefix_cold(const PruneArgs& a, const int32_t* ids, const float* key,
+                                                double* key64, int t, int c, int u0, int TA, int p, float E_rel,
+                                                float E_abs) {
   const float d2a = row_d2<kF32>(a.X + int64_t(ids[t]) * a.row_bytes, a.X + int64_t(ids[c]) * a.row_bytes,
                                  a.row_bytes);
   int u = u0;
@@ -246,14 +282,6 @@ __device__ __forceinline__ int recheck_prefix(const PruneArgs& a, const int32_t*
     if (!(rr >= 0 ? (rr == 1) : fine_dominates(a, ids[t], ids[c], p, &key64[c], double(A2)))) break;
   }
   return u;
-}
-__device__ __forceinline__ int recheck_tests(int u0, int u1, int TA) { return u1 - u0 + (u1 < TA ? 1 : 0); }
-
-// The same, out of line, for the rare pairs decided in place when the queue is full.
-__device__ __noinline__ int recheck_prefix_cold(const PruneArgs& a, const int32_t* ids, const float* key,
-                                                double* key64, int t, int c, int u0, int TA, int p, float E_rel,
-                                                float E_abs) {
-  return recheck_prefix(a, ids, key, key64, t, c, u0, TA, p, E_rel, E_abs);
 }
 
 // ---------------------------------------------------------------------------
@@ -1505,54 +1533,66 @@ __global__ void __launch_bounds__(128 * H + 32, 2) prune_f32_kernel(PruneArgs a)
       }
       if (!any) break;
       {
-        // The slot's open pairs, four at a time: the warp reads the rows together
-        // (a lane per 16-byte chunk; few enough roundings for slice_rel_bound), and
-        // each alpha that removes the column sets its bit in the row's mask.  One
-        // pair per lane, its two rows read chunk by chunk, took longer than all the
-        // rest of a slot on long rows.
+        // The slot's open pairs, 32 at a time, one per lane.  Their single-precision
+        // distances first, four pairs at a time: the warp reads the rows together (a
+        // lane per 16-byte chunk; few enough roundings for slice_rel_bound).  One pair
+        // per lane, its two rows read chunk by chunk, took longer than all the rest of
+        // a slot on long rows.  Each alpha that removes the column sets its bit in the
+        // row's mask.
         const int nq = min(rq_count[s], L::rq_cap), nch = int(a.row_bytes / 16);
-        for (int i0 = 0; i0 < nq; i0 += 4) {
-          const uint4 *pu[4], *pv[4];
+        for (int i0 = 0; i0 < nq; i0 += 32) {
+          const int nb = min(32, nq - i0);
+          float d2a = 0.f;  // of the lane's own pair
+          for (int j0 = 0; j0 < nb; j0 += 4) {
+            const uint4 *pu[4], *pv[4];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const uint32_t e = rq[s * L::rq_cap + min(i0 + j, nq - 1)];
-            const int tr = int(e >> 16), c = int((e >> 5) & 0x7ffu);
-            const int32_t* idq = reinterpret_cast<const int32_t*>(slot_base(s, tr / MAXM) + L::s_ids);
-            pu[j] = reinterpret_cast<const uint4*>(a.X + int64_t(idq[tr % MAXM]) * a.row_bytes);
-            pv[j] = reinterpret_cast<const uint4*>(a.X + int64_t(idq[c]) * a.row_bytes);
-          }
-          float d2a[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 2
-          for (int c = lane; c < nch; c += 32) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) d2a[j] = Acc<kF32>::step4(__ldg(pu[j] + c), __ldg(pv[j] + c), d2a[j]);
-          }
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) d2a[j] += __shfl_xor_sync(0xffffffffu, d2a[j], o);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            if (i0 + j >= nq) break;
-            const uint32_t e = rq[s * L::rq_cap + i0 + j];
-            const int tr = int(e >> 16), c = int((e >> 5) & 0x7ffu), u0 = int(e & 31u);
-            const int gq = tr / MAXM, tq = tr % MAXM;
-            unsigned char* sbq = slot_base(s, gq);
-            const int32_t* idq = reinterpret_cast<const int32_t*>(sbq + L::s_ids);
-            const float kc = reinterpret_cast<const float*>(sbq + L::s_key)[c];
-            double* k64 = reinterpret_cast<double*>(sbq + L::s_key64) + c;
-            int u1 = u0;  // removal is monotone in alpha (recheck_prefix)
-            for (; u1 < a.TA; ++u1) {
-              const int64_t A2 = int64_t(a.Ad[u1]) * a.Ad[u1];
-              const int rr = sure_dominates(float(A2), d2a[j], kc, E_rel, E_abs);
-              if (!(rr >= 0 ? (rr == 1)
-                            : fine_dominates_warp(a, idq[tq], idq[c], point_of_row(a, misc[s * 2 + gq]), k64, double(A2))))
-                break;
+            for (int j = 0; j < 4; ++j) {
+              const uint32_t e = rq[s * L::rq_cap + i0 + min(j0 + j, nb - 1)];
+              const int tr = int(e >> 16), c = int((e >> 5) & 0x7ffu);
+              const int32_t* idq = reinterpret_cast<const int32_t*>(slot_base(s, tr / MAXM) + L::s_ids);
+              pu[j] = reinterpret_cast<const uint4*>(a.X + int64_t(idq[tr % MAXM]) * a.row_bytes);
+              pv[j] = reinterpret_cast<const uint4*>(a.X + int64_t(idq[c]) * a.row_bytes);
             }
-            if (lane == 0) n_rechecks += recheck_tests(u0, u1, a.TA);
-            unsigned long long* mrow = reinterpret_cast<unsigned long long*>(sbq + L::s_masks) + tq * MW + (c >> 6);
-            if (lane >= u0 && lane < u1) atomicOr(mrow + lane * MAXM * MW, 1ull << (c & 63));
+            float f[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+            for (int c = lane; c < nch; c += 32) {
+#pragma unroll
+              for (int j = 0; j < 4; ++j) f[j] = Acc<kF32>::step4(__ldg(pu[j] + c), __ldg(pv[j] + c), f[j]);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) f[j] += __shfl_xor_sync(0xffffffffu, f[j], o);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) d2a = lane == j0 + j ? f[j] : d2a;
           }
+          const uint32_t e = rq[s * L::rq_cap + i0 + min(lane, nb - 1)];
+          const int tr = int(e >> 16), c = int((e >> 5) & 0x7ffu), u0 = int(e & 31u);
+          const int gq = tr / MAXM, tq = tr % MAXM;
+          unsigned char* sbq = slot_base(s, gq);
+          const int32_t* idq = reinterpret_cast<const int32_t*>(sbq + L::s_ids);
+          const float kc = reinterpret_cast<const float*>(sbq + L::s_key)[c];
+          int u1 = u0;  // removal is monotone in alpha
+          bool open = false;
+          while (lane < nb && u1 < a.TA) {
+            const int64_t A2 = int64_t(a.Ad[u1]) * a.Ad[u1];
+            const int rr = sure_dominates(float(A2), d2a, kc, E_rel, E_abs);
+            open = rr < 0;
+            if (rr != 1) break;
+            ++u1;
+          }
+          if (__any_sync(0xffffffffu, open)) {
+            const int32_t ppt = point_of_row(a, misc[s * 2 + gq]);
+            const int f1 = fine_prefix(a, open, idq[tq], idq[c], ppt, reinterpret_cast<double*>(sbq + L::s_key64) + c,
+                                       d2a, kc, u1, E_rel, E_abs);
+            u1 = open ? f1 : u1;
+          }
+          if (lane < nb) {
+            n_rechecks += recheck_tests(u0, u1, a.TA);
+            unsigned long long* mrow = reinterpret_cast<unsigned long long*>(sbq + L::s_masks) + tq * MW + (c >> 6);
+            for (int u = u0; u < u1; ++u) atomicOr(mrow + u * MAXM * MW, 1ull << (c & 63));
+          }
+          __syncwarp();
         }
         __syncwarp();
       }
