@@ -187,7 +187,16 @@ __device__ __forceinline__ double slot_canon(const float* xp, const float* xv, i
   return d2b;
 }
 
-__device__ __forceinline__ bool fine_dominates(const PruneArgs& a, int32_t u, int32_t v, int32_t p,
+// Two float rows of equal values.
+__device__ __forceinline__ bool same_row(const float* a, const float* b, int64_t row_bytes) {
+  for (int64_t i = 0; i < row_bytes / 16; ++i) {
+    const float4 x = __ldg(reinterpret_cast<const float4*>(a) + i), y = __ldg(reinterpret_cast<const float4*>(b) + i);
+    if (x.x != y.x || x.y != y.y || x.z != y.z || x.w != y.w) return false;
+  }
+  return true;
+}
+
+__device__ __noinline__ bool fine_dominates(const PruneArgs& a, int32_t u, int32_t v, int32_t p,
                                                double* key64_v, double A2) {
   const float* X = reinterpret_cast<const float*>(a.X);
   const int64_t stride = a.row_bytes / 4;
@@ -199,6 +208,8 @@ __device__ __forceinline__ bool fine_dominates(const PruneArgs& a, int32_t u, in
   }
   const int o = slot_dominates(A2, -ff_d2(X + int64_t(u) * stride, xv, a.row_bytes), sb, ff_bound(a.d));
   if (o >= 0) return o == 1;
+  // a copy of the pivot: the same distance on both sides
+  if (A2 <= 1.0e6 && same_row(X + int64_t(u) * stride, X + int64_t(p) * stride, a.row_bytes)) return true;
   const double d2a = canon_d2_f32(X + int64_t(u) * stride, xv, a.d);
   atomicAdd(&a.status->fp64_decisions, 1ull);
   return canon_dominates(A2, d2a, slot_canon(X + int64_t(p) * stride, xv, a.d, key64_v));
@@ -1664,7 +1675,7 @@ struct GenericLayout {
   // ids, the order, the keys, the kept ranks, near-tie links; per batch: one mask
   // per candidate, the dominated ones; misc
   __host__ __device__ static size_t masks(int M2) { return size_t(M2) * 23 + (size_t(M2) & 3); }
-  __host__ __device__ static size_t rows(int M2) { return (masks(M2) + (kGenBatch + 2 + 16) * 4 + 127) & ~size_t(127); }
+  __host__ __device__ static size_t rows(int M2) { return (masks(M2) + (kGenBatch + 4 + 16) * 4 + 127) & ~size_t(127); }
 };
 
 // d2 of row `b` from rows a0 and a1 (any of them in shared memory, plain loads),
@@ -1690,8 +1701,27 @@ __device__ __forceinline__ void row_d2_two(const uint8_t* a0, const uint8_t* a1,
   }
 }
 
+// The general prune's open candidates (bits of `todo`; this lane's is point v at
+// distance key from the pivot) against the points kept so far, a warp every eighth:
+// bit `lane` of *found if one removes it.  Out of line, since it is rare.
+__device__ __noinline__ void settle_open(const PruneArgs& a, unsigned todo, int kept, const uint16_t* kept_at,
+                                         const int32_t* perm, const int32_t* ids, int32_t v, int32_t p, float key,
+                                         double* key64_v, int64_t A2, unsigned* found) {
+  const int lane = threadIdx.x & 31;
+  const float E = rel_bound(a.d), Eabs = abs_bound(a.d);
+  const uint8_t* xv = a.X + int64_t(v) * a.row_bytes;
+#pragma unroll 1
+  for (int k = int(threadIdx.x >> 5); k < kept; k += kGenWarps) {
+    if (!(((todo & ~*static_cast<volatile unsigned*>(found)) >> lane) & 1u)) continue;
+    const int32_t u = ids[perm[kept_at[k]]];
+    int r = sure_dominates(float(A2), row_d2<kF32>(a.X + int64_t(u) * a.row_bytes, xv, a.row_bytes), key, E, Eabs);
+    if (r < 0) r = fine_dominates(a, u, v, p, key64_v, double(A2));
+    if (r == 1) atomicOr(found, 1u << lane);
+  }
+}
+
 template <int DT>
-__global__ void __launch_bounds__(kGenThreads) prune_generic_kernel(PruneArgs a, int M2, int stage_rows) {
+__global__ void __launch_bounds__(kGenThreads, 4) prune_generic_kernel(PruneArgs a, int M2, int stage_rows) {
   using AT = typename Acc<DT>::T;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned long long* skey = reinterpret_cast<unsigned long long*>(smem_raw);
@@ -1702,8 +1732,8 @@ __global__ void __launch_bounds__(kGenThreads) prune_generic_kernel(PruneArgs a,
   uint16_t* kept_at = reinterpret_cast<uint16_t*>(smem_raw + size_t(M2) * 20);  // ranks of the kept points
   unsigned char* lnk = smem_raw + size_t(M2) * 22;
   unsigned* dmask = reinterpret_cast<unsigned*>(smem_raw + GenericLayout::masks(M2));  // [kGenBatch]
-  unsigned* dword = dmask + kGenBatch;                                                 // [2] dominated by kept points
-  int* misc = reinterpret_cast<int*>(dword + 2);
+  unsigned* dword = dmask + kGenBatch;  // [3] removed by kept points: for sure; open against some; found after all
+  int* misc = reinterpret_cast<int*>(dword + 4);
   unsigned char* stage = smem_raw + GenericLayout::rows(M2);
   const int64_t stride = a.row_bytes + 16;  // of a staged row
   // staged rows: one or two batches, the rest for kept points
@@ -1847,7 +1877,7 @@ __global__ void __launch_bounds__(kGenThreads) prune_generic_kernel(PruneArgs a,
       for (int i0 = 0, round = 0; i0 < m && kept < R; i0 += kGenBatch, ++round) {
         const int nb = min(kGenBatch, m - i0), b = nbuf == 2 ? round & 1 : 0;
         if (nbuf > 0) cp_async_wait<0>();
-        if (t == 0) *dword = 0u;
+        if (t < 3) dword[t] = 0u;
         __syncthreads();  // this batch's rows; the kept rows; every reader of the other buffer is done
         if (nbuf == 2 && i0 + kGenBatch < m) load_batch(i0 + kGenBatch, b ^ 1);
         auto batch_row = [&](int c) -> const uint8_t* {
@@ -1861,40 +1891,75 @@ __global__ void __launch_bounds__(kGenThreads) prune_generic_kernel(PruneArgs a,
         const int pc = perm[i0 + c];
         const AT kc = key[pc];
         const uint8_t* xc = batch_row(c);
-        // whether point u (stored position pu) removes it
-        auto removes = [&](int pu, AT d2a) -> bool {
-          if constexpr (DT == kU8) {
+        // whether a point at distance d2a removes it: 1, 0 or, for floats, -1 (open)
+        auto sure = [&](AT d2a) -> int {
+          if constexpr (DT == kU8)
             return static_cast<unsigned long long>(A2) * d2a <= 1000000ull * static_cast<unsigned long long>(kc);
-          } else {
-            const int r = sure_dominates(float(A2), d2a, kc, E, Eabs);
-            return r >= 0 ? r == 1 : fine_dominates(a, ids[pu], ids[pc], ppt, &key64[pc], double(A2));
-          }
+          else
+            return sure_dominates(float(A2), d2a, kc, E, Eabs);
         };
-        // ---- the batch against the points kept so far
-        bool dom = lane >= nb;
+        // the same of point u (stored position pu), settled
+        auto removes = [&](int pu, AT d2a) -> bool {
+          const int r = sure(d2a);
+          if constexpr (DT == kF32)
+            if (r < 0) return fine_dominates(a, ids[pu], ids[pc], ppt, &key64[pc], double(A2));
+          return r == 1;
+        };
+        // ---- the batch against the points kept so far.  What is open is left until
+        // every warp has looked: most of it is surely removed by another point
+        bool dom = lane >= nb, open = false;
         for (int k = warp; k < kept && !__all_sync(0xffffffffu, dom); k += 2 * kGenWarps) {
           const int k1 = k + kGenWarps < kept ? k + kGenWarps : k;
           if (!dom) {
             AT d0, d1;
             row_d2_two<DT>(kept_row(k), kept_row(k1), xc, a.row_bytes, d0, d1);
-            dom = removes(perm[kept_at[k]], d0) || removes(perm[kept_at[k1]], d1);
+            const int r0 = sure(d0), r1 = sure(d1);
+            dom = r0 == 1 || r1 == 1;
+            open |= r0 < 0 || r1 < 0;
           }
         }
-        const unsigned db = __ballot_sync(0xffffffffu, dom);
+        const unsigned db = __ballot_sync(0xffffffffu, dom), ob = __ballot_sync(0xffffffffu, open);
         if (lane == 0 && db) atomicOr(dword, db);
+        if (DT == kF32 && lane == 0 && ob) atomicOr(dword + 1, ob);
         __syncthreads();
-        const unsigned alive = ~*dword;
-        // ---- the survivors against one another
-        int at = 0;
+        unsigned alive = ~dword[0];
+        if constexpr (DT == kF32) {
+          if (const unsigned todo = alive & dword[1]) {  // the same in every thread
+            settle_open(a, todo, kept, kept_at, perm, ids, ids[pc], ppt, kc, &key64[pc], A2, dword + 2);
+            __syncthreads();
+            alive &= ~dword[2];
+          }
+        }
+        // ---- the survivors against one another, two of a warp's at a time
+        int at = 0, held = -1;
+        auto against = [&](int u, int u2) {  // u < u2; u2 < 0: u alone
+          const bool live = (alive >> lane) & 1u;
+          bool rm = false, rm2 = false;
+          if (live && lane > u) {
+            if (u2 < 0) {
+              rm = removes(perm[i0 + u], row_d2_any<DT>(batch_row(u), xc, a.row_bytes));
+            } else {
+              AT d0, d1;
+              row_d2_two<DT>(batch_row(u), batch_row(u2), xc, a.row_bytes, d0, d1);
+              rm = removes(perm[i0 + u], d0);
+              rm2 = lane > u2 && removes(perm[i0 + u2], d1);
+            }
+          }
+          const unsigned rb = __ballot_sync(0xffffffffu, rm), rb2 = __ballot_sync(0xffffffffu, rm2);
+          if (lane == 0) dmask[u] = rb;
+          if (lane == 0 && u2 >= 0) dmask[u2] = rb2;
+        };
         for (unsigned mm = alive; mm; mm &= mm - 1, ++at) {
           if (at % kGenWarps != warp) continue;
           const int u = __ffs(int(mm)) - 1;
-          bool rm = false;
-          if (lane > u && ((alive >> lane) & 1u))
-            rm = removes(perm[i0 + u], row_d2_any<DT>(batch_row(u), xc, a.row_bytes));
-          const unsigned rb = __ballot_sync(0xffffffffu, rm);
-          if (lane == 0) dmask[u] = rb;
+          if (held < 0) {
+            held = u;
+          } else {
+            against(held, u);
+            held = -1;
+          }
         }
+        if (held >= 0) against(held, -1);
         __syncthreads();
         // ---- the batch's greedy scan (every thread; the masks are the same for all)
         unsigned keep = 0;
@@ -2227,6 +2292,12 @@ static cudaError_t run_generic(const PruneArgs& args, int num_sms, int64_t host_
   const size_t half = size_t(113) * 1024, whole = size_t(227) * 1024;
   size_t rows = std::min<size_t>(2 * kGenBatch + 64, head < half ? (half - head) / row : 0);
   if (rows < 2 * kGenBatch + 32) rows = std::min<size_t>(2 * kGenBatch + 64, head < whole ? (whole - head) / row : 0);
+  // Many nodes on long rows: a batch and as many kept points, where more would leave
+  // fewer than the four CTAs on an SM that the registers allow (2,000 lists of 150 to
+  // 300 over 128 floats, one target: 128 rows 0.61 ms, 64 0.50; 10,000 of 40 to 64 over
+  // 384 uint8: 0.51, 0.47; over 17 floats all fit, and 64 rows would cost 7%).
+  if (host_count > 2 * int64_t(num_sms) && head + rows * row > size_t(227) * 1024 / 4 - 1024)
+    rows = std::min<size_t>(rows, 2 * kGenBatch);
   if (rows < size_t(kGenBatch)) rows = 0;
   const size_t bytes = head + rows * row;
   auto kern = prune_generic_kernel<DT>;

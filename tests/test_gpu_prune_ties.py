@@ -54,8 +54,8 @@ def test_rows_are_the_oracles(ctx, kind, d, lo, hi):
     rp.rp_graph_free(ctx, g)
 
 
-@pytest.mark.parametrize("kind", ["bits", "rows"])
-@pytest.mark.parametrize("lo,hi,times", [(40, 64, 40), (70, 128, 60)])
+@pytest.mark.parametrize("kind,lo,hi,times", [("bits", 40, 64, 40), ("rows", 40, 64, 40), ("bits", 70, 128, 60),
+                                              ("rows", 70, 128, 60), ("bits", 150, 300, 9)])
 def test_time_stays_within_a_multiple(ctx, kind, lo, hi, times):
     ms = {}
     for k in (kind, "none"):
