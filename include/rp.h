@@ -237,6 +237,9 @@ rp_status rp_graph_export(rp_ctx *ctx, rp_graph g, int64_t *row_ptr, int32_t *co
  *   dists: float[nq * k] squared distances (exact integers for RP_U8; for
  *     RP_F32 single precision, with orderings decided as in binary64), +inf
  *     where ids is -1.  dists may be NULL.
+ * With RP_MEM_DEVICE the call queues its work on the context's stream: the
+ * queries must stay as they are until that work is done (rows of a multiple of
+ * 128 bytes are read where they lie).  ids and dists may lie over the queries.
  * Errors: RP_ENOTFOUND, RP_EINVAL (nq < 0, k < 1, L < k, L > RP_MAX_L),
  *   RP_ENOMEM, RP_ECUDA.
  */

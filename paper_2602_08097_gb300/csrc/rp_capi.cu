@@ -773,19 +773,27 @@ rp_status search_impl(rp_ctx* c, const rp_graph* graphs, int32_t ngraphs, const 
   if (!queries || !ids) return fail(c, RP_EINVAL, "null argument");
   const Dataset& D = *Gs[0]->data;
   rp_status s;
-  const int64_t qbytes = nq * D.row_bytes;
+  // Device rows that already have the padded layout are read in place, unless the
+  // results go over them; a few host rows are padded into pinned memory and go up in
+  // one copy.
+  const size_t packed = size_t(D.d) * elem_size(D.dtype);
+  const int64_t row_area = nq * D.row_bytes;
+  auto over_queries = [&](const void* p) {
+    const auto q = reinterpret_cast<uintptr_t>(queries), o = reinterpret_cast<uintptr_t>(p);
+    return p && o < q + uintptr_t(row_area) && q < o + uintptr_t(nq * k * 4);
+  };
+  const bool in_place = mem_flags == RP_MEM_DEVICE && int64_t(packed) == D.row_bytes &&
+                        reinterpret_cast<uintptr_t>(queries) % 16 == 0 && !over_queries(ids) && !over_queries(dists);
+  const int64_t qbytes = in_place ? 0 : row_area;  // of qbuf
   const int64_t out_bytes = mem_flags == RP_MEM_HOST ? nq * k * 8 : 0;
   // per-query tables of a mixed launch: graph refs, then graph index and L per query
   const int64_t table_off = (qbytes + out_bytes + 255) / 256 * 256;
   const int64_t table_bytes = q_graph ? int64_t(ngraphs) * int64_t(sizeof(SearchGraph)) + 8 * nq + 16 : 0;
   if ((s = grow(c, &c->qbuf, &c->qbuf_bytes, table_off + table_bytes)) != RP_OK) return s;
-  // Device rows that already have the padded layout are read in place; a few
-  // host rows are padded into pinned memory and go up in one copy.
-  const size_t packed = size_t(D.d) * elem_size(D.dtype);
   const uint8_t* rows = c->qbuf;
   const bool small = mem_flags == RP_MEM_HOST && size_t(qbytes + out_bytes) <= kPinData;
   uint8_t* const pin_rows = c->pin + kPinHead;
-  if (mem_flags == RP_MEM_DEVICE && int64_t(packed) == D.row_bytes && reinterpret_cast<uintptr_t>(queries) % 16 == 0) {
+  if (in_place) {
     rows = static_cast<const uint8_t*>(queries);
   } else if (small) {
     for (int64_t i = 0; i < nq; ++i) {

@@ -79,3 +79,25 @@ def test_queries_that_hold_no_numbers_return(ctx, nq):
     ref, _, _ = oracle.greedy_search(X, row_ptr, col, 0, Q[2::3], 64, 10)
     assert np.array_equal(ids[2::3], ref)
     rp.rp_graph_free(ctx, g)
+
+
+@pytest.mark.parametrize("nq", [16, 20000])
+@pytest.mark.parametrize("dtype,d", [("u8", 128), ("f32", 32), ("f32", 24)])
+def test_results_may_lie_over_the_queries(ctx, dtype, d, nq):
+    # ids over the second half of the queries, distances over the first: the ids of
+    # the first queries lie over rows that are searched much later
+    torch = pytest.importorskip("torch")
+    X, Q = _data(dtype, d, 500, nq, 2, False)
+    row_ptr, col = datagen.random_graph(500, 5, 40, seed=3)
+    g = rp.rp_load_graph(ctx, X, row_ptr, col, start=0)
+    k = Q.nbytes // nq // 8
+    q = torch.from_numpy(Q).cuda()
+    ref, refd = rp.rp_search(ctx, g, q.clone(), 32, k)
+    rp.rp_sync(ctx)
+    words = q.view(torch.int32).flatten()
+    ids, dists = words[nq * k:].view(nq, k), words[:nq * k].view(torch.float32).view(nq, k)
+    torch.cuda.synchronize()
+    rp.rp_search(ctx, g, q, 32, k, ids=ids, dists=dists)
+    rp.rp_sync(ctx)
+    assert torch.equal(ids, ref) and torch.equal(dists, refd)
+    rp.rp_graph_free(ctx, g)
