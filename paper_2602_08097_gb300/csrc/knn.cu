@@ -416,10 +416,11 @@ __device__ __forceinline__ float tc_err(const KnnTcArgs& a, float nq, float sq, 
 }
 
 // tc_err as linear in np, for the scan's test: err <= (1 - f) np + c, since
-// 2 sq sp <= nq + np and 2 sp <= np / sq + sq (2 sp <= np + 1 where sq is 0).  Both
-// also carry 2^-21 of nq and np for the roundings of the test.
+// 2 sq sp <= nq + np and 2 sp <= np / s + s for any s > 0: sq, or 2^-20 for queries
+// so small that sub_abs / sq would count.  Both also carry 2^-21 of nq and np for the
+// roundings of the test.
 __device__ __forceinline__ void tc_err_linear(const KnnTcArgs& a, float nq, float& f, float& c) {
-  const float sq = sqrtf(nq), s = sq > 0.f ? sq : 1.f;
+  const float sq = sqrtf(nq), s = fmaxf(sq, 9.5367432e-07f);
   const float g = a.eps_ip * 1.001f + a.eps_n + 9.5367432e-07f;
   f = 1.f - (g + 0.5f * a.sub_abs / s) * 1.0002f;
   c = (g * nq + a.sub_abs * (sq + 0.5f * s)) * 1.0002f + 2e-30f;

@@ -58,6 +58,16 @@ def test_one_row_of_large_norm(ctx, at, times, k):
     _check(ctx, X, Q, k, min(row, 3000))
 
 
+@pytest.mark.parametrize("size", [0.0, 1e-12, 1e-9, 1e-6, 1e-3, 1e3])
+def test_queries_far_smaller_or_larger_than_the_points(ctx, size):
+    rng = np.random.default_rng(3)
+    X = rng.normal(size=(20000, 48)).astype(np.float32)
+    Q = (rng.normal(size=(200, 48)) * size).astype(np.float32)
+    if size > 1:  # all points lie alike from afar: few enough of them to be told apart
+        X = X[:300].copy()
+    _check(ctx, X, Q, 10, 0)
+
+
 @pytest.mark.parametrize("d,k", [(16, 10), (32, 100), (96, 128)])
 def test_norms_over_many_sizes(ctx, d, k):
     rng = np.random.default_rng(d)
