@@ -691,13 +691,6 @@ struct RegList {
     for (int i = 0; i < S; ++i) v |= i == j ? key[i] : 0u;
     return __shfl_sync(kFull, v, l);
   }
-  // The same for the point there.
-  __device__ __forceinline__ unsigned id_at(int l, int j) const {
-    unsigned v = 0;
-#pragma unroll
-    for (int i = 0; i < S; ++i) v |= i == j ? idv[i] : 0u;
-    return __shfl_sync(kFull, v, l) & kIdMask;
-  }
   // This lane's unexpanded entries before L, as bits.
   __device__ __forceinline__ unsigned open_bits() const {
     unsigned v = 0;
@@ -1010,14 +1003,6 @@ __global__ void __launch_bounds__(W == 1 ? kWarps * 32 : W * 32, W == 1 ? 8 : W 
 #pragma unroll 1
         for (int base = 0; base < nf; base += 32) {
           unsigned todo = __ballot_sync(full, enters(base + lane));
-          // at the L-th entry's distance only a smaller id comes before it
-          if constexpr (DT == kU8) {
-            const bool level = base + lane < nf && M.ckey[base + lane] == kth;
-            if (__any_sync(full, level)) {
-              const unsigned kth_id = list.id_at((L - 1) / S, (L - 1) % S);
-              todo &= ~__ballot_sync(full, level && M.cid[base + lane] >= kth_id);
-            }
-          }
           while (todo) {
             const int at = base + __ffs(todo) - 1;
             todo &= todo - 1;

@@ -85,20 +85,3 @@ def test_a_vamana_build_over_ties_matches_the_oracle(ctx):
     assert cut == ref_cut and np.array_equal(got[0], ref_rp) and np.array_equal(got[1], ref_col)
     rp.rp_graph_free(ctx, v)
     rp.rp_graph_free(ctx, g)
-
-
-def test_uint8_points_at_one_distance_take_no_longer_than_others(ctx):
-    rng = np.random.default_rng(8)
-    row_ptr, col = datagen.random_graph(5000, 20, 64, seed=4)
-    Q = rng.integers(0, 256, (2000, 64)).astype(np.uint8)
-    ms = {}
-    for kind in ("same", "random"):
-        X = rng.integers(0, 256, (5000, 64)).astype(np.uint8) * (kind == "random")
-        g = rp.rp_load_graph(ctx, X, row_ptr, col, start=3)
-        clean = rp.rp_graph_export(ctx, g)
-        for _ in range(3):
-            ids, _ = rp.rp_search(ctx, g, Q, 100, 50)
-            ms[kind] = min(ms.get(kind, np.inf), rp.rp_stats(ctx)["last_search_ms"])
-        assert np.array_equal(ids[:40], oracle.greedy_search(X, *clean, 3, Q[:40], 100, 50)[0])
-        rp.rp_graph_free(ctx, g)
-    assert ms["same"] < 1.6 * ms["random"], ms
