@@ -314,6 +314,9 @@ __device__ __forceinline__ bool entry_less(unsigned ka, unsigned ia, double* d64
 // the id cache does not hold get their distances, those that enter the list
 // are sorted by a bitonic network and merged in place.
 // REDO: any L, only the queries that hold kSearchRedo (spread over the grid's warps).
+// With a lane per row before and its rows shared by lanes now, 300 queries on 20,000
+// rows, L = 300 and 1,024: 96 floats 3.78 and 17.2 ms, now 3.21 and 13.5; 960 floats 20.8
+// and 126, 15.5 and 75.5; 128 uint8 1.46 and 6.28, 1.49 and 6.27.
 template <int DT, bool REDO>
 __global__ void __launch_bounds__(kWarps * 32, 8) search_list_kernel(SearchArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -651,7 +654,10 @@ __device__ __noinline__ bool precedes_fine(const uint8_t* Xb, int64_t row_bytes,
   // the end, and ptxas spills in the search's loop, 1.43 to 1.58 ms where it takes 0.95)
   bool differ = false;
 #pragma unroll 1
-  for (int i = threadIdx.x & 31; i < 4 * nch; i += 32) differ |= __ldg(xm + i) != __ldg(xc + i);
+  for (int i = threadIdx.x & 31; i < nch; i += 32) {
+    const float4 a = __ldg(reinterpret_cast<const float4*>(xm) + i), b = __ldg(reinterpret_cast<const float4*>(xc) + i);
+    differ |= a.x != b.x || a.y != b.y || a.z != b.z || a.w != b.w;
+  }
   const bool same = !__any_sync(0xffffffffu, differ);
   bool em, ec;
   const double dm = ff_d2_exact(q, xm, nch, em), dc = ff_d2_exact(q, xc, nch, ec);
@@ -825,11 +831,11 @@ struct RegList {
 // Measured, a list sorted in shared memory (32 neighbours at a time, one lane per
 // row) -> this kernel: 400,000 x 96 floats, L = 100, one query 585 -> 142 us,
 // 10,000 queries 2.57 -> 0.89 ms; 400,000 x 128 uint8, L = 128, 10,000 queries
-// 2.11 -> 1.13 ms; 30,000 x 960 floats, L = 200, 1,000 queries 23.2 -> 4.6 ms (36
-// GB of rows).  Also measured: an unordered list with its minimum and maximum by
-// warp reductions (one query 216 us, 10,000 1.84 ms).  Eight CTAs per SM of
-// one-warp queries (64 registers) beat six and ten (0.89 against 0.98 and 1.09 ms
-// on the float rows).
+// 2.11 -> 1.13 ms; 30,000 x 960 floats, L = 200, 1,000 queries 23.2 -> 4.6 ms (by
+// the counters 37 GB from L2, 7.9 TB/s; the two before 4.1 and 7.3 GB).  Also
+// measured: an unordered list with its minimum and maximum by warp reductions (one
+// query 216 us, 10,000 1.84 ms).  Eight CTAs per SM of one-warp queries (64 registers)
+// beat six and ten (0.89 against 0.98 and 1.09 ms on the float rows).
 template <int DT, int S, int W>
 __global__ void __launch_bounds__(W == 1 ? kWarps * 32 : W * 32, W == 1 ? 8 : W == kTeam ? 3 : kSmallTeamCtas)
     search_reg_kernel(SearchArgs a) {
@@ -996,13 +1002,14 @@ __global__ void __launch_bounds__(W == 1 ? kWarps * 32 : W * 32, W == 1 ? 8 : W 
         const unsigned kth = list.key_at((L - 1) / S, (L - 1) % S);
         const float last = __uint_as_float(kth) * (1.0f + E2) + A2;
         auto enters = [&](int i) {
-          if (i >= nf || (DT == kF32 && M.ctl[2] < 0)) return false;
+          if (i >= nf || (W == 1 && DT == kF32 && M.ctl[2] < 0)) return false;
           if constexpr (DT == kU8) return M.ckey[i] <= kth;
           else return __uint_as_float(M.ckey[i]) <= last || kth == 0x7f800000u;
         };
 #pragma unroll 1
         for (int base = 0; base < nf; base += 32) {
           unsigned todo = __ballot_sync(full, enters(base + lane));
+          if (W > 1 && DT == kF32 && todo && M.ctl[2] < 0) break;
           while (todo) {
             const int at = base + __ffs(todo) - 1;
             todo &= todo - 1;
@@ -1065,9 +1072,11 @@ __global__ void recall_kernel(const int32_t* __restrict__ found, int ld_found, c
 // The CTAs per SM a configured plan may ask for.
 constexpr int kMaxCtasPerSmCap = 16;
 constexpr int kMinCacheBits = 8, kMaxCacheBits = 12;
-// The default plan stops at 512 entries: a larger cache takes shared memory
-// that L1 would otherwise give to the neighbour rows and vectors, and measured
-// slower on 1M x 128 uint8 at L = 128 (1,024 entries 6% slower, 4,096 50%).
+// The default plan stops at 1,024 entries for one warp per query, whose caches
+// share an SM with 31 others, and at the most for a team (L = 100 to 256, one pass of
+// 512 / 1,024 / the default, in ms: 10,000 queries on 400,000 x 128 uint8 1.19 / 1.14 /
+// 1.13, on 400,000 x 96 floats 1.04 / 0.93 / 0.93; by teams, 1,000 on 30,000 x 960
+// floats 5.67 / 5.42 / 4.69, 333 on 200,000 x 128 uint8 0.57 / 0.52 / 0.45).
 constexpr int kDefaultMaxCacheBits = 10;
 
 using SearchKernel = void (*)(SearchArgs);
@@ -1108,8 +1117,9 @@ cudaError_t prepare_kernels() {
 
 // Default plan: the queries in flight hide the latency of each expansion, so
 // the search first maximises the CTAs per SM, then takes the largest id cache
-// (256 or 512 entries per query) that keeps that many.  Plans are remembered
-// per (kernel, L, row bytes); the occupancy queries run once for each.
+// (256 to 1,024 entries per query, a team's up to 4,096) that keeps that many.
+// Plans are remembered per (kernel, L, row bytes); the occupancy queries run once for
+// each.
 struct SearchPlan {
   int bits = kMinCacheBits;
   int ctas = 1;
@@ -1195,8 +1205,8 @@ cudaError_t launch_search(const SearchLaunch& L, cudaStream_t s, int* kernels) {
   // Few queries: a team per query.  400,000 x 96 floats, one warp / team of
   // three / team of five, in us: 152 queries 198 / 178 / 181, 456: 292 / 256 /
   // 241, 800: 370 / 321 / 450, 1,216: 382 / 342 / 624, 1,824: 399 / 495 / 858;
-  // 128-byte uint8 rows alike.  The lines lie where a team's CTAs (3 and 7 per
-  // SM) no longer hold all queries at once.
+  // 128-byte uint8 rows alike.  The lines lie at 3 and 8 queries per SM: a team's
+  // CTAs (3 and 7 per SM) then hold all or nearly all of them at once.
   const int warps = !F.reg ? 0
                     : L.nq <= int64_t(L.num_sms) * kTeamQueriesPerSm      ? kTeam
                     : L.nq <= int64_t(L.num_sms) * kSmallTeamQueriesPerSm ? kSmallTeam
