@@ -78,8 +78,8 @@ __device__ __forceinline__ void acc_pair(uint2 x, uint2 y, unsigned& acc) {
 // Runs of single-precision keys in b[0, m) (sorted ascending) whose intervals
 // overlap are re-ordered by (binary64 distance, id); lane 0 alone, runs are
 // rare.  Returns the end of the run holding position k - 1 (or -1).
-__device__ int fix_near_ties(const uint8_t* Xb, int64_t row_bytes, int d, DevStatus* status,
-                             unsigned long long* b, int m, const float* qv, int64_t qg, int k = 0) {
+__device__ __forceinline__ int fix_near_ties(const uint8_t* Xb, int64_t row_bytes, int d, DevStatus* status,
+                                             unsigned long long* b, int m, const float* qv, int64_t qg, int k = 0) {
   const float E = slice_rel_bound(d), Eabs = abs_bound(d);
   const float* X = reinterpret_cast<const float*>(Xb);
   const int64_t stride = row_bytes / 4;
@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(kThreads) knn_kernel(KnnArgs a) {
 // What bounds the scan: the threads' 64 columns a step, read, tested and now and
 // then stored, about 2,400 of a step's 4,000 cycles (its products: 1,150 at d = 96),
 // and the cuts, which hold the other warps up through the accumulators.  10,000
-// queries x 400,000 points x 96 dims, k 100: 3.7 ms, of which the ranking 0.34; one
+// queries x 400,000 points x 96 dims, k 100: 3.6 ms, of which the ranking 0.34; one
 // CTA per query tile, a lane per query row and the tile's loads, products and cuts
 // in turn took 47.6 (79 CTAs of 152, the tensor cores idle through every cut).  With
 // the exact k-th in a cut, its entries read twice, and a vote per eight columns it
@@ -517,6 +517,40 @@ __device__ __forceinline__ unsigned kth_key(const unsigned (&u)[PER], int m, int
   return hi;
 }
 
+// The cut of a part by every entry's own bound: tau = the k-th smallest d2~ + err of
+// the m entries (the first n0 from the start of e, the rest `gap` places on), those
+// with d2~ - err above it dropped and the others moved to the start; returns how many.
+// Out of line, since it is rare and a small call's scan runs cold (inlined, 4 us more).
+// One warp.
+__device__ __noinline__ int cut_own(const KnnTcArgs& a, uint2* e, int m, int k, float nq, int n0, int gap, float& tau) {
+  const int lane = threadIdx.x & 31;
+  const float sq = sqrtf(nq);
+  auto err = [&](uint2 v) { return own_err(a, nq, sq, v.y); };
+  unsigned u[kTcCand / 32];
+#pragma unroll
+  for (int i = 0; i < kTcCand / 32; ++i) {
+    u[i] = 0xffffffffu;
+    if (32 * i + lane < m) {
+      const uint2 v = e[entry_at(32 * i + lane, n0, gap)];
+      u[i] = fkey(__uint_as_float(v.x) + err(v));
+    }
+  }
+  tau = fkey_inv(kth_key<kTcCand / 32>(u, m, k, 0));
+  int kept = 0;
+  for (int i0 = 0; i0 < m; i0 += 32) {
+    const int i = i0 + lane;
+    uint2 v = make_uint2(0, 0);
+    if (i < m) v = e[entry_at(i, n0, gap)];  // never before the place it may be moved to
+    const bool keep = i < m && __uint_as_float(v.x) - err(v) <= tau;
+    const unsigned km = __ballot_sync(0xffffffffu, keep);
+    __syncwarp();
+    if (keep) e[kept + __popc(km & ((1u << lane) - 1))] = v;
+    kept += __popc(km);
+    __syncwarp();
+  }
+  return kept;
+}
+
 // A part's m >= k candidates (`n0` of them at the buffer's start, the rest up to its
 // end), PER per lane, read once: tau = an upper bound of the k-th smallest d2~, plus
 // w; the entries whose lower bound lies above it are dropped and the rest moved to
@@ -539,30 +573,18 @@ __device__ __forceinline__ int cut_part(const KnnTcArgs& a, uint2* e, int m, flo
     id[i] = v.y;
   }
   tau = fkey_inv(kth_key<PER>(u, m, k, REDO ? 0 : kCutSlack)) + w;
-  unsigned drop = 0;  // bit i: entry 32 i + lane goes
   if (DT == kF32 && (REDO || w > kNarrow * tau)) {
     int c = 0;
 #pragma unroll
     for (int i = 0; i < PER; ++i) c += 32 * i + lane < m && fkey_inv(u[i]) - w <= tau;
-    if (__reduce_add_sync(0xffffffffu, c) > k + kOwnSlack) {
-      const float sq = sqrtf(nq);
-      unsigned ub[PER];
-#pragma unroll
-      for (int i = 0; i < PER; ++i)
-        ub[i] = 32 * i + lane < m ? fkey(fkey_inv(u[i]) + own_err(a, nq, sq, id[i])) : 0xffffffffu;
-      tau = fkey_inv(kth_key<PER>(ub, m, k, 0));
-#pragma unroll
-      for (int i = 0; i < PER; ++i)
-        if (32 * i + lane < m && !(fkey_inv(u[i]) - own_err(a, nq, sq, id[i]) <= tau)) drop |= 1u << i;
-      w = __int_as_float(0x7f800000);  // the test below keeps the rest
-    }
+    if (__reduce_add_sync(0xffffffffu, c) > k + kOwnSlack) return cut_own(a, e, m, k, nq, n0, gap, tau);
   }
   int kept = 0;
   __syncwarp();  // every entry has been read
 #pragma unroll
   for (int i = 0; i < PER; ++i) {
     const float x = fkey_inv(u[i]);
-    const bool keep = 32 * i + lane < m && x - w <= tau && !((drop >> i) & 1u);
+    const bool keep = 32 * i + lane < m && x - w <= tau;
     const unsigned km = __ballot_sync(0xffffffffu, keep);
     if (keep) e[kept + __popc(km & ((1u << lane) - 1))] = make_uint2(__float_as_uint(x), id[i]);
     kept += __popc(km);
@@ -878,12 +900,11 @@ __device__ __forceinline__ void rank_query(const KnnTcArgs& a, int64_t ql, uint2
   const int t = int(ql % kTcQ);
   const float inf = __int_as_float(0x7f800000);
   float tau = fminf(inf, fkey_inv(__ldcg(a.tauq + ql)));  // never lowered: all ones, not a number
-  float w = 0.f, nqq = 0.f, sq = 0.f;
+  float w = 0.f, nqq = 0.f;
   if (!a.exact) {
     nqq = a.qnorm[qg];
-    sq = sqrtf(nqq);
     const float2 tm = *a.tmax;
-    w = cut_width(tc_err(a, nqq, sq, tm.x, tm.y), nqq + tm.x);
+    w = cut_width(tc_err(a, nqq, sqrtf(nqq), tm.x, tm.y), nqq + tm.x);
   }
   // ---- the candidates of the query's parts, cut to the smallest tau
   int m = 0;
@@ -896,6 +917,7 @@ __device__ __forceinline__ void rank_query(const KnnTcArgs& a, int64_t ql, uint2
     m = cut_above(e, m, tau, [&](uint2 v) { return __uint_as_float(v.x) - w; });
     if constexpr (DT == kF32) {
       if (!REDO && m <= a.k + kOwnSlack) return;
+      const float sq = sqrtf(nqq);
       const float own = fkey_inv(kth_of<kRankCand / 32>(
           e, m, a.k, [&](uint2 v) { return __uint_as_float(v.x) + own_err(a, nqq, sq, v.y); }));
       tau = fminf(tau, own);
@@ -986,8 +1008,15 @@ __device__ __forceinline__ void rank_query(const KnnTcArgs& a, int64_t ql, uint2
   warp_sort(keys, m);
   const int nc = min(m, a.k);
   if constexpr (DT == kF32) {
-    if (lane == 0) fix_near_ties(a.X, a.row_bytes, a.d, a.status, keys, m, reinterpret_cast<const float*>(qrow), qg);
-    __syncwarp();
+    // near-tie runs are rare: one lane walks the list only if there is any
+    const float E = slice_rel_bound(a.d), Eabs = abs_bound(a.d);
+    bool near = false;
+    for (int i = lane; i + 1 < m; i += 32)
+      near |= !sure_less(__uint_as_float(unsigned(keys[i] >> 32)), __uint_as_float(unsigned(keys[i + 1] >> 32)), E, Eabs);
+    if (__any_sync(0xffffffffu, near)) {
+      if (lane == 0) fix_near_ties(a.X, a.row_bytes, a.d, a.status, keys, m, reinterpret_cast<const float*>(qrow), qg);
+      __syncwarp();
+    }
   }
   for (int j = lane; j < a.k; j += 32) {
     const bool have = j < nc;
