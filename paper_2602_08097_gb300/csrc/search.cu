@@ -57,14 +57,17 @@ constexpr unsigned kVisited = 0x80000000u;
 constexpr unsigned kIdMask = 0x7fffffffu;
 // A float query's close decisions in search_reg_kernel are made one at a time by the
 // whole warp, which is dear where distances tie all the time (rows of zeros and ones,
-// rows many times over).  A query that has made more than kFineBudget of them, or met
-// one that binary64 has to settle, leaves kSearchRedo as its first id and is searched
-// again by search_list_kernel, which keeps such distances and settles 32 at a time.
-// The benchmark's shapes make 0.2 (400,000 x 96, L = 100) to 20 a query (30,000 x 960,
-// L = 200), and none of their queries is given up.  20,000 x 96 zeros and ones, L =
-// 100, 5,000 queries: every decision made here 2,963 ms, with the budget 55, by the
-// list kernel alone 55.
+// rows many times over).  A query that has spent more than kFineBudget on them leaves
+// kSearchRedo as its first id and is searched again by search_list_kernel, which keeps
+// such distances and settles 32 at a time.  The benchmark's shapes make 0.2 (400,000 x
+// 96, L = 100) to 20 a query (30,000 x 960, L = 200; no query above 47).  20,000 x 96
+// zeros and ones, L = 100, 5,000 queries: every decision made here 2,963 ms, with the
+// budget 55, by the list kernel alone 55.
+// One that binary64 has to settle takes two sums in index order, by a lane each, and
+// costs kFineF64.  30,000 x 960 rows give one to a query in 2,200; were that query
+// given up, its call of 1,000 would take 9 to 18 ms where it takes 4.7.
 constexpr int kFineBudget = 128;
+constexpr int kFineF64 = 32;
 
 struct SearchArgs {
   const uint8_t* X;
@@ -617,7 +620,7 @@ struct RegSmem {
   uint8_t* q;
   unsigned* cid;   // [kNbr] new ids
   unsigned* ckey;  // [kNbr] their distances
-  int* ctl;        // team form: rows to read (-1: the query is done); [1] the query; [2] what is left of kFineBudget
+  int* ctl;        // team form: rows to read (-1: the query is done); [1] the query; [2] what is left of kFineBudget, [3] binary64 decisions
 };
 
 __host__ __device__ inline size_t reg_bytes(int64_t row_bytes, int cache_bits) {
@@ -639,10 +642,11 @@ __device__ inline RegSmem reg_carve(unsigned char* p, int64_t row_bytes, int cac
 
 // Whether point `m` precedes point `c` in (distance, id) order, where their
 // single-precision intervals overlap: by float-float distances, by id where those are
-// exact or the rows the same.  Where binary64 would have to decide, the query is given
-// up.  Called by a whole warp; out of line, since it is rare.  q lies in a RegSmem,
-// whose ctl[2] is what the query may still spend: once that is negative, any answer
-// does and rows of no dimensions are compared.
+// exact or the rows the same, else by the canonical binary64 ones.  Called by a whole
+// warp; out of line, since it is rare.  q lies in a RegSmem, whose ctl[2] is what the
+// query may still spend: once that is negative, any answer does and rows of no
+// dimensions are compared.  ctl[3] counts the binary64 decisions.  Where one is no
+// number, so are most that follow: that costs the whole budget.
 __device__ __noinline__ bool precedes_fine(const uint8_t* Xb, int64_t row_bytes, int d, const float* q, unsigned m,
                                            unsigned c) {
   int* left = reinterpret_cast<int*>(const_cast<uint8_t*>(reinterpret_cast<const uint8_t*>(q)) + row_bytes) +
@@ -664,8 +668,23 @@ __device__ __noinline__ bool precedes_fine(const uint8_t* Xb, int64_t row_bytes,
   int o = slot_order(-dm, -dc, ff_bound(d));
   if (em && ec) o = dm < dc || (dm == dc && m < c);
   if (same) o = m < c;
-  __syncwarp();
-  if ((threadIdx.x & 31) == 0) *left = o < 0 ? -1 : *left - 1;
+  const bool f64 = o < 0;
+  // lane 0 of m, lane 1 of c; no steps in the others, or if float-float decided
+  const float* x = reinterpret_cast<const float*>(Xb + int64_t((threadIdx.x & 31) ? c : m) * row_bytes);
+  const int steps = f64 && (threadIdx.x & 31) < 2 ? d : 0;
+  double v = 0.0;
+#pragma unroll 1
+  for (int i = 0; i < steps; ++i) {
+    const double t = __dsub_rn(double(q[i]), double(__ldg(x + i)));
+    v = __dadd_rn(v, __dmul_rn(t, t));
+  }
+  const double vm = __shfl_sync(0xffffffffu, v, 0), vc = __shfl_sync(0xffffffffu, v, 1);
+  if (f64) o = vm < vc || (vm == vc && m < c);
+  if ((threadIdx.x & 31) == 0) {
+    const bool finite = vm + vc < __longlong_as_double(0x7ff0000000000000LL);
+    *left -= !f64 ? 1 : finite ? kFineF64 : kFineBudget + 1;
+    left[1] += f64;
+  }
   __syncwarp();
   return o == 1;
 }
@@ -902,7 +921,7 @@ __global__ void __launch_bounds__(W == 1 ? kWarps * 32 : W * 32, W == 1 ? 8 : W 
     if (lane == 0) {
       M.cid[0] = start;
       M.cache[(start * 0x9E3779B1u) >> cshift] = start;
-      if (DT == kF32) M.ctl[2] = a.fine_budget;
+      if (DT == kF32) M.ctl[2] = a.fine_budget, M.ctl[3] = 0;
     }
     __syncwarp();
     row_keys<DT, 1>(a.X, a.row_bytes, M.q, M.cid, M.ckey, 1, 0, 1, qn);
@@ -1026,6 +1045,7 @@ __global__ void __launch_bounds__(W == 1 ? kWarps * 32 : W * 32, W == 1 ? 8 : W 
     if (a.visited_cnt && lane == 0) a.visited_cnt[qi] = int32_t(iters < INT32_MAX ? iters : INT32_MAX);
     // ---- the k closest members
     const bool redo = DT == kF32 && M.ctl[2] < 0;  // given up for search_list_kernel
+    if (DT == kF32 && lane == 0 && M.ctl[3] != 0) atomicAdd(&a.status->fp64_search, 2ull * unsigned(M.ctl[3]));
 #pragma unroll
     for (int j = 0; j < S; ++j) {
       const int i = lane * S + j;

@@ -75,6 +75,38 @@ def test_a_list_of_100_takes_no_longer_than_one_of_300(ctx, kind):
     rp.rp_graph_free(ctx, g)
 
 
+@pytest.mark.parametrize("all_rows", [False, True])
+@pytest.mark.parametrize("n,d,nq", [(1500, 96, 1), (1500, 96, 300), (1500, 96, 6000), (1500, 960, 300), (200, 20000, 1)])
+def test_sums_that_differ_in_their_order_alone(ctx, n, d, nq, all_rows):
+    """Queries of equal numbers and rows that permute each other: the distances are
+    equal but for the rounding of binary64 sums in index order.  A pair of such rows
+    takes no second launch."""
+    rng = np.random.default_rng(d)
+    X = rng.normal(size=(n, d)).astype(np.float32)
+    row_ptr, col = datagen.random_graph(n, 20, 60, seed=d)
+    u, v = col[row_ptr[3] : row_ptr[3] + 2]  # both met by every search
+    X[u] = 0.5 + 0.1 * X[u]
+    for i in range(n) if all_rows else [v]:
+        X[i] = rng.permutation(X[u])
+    Q = np.repeat(rng.uniform(0.4, 0.6, (nq, 1)), d, axis=1).astype(np.float32)
+    g = rp.rp_load_graph(ctx, X, row_ptr, col, start=3)
+    row_ptr, col = rp.rp_graph_export(ctx, g)
+    other = rng.normal(size=Q.shape).astype(np.float32)
+    count = [rp.rp_stats(ctx)]
+    for q in (other, Q):
+        ids, dists = rp.rp_search(ctx, g, q, 50, 10)
+        count.append(rp.rp_stats(ctx))
+    launches = [b["kernel_launches"] - a["kernel_launches"] for a, b in zip(count, count[1:])]
+    assert count[2]["fp64_search_dists"] - count[1]["fp64_search_dists"] >= 2 * nq
+    if not all_rows:
+        assert launches[1] == launches[0]
+    sel = np.arange(0, nq, max(1, nq // 60))
+    ref, refd, _ = oracle.greedy_search(X, row_ptr, col, 3, np.ascontiguousarray(Q[sel]), 50, 10)
+    assert np.array_equal(ids[sel], ref)
+    np.testing.assert_allclose(dists[sel], refd, rtol=2e-5)
+    rp.rp_graph_free(ctx, g)
+
+
 def test_a_vamana_build_over_ties_matches_the_oracle(ctx):
     X, _ = _data("bits", 600, 1, 24)
     g = rp.rp_load_graph(ctx, X)
