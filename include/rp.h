@@ -504,10 +504,12 @@ rp_status rp_set_knn_method(rp_ctx *ctx, int32_t method);
  * The paper fixes none; results never depend on it.
  *   cache_bits: 8..12, a direct-mapped cache of 2^cache_bits recently met
  *     ids per query in shared memory (a miss only costs one more distance);
- *     0 = 256 or 512 entries, the larger if it keeps the most CTAs (of 4
- *     queries each) resident per SM that registers and shared memory allow.
+ *     0 = 256 to 1,024 entries (few queries: up to 4,096), the most that keep
+ *     as many CTAs resident per SM as registers and shared memory allow.
  *   ctas_per_sm: at most this many CTAs per SM (0 = as many as one SM
- *     holds with the chosen cache, up to 16).
+ *     holds with the chosen cache, up to 16).  A CTA holds four queries, or
+ *     one that several warps share where L <= 256 and there are at most 8
+ *     queries per SM.
  * Errors: RP_EINVAL.
  */
 rp_status rp_set_search_config(rp_ctx *ctx, int32_t cache_bits, int32_t ctas_per_sm);

@@ -76,8 +76,11 @@ __device__ __forceinline__ bool canon_dominates(double A2, double d2a, double d2
 __device__ __forceinline__ float rel_bound(int d) { return (float)(d + 8) * 5.9604645e-08f; }
 // The same for a difference-form squared distance summed per 32-dimension
 // slice (index order within a slice, then the slice sums in order):
-// (min(d, 32) + ceil(d / 32) + 8) ulps.  Every single-precision distance of
-// the float paths is summed this way.
+// (min(d, 32) + ceil(d / 32) + 8) ulps.  Sums in other orders that stay below that
+// many roundings share the bound: the float prune's gather (a slice by four lanes,
+// at most 16 + 1 + 2) and its rechecks (a row by a warp, d / 32 + 3 and five
+// joins).  The search's sums have a bound of their own (lane_rel_bound), the
+// general prune's rel_bound.
 __device__ __forceinline__ float slice_rel_bound(int d) {
   return float((d < 32 ? d : 32) + (d + 31) / 32 + 8) * 5.9604645e-08f;
 }
